@@ -73,7 +73,9 @@ struct mlb_handle {
     void *sval32 = nullptr, *Q32 = nullptr, *F32 = nullptr, *G32 = nullptr, *W32 = nullptr;
     void *x32 = nullptr, *r32 = nullptr, *z32 = nullptr, *b32 = nullptr;
     void *xbest = nullptr;   // refined mode: best FP64 solution so far
-    double *partials = nullptr;
+    // the single solve's exchange: [BarrierState, padded to 256 bytes][slots],
+    // zeroed before every launch
+    Slot *slots = nullptr;
     BarrierState *bar = nullptr;
     DevResult *dres = nullptr;
     double *err_hist = nullptr;
@@ -821,8 +823,8 @@ int create_impl(mlb_handle *h, const mlb_matrix *A, const mlb_matrix *AH, const 
     h->grid = std::max(grid, 1);
     h->grid_max = std::max(maxg, 1);
     h->grid_want = (int)std::max<int64_t>(1, std::min<int64_t>(want, maxg));
-    if ((rc = dev_alloc_t(h, &h->partials, (size_t)2 * maxg * kMaxSums * 8))) return rc;
-    if ((rc = dev_alloc_t(h, &h->bar, sizeof(BarrierState)))) return rc;
+    if ((rc = dev_alloc_t(h, &h->bar, 256 + (size_t)2 * kMaxSums * maxg * sizeof(Slot)))) return rc;
+    h->slots = (Slot *)((char *)h->bar + 256);
     if ((rc = dev_alloc_t(h, &h->dres, sizeof(DevResult)))) return rc;
     if ((rc = dev_alloc_t(h, &h->qd_partials, (size_t)h->grid_max * kQdMaxN * 2 * 8))) return rc;
     if ((rc = dev_alloc_t(h, &h->qd_out, (size_t)(kQdMaxN * 2 + 1) * 8))) return rc;
@@ -1003,7 +1005,7 @@ int mlbicgstab_solve(mlb_handle *h, const void *b, void *x, int32_t on_device, d
     }
     if (int rcs = stage_in(h, b, x, on_device, st)) return rcs;
     if (int rcm = map_solution(h, false)) return rcm;   // y_0 = M x_0
-    MLB_CUDA(cudaMemsetAsync(h->bar, 0, sizeof(BarrierState), st));
+    MLB_CUDA(cudaMemsetAsync(h->bar, 0, 256 + (h->grid > 1 ? (size_t)2 * kMaxSums * h->grid * sizeof(Slot) : 0), st));
     SolveCtl ctl;
     ctl.tol = tol;
     ctl.maxit = maxit;
@@ -1011,7 +1013,7 @@ int mlbicgstab_solve(mlb_handle *h, const void *b, void *x, int32_t on_device, d
     ctl.max_outer = h->max_outer;
     ctl.err_hist = err_hist ? h->err_hist : nullptr;
     ctl.hist_cap = err_hist ? hist_cap : 0;
-    ctl.partials = h->partials;
+    ctl.slots = h->slots;
     ctl.bar = h->bar;
     ctl.res = h->dres;
     ctl.timeout_ns = h->timeout_ns;
@@ -1147,7 +1149,7 @@ int mlbicgstab_solve_batch(mlb_handle *const *hs, int32_t count, const void *con
     const std::vector<int> big(porder.begin(), porder.begin() + nbig), small(porder.begin() + nbig, porder.end());
     // workspace: [queue (256 B)] [order_big] [order_small] [team barriers]
     // [team slots] [solve barriers] [results] (copied from the host:
-    // zeroes, results marked as not run) [items] [team partial sums]
+    // zeroes, results marked as not run) [items] [team slots, zeroed]
     auto up256 = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t off_big = 256;
     const size_t off_small = off_big + up256(big.size() * 4 + 4);
@@ -1156,8 +1158,9 @@ int mlbicgstab_solve_batch(mlb_handle *const *hs, int32_t count, const void *con
     const size_t off_sbar = off_titem + up256((size_t)teams * 8 + 8);
     const size_t off_res = off_sbar + up256(big.size() * sizeof(BarrierState) + 16);
     const size_t off_items = off_res + up256((size_t)count * sizeof(DevResult));
-    const size_t off_spart = off_items + up256((size_t)count * item_bytes);
-    const size_t need = off_spart + big.size() * 2 * kMaxSums * (size_t)team * sizeof(double) + 256;
+    const size_t off_slots = off_items + up256((size_t)count * item_bytes);
+    const size_t slot_bytes = big.size() * 2 * kMaxSums * (size_t)team * sizeof(Slot);
+    const size_t need = off_slots + slot_bytes + 256;
     if (need > h0->bws_bytes) {
         if (h0->bws) cudaFree(h0->bws);
         h0->bws = nullptr;
@@ -1237,13 +1240,14 @@ int mlbicgstab_solve_batch(mlb_handle *const *hs, int32_t count, const void *con
     plan.tbar = (BarrierState *)(dws + off_tbar);
     plan.team_item = (int *)(dws + off_titem);
     plan.sbar = (BarrierState *)(dws + off_sbar);
-    plan.spart = (double *)(dws + off_spart);
+    plan.sslots = (Slot *)(dws + off_slots);
     plan.timeout_ns = max_timeout;
     for (int s = 0; s < count; ++s) {
         if (int rcs = stage_in(hs[s], b[s], x[s], on_device, st)) return rcs;
         if (int rcm = map_solution(hs[s], false, st)) return rcm;
     }
-    MLB_CUDA(cudaMemcpyAsync(dws, hws, off_spart, cudaMemcpyHostToDevice, st));
+    MLB_CUDA(cudaMemcpyAsync(dws, hws, off_slots, cudaMemcpyHostToDevice, st));
+    if (slot_bytes) MLB_CUDA(cudaMemsetAsync(dws + off_slots, 0, slot_bytes, st));
     bool any_ilu = false;
     for (int q = 0; q < count; ++q) any_ilu = any_ilu || has_ilu(hs[q]);
     const void *ditems = dws + off_items;
@@ -1770,9 +1774,11 @@ int mlbicgstab_selftest_barrier_timeout(int32_t grid, int64_t timeout_ns) {
         return MLB_ERR_CUDA;
     }
     BarrierState *bs = nullptr;
-    MLB_CUDA(cudaMalloc(&bs, sizeof(BarrierState)));
-    cudaError_t e = cudaMemset(bs, 0, sizeof(BarrierState));
-    if (e == cudaSuccess) e = launch_barrier_selftest(grid, bs, (uint64_t)timeout_ns, nullptr);
+    const size_t bytes = 256 + (size_t)(grid + 1) * sizeof(Slot);
+    MLB_CUDA(cudaMalloc(&bs, bytes));
+    cudaError_t e = cudaMemset(bs, 0, bytes);
+    if (e == cudaSuccess)
+        e = launch_barrier_selftest(grid, bs, (Slot *)((char *)bs + 256), (uint64_t)timeout_ns, nullptr);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     BarrierState hb;
     memset(&hb, 0, sizeof(hb));

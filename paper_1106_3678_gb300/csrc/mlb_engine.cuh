@@ -5,11 +5,18 @@
 // Every step of the method is a "pass" over the rows: a streaming update of
 // a few N-vectors fused with the inner product(s) the next step needs, or a
 // SELL-32 SpMV fused with its inner products.  Each pass ends in a
-// deterministic reduction: per-CTA partial sums, a grid barrier, then every
-// CTA sums the partials in the same fixed order.  All scalars (alpha,
-// beta~, beta, omega, c, e, err) are therefore bit-identical in every CTA,
-// and every CTA takes the same branches (convergence, breakdown, g_n/r_n
-// bookkeeping) without any host round trip.
+// deterministic reduction over the team (GridSync::reduce).  All scalars
+// (alpha, beta~, beta, omega, c, e, err) are therefore bit-identical in
+// every CTA, and every CTA takes the same branches (convergence, breakdown,
+// g_n/r_n bookkeeping) without any host round trip.
+//
+// The iteration is an interpreter: the sequence of passes depends on n
+// alone (Step), each pass is one case of one switch, and everything that
+// lives from one pass to the next is in shared memory (Scalars, c, bt).  So
+// a pass has the registers to itself (inlined into nested loops, the
+// passes' values crowded each other out into local memory, which misses
+// the small L1 beside the tile ring), and the producer warp follows the
+// same sequence on its own, one pass ahead of the sums.
 //
 // Work distribution: every CTA of the team owns a contiguous, balanced range
 // of 32-row slices (and the matching rows of every vector).  Every pass
@@ -47,8 +54,13 @@ namespace mlb {
 
 constexpr int kThreads = kTileThreads;   // 15 consumer warps + 1 producer warp
 constexpr int kMaxN = 64;       // largest number of shadow vectors
-constexpr int kMaxSums = 8;     // doubles reduced per pass (max)
-constexpr int kRedDoubles = kMaxSums * (kThreads / 2 + 1);   // shared reduction scratch
+constexpr int kMaxSums = 5;     // doubles reduced per pass (max)
+// Shared scratch of a team's reductions.
+struct RedScratch {
+    double part[kMaxSums][kConsumers / 2];
+    double total[kMaxSums];
+    int fail;
+};
 
 // Result record written by CTA 0 at the end of a solve.
 struct DevResult {
@@ -62,22 +74,38 @@ struct DevResult {
 
 enum { OP_MATVEC = 0, OP_DOT = 1, OP_SAXPY = 2, OP_SCALE = 3, OP_NORM = 4 };
 
-// Per-CTA accounting in shared memory (identical in every CTA).
+// Per-CTA accounting in shared memory (identical in every CTA), kept by
+// consumer thread kAcctThread: integer adds, beside the threads that work
+// out the pass's scalars.
+constexpr int kAcctThread = 64;
 struct Acct {
     int64_t ops[5];   // Table 4.3 categories of the current inner call
     int64_t spmv;     // all sparse products of the solve
-    // Algorithmic bytes and floating-point operations of the solve, kept
-    // in integer arithmetic: thread 0 adds to them in every pass, on the
-    // pass's critical path, where FP64 adds would cost ~60 cycles each.
+    // Algorithmic bytes and floating-point operations of the solve.
     int64_t bytes;
     int64_t flops;
-    // Scalars evaluated by thread 0 and read by every thread after a
-    // __syncthreads: FP64 division and square root are costly on this GPU,
-    // so they are not repeated by all threads.  Calls rotate through the
-    // slots, so a slot is rewritten only after three more __syncthreads,
-    // which every reader of its previous value has already passed.
-    double d[4];
-    cdouble z[4];
+};
+
+// Scalars of the iteration, in shared memory.  After a pass's reduction
+// consumer thread 0 works out the coefficient of the next pass (one FP64
+// division, ~0.3 us on this GPU) while thread kErrThread takes the residual
+// norm's decisions; the other threads only read `coef` and `exit`, so no
+// FP64 instruction of 480 threads sits between two passes.
+constexpr int kErrThread = 32;
+template <typename S>
+struct Scalars {
+    S coef;          // coefficient of the next pass
+    S e;             // q_{i+1}^H r
+    S omega, inv_omega;
+    double bnrm2;    // ||b|| (1 when b = 0)
+    double rr;       // ||r||^2 (or ||u||^2) of the last update
+    double far;      // a ||r||^2 above this is certainly not below tol
+    double err;      // ||r|| / ||b|| where it was worked out
+    int64_t iter;
+    int exit;        // the iteration ends
+    int flag, j, i;  // its result
+    int act;         // (refined mode) replace the residual
+    int conv;        // (refined mode) the true residual met its tolerance
 };
 
 // ILU(0) preconditioner M = L U of Algorithm 7.1 (the preconditioner of
@@ -134,7 +162,7 @@ struct SolveCtl {
     int max_outer;
     double *err_hist;           // device, may be null
     int64_t hist_cap;
-    double *partials;           // [2][kMaxSums][gridDim]
+    Slot *slots;                // [2][kMaxSums][gridDim], zeroed before the launch
     BarrierState *bar;
     DevResult *res;
     uint64_t timeout_ns;
@@ -304,12 +332,13 @@ __device__ __noinline__ T sell_slice_sum_wide(const int32_t *cp, const T *vp, in
 // widths then count blocks.  Slices up to PW entries wide take the
 // pipelined path (PW registers of gathered x per thread), wider ones a
 // direct loop.  Returns false when a tile wait timed out.
+//
+// sell_consume is the consumer warps' part.
 template <int NE, int EW = 1, int PW = 8, typename T, typename Fin, typename AccArr>
-__device__ __forceinline__ bool sell_spmv(TileRing *R, unsigned &pseq, unsigned &cseq, uint64_t timeout_ns,
-                                          int64_t s_lo, int64_t s_hi, int spt, const int64_t *slice_ptr,
-                                          const int32_t *scol, const T *sval, const T *xin,
-                                          const T *const (&epi)[NE > 0 ? NE : 1], int lane, Fin fin,
-                                          AccArr &acc) {
+__device__ __forceinline__ bool sell_consume(TileRing *R, unsigned &cseq, uint64_t timeout_ns, int64_t s_lo,
+                                             int64_t s_hi, int spt, const int64_t *slice_ptr, const int32_t *scol,
+                                             const T *sval, const T *xin, const T *const (&epi)[NE > 0 ? NE : 1],
+                                             int lane, Fin fin, AccArr &acc) {
     static_assert(EW == 1 || EW == 3, "scalar entries or 3x3 blocks");
     constexpr int kPipeW = PW;
     constexpr int NEA = NE > 0 ? NE : 1;
@@ -318,32 +347,20 @@ __device__ __forceinline__ bool sell_spmv(TileRing *R, unsigned &pseq, unsigned 
     bool ok = true;
     if (spt <= 0) {
         // slices too wide for one stage: direct loads, no pipeline
-        if (cw < kConsumerWarps) {
-            for (int64_t s = s_lo + cw; s < s_hi; s += kConsumerWarps) {
-                const int64_t o = off(s);
-                const int w = (int)((off(s + 1) - o) >> 5);
-                const int64_t row = s * 32 + lane;
-                T e[NEA];
+        for (int64_t s = s_lo + cw; s < s_hi; s += kConsumerWarps) {
+            const int64_t o = off(s);
+            const int w = (int)((off(s + 1) - o) >> 5);
+            const int64_t row = s * 32 + lane;
+            T e[NEA];
 #pragma unroll
-                for (int i = 0; i < NE; ++i) e[i] = epi[i][row];
-                if constexpr (EW == 3)
-                    fin(row, sell_slice_sum3(scol + o + lane, sval + 3 * (o + lane), w, xin), e, acc);
-                else
-                    fin(row, sell_slice_sum(scol + o + lane, sval + o + lane, w, xin), e, acc);
-            }
+            for (int i = 0; i < NE; ++i) e[i] = epi[i][row];
+            if constexpr (EW == 3)
+                fin(row, sell_slice_sum3(scol + o + lane, sval + 3 * (o + lane), w, xin), e, acc);
+            else
+                fin(row, sell_slice_sum(scol + o + lane, sval + o + lane, w, xin), e, acc);
         }
         fence_proxy_async_global();
         return true;
-    }
-    if (cw == kConsumerWarps) {
-        if (lane == 0) {
-            const void *ep[NEA];
-#pragma unroll
-            for (int i = 0; i < NE; ++i) ep[i] = epi[i];
-            ok = produce_sell(R, s_lo, s_hi, spt, off, sval, EW * (int)sizeof(T), (int)sizeof(T), scol, ep, NE, pseq,
-                              timeout_ns);
-        }
-        return ok;
     }
     // one slice of one tile, as seen by this warp: stage, entry offset of
     // the slice in the stage (o), entries of the tile (nv), slice width w
@@ -454,6 +471,27 @@ __device__ __forceinline__ bool sell_spmv(TileRing *R, unsigned &pseq, unsigned 
     return ok;
 }
 
+// Producer and consumers of one product in one call (the fused product's
+// kernel): pseq is the producer lane's tile counter, cseq a consumer's.
+template <int NE, int EW = 1, int PW = 8, typename T, typename Fin, typename AccArr>
+__device__ __forceinline__ bool sell_spmv(TileRing *R, unsigned &pseq, unsigned &cseq, uint64_t timeout_ns,
+                                          int64_t s_lo, int64_t s_hi, int spt, const int64_t *slice_ptr,
+                                          const int32_t *scol, const T *sval, const T *xin,
+                                          const T *const (&epi)[NE > 0 ? NE : 1], int lane, Fin fin, AccArr &acc) {
+    constexpr int NEA = NE > 0 ? NE : 1;
+    if ((threadIdx.x >> 5) == kConsumerWarps) {
+        if (lane != 0 || spt <= 0) return true;
+        const SliceOffsets off(R, slice_ptr, s_lo, s_hi);
+        const void *ep[NEA];
+#pragma unroll
+        for (int i = 0; i < NE; ++i) ep[i] = epi[i];
+        return produce_sell(R, s_lo, s_hi, spt, off, sval, EW * (int)sizeof(T), (int)sizeof(T), scol, ep, NE, pseq,
+                            timeout_ns);
+    }
+    return sell_consume<NE, EW, PW>(R, cseq, timeout_ns, s_lo, s_hi, spt, slice_ptr, scol, sval, xin, epi, lane, fin,
+                                    acc);
+}
+
 // A 16-byte chunk of input i of a tile, from shared memory.
 template <typename T>
 __device__ __forceinline__ Pack<T> lds(const unsigned char *stage, int tc, int i, int k) {
@@ -473,155 +511,190 @@ __device__ __forceinline__ typename coef_of<T>::type mk_coef(const double *v) {
 // system: the whole grid (a single solve), a group of CTAs of a batch
 // launch (a large system of a batch), or the CTA alone (the other systems
 // of a batch).  Every CTA of a team passes the same sequence of
-// barriers and reductions, so `epoch` and the slots advance in lock step.
-// Several engines in one kernel share one GridSync.
+// barriers and reductions, so the epochs advance in lock step.
+// Several engines in one kernel share one GridSync.  Its members are called
+// by every consumer thread; the producer warp takes no part.
 //
 // The object lives in shared memory, one per CTA (thread-private copies
 // would sit in local memory, which the L1 left beside the tile ring cannot
-// hold for 512 threads, so every access would go to L2).  Writers: `epoch`
-// and `slot` thread 0; `ok` any thread (only ever set to false).  The tile
+// hold for 512 threads, so every access would go to L2).  Writers: the
+// epochs thread 0; `ok` any thread (only ever set to false).  The tile
 // sequence counters are per thread, in `seqs[threadIdx.x]` (the producer
-// lane counts issued tiles, a consumer thread consumed ones): one shared
+// warp counts issued tiles, a consumer thread consumed ones): one shared
 // counter would race, since in a pass of at most kStages tiles a fast warp
 // can finish the pass before a slow one has read where it starts.
 struct GridSync {
     unsigned nblocks;   // CTAs in the team
     unsigned bid;       // this CTA's rank in the team
     BarrierState *bar;
-    double *partials;   // [2][kMaxSums][gridDim]
-    double *red;        // shared, kRedDoubles
-    int *sflag;         // shared
+    Slot *slots;        // [2][kMaxSums][nblocks]: exchange e uses half e & 1
+    RedScratch *red;    // shared
     uint64_t timeout_ns;
-    unsigned epoch;
-    int slot;
+    unsigned epoch;     // exchanges this CTA has passed
+    unsigned bepoch;    // barriers (sync) this CTA has passed
     bool ok;            // false once a barrier or a tile wait failed
     TileRing *ring;     // shared-memory tile pipeline of this CTA
     unsigned *seqs;     // shared, kThreads per-thread tile counters
 
     __device__ __forceinline__ unsigned &seq() const { return seqs[threadIdx.x]; }
 
-    // Team = the whole grid.
-    __device__ GridSync(BarrierState *b, double *p, double *r, int *f, uint64_t to, TileRing *rg, unsigned *sq)
-        : nblocks(gridDim.x), bid(blockIdx.x), bar(b), partials(p), red(r), sflag(f), timeout_ns(to), epoch(0),
-          slot(0), ok(true), ring(rg), seqs(sq) {}
-    // Team = `nb` CTAs of a batch launch (rank `id`) with their own
-    // barrier state and partial sums ([2][kMaxSums][nb] doubles).
-    __device__ GridSync(BarrierState *b, double *p, unsigned nb, unsigned id, double *r, int *f, uint64_t to,
-                        TileRing *rg, unsigned *sq)
-        : nblocks(nb), bid(id), bar(b), partials(p), red(r), sflag(f), timeout_ns(to), epoch(0), slot(0), ok(true),
-          ring(rg), seqs(sq) {}
-    // Team = this CTA alone.
-    __device__ GridSync(double *r, int *f, uint64_t to, TileRing *rg, unsigned *sq)
-        : nblocks(1), bid(0), bar(nullptr), partials(nullptr), red(r), sflag(f), timeout_ns(to), epoch(0), slot(0),
-          ok(true), ring(rg), seqs(sq) {}
-
-    // Thread 0 arrives/waits; all threads of the CTA then proceed.  Returns
-    // false (uniformly) when the barrier failed.
-    __device__ __forceinline__ bool gbar() {
-        if (threadIdx.x == 0) *sflag = grid_arrive_wait(bar, epoch, nblocks, timeout_ns) ? 1 : 0;
-        __syncthreads();
-        if (*sflag == 0) { ok = false; return false; }
-        return true;
+    // Team of `nb` CTAs (rank `id`) with their own barrier state and slots;
+    // nb = 1: this CTA alone (b and p null).
+    __device__ GridSync(BarrierState *b, Slot *p, unsigned nb, unsigned id, RedScratch *r, uint64_t to, TileRing *rg,
+                        unsigned *sq)
+        : nblocks(nb), bid(id), bar(b), slots(p), red(r), timeout_ns(to), epoch(0), bepoch(0), ok(!rg->failed),
+          ring(rg), seqs(sq) {
+        r->fail = 0;
     }
 
-    // Sum K values over the team; every thread of every CTA receives the
-    // same bits.  A dependent FP64 add costs about 60 cycles on this GPU and
+    // Slots of sum k of the exchange `ep`.  Two halves suffice: a CTA
+    // puts exchange ep + 2 only after it has seen every slot of ep + 1,
+    // which a CTA puts after it has read every slot of ep.
+    __device__ __forceinline__ Slot *slot_of(unsigned ep, int k) const {
+        return slots + ((size_t)(ep & 1u) * kMaxSums + k) * nblocks;
+    }
+
+    // The last levels of reduce(), by one warp.  Out of line: its registers
+    // stay out of the passes.
+    __device__ __noinline__ void team_total(int k, bool fence) {
+        const int lane = threadIdx.x & 31;
+        const double *p = red->part[k] + lane;
+        double t = p[0] + p[32];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (nblocks > 1) {
+            const unsigned ep = epoch + 1;
+            Slot *const q = slot_of(ep, k);
+            if (lane == 0) {
+                if (fence) fence_acq_rel_gpu();   // this CTA's writes before its slot
+                slot_put(q + bid, t, ep);
+            }
+            const bool got = slots_sum(q, nblocks, ep, bar, timeout_ns, t);
+            if (fence) fence_acq_rel_gpu();       // the other CTAs' writes after their slots
+            if (!got && lane == 0) red->fail = 1;
+        }
+        if (lane == 0) red->total[k] = t;
+    }
+
+    // Sum K values over the team into red->total[0, K), the same bits in
+    // every CTA.  A dependent FP64 add costs about 60 cycles on this GPU and
     // one warp issues at most one FP64 instruction per ~60 cycles, so the
     // sums are short trees spread over many warps, independent sums
     // interleaved:
     //   CTA level 0: lanes l < 16 of every warp add their value to lane
-    //                l+16's (256 partials per sum);
+    //                l+16's (240 partials per sum);
     //   CTA level 1: task (k, g), g < 64, on its own thread, adds partials
     //                g, g+64, g+128, g+192 as a pair tree;
     //   CTA level 2: warp k adds the 64 level-1 results of sum k (lane l:
     //                l and l+32), then an xor tree over the lanes;
     //   team:        with several CTAs, warp k of every CTA adds the CTA
-    //                totals of sum k the same way (lane l: CTAs l, l+32, ...
-    //                as a pair tree, then the xor tree).
+    //                totals of sum k the same way, from their slots.
     // Fixed order for a given team size: deterministic.
+    // fence: what any CTA of the team wrote before is visible to all of them
+    // after (needed before a pass that gathers; the streaming passes read
+    // their own CTA's rows only).  False (uniformly) when a wait failed.
     template <int K>
-    __device__ __forceinline__ bool reduce(double (&v)[K]) {
-        static_assert(K <= kMaxSums && kThreads == 512, "reduction layout");
-        constexpr int P0 = kThreads / 2, G1 = P0 / 4;
+    __device__ __forceinline__ bool reduce(const double (&v)[K], bool fence) {
+        static_assert(K <= kMaxSums && kMaxSums <= kConsumerWarps && kConsumers == 480, "reduction layout");
+        constexpr int G1 = 64;
         const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-        double *sv = red;                     // K * P0 partials
-        double *bc = red + kMaxSums * P0;     // K totals
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const double h = v[k] + __shfl_down_sync(0xffffffffu, v[k], 16);
-            if (lane < 16) sv[k * P0 + warp * 16 + lane] = h;
+            if (lane < 16) red->part[k][warp * 16 + lane] = h;
         }
-        __syncthreads();
-        for (int task = tid; task < K * G1; task += kThreads) {
-            double *p = sv + (task / G1) * P0 + task % G1;
-            const double a0 = p[0], a1 = p[G1], a2 = p[2 * G1], a3 = p[3 * G1];
-            p[0] = (a0 + a1) + (a2 + a3);      // only this task reads slot 0
+        consumer_sync();
+        if (tid < K * G1) {
+            double *p = red->part[tid / G1] + tid % G1;
+            const double a0 = p[0], a1 = p[G1], a2 = p[2 * G1];
+            // the last group has 48 partials
+            p[0] = (a0 + a1) + (tid % G1 < 48 ? a2 + p[3 * G1] : a2);   // only this task reads slot 0
         }
-        __syncthreads();
-        if (warp < K) {
-            const double *p = sv + warp * P0 + lane;
-            double t = p[0] + p[32];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) bc[warp] = t;
-        }
-        __syncthreads();
-        if (nblocks == 1) {
-#pragma unroll
-            for (int k = 0; k < K; ++k) v[k] = bc[k];
-            return true;
-        }
-        const unsigned G = nblocks;
-        double *part = partials + (size_t)slot * kMaxSums * G;
-        if (tid == 0) {
-#pragma unroll
-            for (int k = 0; k < K; ++k) part[(size_t)k * G + bid] = bc[k];
-        }
-        if (!gbar()) return false;
-        if (tid == 0) slot ^= 1;   // every thread has read it (gbar synchronises)
-        if (warp < K) {
-            const double *p = part + (size_t)warp * G;
-            double t = 0.0;
-            for (unsigned b0 = 0; b0 < G; b0 += 256) {
-                double x[8];
-#pragma unroll
-                for (int m = 0; m < 8; ++m) {
-                    const unsigned b = b0 + lane + 32 * m;
-                    x[m] = b < G ? p[b] : 0.0;
-                }
-                const double s8 = ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
-                t = b0 == 0 ? s8 : t + s8;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) bc[warp] = t;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] = bc[k];
+        consumer_sync();
+        if (warp < K) team_total(warp, fence);
+        consumer_sync();
+        if (tid == 0) epoch += 1;   // read again only after another barrier
+        if (red->fail) { ok = false; return false; }
         return true;
     }
 
+    // Team barrier (a counter: cheaper than an exchange where no value goes
+    // with it).
     __device__ __forceinline__ bool sync() {
-        __syncthreads();
-        if (nblocks == 1) return true;
-        return gbar();
+        arrive();
+        return wait();
     }
 
     // sync() in two halves: arrive() once this CTA's writes are done,
     // wait() before reading other CTAs' writes; work between the two that
-    // reads nothing written in this step overlaps the wait.  Every thread
-    // calls both; wait() returns false (uniformly) when the barrier failed.
+    // reads nothing written in this step overlaps the wait.  wait() returns
+    // false (uniformly) when the barrier failed.
     __device__ __forceinline__ void arrive() {
-        __syncthreads();
-        if (nblocks > 1 && threadIdx.x == 0) grid_arrive(bar, epoch);
+        consumer_sync();
+        if (nblocks > 1 && threadIdx.x == 0) grid_arrive(bar, bepoch);
     }
     __device__ __forceinline__ bool wait() {
-        if (nblocks == 1) return true;   // arrive()'s __syncthreads ordered the CTA
-        if (threadIdx.x == 0) *sflag = grid_wait(bar, epoch, nblocks, timeout_ns) ? 1 : 0;
-        __syncthreads();
-        if (*sflag == 0) { ok = false; return false; }
+        if (nblocks == 1) return true;   // arrive()'s barrier ordered the CTA
+        if (threadIdx.x == 0 && !grid_wait(bar, bepoch, nblocks, timeout_ns)) red->fail = 1;
+        consumer_sync();
+        if (red->fail) { ok = false; return false; }
         return true;
+    }
+
+    // Hand a command to the producer warp (every consumer thread calls it).
+    __device__ __forceinline__ void post(int cmd) {
+        if (threadIdx.x == 0) {
+            ring->cmd = cmd;
+            ring->stop = 0;
+        }
+        __syncthreads();
+    }
+    // End of an iteration: stop the producer, meet it, and discard the tiles
+    // it has issued ahead (their stages are released as if consumed).
+    // `passes`: passes this CTA's consumers have finished.
+    __device__ __forceinline__ void end_inner(unsigned &sq, unsigned passes) {
+        if (threadIdx.x == 0) {
+            *(volatile int *)&ring->stop = 1;
+            ring->passes = passes;
+        }
+        __syncthreads();
+        for (const unsigned last = ring->issued; sq != last; ++sq) {
+            if (!mbar_wait(&ring->full[sq % kStages], (sq / kStages) & 1u, timeout_ns)) {
+                ring->failed = 1;
+                ok = false;
+                break;
+            }
+            __syncwarp();
+            if ((threadIdx.x & 31) == 0) mbar_arrive(&ring->empty[sq % kStages]);
+        }
+        consumer_sync();
+    }
+};
+
+// One pass of the iteration (Engine::inner) and the pass after it: a
+// function of n alone, which the producer warp follows too.  i: the slot the
+// step builds (ALPHA uses slot i - 1; i = n: the block's last update); s:
+// the column a sweep's pass uses; first: block 0.
+enum { P_SPMV_C, P_ALPHA, P_SPMV_Z, P_OMEGA, P_W_FIRST, P_W_ROUND, P_W_LAST, P_F_ROUND, P_G_J0 };
+struct Step {
+    int op = P_SPMV_C, i = 0, s = 0;
+    bool first = true;
+    __device__ __forceinline__ void advance(int n) {
+        switch (op) {
+        case P_SPMV_C: ++i; op = P_ALPHA; break;
+        case P_ALPHA: op = i == n ? P_SPMV_Z : first ? P_G_J0 : i == n - 1 ? P_W_LAST : P_W_FIRST; break;
+        case P_SPMV_Z: op = P_OMEGA; break;
+        case P_OMEGA:
+            i = 0;
+            first = false;
+            op = n == 1 ? P_W_LAST : P_W_FIRST;
+            break;
+        case P_W_FIRST: s = i + 1; op = s < n - 1 ? P_W_ROUND : P_W_LAST; break;
+        case P_W_ROUND: ++s; op = s < n - 1 ? P_W_ROUND : P_W_LAST; break;
+        case P_W_LAST: s = 0; op = i == 0 ? P_SPMV_C : P_F_ROUND; break;
+        case P_F_ROUND: ++s; op = s <= i - 1 ? P_F_ROUND : P_SPMV_C; break;
+        default: s = 1; op = i >= 2 ? P_F_ROUND : P_SPMV_C; break;   // P_G_J0
+        }
     }
 };
 
@@ -635,6 +708,9 @@ struct NoHook {
 // product passes' switch to M^{-1} of their input); without it none of
 // that code is reachable.  EW: the matrix storage of the products (1:
 // scalar SELL-32; 3: 3x3 blocks, see sell_slice_sum3).
+//
+// The consumer threads run inner() and the other members; the producer warp
+// runs serve() beside them.
 template <typename T, bool PC = false, int EW = 1>
 struct Engine {
     using S = typename coef_of<T>::type;                      // FP64 coefficient
@@ -649,14 +725,16 @@ struct Engine {
     // shared memory
     S *c;            // kMaxN
     S *bt;           // kMaxN
-    Acct *acct;      // accounting, kept by thread 0 (uniform in the grid)
+    Acct *acct;
+    Scalars<S> *sc;
     // ownership: slices [s_lo, s_hi), chunks [c_lo, c_hi)
     int64_t s_lo, s_hi, c_lo, c_hi;
 
     // Constructed by one thread in shared memory (one engine per CTA; see
     // GridSync); every thread then calls attach().
-    __device__ Engine(const SysView<T> &s, const SolveCtl &k, GridSync &g, S *c_, S *bt_, Acct *acct_)
-        : sys(s), ctl(k), gs(g), c(c_), bt(bt_), acct(acct_) {
+    __device__ Engine(const SysView<T> &s, const SolveCtl &k, GridSync &g, S *c_, S *bt_, Acct *acct_,
+                      Scalars<S> *sc_)
+        : sys(s), ctl(k), gs(g), c(c_), bt(bt_), acct(acct_), sc(sc_) {
         own_range(s.nslices, g.nblocks, g.bid, s_lo, s_hi);
         c_lo = s_lo * CPS;
         c_hi = s_hi * CPS;
@@ -668,7 +746,7 @@ struct Engine {
     // Complex values: a multiply-add is 8 real operations, |v|^2 4, a
     // scaling 6.
     __device__ __forceinline__ void op(int which, int cnt = 1) {
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == kAcctThread) {
             acct->ops[which] += cnt;
             constexpr bool cx_ = is_cx<T>::value;
             const int64_t N = sys.N;
@@ -681,161 +759,208 @@ struct Engine {
         }
     }
 
-    // Evaluate fn() in thread 0 only and give the value to every thread.
-    // Back-to-back calls use rotating slots; `bs` is the caller's counter
-    // (a register, the same sequence in every thread).
-    template <typename Fn>
-    __device__ __forceinline__ S once_s(unsigned &bs, Fn fn) {
-        const int k = bs++ & 3;
-        if constexpr (is_cx<T>::value) {
-            if (threadIdx.x == 0) acct->z[k] = fn();
-            __syncthreads();
-            return acct->z[k];
-        } else {
-            if (threadIdx.x == 0) acct->d[k] = fn();
-            __syncthreads();
-            return acct->d[k];
-        }
-    }
-    template <typename Fn>
-    __device__ __forceinline__ double once_d(unsigned &bs, Fn fn) {
-        const int k = bs++ & 3;
-        if (threadIdx.x == 0) acct->d[k] = fn();
-        __syncthreads();
-        return acct->d[k];
-    }
-
     __device__ __forceinline__ const T *Qc(int k) const { return sys.Q + (int64_t)k * sys.ld; }
     __device__ __forceinline__ const T *Fc(int k) const { return sys.F + (int64_t)k * sys.ld; }
     __device__ __forceinline__ T *Gc(int k) const { return sys.G + (int64_t)k * sys.ld; }
     __device__ __forceinline__ T *Wc(int k) const { return sys.W + (int64_t)k * sys.ld; }
 
     __device__ __forceinline__ void vbytes(int nvec) {
-        if (threadIdx.x == 0) acct->bytes += nvec * sys.N * (int64_t)sizeof(T);
+        if (threadIdx.x == kAcctThread) acct->bytes += nvec * sys.N * (int64_t)sizeof(T);
     }
     __device__ __forceinline__ void sbytes(int nextra) {
         // SpMV: entries (values, and a column index per stored entry of EW
         // values), row_ptr-equivalent, x read once, y written once, plus
         // `nextra` epilogue vectors.
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == kAcctThread) {
             acct->bytes += sys.nnz * (int64_t)sizeof(T) + sys.nnz / EW * 4 + 4 * (sys.N + 1) +
                            (2 + nextra) * sys.N * (int64_t)sizeof(T);
             acct->spmv++;
         }
     }
 
-    template <int K>
-    __device__ __forceinline__ bool reduce(double (&v)[K]) { return gs.template reduce<K>(v); }
-    __device__ __forceinline__ bool sync() { return gs.sync(); }
+    // ------------------------------------------------------------------
+    // the producer warp
+    // ------------------------------------------------------------------
 
-    // Inputs of a streaming pass: only the producer lane reads the list (it
-    // issues the copies); every thread derives the tile geometry from the
-    // count, so the consumers keep it in registers.
-    struct PassIn {
-        const T *const *in;
-        int ni;
-    };
-    __device__ __forceinline__ TileGeom geom(const PassIn &P) const {
-        return TileGeom{tile_chunks_for(P.ni), c_lo, c_hi};
-    }
-    // The producer lane's copy descriptor.
-    __device__ __forceinline__ void tile_pass(TilePass &D, const PassIn &P) const {
-        D.ni = P.ni;
-        for (int i = 0; i < P.ni; ++i) D.in[i] = P.in[i];
-        D.tc = tile_chunks_for(P.ni);
-        D.c_lo = c_lo;
-        D.c_hi = c_hi;
-    }
-
-    // Streaming pass through the tile pipeline: fn(chunk, stage, k, acc)
-    // for every chunk of this CTA, then a team reduction of K sums.
-    template <int K, typename Fn>
-    __device__ __forceinline__ bool tsum(const PassIn &P, Fn fn, double (&out)[K]) {
-        ACC acc[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) acc[k] = ACC(0);
-        bool okw = true;
-        TileRing *const ring = gs.ring;
-        const uint64_t to = gs.timeout_ns;
-        if ((threadIdx.x >> 5) == kConsumerWarps) {
-            if ((threadIdx.x & 31) == 0) {
-                TilePass D;
-                tile_pass(D, P);
-                unsigned sq = gs.seq();
-                okw = produce(ring, D, sq, to);
-                gs.seq() = sq;
-            }
-        } else {
-            unsigned sq = gs.seq();
-            okw = consume(ring, geom(P), sq, to, [&](int64_t ch, const unsigned char *st, int k) { fn(ch, st, k, acc); });
-            gs.seq() = sq;
+    // Issue the tiles of pass `st` (the input order of each pass is that of
+    // its consumer side below).
+    __device__ __forceinline__ int issue(const Step &st, unsigned &sq) {
+        const int lane = threadIdx.x & 31, n = sys.n, i = st.i, s = st.s;
+        TileRing *const R = gs.ring;
+        const T *p = nullptr;
+        int ni = 0;
+        switch (st.op) {
+        case P_SPMV_C:
+        case P_SPMV_Z:
+            return issue_product(st.op == P_SPMV_C ? Qc(i) : sys.r, 1, sq);
+        case P_ALPHA: {
+            const bool hq = i < n, f0 = st.first && hq;
+            ni = 4 + (hq ? 1 : 0) + (f0 ? 1 : 0);
+            p = lane == 0 ? sys.x : lane == 1 ? Gc(i - 1) : lane == 2 ? sys.r : lane == 3 ? Wc(i - 1)
+                : lane == 4 && hq ? Qc(i) : sys.F;
+            break;
         }
-        if (!okw) gs.ring->failed = 1;
-#pragma unroll
-        for (int k = 0; k < K; ++k) out[k] = (double)acc[k];
-        if (!reduce<K>(out)) return false;
-        if (gs.ring->failed) { gs.ok = false; return false; }
-        return true;
+        case P_OMEGA:
+            ni = 4;
+            p = lane == 0 ? sys.x : lane == 1 ? sys.r : lane == 2 ? sys.z : sys.Q;
+            break;
+        case P_W_FIRST:
+            ni = 3;
+            p = lane == 0 ? sys.r : lane == 1 ? Wc(i) : Qc(i + 1);
+            break;
+        case P_W_ROUND:
+            ni = 3;
+            p = lane == 0 ? Wc(i) : lane == 1 ? Wc(s) : Qc(s + 1);
+            break;
+        case P_W_LAST: {
+            const int nt = n - 1 - i, ntile = nt < kMaxInputs - 4 ? nt : kMaxInputs - 4, f = i > 0 ? 1 : 0;
+            ni = 3 + f + ntile;
+            p = lane == 0 ? Wc(i) : lane == 1 ? Gc(i) : lane == 2 ? (i == n - 1 ? sys.r : Wc(n - 1))
+                : lane == 3 && f ? sys.F : Gc(i + 1 + lane - 3 - f);
+            break;
+        }
+        case P_F_ROUND:
+            ni = s + 1 <= i - 1 ? 3 : 2;
+            p = lane == 0 ? Gc(i) : lane == 1 ? Gc(s) : Fc(s + 1);
+            break;
+        default:   // P_G_J0
+            ni = i >= 2 ? 3 : 2;
+            p = lane == 0 ? sys.r : lane == 1 ? sys.G : Fc(1);
+            break;
+        }
+        return produce_lanes(R, p, ni, c_lo, c_hi, sq, gs.timeout_ns);
     }
-    // Streaming pass with no inner product: the tiles, then only a team
-    // barrier (the next pass gathers what this one wrote), no reduction.
+    // Tiles of a product with `ne` epilogue vectors (lane 2 + k copies
+    // vector k, its own `epi`).
+    __device__ __forceinline__ int issue_product(const T *epi, int ne, unsigned &sq) {
+        if (sys.spt[ne] <= 0) return 0;
+        const SliceOffsets off(gs.ring, sys.slice_ptr, s_lo, s_hi);
+        return produce_sell_lanes(gs.ring, s_lo, s_hi, sys.spt[ne], off, sys.sval, EW * (int)sizeof(T),
+                                  (int)sizeof(T), sys.scol, epi, ne, sq, gs.timeout_ns);
+    }
+    // Wait until the consumers have finished the pass.
+    __device__ __forceinline__ int wait_done(unsigned &passes) {
+        int st = 0;
+        if ((threadIdx.x & 31) == 0) st = producer_wait(gs.ring, &gs.ring->done, passes & 1u, gs.timeout_ns);
+        st = __shfl_sync(0xffffffffu, st, 0);
+        if (st == 0) passes += 1;
+        return st;
+    }
+    // The producer warp's side of a system: commands of the consumers until
+    // kCmdExit.  Decide: the iteration asks the consumers after every update
+    // of r (refined mode).  residual64 issues the FP64 residual's tiles.
+    template <bool Decide, typename Fn>
+    __device__ __forceinline__ void serve(Fn residual64) {
+        TileRing *const R = gs.ring;
+        unsigned sq = gs.seq(), passes = R->passes;
+        for (;;) {
+            __syncthreads();
+            const int cmd = R->cmd;
+            if (cmd == kCmdExit) break;
+            int st = 0;
+            if (cmd == kCmdResidual) {
+                st = issue_product((threadIdx.x & 31) == 2 ? sys.b : sys.Q, 2, sq);
+                if (st == 0) st = wait_done(passes);
+            } else if (cmd == kCmdResidual64) {
+                st = residual64(sq);
+                if (st == 0) st = wait_done(passes);
+            } else {
+                const int n = sys.n;
+                bool met = false;   // the consumers' end_inner has been met at a decision
+                for (Step p; st == 0; p.advance(n)) {
+                    st = issue(p, sq);
+                    if (st == 0) st = wait_done(passes);
+                    if constexpr (Decide) {
+                        if (st == 0 && (p.op == P_ALPHA || p.op == P_OMEGA)) {
+                            if ((threadIdx.x & 31) == 0) R->issued = sq;
+                            __syncthreads();
+                            if (R->stop) {
+                                met = true;
+                                break;
+                            }
+                            if (R->cmd == kCmdResidual64) {
+                                st = residual64(sq);
+                                if (st == 0) st = wait_done(passes);
+                                if (st == 0) {
+                                    if ((threadIdx.x & 31) == 0) R->issued = sq;
+                                    __syncthreads();
+                                    if (R->stop) {
+                                        met = true;
+                                        break;
+                                    }
+                                }
+                            }
+                        }
+                    }
+                }
+                if (st == 2) R->failed = 1;
+                if (!met) {
+                    if ((threadIdx.x & 31) == 0) R->issued = sq;
+                    __syncthreads();
+                }
+                passes = R->passes;
+                continue;
+            }
+            if (st == 2) R->failed = 1;
+            if ((threadIdx.x & 31) == 0) R->passes = passes;
+        }
+        gs.seq() = sq;
+        if ((threadIdx.x & 31) == 0) R->passes = passes;
+    }
+
+    // ------------------------------------------------------------------
+    // the consumers' side of the passes
+    // ------------------------------------------------------------------
+
+    // Streaming pass through the tile pipeline: fn(chunk, stage, k) for
+    // every chunk of this CTA.
     template <typename Fn>
-    __device__ __forceinline__ bool tpass(const PassIn &P, Fn fn) {
-        bool okw = true;
+    __device__ __forceinline__ void tiles(int tc, unsigned &sq, Fn fn) {
         TileRing *const ring = gs.ring;
-        const uint64_t to = gs.timeout_ns;
-        if ((threadIdx.x >> 5) == kConsumerWarps) {
-            if ((threadIdx.x & 31) == 0) {
-                TilePass D;
-                tile_pass(D, P);
-                unsigned sq = gs.seq();
-                okw = produce(ring, D, sq, to);
-                gs.seq() = sq;
-            }
-        } else {
-            unsigned sq = gs.seq();
-            okw = consume(ring, geom(P), sq, to, [&](int64_t ch, const unsigned char *st, int k) { fn(ch, st, k); });
-            gs.seq() = sq;
-        }
-        if (!okw) gs.ring->failed = 1;
-        if (!sync()) return false;
+        if (!consume(ring, TileGeom{tc, c_lo, c_hi}, sq, gs.timeout_ns, fn)) ring->failed = 1;
+        pass_done(ring);
+    }
+    template <int K>
+    __device__ __forceinline__ bool reduce(const ACC (&acc)[K], bool fence) {
+        double v[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) v[k] = (double)acc[k];
+        return gs.template reduce<K>(v, fence) && ring_ok();
+    }
+    // A failed tile wait marks the ring; the pass's reduction or barrier
+    // then reports it.
+    __device__ __forceinline__ bool ring_ok() {
         if (gs.ring->failed) { gs.ok = false; return false; }
         return true;
     }
 
     // SELL-32 SpMV pass over the owned slices (matrix tiles through the
-    // ring).  A failed tile wait marks the ring; the pass's reduction then
-    // reports it.
-    template <int K, int NE, typename Fin>
-    __device__ __forceinline__ void spmv_rows(const T *xin, const T *const (&epi)[NE], Fin fin, ACC (&acc)[K]) {
+    // ring).
+    template <int NE, typename Fin, int K>
+    __device__ __forceinline__ void spmv_rows(const T *xin, const T *const (&epi)[NE], unsigned &sq, Fin fin,
+                                              ACC (&acc)[K]) {
         // with ILU(0) the product is A t, t = M^{-1} xin formed by the
         // caller (ilu_pre) before the pass
         if constexpr (PC) {
             if (sys.ilu.lu) xin = sys.ilu.t;
         }
-        unsigned sq = gs.seq();   // issued (producer lane) or consumed (consumers) tiles
         bool okw;
         // FP32 and complex engines: a pipelined width of 7 where the rows
-        // allow it (gathered x registers fewer: the refined solve 3 %, the
-        // complex one 3.5 % less time per iteration); the real FP64 engine
+        // allow it (fewer registers of gathered x); the real FP64 engine
         // keeps 8 (no gain at 7)
         if constexpr (is_narrow<T>::value || is_cx<T>::value) {
             if (sys.narrow_rows)
-                okw = sell_spmv<NE, EW, 7>(gs.ring, sq, sq, gs.timeout_ns, s_lo, s_hi, sys.spt[NE], sys.slice_ptr,
-                                           sys.scol, sys.sval, xin, epi, threadIdx.x & 31, fin, acc);
+                okw = sell_consume<NE, EW, 7>(gs.ring, sq, gs.timeout_ns, s_lo, s_hi, sys.spt[NE], sys.slice_ptr,
+                                              sys.scol, sys.sval, xin, epi, threadIdx.x & 31, fin, acc);
             else
-                okw = sell_spmv<NE, EW>(gs.ring, sq, sq, gs.timeout_ns, s_lo, s_hi, sys.spt[NE], sys.slice_ptr,
-                                        sys.scol, sys.sval, xin, epi, threadIdx.x & 31, fin, acc);
+                okw = sell_consume<NE, EW>(gs.ring, sq, gs.timeout_ns, s_lo, s_hi, sys.spt[NE], sys.slice_ptr,
+                                           sys.scol, sys.sval, xin, epi, threadIdx.x & 31, fin, acc);
         } else {
-            okw = sell_spmv<NE, EW>(gs.ring, sq, sq, gs.timeout_ns, s_lo, s_hi, sys.spt[NE], sys.slice_ptr,
-                                    sys.scol, sys.sval, xin, epi, threadIdx.x & 31, fin, acc);
+            okw = sell_consume<NE, EW>(gs.ring, sq, gs.timeout_ns, s_lo, s_hi, sys.spt[NE], sys.slice_ptr, sys.scol,
+                                       sys.sval, xin, epi, threadIdx.x & 31, fin, acc);
         }
-        gs.seq() = sq;
         if (!okw) gs.ring->failed = 1;
-    }
-    __device__ __forceinline__ bool ring_ok() {
-        if (gs.ring->failed) { gs.ok = false; return false; }
-        return true;
+        pass_done(gs.ring);
     }
 
     // ------------------------------------------------------------------
@@ -942,7 +1067,7 @@ struct Engine {
         ilu_fetch_l(q0 + tid, q1, v, R);
         for (int l = 0; l < nl; ++l) {
             if (R.i >= 0) out[R.i] = ilu_row_sum(R, R.v, out);
-            for (int64_t q = q0 + tid + kThreads; q < q1; q += kThreads) {   // more rows than threads
+            for (int64_t q = q0 + tid + kConsumers; q < q1; q += kConsumers) {   // more rows than threads
                 const int i = M.lrows[q];
                 const int64_t k0 = M.rp[i], kd = k0 + M.dpos[i];
                 T t = v[i];
@@ -961,7 +1086,7 @@ struct Engine {
         }
         for (int l = 0; l < nu; ++l) {
             if (R.i >= 0) out[R.i] = ilu_row_sum(R, ldcg_val(out + R.i), out) / R.v;
-            for (int64_t q = q0 + tid + kThreads; q < q1; q += kThreads) {
+            for (int64_t q = q0 + tid + kConsumers; q < q1; q += kConsumers) {
                 const int i = M.urows[q];
                 const int64_t kd = M.rp[i] + M.dpos[i], k1 = M.rp[i + 1];
                 T t = ldcg_val(out + i);
@@ -975,7 +1100,7 @@ struct Engine {
             }
             if (!gs.wait()) return false;
         }
-        if (threadIdx.x == 0) {   // factors and row data once, v read, out written and re-read
+        if (threadIdx.x == kAcctThread) {   // factors and row data once, v read, out written and re-read
             acct->bytes += M.nnz * (int64_t)(sizeof(T) + 4) + sys.N * (int64_t)(8 + 4 + 8 + 3 * sizeof(T));
             acct->flops += (is_cx<T>::value ? 8 : 2) * M.nnz;
         }
@@ -998,8 +1123,8 @@ struct Engine {
     // row-parallel products).
     __device__ __noinline__ bool ilu_to_y() {
         const IluView<T> &M = sys.ilu;
-        const int64_t nth = (int64_t)gs.nblocks * kThreads;
-        const int64_t me = (int64_t)gs.bid * kThreads + threadIdx.x;
+        const int64_t nth = (int64_t)gs.nblocks * kConsumers;
+        const int64_t me = (int64_t)gs.bid * kConsumers + threadIdx.x;
         T *const x = sys.x, *const t = M.t;
         for (int64_t i = me; i < sys.N; i += nth) {
             const int64_t kd = M.rp[i] + M.dpos[i], k1 = M.rp[i + 1];
@@ -1019,8 +1144,8 @@ struct Engine {
 
     // x = M^{-1} y once the final residual pass has formed t = M^{-1} y.
     __device__ __noinline__ bool ilu_to_x() {
-        const int64_t nth = (int64_t)gs.nblocks * kThreads;
-        const int64_t me = (int64_t)gs.bid * kThreads + threadIdx.x;
+        const int64_t nth = (int64_t)gs.nblocks * kConsumers;
+        const int64_t me = (int64_t)gs.bid * kConsumers + threadIdx.x;
         T *const x = sys.x;
         const T *t = sys.ilu.t;
         for (int64_t i = me; i < sys.N; i += nth) x[i] = ldcg_val(t + i);
@@ -1028,22 +1153,23 @@ struct Engine {
     }
 
     // ------------------------------------------------------------------
-    // passes
+    // passes (sums in gs.red->total)
     // ------------------------------------------------------------------
 
-    // r = b - A x, g_0 = r; sums ||b||^2, ||r||^2, q_1^H r.
-    __device__ __forceinline__ bool ph_residual_body(double &bb, double &rr, S &qr, bool write_g0) {
+    // r = b - A x, g_0 = r; sums ||b||^2, ||r||^2, q_1^H r.  The caller has
+    // posted kCmdResidual.
+    __device__ __noinline__ bool ph_residual(bool write_g0) {
         constexpr int K = 2 + DS;
         ACC acc[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) acc[k] = ACC(0);
-        const T *q1 = Qc(0);
         T *g0 = Gc(0);
-        const T *epi[2] = {sys.b, q1};
+        const T *epi[2] = {sys.b, Qc(0)};
         T *const r = sys.r;
+        unsigned sq = gs.seq();
         // epilogues capture by value: a captured reference would keep the
         // pointer in memory, reloaded after every store of the loop
-        spmv_rows<K>(sys.x, epi, [=](int64_t row, T y, const T (&e)[2], ACC(&a)[K]) {
+        spmv_rows<2>(sys.x, epi, sq, [=](int64_t row, T y, const T (&e)[2], ACC(&a)[K]) {
             T rv = subT(e[0], y);
             r[row] = rv;
             if (write_g0) g0[row] = rv;
@@ -1051,15 +1177,9 @@ struct Engine {
             acc_nrm(&a[1], rv);
             acc_dot(&a[2], e[1], rv);
         }, acc);
-        double v[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] = (double)acc[k];
-        if (!reduce<K>(v) || !ring_ok()) return false;
-        bb = v[0];
-        rr = v[1];
-        qr = mk_coef<T>(v + 2);
+        gs.seq() = sq;
         sbytes(write_g0 ? 4 : 3);
-        return true;
+        return reduce<K>(acc, true);
     }
 
     // Refined mode, inner start with x_0 = 0: b = r = g_0 = src * scale
@@ -1080,7 +1200,7 @@ struct Engine {
         T *const rq = sys.r;
         T *const xq = sys.x;
         const int64_t clo = c_lo, chi = c_hi;
-        if ((threadIdx.x >> 5) < kConsumerWarps) {
+        {
             for (int64_t ch = clo + threadIdx.x; ch < chi; ch += kConsumers) {
                 const uint4 *sp = reinterpret_cast<const uint4 *>(src) + 2 * ch;
                 uint4 w2[2] = {sp[0], sp[1]};
@@ -1109,11 +1229,11 @@ struct Engine {
         double v[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) v[k] = (double)acc[k];
-        if (!reduce<K>(v)) return false;
-        bb = v[0];
-        rr = v[1];
-        qr = mk_coef<T>(v + 2);
-        if (threadIdx.x == 0) acct->bytes += sys.N * (int64_t)(sizeof(TW) + 5 * sizeof(T));
+        if (!gs.template reduce<K>(v, true)) return false;
+        bb = gs.red->total[0];
+        rr = gs.red->total[1];
+        qr = mk_coef<T>(gs.red->total + 2);
+        if (threadIdx.x == kAcctThread) acct->bytes += sys.N * (int64_t)(sizeof(TW) + 5 * sizeof(T));
         return true;
     }
 
@@ -1134,7 +1254,7 @@ struct Engine {
         for (int k = 0; k < K; ++k) acc[k] = ACC(0);
         T *const rq = sys.r;
         const int64_t clo = c_lo, chi = c_hi;
-        if ((threadIdx.x >> 5) < kConsumerWarps) {
+        {
             for (int64_t ch = clo + threadIdx.x; ch < chi; ch += kConsumers) {
                 const uint4 *sp = reinterpret_cast<const uint4 *>(src) + 2 * ch;
                 uint4 w2[2] = {sp[0], sp[1]};
@@ -1162,77 +1282,60 @@ struct Engine {
         double v[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) v[k] = (double)acc[k];
-        if (!reduce<K>(v)) return false;
-        rr = v[0];
-        qr = mk_coef<T>(v + 1);
-        fr = mk_coef<T>(v + 1 + DS);
-        if (threadIdx.x == 0)
+        if (!gs.template reduce<K>(v, true)) return false;
+        rr = gs.red->total[0];
+        qr = mk_coef<T>(gs.red->total + 1);
+        fr = mk_coef<T>(gs.red->total + 1 + DS);
+        if (threadIdx.x == kAcctThread)
             acct->bytes += sys.N * (int64_t)(sizeof(TW) + (1 + (qv ? 1 : 0) + (fv ? 1 : 0)) * sizeof(T));
         return true;
     }
 
-    // w_slot = A g_slot; returns c = q_qcol^H w.
-    __device__ __forceinline__ bool ph_spmv_c_body(int sl, int qcol, S &cval) {
-        constexpr int K = DS;
-        ACC acc[K];
+    // w_i = A g_i; sum q_i^H w.
+    __device__ __forceinline__ bool ph_spmv_c(int i, unsigned &sq) {
+        ACC acc[DS];
 #pragma unroll
-        for (int k = 0; k < K; ++k) acc[k] = ACC(0);
-        const T *q = Qc(qcol);
-        T *w = Wc(sl);
-        const T *epi[1] = {q};
-        spmv_rows<K>(Gc(sl), epi, [=](int64_t row, T y, const T (&e)[1], ACC(&a)[K]) {
+        for (int k = 0; k < DS; ++k) acc[k] = ACC(0);
+        T *const w = Wc(i);
+        const T *epi[1] = {Qc(i)};
+        spmv_rows<1>(Gc(i), epi, sq, [=](int64_t row, T y, const T (&e)[1], ACC(&a)[DS]) {
             w[row] = y;
             acc_dot(&a[0], e[0], y);
         }, acc);
-        double v[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] = (double)acc[k];
-        if (!reduce<K>(v) || !ring_ok()) return false;
-        cval = mk_coef<T>(v);
         sbytes(1);
-        return true;
+        return reduce<DS>(acc, false);
     }
 
     // z = A u (u held in r); sums z^H z, z^H u.
-    __device__ __forceinline__ bool ph_spmv_z_body(double &zz, S &zu) {
+    __device__ __forceinline__ bool ph_spmv_z(unsigned &sq) {
         constexpr int K = 1 + DS;
         ACC acc[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) acc[k] = ACC(0);
         const T *epi[1] = {sys.r};
         T *const z = sys.z;
-        spmv_rows<K>(sys.r, epi, [=](int64_t row, T y, const T (&e)[1], ACC(&a)[K]) {
+        spmv_rows<1>(sys.r, epi, sq, [=](int64_t row, T y, const T (&e)[1], ACC(&a)[K]) {
             z[row] = y;
             acc_nrm(&a[0], y);
             acc_dot(&a[1], y, e[0]);
         }, acc);
-        double v[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] = (double)acc[k];
-        if (!reduce<K>(v) || !ring_ok()) return false;
-        zz = v[0];
-        zu = mk_coef<T>(v + 1);
         sbytes(1);
-        return true;
+        return reduce<K>(acc, false);
     }
 
-    // x += alpha g_sl, r -= alpha w_sl; sums ||r||^2, q_qcol^H r and
+    // x += alpha g_sl, r -= alpha w_sl; sums ||r||^2, q_qcol^H r (hq) and
     // (when f0) f_1^H r.
-    __device__ __forceinline__ bool ph_alpha_body(S alpha, int sl, int qcol, bool f0, double &rr, S &qr, S &fr) {
+    __device__ __forceinline__ bool ph_alpha(S alpha, bool hq, bool f0, unsigned &sq) {
         constexpr int K = 1 + 2 * DS;
         const T a = to_t<T>(alpha), na = to_t<T>(-alpha);
-        const bool hq = qcol >= 0;
-        const T *in[6] = {sys.x, Gc(sl), sys.r, Wc(sl), hq ? Qc(qcol) : nullptr, f0 ? Fc(0) : nullptr};
-        int ni = 4;
-        if (hq) in[ni++] = Qc(qcol);
-        if (f0) in[ni++] = Fc(0);
-        const int iq = 4, iff = hq ? 5 : 4;
+        const int ni = 4 + (hq ? 1 : 0) + (f0 ? 1 : 0), iff = hq ? 5 : 4;
         T *const xo = sys.x;
         T *const ro = sys.r;
-        const PassIn P{in, ni};
-        const int tc = tile_chunks_for(P.ni);
-        double v[K];
-        bool okk = tsum<K>(P, [&](int64_t ch, const unsigned char *st, int k, ACC *acc) {
+        const int tc = tile_chunks_for(ni);
+        ACC acc[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) acc[k] = ACC(0);
+        tiles(tc, sq, [&](int64_t ch, const unsigned char *st, int k) {
             Pack<T> xx = lds<T>(st, tc, 0, k), gg = lds<T>(st, tc, 1, k), rv = lds<T>(st, tc, 2, k),
                     ww = lds<T>(st, tc, 3, k);
 #pragma unroll
@@ -1245,7 +1348,7 @@ struct Engine {
 #pragma unroll
             for (int e = 0; e < PW; ++e) acc_nrm(&acc[0], rv.e[e]);
             if (hq) {
-                Pack<T> qq = lds<T>(st, tc, iq, k);
+                Pack<T> qq = lds<T>(st, tc, 4, k);
 #pragma unroll
                 for (int e = 0; e < PW; ++e) acc_dot(&acc[1], qq.e[e], rv.e[e]);
             }
@@ -1254,26 +1357,30 @@ struct Engine {
 #pragma unroll
                 for (int e = 0; e < PW; ++e) acc_dot(&acc[1 + DS], ff.e[e], rv.e[e]);
             }
-        }, v);
-        if (!okk) return false;
-        rr = v[0];
-        qr = mk_coef<T>(v + 1);
-        fr = mk_coef<T>(v + 1 + DS);
+        });
         vbytes(6 + (hq ? 1 : 0) + (f0 ? 1 : 0));
-        return true;
+        if (f0) return reduce<K>(acc, false);
+        // without f the sums are ||r||^2 and q^H r, at the block's end (u in
+        // r, which the next pass gathers) ||u||^2 alone
+        ACC a1[1 + DS];
+#pragma unroll
+        for (int k = 0; k < 1 + DS; ++k) a1[k] = acc[k];
+        if (hq) return reduce<1 + DS>(a1, false);
+        ACC a0[1] = {acc[0]};
+        return reduce<1>(a0, true);
     }
 
     // x += omega u, r = u - omega z (u in r); sums ||r||^2, q_1^H r.
-    __device__ __forceinline__ bool ph_omega_body(S omega, double &rr, S &qr) {
+    __device__ __forceinline__ bool ph_omega(S omega, unsigned &sq) {
         constexpr int K = 1 + DS;
         const T om = to_t<T>(omega), nom = to_t<T>(-omega);
-        const T *in[4] = {sys.x, sys.r, sys.z, Qc(0)};
         T *const xo = sys.x;
         T *const ro = sys.r;
-        const PassIn P{in, 4};
-        const int tc = tile_chunks_for(P.ni);
-        double v[K];
-        bool okk = tsum<K>(P, [&](int64_t ch, const unsigned char *st, int k, ACC *acc) {
+        const int tc = tile_chunks_for(4);
+        ACC acc[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) acc[k] = ACC(0);
+        tiles(tc, sq, [&](int64_t ch, const unsigned char *st, int k) {
             Pack<T> xx = lds<T>(st, tc, 0, k), uu = lds<T>(st, tc, 1, k), zz = lds<T>(st, tc, 2, k),
                     qq = lds<T>(st, tc, 3, k);
 #pragma unroll
@@ -1288,58 +1395,32 @@ struct Engine {
                 acc_nrm(&acc[0], uu.e[e]);
                 acc_dot(&acc[1], qq.e[e], uu.e[e]);
             }
-        }, v);
-        if (!okk) return false;
-        rr = v[0];
-        qr = mk_coef<T>(v + 1);
+        });
         vbytes(6);
-        return true;
+        return reduce<K>(acc, false);
     }
 
-    // z_w = r + bt0 * w_sl (in place); sums q_qcol^H z_w.
-    __device__ __forceinline__ bool ph_w_first_body(S bt0, int sl, int qcol, S &d) {
-        constexpr int K = DS;
-        const T b0 = to_t<T>(bt0);
-        T *wp = Wc(sl);
-        const T *in[3] = {sys.r, wp, Qc(qcol)};
-        const PassIn P{in, 3};
-        const int tc = tile_chunks_for(P.ni);
-        double v[K];
-        bool okk = tsum<K>(P, [&](int64_t ch, const unsigned char *st, int k, ACC *acc) {
-            Pack<T> rv = lds<T>(st, tc, 0, k), ww = lds<T>(st, tc, 1, k), qq = lds<T>(st, tc, 2, k);
+    // z_w = r + bt0 w_i (first) or z_w += bts w_s, in place; sum q^H z_w.
+    __device__ __forceinline__ bool ph_w(bool first, S coef, int i, unsigned &sq) {
+        const T b = to_t<T>(coef);
+        T *const wp = Wc(i);
+        const int tc = tile_chunks_for(3);
+        ACC acc[DS];
 #pragma unroll
-            for (int e = 0; e < PW; ++e) ww.e[e] = efma(b0, ww.e[e], rv.e[e]);
-            stp(wp, ch, ww);
+        for (int k = 0; k < DS; ++k) acc[k] = ACC(0);
+        // inputs: r, w_i, q; or w_i, w_s, q
+        const int ia = first ? 1 : 0, io = first ? 0 : 1;
+        tiles(tc, sq, [&](int64_t ch, const unsigned char *st, int k) {
+            Pack<T> zw = lds<T>(st, tc, ia, k), o = lds<T>(st, tc, io, k), qq = lds<T>(st, tc, 2, k);
+            // first: r + b w_i, else w_i + b w_s
 #pragma unroll
-            for (int e = 0; e < PW; ++e) acc_dot(&acc[0], qq.e[e], ww.e[e]);
-        }, v);
-        if (!okk) return false;
-        d = mk_coef<T>(v);
-        vbytes(4);
-        return true;
-    }
-
-    // z_w += bts * w_s (in place); sums q_qcol^H z_w.
-    __device__ __forceinline__ bool ph_w_round_body(S bts, int s, int sl, int qcol, S &d) {
-        constexpr int K = DS;
-        const T bb = to_t<T>(bts);
-        T *wp = Wc(sl);
-        const T *in[3] = {wp, Wc(s), Qc(qcol)};
-        const PassIn P{in, 3};
-        const int tc = tile_chunks_for(P.ni);
-        double v[K];
-        bool okk = tsum<K>(P, [&](int64_t ch, const unsigned char *st, int k, ACC *acc) {
-            Pack<T> zw = lds<T>(st, tc, 0, k), w2 = lds<T>(st, tc, 1, k), qq = lds<T>(st, tc, 2, k);
-#pragma unroll
-            for (int e = 0; e < PW; ++e) zw.e[e] = efma(bb, w2.e[e], zw.e[e]);
+            for (int e = 0; e < PW; ++e) zw.e[e] = first ? efma(b, zw.e[e], o.e[e]) : efma(b, o.e[e], zw.e[e]);
             stp(wp, ch, zw);
 #pragma unroll
             for (int e = 0; e < PW; ++e) acc_dot(&acc[0], qq.e[e], zw.e[e]);
-        }, v);
-        if (!okk) return false;
-        d = mk_coef<T>(v);
+        });
         vbytes(4);
-        return true;
+        return reduce<DS>(acc, false);
     }
 
     // Last pass of the z_w sweep, fused with every deferred g-update of the
@@ -1349,34 +1430,27 @@ struct Engine {
     //   g = bt[sl] g_sl;  g += bt[t] g_t for t = sl+1..n-1;  g = z_w - g/omega
     // sums f_1^H g when with_f.  The first kMaxInputs-4 columns g_t come
     // through the tile pipeline, any further ones by direct loads.
-    __device__ __forceinline__ bool ph_w_last_body(bool first, int sl, S inv_omega, bool with_f, S &d) {
-        constexpr int K = DS;
+    __device__ __forceinline__ bool ph_w_last(int sl, unsigned &sq) {
         const int n = sys.n;
         const int last = n - 1;
+        const bool first = sl == last, with_f = sl > 0;
         T *wp = Wc(sl);
         T *gp = Gc(sl);
         const T bl = to_t<T>(bt[first ? sl : last]);
         const T b0 = to_t<T>(bt[sl]);
-        const T nio = to_t<T>(-inv_omega);
+        const T nio = to_t<T>(-sc->inv_omega);
         const int t0 = sl + 1;
         const int nt = n - t0;                                     // g_t columns
         const int ntile = nt < kMaxInputs - 4 ? nt : kMaxInputs - 4;
-        const T *in[kMaxInputs];
-        int ni = 0;
-        in[ni++] = wp;
-        in[ni++] = gp;
-        in[ni++] = first ? sys.r : Wc(last);
-        const int i_f = ni;
-        if (with_f) in[ni++] = Fc(0);
-        const int i_t = ni;
-        for (int t = 0; t < ntile; ++t) in[ni++] = Gc(t0 + t);
+        const int i_t = with_f ? 4 : 3;
         const T *const Gb = sys.G;
         const int64_t ldv = sys.ld;
         const S *const btl = bt;
-        const PassIn P{in, ni};
-        const int tc = tile_chunks_for(P.ni);
-        double v[K];
-        bool okk = tsum<K>(P, [&](int64_t ch, const unsigned char *st, int k, ACC *acc) {
+        const int tc = tile_chunks_for(i_t + ntile);
+        ACC acc[DS];
+#pragma unroll
+        for (int k = 0; k < DS; ++k) acc[k] = ACC(0);
+        tiles(tc, sq, [&](int64_t ch, const unsigned char *st, int k) {
             Pack<T> zw = lds<T>(st, tc, 0, k), g = lds<T>(st, tc, 1, k), o = lds<T>(st, tc, 2, k);
             if (first) {
 #pragma unroll
@@ -1398,120 +1472,40 @@ struct Engine {
             stp(wp, ch, zw);
             stp(gp, ch, g);
             if (with_f) {
-                Pack<T> ff = lds<T>(st, tc, i_f, k);
+                Pack<T> ff = lds<T>(st, tc, 3, k);
 #pragma unroll
                 for (int e = 0; e < PW; ++e) acc_dot(&acc[0], ff.e[e], g.e[e]);
             }
-        }, v);
-        if (!okk) return false;
-        d = mk_coef<T>(v);
+        });
         vbytes(5 + nt + (with_f ? 1 : 0));
-        return true;
+        if (!with_f) return gs.sync() && ring_ok();   // the next pass gathers g
+        return reduce<DS>(acc, false);
     }
 
-    // g_sl += beta g_s; sums f_fcol^H g_sl when fcol >= 0 (else no sum).
-    __device__ __forceinline__ bool ph_f_round_body(S beta, int s, int sl, int fcol, S &d) {
+    // g_i += beta g_s, or (block 0's first) g_i = r + beta g_0; sums f^H g_i, or, at the sweep's end (the next pass gathers g_i), a team
+    // barrier.
+    __device__ __forceinline__ bool ph_g(S beta, int i, bool with_f, unsigned &sq) {
         const T bb = to_t<T>(beta);
-        T *gp = Gc(sl);
-        const T *in[3] = {gp, Gc(s), fcol >= 0 ? Fc(fcol) : nullptr};
-        const PassIn P{in, fcol >= 0 ? 3 : 2};
-        const int tc = tile_chunks_for(P.ni);
-        if (fcol < 0) {
-            bool okk = tpass(P, [&](int64_t ch, const unsigned char *st, int k) {
-                Pack<T> g = lds<T>(st, tc, 0, k), g2 = lds<T>(st, tc, 1, k);
+        T *gp = Gc(i);
+        const int tc = tile_chunks_for(with_f ? 3 : 2);
+        ACC acc[DS];
 #pragma unroll
-                for (int e = 0; e < PW; ++e) g.e[e] = efma(bb, g2.e[e], g.e[e]);
-                stp(gp, ch, g);
-            });
-            vbytes(3);
-            return okk;
-        }
-        constexpr int K = DS;
-        double v[K];
-        bool okk = tsum<K>(P, [&](int64_t ch, const unsigned char *st, int k, ACC *acc) {
-            Pack<T> g = lds<T>(st, tc, 0, k), g2 = lds<T>(st, tc, 1, k), ff = lds<T>(st, tc, 2, k);
+        for (int k = 0; k < DS; ++k) acc[k] = ACC(0);
+        tiles(tc, sq, [&](int64_t ch, const unsigned char *st, int k) {
+            Pack<T> g = lds<T>(st, tc, 0, k), g2 = lds<T>(st, tc, 1, k);
 #pragma unroll
             for (int e = 0; e < PW; ++e) g.e[e] = efma(bb, g2.e[e], g.e[e]);
             stp(gp, ch, g);
+            if (with_f) {
+                Pack<T> ff = lds<T>(st, tc, 2, k);
 #pragma unroll
-            for (int e = 0; e < PW; ++e) acc_dot(&acc[0], ff.e[e], g.e[e]);
-        }, v);
-        if (!okk) return false;
-        d = mk_coef<T>(v);
-        vbytes(4);
-        return true;
+                for (int e = 0; e < PW; ++e) acc_dot(&acc[0], ff.e[e], g.e[e]);
+            }
+        });
+        vbytes(with_f ? 4 : 3);
+        if (!with_f) return gs.sync() && ring_ok();
+        return reduce<DS>(acc, false);
     }
-
-    // Block 0: g_sl = r + beta g_0; sums f_fcol^H g_sl when fcol >= 0.
-    __device__ __forceinline__ bool ph_g_j0_body(S beta, int sl, int fcol, S &d) {
-        const T bb = to_t<T>(beta);
-        T *gp = Gc(sl);
-        const T *in[3] = {sys.r, Gc(0), fcol >= 0 ? Fc(fcol) : nullptr};
-        const PassIn P{in, fcol >= 0 ? 3 : 2};
-        const int tc = tile_chunks_for(P.ni);
-        if (fcol < 0) {
-            bool okk = tpass(P, [&](int64_t ch, const unsigned char *st, int k) {
-                Pack<T> rv = lds<T>(st, tc, 0, k), g2 = lds<T>(st, tc, 1, k), g;
-#pragma unroll
-                for (int e = 0; e < PW; ++e) g.e[e] = efma(bb, g2.e[e], rv.e[e]);
-                stp(gp, ch, g);
-            });
-            vbytes(3);
-            return okk;
-        }
-        constexpr int K = DS;
-        double v[K];
-        bool okk = tsum<K>(P, [&](int64_t ch, const unsigned char *st, int k, ACC *acc) {
-            Pack<T> rv = lds<T>(st, tc, 0, k), g2 = lds<T>(st, tc, 1, k), ff = lds<T>(st, tc, 2, k), g;
-#pragma unroll
-            for (int e = 0; e < PW; ++e) g.e[e] = efma(bb, g2.e[e], rv.e[e]);
-            stp(gp, ch, g);
-#pragma unroll
-            for (int e = 0; e < PW; ++e) acc_dot(&acc[0], ff.e[e], g.e[e]);
-        }, v);
-        if (!okk) return false;
-        d = mk_coef<T>(v);
-        vbytes(4);
-        return true;
-    }
-
-    // ------------------------------------------------------------------
-    // helpers
-    // ------------------------------------------------------------------
-    __device__ __forceinline__ void record(bool rec, int64_t iter, double err) {
-        if (rec && ctl.err_hist && iter < ctl.hist_cap && gs.bid == 0 && threadIdx.x == 0)
-            ctl.err_hist[iter] = err;
-    }
-
-    // The streaming passes are inlined into the FP64 engines: no saves and
-    // restores of registers around the calls, whose stack sits in L2
-    // beside the tile ring.  The SELL product passes stay out of line in
-    // the real engines (inlined, their register demand spreads over the
-    // whole loop: n = 1 took 223 instead of 193 us per iteration at 128^3,
-    // and the natural-order ILU(0) solve 4 % longer) but are inlined in the
-    // complex one without ILU(0) (1 % faster).  The FP32 engines call every
-    // pass out of line (their kernels then compile in a fraction of the
-    // time; inlining gained 2 % only where the refined mode does not
-    // converge without a preconditioner).
-    static constexpr bool kInlinePasses = std::is_same<T, double>::value || std::is_same<T, cdouble>::value;
-    static constexpr bool kInlineProducts = std::is_same<T, cdouble>::value && !PC;
-#define MLB_PASS(name, inl, params, args)                                   \
-    __device__ __noinline__ bool name##_ool params { return name##_body args; } \
-    __device__ __forceinline__ bool name params {                            \
-        if constexpr (inl) return name##_body args;                          \
-        else return name##_ool args;                                         \
-    }
-    MLB_PASS(ph_residual, kInlineProducts, (double &bb, double &rr, S &qr, bool write_g0), (bb, rr, qr, write_g0))
-    MLB_PASS(ph_spmv_c, kInlineProducts, (int sl, int qcol, S &cval), (sl, qcol, cval))
-    MLB_PASS(ph_spmv_z, kInlineProducts, (double &zz, S &zu), (zz, zu))
-    MLB_PASS(ph_alpha, kInlinePasses, (S alpha, int sl, int qcol, bool f0, double &rr, S &qr, S &fr), (alpha, sl, qcol, f0, rr, qr, fr))
-    MLB_PASS(ph_omega, kInlinePasses, (S omega, double &rr, S &qr), (omega, rr, qr))
-    MLB_PASS(ph_w_first, kInlinePasses, (S bt0, int sl, int qcol, S &d), (bt0, sl, qcol, d))
-    MLB_PASS(ph_w_round, kInlinePasses, (S bts, int s, int sl, int qcol, S &d), (bts, s, sl, qcol, d))
-    MLB_PASS(ph_w_last, kInlinePasses, (bool first, int sl, S inv_omega, bool with_f, S &d), (first, sl, inv_omega, with_f, d))
-    MLB_PASS(ph_f_round, kInlinePasses, (S beta, int s, int sl, int fcol, S &d), (beta, s, sl, fcol, d))
-    MLB_PASS(ph_g_j0, kInlinePasses, (S beta, int sl, int fcol, S &d), (beta, sl, fcol, d))
-#undef MLB_PASS
 
     // ------------------------------------------------------------------
     // one call of the method (Algorithm 7.1, M = I) from the current x
@@ -1523,266 +1517,324 @@ struct Engine {
         double err;
     };
 
+    __device__ __forceinline__ void record(bool rec, int64_t iter, double err) {
+        if (rec && ctl.err_hist && iter < ctl.hist_cap && gs.bid == 0) ctl.err_hist[iter] = err;
+    }
+    __device__ __forceinline__ S total(int k) const { return mk_coef<T>(gs.red->total + k); }
+
     // `init` (refined mode only): start from x_0 = 0 with b = init * scale
-    // instead of reading b and x.  `hook` (refined mode only): residual
-    // replacement by the FP64 outer iteration.  hook->replace(qcol, f0, rr,
-    // qr, fr, conv) moves the FP32 iterate into the FP64 solution, replaces
-    // r by the scaled FP64 true residual and returns ||r||^2 and the inner
-    // products of the replaced r that the next step needs, and whether the
-    // true residual met the outer tolerance.  It is called when the
-    // recursive residual meets `tol` (instead of stopping: the inner call
-    // stops only once the true residual has met the outer tolerance) and,
-    // at block ends, when hook->want(err) (reliable updates); a block end
-    // also ends the call when hook->stalled(iter, err).
+    // instead of reading b and x.  `hook` (refined mode only, in shared
+    // memory): residual replacement by the FP64 outer iteration.
+    // hook->replace(qcol, f0, rr, qr, fr, conv) moves the FP32 iterate into
+    // the FP64 solution, replaces r by the scaled FP64 true residual and
+    // returns ||r||^2 and the inner products of the replaced r that the next
+    // step needs, and whether the true residual met the outer tolerance.  It
+    // is called when the recursive residual meets `tol` (instead of
+    // stopping: the inner call stops only once the true residual has met the
+    // outer tolerance) and, at block ends, when hook->want(err) (reliable
+    // updates); a block end also ends the call when hook->stalled(iter, err).
+    //
+    // After inner() returns, x and r are visible to their own CTA only: a
+    // team barrier comes before any pass that gathers them.
     template <typename Hook = NoHook>
     __device__ Out inner(int64_t maxit, bool rec, double tol,
                          const typename wide_of<T>::type *init = nullptr, double scale = 1.0,
                          Hook *hook = nullptr) {
         const int n = sys.n;
+        const int tid = threadIdx.x;
+        rec = rec && ctl.err_hist != nullptr;
         Out o{1, 0, 0, 0, 0.0};
-        unsigned bsl = 0;   // rotating broadcast slot of once_s / once_d
-        if (threadIdx.x == 0)
+        if (tid == kAcctThread)
             for (int q = 0; q < 5; ++q) acct->ops[q] = 0;
 
         // r_0 = b - A x_0 (step 2) with the stopping-rule denominator
-        double bb, rr;
-        S e, fr{}, d{};
         bool started = false;
         if constexpr (is_narrow<T>::value) {
             if (init) {
+                double bb, rr;
+                S e;
                 if (!ph_init_narrow(init, scale, bb, rr, e)) return o;
                 op(OP_NORM, 2);
                 started = true;
             }
         }
         if (!started) {
-            if (!ilu_pre(sys.x) || !ph_residual(bb, rr, e, true)) return o;
+            if (!ilu_pre(sys.x)) return o;
+            gs.post(kCmdResidual);
+            if (!ph_residual(true)) return o;
             op(OP_NORM, 2);
             op(OP_MATVEC, 1);
         }
-        const double bnrm2 = once_d(bsl, [&] {
-            double t = sqrt(bb);
-            return t == 0.0 ? 1.0 : t;
-        });
-        double err = once_d(bsl, [&] { return sqrt(rr) / bnrm2; });
-        o.err = err;
-        record(rec, 0, err);
-        if (err < tol) { o.flag = 0; return o; }
-        if constexpr (Hook::kActive) hook->reset(err);
-
-        // w_0 = A g_0, c_0 = q_1^H w_0; e_0 = q_1^H r_0 came with r_0
-        S cv;
-        if (!ilu_pre(Gc(0)) || !ph_spmv_c(0, 0, cv)) return o;
-        op(OP_MATVEC);
-        op(OP_DOT);
-        if (threadIdx.x == 0) c[0] = cv;
-        __syncthreads();
-        if (is_zero(cv) || !finite_of(cv)) { o.flag = -1; return o; }
-        op(OP_DOT);
-
-        S omega{}, inv_omega{};
-        int64_t iter = 0;
-        for (int j = 0;; ++j) {
-            o.j = j;
-            for (int i = 1; i <= n - 1; ++i) {
-                o.i = i;
-                // steps 5-8: alpha, x, r, e (and f_1^H r in block 0)
-                S alpha = once_s(bsl, [&] { return e / c[i - 1]; });
-                double r2;
-                S qr;
-                if (!ph_alpha(alpha, i - 1, i, j == 0, r2, qr, fr)) return o;
-                op(OP_SAXPY, 2);
-                op(OP_NORM);
-                err = once_d(bsl, [&] { return sqrt(r2) / bnrm2; });
-                iter++;
-                o.iter = iter;
-                if constexpr (Hook::kActive) {
-                    hook->track(err);
-                    if (err < tol) {
-                        bool conv;
-                        if (!hook->replace(i, j == 0, r2, qr, fr, conv)) return o;
-                        err = once_d(bsl, [&] { return sqrt(r2) / bnrm2; });
-                        hook->reset(err);
-                        if (conv) { o.err = err; o.flag = 0; return o; }
-                    }
-                }
-                o.err = err;
-                record(rec, iter, err);
-                if (!Hook::kActive && err < tol) { o.flag = 0; return o; }
-                if (iter >= maxit) return o;
-                e = qr;
-                op(OP_DOT);
-
-                if (j >= 1) {
-                    // steps 10-18: sweep the rest of block j-1 with q's
-                    S b0 = once_s(bsl, [&] { return -(e / c[i]); });
-                    if (threadIdx.x == 0) bt[i] = b0;
-                    __syncthreads();
-                    op(OP_SAXPY);
-                    op(OP_SCALE);
-                    if (i == n - 1) {
-                        if (!ph_w_last(true, i, inv_omega, true, d)) return o;
-                    } else {
-                        if (!ph_w_first(b0, i, i + 1, d)) return o;
-                        for (int s = i + 1; s <= n - 1; ++s) {
-                            S bs = once_s(bsl, [&] { return -(d / c[s]); });
-                            if (threadIdx.x == 0) bt[s] = bs;
-                            __syncthreads();
-                            op(OP_DOT);
-                            op(OP_SAXPY, 2);
-                            if (s < n - 1) {
-                                if (!ph_w_round(bs, s, i, s + 1, d)) return o;
-                            } else {
-                                if (!ph_w_last(false, i, inv_omega, true, d)) return o;
-                            }
-                        }
-                    }
-                    op(OP_SAXPY);   // omega-correction
-                    // steps 19-22: sweep block j with f's
-                    for (int s = 0; s <= i - 1; ++s) {
-                        S beta = once_s(bsl, [&] { return -(d / c[s]); });
-                        op(OP_DOT);
-                        op(OP_SAXPY);
-                        if (!ph_f_round(beta, s, i, s + 1 <= i - 1 ? s + 1 : -1, d)) return o;
-                    }
-                } else {
-                    // steps 24-29 (block 0)
-                    S beta = once_s(bsl, [&] { return -(fr / c[0]); });
-                    op(OP_DOT);
-                    op(OP_SAXPY);
-                    if (!ph_g_j0(beta, i, i >= 2 ? 1 : -1, d)) return o;
-                    for (int s = 1; s <= i - 1; ++s) {
-                        beta = once_s(bsl, [&] { return -(d / c[s]); });
-                        op(OP_DOT);
-                        op(OP_SAXPY);
-                        if (!ph_f_round(beta, s, i, s + 1 <= i - 1 ? s + 1 : -1, d)) return o;
-                    }
-                }
-                // steps 31-32: w = A g, c = q_{i+1}^H w
-                if (!ilu_pre(Gc(i)) || !ph_spmv_c(i, i, cv)) return o;
-                op(OP_MATVEC);
-                op(OP_DOT);
-                if (threadIdx.x == 0) c[i] = cv;
-                __syncthreads();
-                if (is_zero(cv) || !finite_of(cv)) { o.flag = -1; return o; }
+        if (tid == 0) {
+            sc->e = total(2);
+            const double t0 = sqrt(gs.red->total[0]);
+            const double bn = t0 == 0.0 ? 1.0 : t0, rr = gs.red->total[1], e0 = sqrt(rr) / bn;
+            sc->bnrm2 = bn;
+            sc->rr = rr;
+            sc->err = e0;
+            // sqrt(rr) / bn < tol is impossible above this (1e-12 covers
+            // the roundings; below 1e-290 the exact test decides)
+            const double t = tol * bn, f = t * t * (1.0 + 1e-12);
+            sc->far = f > 1e-290 ? f : 1e-290;
+            sc->iter = 0;
+            sc->flag = 1;
+            sc->exit = 0;
+            sc->j = sc->i = 0;
+            sc->act = sc->conv = 0;
+            record(rec, 0, e0);
+            if (e0 < tol) {
+                sc->flag = 0;
+                sc->exit = 1;
             }
+            if constexpr (Hook::kActive) hook->reset(e0);
+        }
+        consumer_sync();
+        o.err = sc->err;
+        if (sc->exit) {
+            o.flag = sc->flag;
+            return o;
+        }
+        // the producer's first step is the product w_0 = A g_0
+        gs.post(kCmdInner);
+        unsigned sq = gs.seq(), passes = 0;
+        const unsigned pass0 = gs.ring->passes;
 
-            // steps 34-36: alpha, x, u (u kept in r)
-            o.i = n;
-            {
-                S alpha = once_s(bsl, [&] { return e / c[n - 1]; });
-                double u2;
-                S dummy;
-                if (!ph_alpha(alpha, n - 1, -1, false, u2, dummy, fr)) return o;
-                op(OP_SAXPY, 2);
-                op(OP_NORM);
-                err = once_d(bsl, [&] { return sqrt(u2) / bnrm2; });
-                if constexpr (Hook::kActive) {
-                    hook->track(err);
-                    if (err < tol) {
-                        // u (kept in r) replaced by the true residual; the
-                        // omega step then works on the replaced u
-                        bool conv;
-                        S dq, df;
-                        if (!hook->replace(-1, false, u2, dq, df, conv)) return o;
-                        err = once_d(bsl, [&] { return sqrt(u2) / bnrm2; });
-                        hook->reset(err);
-                        if (conv) {
-                            iter++;
-                            o.iter = iter;
-                            o.err = err;
-                            o.flag = 0;
-                            return o;
-                        }
-                    }
-                }
-                o.err = err;
-                if (!Hook::kActive && err < tol) {
-                    iter++;
-                    o.iter = iter;
-                    record(rec, iter, err);
-                    o.flag = 0;
-                    return o;
-                }
-                // step 38: omega = (A u)^H u / ||A u||^2, Eq. 5.1 guard
-                double zz;
-                S zu;
-                if (!ilu_pre(sys.r) || !ph_spmv_z(zz, zu)) return o;
+        int j = 0;
+        for (Step st;; st.advance(n)) {
+            const int i = st.i;
+            bool good = true;
+            switch (st.op) {
+            case P_SPMV_C:
+                // steps 31-32, 51 (and w_0 = A g_0): w = A g, c = q_{i+1}^H w
+                good = ilu_pre(Gc(i)) && ph_spmv_c(i, sq);
                 op(OP_MATVEC);
                 op(OP_DOT);
-                if (zz == 0.0 || !isfinite(zz)) { o.flag = -1; return o; }
+                if (tid == 0) {
+                    const S cv = total(0);
+                    c[i] = cv;
+                    if (is_zero(cv) || !finite_of(cv)) {
+                        sc->flag = -1;
+                        sc->exit = 1;
+                    }
+                    sc->coef = sc->e / cv;
+                }
+                break;
+            case P_ALPHA: {
+                // steps 5-8: alpha, x, r, e (and f_1^H r in block 0); steps
+                // 34-36 at the block's end (u kept in r)
+                const bool hq = i < n, f0 = st.first && hq;
+                // the inner product of c_0 belongs to the first block's start
+                if (st.first && i == 1) op(OP_DOT);
+                good = ph_alpha(sc->coef, hq, f0, sq);
+                op(OP_SAXPY, 2);
+                op(OP_NORM);
+                if (tid == kErrThread) {
+                    sc->j = j;
+                    sc->i = i;
+                    residual_norm<Hook>(gs.red->total[0], hq, false, maxit, rec, tol, hook);
+                }
+                if (hq && tid == 0) alpha_coef(i, f0);
+                break;
+            }
+            case P_SPMV_Z:
+                // step 38: omega = (A u)^H u / ||A u||^2, Eq. 5.1 guard
+                good = ilu_pre(sys.r) && ph_spmv_z(sq);
+                op(OP_MATVEC);
                 op(OP_DOT);
-                if (ctl.kappa > 0.0) op(OP_NORM, 2);
-                omega = once_s(bsl, [&] {
+                if (tid == 0) {
+                    const double zz = gs.red->total[0];
+                    const S zu = total(1);
+                    const bool bad = zz == 0.0 || !isfinite(zz);
                     S om = zu / zz;
                     if (ctl.kappa > 0.0) {
-                        double arho = abs_of(zu) / (sqrt(zz) * sqrt(u2));
+                        const double arho = abs_of(zu) / (sqrt(zz) * sqrt(sc->rr));
                         if (arho < ctl.kappa && arho != 0.0) om = (ctl.kappa * om) / arho;
                     }
-                    return om;
-                });
-                if (is_zero(omega) || !finite_of(omega)) { o.flag = -1; return o; }
-                inv_omega = once_s(bsl, [&] { return recip(omega); });
+                    if (bad || is_zero(om) || !finite_of(om)) {
+                        sc->flag = -1;
+                        sc->exit = 1;
+                    }
+                    sc->act = bad;   // counted below
+                    sc->coef = om;
+                    sc->omega = om;
+                }
+                break;
+            case P_OMEGA:
                 // steps 39-41: x += omega u, r = u - omega A u, e = q_1^H r
-                S q1r;
-                double r2;
-                if (!ph_omega(omega, r2, q1r)) return o;
+                good = ph_omega(sc->coef, sq);
                 op(OP_SAXPY, 2);
                 op(OP_NORM);
-                err = once_d(bsl, [&] { return sqrt(r2) / bnrm2; });
-                iter++;
-                o.iter = iter;
-                if constexpr (Hook::kActive) {
-                    hook->track(err);
-                    if (err < tol || hook->want(err)) {
-                        bool conv;
-                        S df;
-                        if (!hook->replace(0, false, r2, q1r, df, conv)) return o;
-                        err = once_d(bsl, [&] { return sqrt(r2) / bnrm2; });
-                        hook->reset(err);
-                        if (conv) { o.err = err; o.flag = 0; return o; }
-                    }
-                    if (hook->stalled(iter, err)) { o.err = err; return o; }
-                }
-                o.err = err;
-                record(rec, iter, err);
-                if (!Hook::kActive && err < tol) { o.flag = 0; return o; }
-                if (iter >= maxit) return o;
-                e = q1r;
-                op(OP_DOT);
-            }
-            // steps 42-50: sweep block j with q's into slot 0
-            {
-                S b0 = once_s(bsl, [&] { return -(e / c[0]); });
-                if (threadIdx.x == 0) bt[0] = b0;
-                __syncthreads();
-                op(OP_SAXPY);
-                op(OP_SCALE);
-                if (n == 1) {
-                    if (!ph_w_last(true, 0, inv_omega, false, d)) return o;
+                if (tid == kErrThread) residual_norm<Hook>(gs.red->total[0], true, true, maxit, rec, tol, hook);
+                if (tid == 2 * kErrThread) sc->inv_omega = recip(sc->omega);
+                if (tid == 0) omega_coef();
+                break;
+            case P_W_FIRST:
+            case P_W_ROUND: {
+                // steps 10-17, 42-48: sweep the rest of block j-1 with q's
+                const bool wf = st.op == P_W_FIRST;
+                if (wf) {
+                    op(OP_SAXPY);
+                    op(OP_SCALE);
                 } else {
-                    if (!ph_w_first(b0, 0, 1, d)) return o;
-                    for (int s = 1; s <= n - 1; ++s) {
-                        S bs = once_s(bsl, [&] { return -(d / c[s]); });
-                        if (threadIdx.x == 0) bt[s] = bs;
-                        __syncthreads();
-                        op(OP_DOT);
-                        op(OP_SAXPY, 2);
-                        if (s < n - 1) {
-                            if (!ph_w_round(bs, s, 0, s + 1, d)) return o;
-                        } else {
-                            if (!ph_w_last(false, 0, inv_omega, false, d)) return o;
-                        }
-                    }
+                    op(OP_DOT);
+                    op(OP_SAXPY, 2);
                 }
-                op(OP_SAXPY);   // omega-correction
-                // step 51: w = A g, c = q_1^H w
-                if (!ilu_pre(Gc(0)) || !ph_spmv_c(0, 0, cv)) return o;
-                op(OP_MATVEC);
+                good = ph_w(wf, sc->coef, i, sq);
+                if (tid == 0) {
+                    const int s = wf ? i + 1 : st.s + 1;
+                    const S b = -(total(0) / c[s]);
+                    bt[s] = b;
+                    sc->coef = b;
+                }
+                break;
+            }
+            case P_W_LAST:
+                if (i == n - 1) {
+                    op(OP_SAXPY);
+                    op(OP_SCALE);
+                } else {
+                    op(OP_DOT);
+                    op(OP_SAXPY, 2);
+                }
+                op(OP_SAXPY);   // omega-correction (steps 18, 50)
+                good = ph_w_last(i, sq);
+                if (i > 0 && tid == 0) sc->coef = -(total(0) / c[0]);
+                break;
+            default: {   // P_F_ROUND, P_G_J0
+                // steps 19-22 (24-28 in block 0): sweep block j with f's
+                const int s1 = st.op == P_F_ROUND ? st.s + 1 : 1;
+                const bool more = s1 <= i - 1;
                 op(OP_DOT);
-                if (threadIdx.x == 0) c[0] = cv;
-                __syncthreads();
-                if (is_zero(cv) || !finite_of(cv)) { o.flag = -1; return o; }
+                op(OP_SAXPY);
+                good = ph_g(sc->coef, i, more, sq);
+                if (more && tid == 0) sc->coef = -(total(0) / c[s1]);
+                break;
+            }
+            }
+            ++passes;
+            consumer_sync();
+            if (!good) break;
+            if (st.op == P_SPMV_Z) {
+                if (!sc->act) op(OP_DOT);
+                if (!sc->act && ctl.kappa > 0.0) op(OP_NORM, 2);
+            }
+            if constexpr (Hook::kActive) {
+                if (st.op == P_ALPHA || st.op == P_OMEGA) {
+                    if (sc->exit) break;
+                    const bool hq = st.op == P_OMEGA || i < n;
+                    if (sc->act) {
+                        const bool f0 = st.op == P_ALPHA && st.first && hq;
+                        gs.seq() = sq;
+                        double rr;
+                        S qr, fr;
+                        bool conv;
+                        good = hook->replace(st.op == P_OMEGA ? 0 : hq ? i : -1, f0, rr, qr, fr, conv);
+                        sq = gs.seq();
+                        ++passes;
+                        if (!good) break;
+                        if (tid == kErrThread) replaced<Hook>(rr, conv, st.op, hq, maxit, hook);
+                        if (tid == 0 && hq) {
+                            if (st.op == P_OMEGA) omega_coef();
+                            else alpha_coef(i, f0);
+                        }
+                        consumer_sync();
+                        if (sc->exit) break;
+                    }
+                    gs.post(kCmdGo);
+                }
+            }
+            if (sc->exit) break;
+            if (st.op == P_ALPHA && i < n) op(OP_DOT);
+            if (st.op == P_OMEGA) {
+                op(OP_DOT);
+                ++j;
+            }
+        }
+        gs.end_inner(sq, pass0 + passes);
+        gs.seq() = sq;
+        o.flag = gs.ok ? sc->flag : 1;
+        o.iter = sc->iter;
+        o.j = sc->j;
+        o.i = sc->i;
+        o.err = sqrt(sc->rr) / sc->bnrm2;
+        return o;
+    }
+
+    // Thread 0: the coefficient after an update of r within a block
+    // (i: the step's slot): e, then beta~ of the sweep with q's (bt[i]) or,
+    // in block 0, beta of the one with f's.
+    __device__ __forceinline__ void alpha_coef(int i, bool f0) {
+        const S e = total(1);
+        sc->e = e;
+        if (f0) {
+            sc->coef = -(total(1 + DS) / c[0]);
+        } else {
+            const S b = -(e / c[i]);
+            bt[i] = b;
+            sc->coef = b;
+        }
+    }
+    // Thread 0: the coefficient after the omega step.
+    __device__ __forceinline__ void omega_coef() {
+        const S e = total(1);
+        sc->e = e;
+        const S b = -(e / c[0]);
+        bt[0] = b;
+        sc->coef = b;
+    }
+    // Thread kErrThread, after an update of r (or of u at the block's end,
+    // counts = false): iteration count, stopping rule, iteration limit.
+    // The division and the square root of ||r|| / ||b|| are only taken where
+    // the value is recorded or can decide.
+    template <typename Hook>
+    __device__ __forceinline__ void residual_norm(double rr, bool counts, bool block_end, int64_t maxit, bool rec,
+                                                  double tol, Hook *hook) {
+        sc->rr = rr;
+        int64_t iter = sc->iter + (counts ? 1 : 0);
+        sc->iter = iter;
+        bool conv = false;
+        if (Hook::kActive || rec || !(rr > sc->far)) {
+            const double err = sqrt(rr) / sc->bnrm2;
+            conv = err < tol;
+            if constexpr (Hook::kActive) {
+                hook->track(err);
+                sc->act = conv || (block_end && hook->want(err));
+                if (!sc->act) after_norm(err, counts, block_end, maxit, hook);
+                return;
+            }
+            if (conv && !counts) {
+                iter++;
+                sc->iter = iter;
+            }
+            if (counts || conv) record(rec, iter, err);
+        }
+        if (conv) {
+            sc->flag = 0;
+            sc->exit = 1;
+        } else if (counts && iter >= maxit) {
+            sc->exit = 1;
+        }
+    }
+    // Refined mode: the tests that follow the (possibly replaced) residual.
+    template <typename Hook>
+    __device__ __forceinline__ void after_norm(double err, bool counts, bool block_end, int64_t maxit, Hook *hook) {
+        if constexpr (Hook::kActive) {
+            if (block_end && hook->stalled(sc->iter, err)) sc->exit = 1;
+            else if (counts && sc->iter >= maxit) sc->exit = 1;
+        }
+    }
+    template <typename Hook>
+    __device__ __forceinline__ void replaced(double rr, bool conv, int op_, bool hq, int64_t maxit, Hook *hook) {
+        if constexpr (Hook::kActive) {
+            sc->rr = rr;
+            const double err = sqrt(rr) / sc->bnrm2;
+            hook->reset(err);
+            if (conv) {
+                if (!hq) sc->iter += 1;   // the converged half step counts
+                sc->flag = 0;
+                sc->exit = 1;
+            } else {
+                after_norm(err, hq, op_ == P_OMEGA, maxit, hook);
             }
         }
     }

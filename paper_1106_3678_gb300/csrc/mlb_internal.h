@@ -74,8 +74,8 @@ struct BatchPlan {
     unsigned *queue;         // [0]: next of order_small, [1]: next of order_big (zeroed)
     BarrierState *tbar;      // per team: barrier of the team's turns (zeroed)
     int *team_item;          // per team: 2 slots, the turn's position in order_big
-    BarrierState *sbar;      // per position of order_big: the solve's barrier (zeroed)
-    double *spart;           // per position of order_big: 2 * kMaxSums * team doubles
+    BarrierState *sbar;      // per position of order_big: the solve's failure word (zeroed)
+    Slot *sslots;            // per position of order_big: 2 * kMaxSums * team slots (zeroed)
     uint64_t timeout_ns;     // limit of the waits between turns
 };
 // ilu: some item has an ILU(0) preconditioner (the kernel with those passes
@@ -180,7 +180,8 @@ cudaError_t launch_permute(const void *src, void *dst, const int32_t *perm, int6
                            cudaStream_t st);
 
 // Failure-detection self-test of the grid barrier (see the C ABI).
-cudaError_t launch_barrier_selftest(int grid, BarrierState *bs,
+// `slots`: grid + 1 slots, zeroed.
+cudaError_t launch_barrier_selftest(int grid, BarrierState *bs, Slot *slots,
                                     uint64_t timeout_ns, cudaStream_t st);
 
 }  // namespace mlb

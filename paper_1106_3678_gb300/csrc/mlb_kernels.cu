@@ -408,14 +408,15 @@ cudaError_t launch_spmv_qdot_tiled(const SysView<T> &sys, int ne, int64_t maxw, 
 // ===========================================================================
 // failure-detection self-test: a barrier one participant never reaches
 // ===========================================================================
-__global__ void barrier_selftest_kernel(BarrierState *bs, uint64_t timeout_ns) {
-    __shared__ int flag;
-    unsigned epoch = 0;
-    grid_barrier(bs, epoch, gridDim.x + 1, timeout_ns, &flag);
+__global__ void barrier_selftest_kernel(BarrierState *bs, Slot *slots, uint64_t timeout_ns) {
+    if (threadIdx.x >= 32) return;
+    if (threadIdx.x == 0) slot_put(slots + blockIdx.x, 0.0, 1u);
+    double t;
+    slots_sum(slots, gridDim.x + 1, 1u, bs, timeout_ns, t);
 }
 
-cudaError_t launch_barrier_selftest(int grid, BarrierState *bs, uint64_t timeout_ns, cudaStream_t st) {
-    void *args[] = {(void *)&bs, (void *)&timeout_ns};
+cudaError_t launch_barrier_selftest(int grid, BarrierState *bs, Slot *slots, uint64_t timeout_ns, cudaStream_t st) {
+    void *args[] = {(void *)&bs, (void *)&slots, (void *)&timeout_ns};
     return cudaLaunchCooperativeKernel((const void *)barrier_selftest_kernel, dim3(grid), dim3(64), args, 0,
                                        st);
 }

@@ -73,28 +73,38 @@ struct Refiner {
         own_range(v_.nslices, g.nblocks, g.bid, s_lo, s_hi);
     }
 
+    // Producer warp: the tiles of residual().
+    __device__ __forceinline__ int issue(unsigned &sq) {
+        if (v.spt[1] <= 0) return 0;
+        const SliceOffsets off(gs.ring, v.slice_ptr, s_lo, s_hi);
+        return produce_sell_lanes(gs.ring, s_lo, s_hi, v.spt[1], off, v.sval, EW * (int)sizeof(T64), (int)sizeof(T64),
+                                  v.scol, v.b, 1, sq, gs.timeout_ns);
+    }
+
     // r = b - A x in FP64; sums ||b||^2, ||r||^2.
     __device__ __noinline__ bool residual(double &bb, double &rr) {
+        gs.post(kCmdResidual64);
         double acc[2] = {0.0, 0.0};
         const T64 *epi[1] = {v.b};
         T64 *const r = v.r;
-        unsigned sq = gs.seq();   // issued (producer lane) or consumed (consumers) tiles
-        bool okt = sell_spmv<1, EW>(gs.ring, sq, sq, gs.timeout_ns, s_lo, s_hi, v.spt[1], v.slice_ptr, v.scol, v.sval,
-                                v.x, epi, threadIdx.x & 31,
-                                [=](int64_t row, T64 y, const T64 (&e)[1], double(&a)[2]) {
-                                    T64 rv = subT(e[0], y);
-                                    r[row] = rv;
-                                    acc_nrm(&a[0], e[0]);
-                                    acc_nrm(&a[1], rv);
-                                },
-                                acc);
+        unsigned sq = gs.seq();
+        const bool okt = sell_consume<1, EW>(gs.ring, sq, gs.timeout_ns, s_lo, s_hi, v.spt[1], v.slice_ptr, v.scol,
+                                             v.sval, v.x, epi, threadIdx.x & 31,
+                                             [=](int64_t row, T64 y, const T64 (&e)[1], double(&a)[2]) {
+                                                 T64 rv = subT(e[0], y);
+                                                 r[row] = rv;
+                                                 acc_nrm(&a[0], e[0]);
+                                                 acc_nrm(&a[1], rv);
+                                             },
+                                             acc);
         gs.seq() = sq;
         if (!okt) gs.ring->failed = 1;
-        if (!gs.template reduce<2>(acc)) return false;
+        pass_done(gs.ring);
+        if (!gs.template reduce<2>(acc, true)) return false;
         if (gs.ring->failed) { gs.ok = false; return false; }
-        bb = acc[0];
-        rr = acc[1];
-        if (threadIdx.x == 0) {
+        bb = gs.red->total[0];
+        rr = gs.red->total[1];
+        if (threadIdx.x == kAcctThread) {
             acct->bytes += v.nnz * (int64_t)sizeof(T64) + v.nnz / EW * 4 + 4 * (v.N + 1) +
                            3 * v.N * (int64_t)sizeof(T64);
             acct->flops += (DS == 2 ? 8 : 2) * v.nnz + (DS == 2 ? 10 : 5) * v.N;
@@ -112,7 +122,7 @@ struct Refiner {
         static_assert(PW * sizeof(T64) == 32, "an FP32 chunk maps to two FP64 chunks");
         constexpr int CPS = 32 * sizeof(T32) / 16;   // FP32 chunks per slice
         const int64_t c_hi = s_hi * CPS;
-        const int64_t c_start = s_lo * CPS + ((threadIdx.x >> 5) < kConsumerWarps ? threadIdx.x : c_hi);
+        const int64_t c_start = s_lo * CPS + threadIdx.x;
         T64 *const x64 = v.x;
         for (int64_t ch = c_start; ch < c_hi; ch += kConsumers) {
             Pack<T32> d;
@@ -129,7 +139,7 @@ struct Refiner {
             if (zero) reinterpret_cast<uint4 *>(zero)[ch] = make_uint4(0u, 0u, 0u, 0u);
         }
         fence_proxy_async_global();
-        if (threadIdx.x == 0)
+        if (threadIdx.x == kAcctThread)
             acct->bytes += v.N * (int64_t)(2 * sizeof(T64) + (zero ? 2 : 1) * sizeof(T32));
         return gs.sync();
     }
@@ -138,11 +148,11 @@ struct Refiner {
     __device__ __noinline__ bool keep(bool save) {
         constexpr int CPS64 = 32 * sizeof(T64) / 16;   // FP64 chunks per slice
         const int64_t c_hi = s_hi * CPS64;
-        const int64_t c_start = s_lo * CPS64 + ((threadIdx.x >> 5) < kConsumerWarps ? threadIdx.x : c_hi);
+        const int64_t c_start = s_lo * CPS64 + threadIdx.x;
         uint4 *dst = reinterpret_cast<uint4 *>(save ? v.xbest : v.x);
         const uint4 *src = reinterpret_cast<const uint4 *>(save ? v.x : v.xbest);
         for (int64_t ch = c_start; ch < c_hi; ch += kConsumers) dst[ch] = src[ch];
-        if (threadIdx.x == 0) acct->bytes += 2 * v.N * (int64_t)sizeof(T64);
+        if (threadIdx.x == kAcctThread) acct->bytes += 2 * v.N * (int64_t)sizeof(T64);
         return gs.sync();
     }
 
@@ -160,7 +170,8 @@ struct RefineOut {
 };
 
 // Residual replacement of one inner call (see the file comment and
-// Engine::inner).  A per-thread object: every thread holds the same values.
+// Engine::inner).  In shared memory; its state is kept by the engine's
+// kErrThread (thread 0 at the start).
 template <typename T32, typename T64, bool PC, int EW = 1>
 struct RelUpdate {
     static constexpr bool kActive = true;
@@ -199,18 +210,21 @@ struct RelUpdate {
         const T32 *d = E->sys.x;
         if constexpr (PC) {
             if (E->sys.ilu.lu) {
-                if (!E->ilu_solve(E->sys.x, E->sys.ilu.t)) return false;
+                // the iterate's rows of every CTA are read
+                if (!E->gs.sync() || !E->ilu_solve(E->sys.x, E->sys.ilu.t)) return false;
                 d = E->sys.ilu.t;
             }
         }
         if (!R->update(sigma, d, E->sys.x)) return false;
         double bb, r64;
         if (!R->residual(bb, r64)) return false;
-        true_err = sqrt(r64) / bn;
-        conv = true_err < tol;
-        if (!E->ph_replace_narrow(R->v.r, 1.0 / sigma, qcol, f0, rr, qr, fr)) return false;
-        updates++;
-        return true;
+        const double te = sqrt(r64) / bn;
+        conv = te < tol;
+        if (threadIdx.x == 0) {
+            true_err = te;
+            updates++;
+        }
+        return E->ph_replace_narrow(R->v.r, 1.0 / sigma, qcol, f0, rr, qr, fr);
     }
 };
 
@@ -219,7 +233,7 @@ struct RelUpdate {
 // one.
 template <typename T32, typename T64, bool PC, int EW = 1>
 __device__ RefineOut refine_solve(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> &R, const SolveCtl &ctl,
-                                  const RefCtl &rc) {
+                                  const RefCtl &rc, RelUpdate<T32, T64, PC, EW> &hk) {
     RefineOut out{1, 0, 0, __longlong_as_double(0x7ff8000000000000LL)};
     double prev = 0.0;   // true residual at the start of the last inner call
     double best = 0.0;   // true residual of the saved solution xbest
@@ -265,7 +279,10 @@ __device__ RefineOut refine_solve(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> 
         int64_t budget = ctl.maxit - out.iter;
         if (budget > rc.inner_maxit) budget = rc.inner_maxit;
         const double rn = sqrt(rr);
-        RelUpdate<T32, T64, PC, EW> hk{&E, &R, rn, bn, ctl.tol, rc.delta, rc.window, 0.0, INFINITY, 0, err, 0};
+        consumer_sync();   // no thread still reads the last call's state
+        if (threadIdx.x == 0)
+            hk = RelUpdate<T32, T64, PC, EW>{&E, &R, rn, bn, ctl.tol, rc.delta, rc.window, 0.0, INFINITY, 0, err, 0};
+        consumer_sync();
         auto o = E.inner(budget, false, ctl.tol * bn / rn, R.v.r, 1.0 / rn, &hk);
         if (!E.gs.ok) return out;
         out.iter += o.iter;
@@ -282,7 +299,7 @@ __device__ RefineOut refine_solve(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> 
         const T32 *d = E.sys.x;
         if constexpr (PC) {
             if (E.sys.ilu.lu) {
-                if (!E.ilu_solve(E.sys.x, E.sys.ilu.t)) return out;
+                if (!E.gs.sync() || !E.ilu_solve(E.sys.x, E.sys.ilu.t)) return out;
                 d = E.sys.ilu.t;
             }
         }

@@ -20,10 +20,9 @@ namespace mlb {
 // from the current x while the recursive residual met tol but the true
 // residual did not (restart rule of this library), all iterations counted
 // against one maxit; then the true residual; the team's rank-0 CTA writes
-// the result record.
+// the result record.  Consumer threads only.
 template <typename T, bool PC, int EW>
 __device__ void run_fp64_solve(Engine<T, PC, EW> &E, GridSync &gs, const SolveCtl &ctl, Acct &acct, DevResult *res) {
-    using S = typename coef_of<T>::type;
     int64_t total = 0;
     int outer = 0;
     typename Engine<T, PC, EW>::Out o{1, 0, 0, 0, 0.0};
@@ -37,24 +36,23 @@ __device__ void run_fp64_solve(Engine<T, PC, EW> &E, GridSync &gs, const SolveCt
         o = E.inner(ctl.maxit - total, outer == 0, ctl.tol);
         if (!gs.ok) break;
         total += o.iter;
+        gs.sync();   // the residual pass that follows gathers x
         if (o.flag != 0 || o.iter == 0 || total >= ctl.maxit || outer >= ctl.max_outer) break;
         outer++;
     }
-    int64_t ops_last[5];
-    for (int q = 0; q < 5; ++q) ops_last[q] = acct.ops[q];
     double true_rel = __longlong_as_double(0x7ff8000000000000LL);
-    if (gs.ok) {
-        double bb, rr;
-        S qr;
-        if (E.ilu_pre(E.sys.x) && E.ph_residual(bb, rr, qr, false)) {
-            double bn = sqrt(bb);
+    if (gs.ok && E.ilu_pre(E.sys.x)) {
+        gs.post(kCmdResidual);
+        if (E.ph_residual(false)) {
+            double bn = sqrt(gs.red->total[0]);
             if (bn == 0.0) bn = 1.0;
-            true_rel = sqrt(rr) / bn;
+            true_rel = sqrt(gs.red->total[1]) / bn;
             if constexpr (PC) {
                 if (E.sys.ilu.lu) E.ilu_to_x();
             }
         }
     }
+    consumer_sync();   // the accounting is complete
     if (gs.bid == 0 && threadIdx.x == 0) {
         res->flag = o.flag;
         res->j = o.j;
@@ -68,7 +66,7 @@ __device__ void run_fp64_solve(Engine<T, PC, EW> &E, GridSync &gs, const SolveCt
         res->true_relres = true_rel;
         res->bytes = (double)acct.bytes;
         res->flops = (double)acct.flops;
-        for (int q = 0; q < 5; ++q) res->ops[q] = ops_last[q];
+        for (int q = 0; q < 5; ++q) res->ops[q] = acct.ops[q];
         res->ctas = (int32_t)gs.nblocks;
     }
 }
@@ -96,15 +94,27 @@ __device__ __forceinline__ void acct_reset(Acct &acct) {
     __syncthreads();
 }
 
+// One FP64 solve by a CTA: its producer warp and its consumer warps.
+template <typename T, bool PC, int EW>
+__device__ __forceinline__ void run_cta(Engine<T, PC, EW> &E, GridSync &gs, const SolveCtl &ctl, Acct &acct) {
+    if ((threadIdx.x >> 5) == kConsumerWarps) {
+        E.template serve<false>([](unsigned &) { return 0; });
+    } else {
+        run_fp64_solve(E, gs, ctl, acct, ctl.res);
+        gs.post(kCmdExit);
+    }
+    __syncthreads();
+}
+
 template <typename T, bool PC, int EW = 1>
 __global__ void __launch_bounds__(kThreads, 1) solve_kernel(SysView<T> sys, SolveCtl ctl) {
     using S = typename coef_of<T>::type;
     extern __shared__ unsigned char dsm[];
-    __shared__ double red[kRedDoubles];
+    __shared__ RedScratch red;
     __shared__ S cbuf[kMaxN];
     __shared__ S btbuf[kMaxN];
-    __shared__ int sflag;
     __shared__ Acct acct;
+    __shared__ Scalars<S> scal;
     __shared__ TileRing ring;
     __shared__ SysView<T> s_sys;
     __shared__ SolveCtl s_ctl;
@@ -116,15 +126,14 @@ __global__ void __launch_bounds__(kThreads, 1) solve_kernel(SysView<T> sys, Solv
     if (threadIdx.x == 0) {
         s_sys = sys;
         s_ctl = ctl;
-        new (gs_slot.get()) GridSync(ctl.bar, ctl.partials, red, &sflag, ctl.timeout_ns, &ring, seqs);
-        new (e_slot.get()) Engine<T, PC, EW>(s_sys, s_ctl, *gs_slot.get(), cbuf, btbuf, &acct);
+        new (gs_slot.get()) GridSync(ctl.bar, ctl.slots, gridDim.x, blockIdx.x, &red, ctl.timeout_ns, &ring, seqs);
+        new (e_slot.get()) Engine<T, PC, EW>(s_sys, s_ctl, *gs_slot.get(), cbuf, btbuf, &acct, &scal);
     }
     acct_reset(acct);   // includes the __syncthreads that publishes the objects
     GridSync &gs = *gs_slot.get();
     Engine<T, PC, EW> &E = *e_slot.get();
     E.attach();
-    run_fp64_solve(E, gs, s_ctl, acct, s_ctl.res);
-    __syncthreads();
+    run_cta(E, gs, s_ctl, acct);
     ring_drain(&ring, seqs[kConsumers], seqs[0], s_ctl.timeout_ns);
 }
 
@@ -148,7 +157,7 @@ __device__ __forceinline__ int team_next(const BatchPlan &p, unsigned team, unsi
     return q < p.count_big ? q : -1;
 }
 
-// Runs the plan: solve(item index, team size, rank, barrier, partials) for
+// Runs the plan: solve(item index, team size, rank, barrier, slots) for
 // each system this CTA takes (team size 1: this CTA alone).
 template <typename Solve>
 __device__ __forceinline__ void run_batch_plan(const BatchPlan &p, int *sflag, int *s_next, Solve solve) {
@@ -159,7 +168,7 @@ __device__ __forceinline__ void run_batch_plan(const BatchPlan &p, int *sflag, i
             const int q = team_next(p, team, rank, tepoch, turn, sflag, s_next);
             if (q < 0) break;
             solve(p.order_big[q], (unsigned)p.team, rank, p.sbar + q,
-                  p.spart + (size_t)q * 2 * kMaxSums * p.team);
+                  p.sslots + (size_t)q * 2 * kMaxSums * p.team);
         }
     }
     for (;;) {
@@ -167,7 +176,7 @@ __device__ __forceinline__ void run_batch_plan(const BatchPlan &p, int *sflag, i
         __syncthreads();
         const int q = *s_next;
         if (q >= p.count_small) break;
-        solve(p.order_small[q], 1u, 0u, (BarrierState *)nullptr, (double *)nullptr);
+        solve(p.order_small[q], 1u, 0u, (BarrierState *)nullptr, (Slot *)nullptr);
     }
 }
 
@@ -179,11 +188,12 @@ __global__ void __launch_bounds__(kThreads, 1) batch_kernel(const BatchItem<T> *
     using S = typename coef_of<T>::type;
     extern __shared__ unsigned char dsm[];
     __shared__ TileRing ring;
-    __shared__ double red[kRedDoubles];
+    __shared__ RedScratch red;
     __shared__ S cbuf[kMaxN];
     __shared__ S btbuf[kMaxN];
-    __shared__ int sflag;
     __shared__ Acct acct;
+    __shared__ Scalars<S> scal;
+    __shared__ int sflag;
     __shared__ int s_next;
     __shared__ BatchItem<T> item;
     __shared__ SharedSlot<GridSync> gs_slot;
@@ -192,21 +202,19 @@ __global__ void __launch_bounds__(kThreads, 1) batch_kernel(const BatchItem<T> *
     ring_init(&ring, ring_buffer(dsm));
     seqs[threadIdx.x] = 0;
     uint64_t timeout = plan.timeout_ns;
-    run_batch_plan(plan, &sflag, &s_next, [&](int idx, unsigned nb, unsigned rk, BarrierState *bar, double *part) {
+    run_batch_plan(plan, &sflag, &s_next, [&](int idx, unsigned nb, unsigned rk, BarrierState *bar, Slot *slots) {
         if (threadIdx.x == 0) item = items[idx];
         acct_reset(acct);   // includes the __syncthreads that publishes `item`
         timeout = item.ctl.timeout_ns;
         if (threadIdx.x == 0) {
-            GridSync *g = nb > 1 ? new (gs_slot.get()) GridSync(bar, part, nb, rk, red, &sflag, timeout, &ring, seqs)
-                                 : new (gs_slot.get()) GridSync(red, &sflag, timeout, &ring, seqs);
-            new (e_slot.get()) Engine<T, PC>(item.sys, item.ctl, *g, cbuf, btbuf, &acct);
+            GridSync *g = new (gs_slot.get()) GridSync(bar, slots, nb, rk, &red, timeout, &ring, seqs);
+            new (e_slot.get()) Engine<T, PC>(item.sys, item.ctl, *g, cbuf, btbuf, &acct, &scal);
         }
         __syncthreads();
         GridSync &gs = *gs_slot.get();
         Engine<T, PC> &E = *e_slot.get();
         E.attach();
-        run_fp64_solve(E, gs, item.ctl, acct, item.ctl.res);
-        __syncthreads();
+        run_cta(E, gs, item.ctl, acct);
     });
     ring_drain(&ring, seqs[kConsumers], seqs[0], timeout);
 }
@@ -260,34 +268,51 @@ int solve_blocks_per_sm_pc() {
 // ===========================================================================
 // FP32-inner / FP64-refined persistent solve and batch kernels
 // ===========================================================================
+// One refined solve by a CTA: its producer warp and its consumer warps.
+template <typename T32, typename T64, bool PC, int EW>
+__device__ __forceinline__ RefineOut refine_cta(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> &R,
+                                                const SolveCtl &ctl, const RefCtl &rc,
+                                                RelUpdate<T32, T64, PC, EW> &hk) {
+    RefineOut o{1, 0, 0, 0.0};
+    if ((threadIdx.x >> 5) == kConsumerWarps) {
+        E.template serve<true>([&](unsigned &sq) { return R.issue(sq); });
+    } else {
+        o = refine_solve<T32, T64, PC, EW>(E, R, ctl, rc, hk);
+        E.gs.post(kCmdExit);
+    }
+    __syncthreads();
+    return o;
+}
+
 template <typename T32, typename T64, bool PC>
 __global__ void __launch_bounds__(kThreads, 1)
     batch_refine_kernel(const BatchItemR<T32, T64> *items, BatchPlan plan) {
     using S = typename coef_of<T32>::type;
     extern __shared__ unsigned char dsm[];
     __shared__ TileRing ring;
-    __shared__ double red[kRedDoubles];
+    __shared__ RedScratch red;
     __shared__ S cbuf[kMaxN];
     __shared__ S btbuf[kMaxN];
-    __shared__ int sflag;
     __shared__ Acct acct;
+    __shared__ Scalars<S> scal;
+    __shared__ int sflag;
     __shared__ int s_next;
     __shared__ BatchItemR<T32, T64> item;
     __shared__ SharedSlot<GridSync> gs_slot;
     __shared__ SharedSlot<Engine<T32, PC>> e_slot;
     __shared__ SharedSlot<Refiner<T64, T32>> r_slot;
+    __shared__ SharedSlot<RelUpdate<T32, T64, PC>> h_slot;
     __shared__ unsigned seqs[kThreads];   // tile counters, kept across systems
     ring_init(&ring, ring_buffer(dsm));
     seqs[threadIdx.x] = 0;
     uint64_t timeout = plan.timeout_ns;
-    run_batch_plan(plan, &sflag, &s_next, [&](int idx, unsigned nb, unsigned rk, BarrierState *bar, double *part) {
+    run_batch_plan(plan, &sflag, &s_next, [&](int idx, unsigned nb, unsigned rk, BarrierState *bar, Slot *slots) {
         if (threadIdx.x == 0) item = items[idx];
         acct_reset(acct);
         timeout = item.ctl.timeout_ns;
         if (threadIdx.x == 0) {
-            GridSync *g = nb > 1 ? new (gs_slot.get()) GridSync(bar, part, nb, rk, red, &sflag, timeout, &ring, seqs)
-                                 : new (gs_slot.get()) GridSync(red, &sflag, timeout, &ring, seqs);
-            new (e_slot.get()) Engine<T32, PC>(item.sys, item.ctl, *g, cbuf, btbuf, &acct);
+            GridSync *g = new (gs_slot.get()) GridSync(bar, slots, nb, rk, &red, timeout, &ring, seqs);
+            new (e_slot.get()) Engine<T32, PC>(item.sys, item.ctl, *g, cbuf, btbuf, &acct, &scal);
             new (r_slot.get()) Refiner<T64, T32>(item.rv, *g, &acct);
         }
         __syncthreads();
@@ -295,8 +320,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         Engine<T32, PC> &E = *e_slot.get();
         Refiner<T64, T32> &R = *r_slot.get();
         E.attach();
-        RefineOut o = refine_solve<T32, T64, PC>(E, R, item.ctl, item.rc);
-        __syncthreads();
+        const RefineOut o = refine_cta<T32, T64, PC, 1>(E, R, item.ctl, item.rc, *h_slot.get());
         if (gs.bid == 0 && threadIdx.x == 0) {
             DevResult *res = item.ctl.res;
             res->flag = o.flag;
@@ -353,11 +377,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     using S = typename coef_of<T32>::type;
     extern __shared__ unsigned char dsm[];
     __shared__ TileRing ring;
-    __shared__ double red[kRedDoubles];
+    __shared__ RedScratch red;
     __shared__ S cbuf[kMaxN];
     __shared__ S btbuf[kMaxN];
-    __shared__ int sflag;
     __shared__ Acct acct;
+    __shared__ Scalars<S> scal;
     __shared__ SysView<T32> s_sys;
     __shared__ RefView<T64> s_rv;
     __shared__ SolveCtl s_ctl;
@@ -365,6 +389,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __shared__ SharedSlot<GridSync> gs_slot;
     __shared__ SharedSlot<Engine<T32, PC, EW>> e_slot;
     __shared__ SharedSlot<Refiner<T64, T32, EW>> r_slot;
+    __shared__ SharedSlot<RelUpdate<T32, T64, PC, EW>> h_slot;
     __shared__ unsigned seqs[kThreads];
     ring_init(&ring, ring_buffer(dsm));
     seqs[threadIdx.x] = 0;
@@ -373,8 +398,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         s_rv = rv;
         s_ctl = ctl;
         s_rc = rc;
-        GridSync *g = new (gs_slot.get()) GridSync(ctl.bar, ctl.partials, red, &sflag, ctl.timeout_ns, &ring, seqs);
-        new (e_slot.get()) Engine<T32, PC, EW>(s_sys, s_ctl, *g, cbuf, btbuf, &acct);
+        GridSync *g = new (gs_slot.get()) GridSync(ctl.bar, ctl.slots, gridDim.x, blockIdx.x, &red, ctl.timeout_ns, &ring, seqs);
+        new (e_slot.get()) Engine<T32, PC, EW>(s_sys, s_ctl, *g, cbuf, btbuf, &acct, &scal);
         new (r_slot.get()) Refiner<T64, T32, EW>(s_rv, *g, &acct);
     }
     acct_reset(acct);   // includes the __syncthreads that publishes the objects
@@ -382,8 +407,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     Engine<T32, PC, EW> &E = *e_slot.get();
     Refiner<T64, T32, EW> &R = *r_slot.get();
     E.attach();
-    RefineOut o = refine_solve<T32, T64, PC, EW>(E, R, s_ctl, s_rc);
-    __syncthreads();
+    const RefineOut o = refine_cta<T32, T64, PC, EW>(E, R, s_ctl, s_rc, *h_slot.get());
     ring_drain(&ring, seqs[kConsumers], seqs[0], ctl.timeout_ns);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         DevResult *res = ctl.res;

@@ -9,12 +9,19 @@
 // mbarrier (transaction count of the bulk copies) and an "empty" mbarrier
 // (one arrival per consumer warp).  Every wait is bounded.
 //
+// In the solve kernels the producer warp follows the sequence of passes by
+// itself (it depends on n alone) and starts a pass's tiles as soon as every
+// consumer warp has finished the pass before (the "done" mbarrier), while
+// the consumers still reduce that pass's sums over the CTA and the team and
+// work out the next coefficient.  It takes no part in the consumers'
+// barriers, so a copy that waits for the memory system delays nobody.
+//
 // A CTA only ever bulk-loads vector ranges it owns (or read-only data), and
 // a pass never bulk-loads what the same pass writes.  So the only
 // cross-proxy ordering needed is CTA-local and per pass: each consumer
 // thread fences its generic-proxy stores with fence.proxy.async once at the
-// end of a pass, before the CTA barrier after which the producer may issue
-// bulk copies of that data.
+// end of a pass, before its warp's arrival on "done" (or a CTA barrier),
+// after which the producer may issue bulk copies of that data.
 #pragma once
 
 #include <cstdint>
@@ -55,6 +62,17 @@ __device__ __forceinline__ bool mbar_test(uint64_t *b, unsigned phase) {
         : "memory");
     return ok != 0;
 }
+// The same without the hardware's suspended wait (for a waiter that also
+// watches a flag).
+__device__ __forceinline__ bool mbar_probe(uint64_t *b, unsigned phase) {
+    uint32_t ok;
+    asm volatile(
+        "{ .reg .pred p; mbarrier.test_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok)
+        : "r"(smem_addr(b)), "r"(phase)
+        : "memory");
+    return ok != 0;
+}
 // Bounded wait for the phase with parity `phase` to complete.
 __device__ __forceinline__ bool mbar_wait(uint64_t *b, unsigned phase, uint64_t timeout_ns) {
     if (mbar_test(b, phase)) return true;
@@ -87,14 +105,28 @@ __device__ __forceinline__ uint64_t l2_evict_first_policy() {
 }
 __device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
+// Commands of the consumers to the producer warp (TileRing::cmd), handed
+// over by a __syncthreads of the whole CTA.
+enum {
+    kCmdExit,        // this system is done
+    kCmdResidual,    // one residual pass of the engine
+    kCmdResidual64,  // one residual pass of the refined mode's FP64 side
+    kCmdInner,       // the iteration from its first product on
+    kCmdGo,          // (refined mode) go on with the iteration
+};
+
 // Ring state of one CTA (in shared memory; producer and consumers advance
 // their own sequence counters in lock step over the same tiles).
 struct TileRing {
     uint64_t full[kStages];
     uint64_t empty[kStages];
+    uint64_t done;           // completed passes (one arrival per consumer warp)
     unsigned char *buf;      // kStages * kStageBytes, 128-byte aligned
-    unsigned issued;         // tiles issued (producer lane 0 only)
-    unsigned consumed;       // tiles consumed (every consumer thread, uniform)
+    unsigned issued;         // tiles issued (written by the producer where both sides meet)
+    unsigned consumed;       // tiles and passes consumed (written by the consumers there)
+    unsigned passes;
+    int cmd;
+    int stop;                // the iteration ended: the producer returns from its waits
     int failed;              // set when a wait timed out
     // Cache of the SELL-32 slice offsets of this CTA's slice range:
     // soff[i] = slice_ptr[soff_lo + i] - soff_base for i = 0..soff_hi-soff_lo
@@ -110,13 +142,34 @@ __device__ __forceinline__ void ring_init(TileRing *R, unsigned char *buf) {
             mbar_init(&R->full[s], 1);
             mbar_init(&R->empty[s], kConsumerWarps);
         }
+        mbar_init(&R->done, kConsumerWarps);
         R->buf = buf;
         R->failed = 0;
+        R->stop = 0;
+        R->passes = 0;
         R->soff = reinterpret_cast<int32_t *>(buf + (size_t)kStages * kStageBytes);
         R->soff_src = nullptr;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+}
+
+// Barrier of the consumer warps alone.
+__device__ __forceinline__ void consumer_sync() {
+    asm volatile("bar.sync 1, %0;" ::"n"(kConsumers) : "memory");
+}
+
+// Bounded wait of the producer's lane 0: 0 when the phase completed, 1 when
+// the consumers ended the iteration, 2 on a timeout.  Twice the consumers'
+// limit, so that a wait of theirs that gives up is reported as such.
+__device__ __forceinline__ int producer_wait(TileRing *R, uint64_t *b, unsigned phase, uint64_t timeout_ns) {
+    if (mbar_probe(b, phase)) return 0;
+    const uint64_t t0 = globaltimer_ns();
+    for (unsigned it = 1;; ++it) {
+        if (mbar_probe(b, phase)) return 0;
+        if (*(volatile int *)&R->stop) return 1;
+        if ((it & 63u) == 0 && globaltimer_ns() - t0 > 2 * timeout_ns) return 2;
+    }
 }
 
 // Slice offsets cached per CTA (slices of one CTA's share, plus one).
@@ -252,6 +305,74 @@ __device__ __forceinline__ bool consume(TileRing *R, const TileGeom g, unsigned 
     seq = sq;
     fence_proxy_async_global();
     return true;
+}
+
+// End of a consumer's part of a pass in the solve kernels (its stores are
+// fenced for the async proxy): the producer may start the next pass.
+__device__ __forceinline__ void pass_done(TileRing *R) {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(&R->done);
+}
+
+// Producer warp (all 32 lanes): issue every tile of a streaming pass over
+// the chunks [c_lo, c_hi), lane i < ni copying input i from `src` (its own
+// pointer).  Returns 0, 1 (stopped) or 2 (timeout), the same in every lane.
+__device__ __forceinline__ int produce_lanes(TileRing *R, const void *src, int ni, int64_t c_lo, int64_t c_hi,
+                                             unsigned &seq, uint64_t timeout_ns) {
+    const int lane = threadIdx.x & 31, tc = tile_chunks_for(ni);
+    for (int64_t c0 = c_lo; c0 < c_hi; c0 += tc, ++seq) {
+        const int s = (int)(seq % kStages);
+        const unsigned use = seq / kStages;
+        int st = 0;
+        if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u, timeout_ns);
+        st = __shfl_sync(0xffffffffu, st, 0);
+        if (st) return st;
+        const unsigned bytes = (unsigned)(c_hi - c0 < tc ? c_hi - c0 : tc) * 16u;
+        if (lane == 0) mbar_arrive_expect_tx(&R->full[s], bytes * (unsigned)ni);
+        __syncwarp();
+        if (lane < ni)
+            bulk_g2s(R->buf + (size_t)s * kStageBytes + (size_t)lane * tc * 16, (const unsigned char *)src + c0 * 16,
+                     bytes, &R->full[s]);
+    }
+    return 0;
+}
+
+// The same for SELL-32 tiles (see produce_sell): lane 0 copies the values,
+// lane 1 the column indices, lane 2 + i epilogue vector i from `epi` (its
+// own pointer).
+__device__ __forceinline__ int produce_sell_lanes(TileRing *R, int64_t s_lo, int64_t s_hi, int spt,
+                                                  const SliceOffsets &off, const void *sval, int vbytes, int ebytes,
+                                                  const int32_t *scol, const void *epi, int ne, unsigned &seq,
+                                                  uint64_t timeout_ns) {
+    const uint64_t pol = l2_evict_first_policy();
+    const int lane = threadIdx.x & 31;
+    for (int64_t s0 = s_lo; s0 < s_hi; s0 += spt, ++seq) {
+        const int s = (int)(seq % kStages);
+        const unsigned use = seq / kStages;
+        int st = 0;
+        if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u, timeout_ns);
+        st = __shfl_sync(0xffffffffu, st, 0);
+        if (st) return st;
+        const int64_t s1 = s0 + spt < s_hi ? s0 + spt : s_hi;
+        const int64_t e0 = off(s0);
+        const unsigned nv = (unsigned)(off(s1) - e0);
+        const unsigned bv = nv * (unsigned)vbytes, bc = nv * 4u;
+        const unsigned be = (unsigned)(s1 - s0) * 32u * (unsigned)ebytes;
+        if (lane == 0) mbar_arrive_expect_tx(&R->full[s], bv + bc + be * (unsigned)ne);
+        __syncwarp();
+        unsigned char *const dst = R->buf + (size_t)s * kStageBytes;
+        if (lane < 2) {
+            if (nv > 0)
+                bulk_g2s_hint(lane == 0 ? dst : dst + bv,
+                              lane == 0 ? (const unsigned char *)sval + e0 * vbytes
+                                        : (const unsigned char *)(scol + e0),
+                              lane == 0 ? bv : bc, &R->full[s], pol);
+        } else if (lane < 2 + ne) {
+            bulk_g2s(dst + bv + bc + (size_t)(lane - 2) * spt * 32 * ebytes,
+                     (const unsigned char *)epi + s0 * 32 * ebytes, be, &R->full[s]);
+        }
+    }
+    return 0;
 }
 
 // SELL-32 tiles: `spt` consecutive slices [s0, s0+spt) of this CTA's slice
