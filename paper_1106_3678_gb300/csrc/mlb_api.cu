@@ -38,6 +38,10 @@ struct mlb_handle {
     int64_t ilu_nnz = 0;
     int32_t *ilu_lcnt = nullptr, *ilu_ucnt = nullptr, *ilu_lell_c = nullptr, *ilu_uell_c = nullptr;
     void *ilu_lell_a = nullptr, *ilu_uell_a = nullptr, *ilu_udiag = nullptr;
+    IluLevel *ilu_llev = nullptr, *ilu_ulev = nullptr;    // few levels: the streamed form
+    int32_t *ilu_lmeta = nullptr, *ilu_umeta = nullptr;
+    int ilu_maxw = 0;
+    int64_t ilu_nel = 0, ilu_neu = 0, ilu_ndiag = 0;      // values in lell, uell, udiag
     // refined mode with ILU(0): FP32 copies of the factor values and an
     // FP32 work vector for M^{-1}
     void *ilu_lu32 = nullptr, *ilu_t32 = nullptr, *ilu_lell_a32 = nullptr, *ilu_uell_a32 = nullptr,
@@ -304,7 +308,6 @@ SysView<T> make_view(const mlb_handle *h) {
     v.sval = (const T *)h->sval;
     set_spt(v.spt, h->maxw, sizeof(T), h->spt_cap, h->ew);
     v.ew = h->ew;
-    v.narrow_rows = h->maxw <= 7 ? 1 : 0;
     v.Q = (const T *)h->Q;
     v.F = (const T *)h->F;
     v.G = (T *)h->G;
@@ -330,6 +333,11 @@ SysView<T> make_view(const mlb_handle *h) {
         v.ilu.t = (T *)h->ilu_t;
         v.ilu.lcnt = h->ilu_lcnt;
         v.ilu.ucnt = h->ilu_ucnt;
+        v.ilu.llev = h->ilu_llev;
+        v.ilu.ulev = h->ilu_ulev;
+        v.ilu.lmeta = (const int2 *)h->ilu_lmeta;
+        v.ilu.umeta = (const int2 *)h->ilu_umeta;
+        v.ilu.spt = ilu_slices_per_tile(h->ilu_maxw, sizeof(v.Q[0]));
         v.ilu.lell_c = h->ilu_lell_c;
         v.ilu.uell_c = h->ilu_uell_c;
         v.ilu.lell_a = (const T *)h->ilu_lell_a;
@@ -351,7 +359,6 @@ SysView<T32> make_view32(const mlb_handle *h) {
     v.sval = (const T32 *)h->sval32;
     set_spt(v.spt, h->maxw, sizeof(T32), h->spt_cap, h->ew);
     v.ew = h->ew;
-    v.narrow_rows = h->maxw <= 7 ? 1 : 0;
     v.Q = (const T32 *)h->Q32;
     v.F = (const T32 *)h->F32;
     v.G = (T32 *)h->G32;
@@ -377,6 +384,11 @@ SysView<T32> make_view32(const mlb_handle *h) {
         v.ilu.t = (T32 *)h->ilu_t32;
         v.ilu.lcnt = h->ilu_lcnt;
         v.ilu.ucnt = h->ilu_ucnt;
+        v.ilu.llev = h->ilu_llev;
+        v.ilu.ulev = h->ilu_ulev;
+        v.ilu.lmeta = (const int2 *)h->ilu_lmeta;
+        v.ilu.umeta = (const int2 *)h->ilu_umeta;
+        v.ilu.spt = ilu_slices_per_tile(h->ilu_maxw, sizeof(v.Q[0]));
         v.ilu.lell_c = h->ilu_lell_c;
         v.ilu.uell_c = h->ilu_uell_c;
         v.ilu.lell_a = (const T32 *)h->ilu_lell_a32;
@@ -669,21 +681,37 @@ int create_impl(mlb_handle *h, const mlb_matrix *A, const mlb_matrix *AH, const 
         MLB_CUDA(cudaMemcpy(h->ilu_urows, ih.urows.data(), (size_t)N * 4, cudaMemcpyHostToDevice));
         MLB_CUDA(cudaMemcpy(h->ilu_uptr, ih.uptr.data(), ih.uptr.size() * 4, cudaMemcpyHostToDevice));
         MLB_CUDA(cudaMemsetAsync(h->ilu_t, 0, vb, st));
-        const size_t ne = (size_t)kIluEll * N;
+        const size_t nel = ih.lell_c.size(), neu = ih.uell_c.size();
+        h->ilu_nel = (int64_t)nel;
+        h->ilu_neu = (int64_t)neu;
+        const size_t ndiag = ih.udiag.size() / es;
+        h->ilu_ndiag = (int64_t)ndiag;
+        h->ilu_maxw = ih.maxw;
+        auto up = [&](auto **p, const auto &v) {
+            using E = typename std::decay_t<decltype(v)>::value_type;
+            if (const int rca = dev_alloc_t(h, p, v.size() * sizeof(E))) return rca;
+            MLB_CUDA(cudaMemcpy(*p, v.data(), v.size() * sizeof(E), cudaMemcpyHostToDevice));
+            return MLB_OK;
+        };
+        if (ih.wide) {
+            if ((rc = up(&h->ilu_llev, ih.llev)) || (rc = up(&h->ilu_ulev, ih.ulev)) ||
+                (rc = up(&h->ilu_lmeta, ih.lmeta)) || (rc = up(&h->ilu_umeta, ih.umeta)))
+                return rc;
+        }
         if ((rc = dev_alloc_t(h, &h->ilu_lcnt, (size_t)N * 4))) return rc;
         if ((rc = dev_alloc_t(h, &h->ilu_ucnt, (size_t)N * 4))) return rc;
-        if ((rc = dev_alloc_t(h, &h->ilu_lell_c, ne * 4))) return rc;
-        if ((rc = dev_alloc_t(h, &h->ilu_uell_c, ne * 4))) return rc;
-        if ((rc = dev_alloc(h, &h->ilu_lell_a, ne * es))) return rc;
-        if ((rc = dev_alloc(h, &h->ilu_uell_a, ne * es))) return rc;
-        if ((rc = dev_alloc(h, &h->ilu_udiag, (size_t)N * es))) return rc;
+        if ((rc = dev_alloc_t(h, &h->ilu_lell_c, nel * 4))) return rc;
+        if ((rc = dev_alloc_t(h, &h->ilu_uell_c, neu * 4))) return rc;
+        if ((rc = dev_alloc(h, &h->ilu_lell_a, nel * es))) return rc;
+        if ((rc = dev_alloc(h, &h->ilu_uell_a, neu * es))) return rc;
+        if ((rc = dev_alloc(h, &h->ilu_udiag, ndiag * es))) return rc;
         MLB_CUDA(cudaMemcpy(h->ilu_lcnt, ih.lcnt.data(), (size_t)N * 4, cudaMemcpyHostToDevice));
         MLB_CUDA(cudaMemcpy(h->ilu_ucnt, ih.ucnt.data(), (size_t)N * 4, cudaMemcpyHostToDevice));
-        MLB_CUDA(cudaMemcpy(h->ilu_lell_c, ih.lell_c.data(), ne * 4, cudaMemcpyHostToDevice));
-        MLB_CUDA(cudaMemcpy(h->ilu_uell_c, ih.uell_c.data(), ne * 4, cudaMemcpyHostToDevice));
-        MLB_CUDA(cudaMemcpy(h->ilu_lell_a, ih.lell_a.data(), ne * es, cudaMemcpyHostToDevice));
-        MLB_CUDA(cudaMemcpy(h->ilu_uell_a, ih.uell_a.data(), ne * es, cudaMemcpyHostToDevice));
-        MLB_CUDA(cudaMemcpy(h->ilu_udiag, ih.udiag.data(), (size_t)N * es, cudaMemcpyHostToDevice));
+        MLB_CUDA(cudaMemcpy(h->ilu_lell_c, ih.lell_c.data(), nel * 4, cudaMemcpyHostToDevice));
+        MLB_CUDA(cudaMemcpy(h->ilu_uell_c, ih.uell_c.data(), neu * 4, cudaMemcpyHostToDevice));
+        MLB_CUDA(cudaMemcpy(h->ilu_lell_a, ih.lell_a.data(), nel * es, cudaMemcpyHostToDevice));
+        MLB_CUDA(cudaMemcpy(h->ilu_uell_a, ih.uell_a.data(), neu * es, cudaMemcpyHostToDevice));
+        MLB_CUDA(cudaMemcpy(h->ilu_udiag, ih.udiag.data(), ndiag * es, cudaMemcpyHostToDevice));
     }
 
     // reordering (multicolour ILU(0)): the permutation and a staging vector
@@ -793,19 +821,17 @@ int create_impl(mlb_handle *h, const mlb_matrix *A, const mlb_matrix *AH, const 
             MLB_CUDA(launch_narrow((const double *)h->F, (float *)h->F32, ld * (int64_t)(n - 1) * (int64_t)es / 8,
                                    st));
         if (has_ilu(h)) {
-            const int64_t N = h->N;
-            const size_t ne = (size_t)kIluEll * N;
             if ((rc = dev_alloc(h, &h->ilu_lu32, (size_t)h->ilu_nnz * es / 2))) return rc;
             if ((rc = dev_alloc(h, &h->ilu_t32, vb32))) return rc;
-            if ((rc = dev_alloc(h, &h->ilu_lell_a32, ne * es / 2))) return rc;
-            if ((rc = dev_alloc(h, &h->ilu_uell_a32, ne * es / 2))) return rc;
-            if ((rc = dev_alloc(h, &h->ilu_udiag32, (size_t)N * es / 2))) return rc;
+            if ((rc = dev_alloc(h, &h->ilu_lell_a32, (size_t)h->ilu_nel * es / 2))) return rc;
+            if ((rc = dev_alloc(h, &h->ilu_uell_a32, (size_t)h->ilu_neu * es / 2))) return rc;
+            if ((rc = dev_alloc(h, &h->ilu_udiag32, (size_t)h->ilu_ndiag * es / 2))) return rc;
             MLB_CUDA(cudaMemsetAsync(h->ilu_t32, 0, vb32, st));
             const int64_t dpe = (int64_t)es / 8;   // doubles per value
             MLB_CUDA(launch_narrow((const double *)h->ilu_lu, (float *)h->ilu_lu32, h->ilu_nnz * dpe, st));
-            MLB_CUDA(launch_narrow((const double *)h->ilu_lell_a, (float *)h->ilu_lell_a32, (int64_t)ne * dpe, st));
-            MLB_CUDA(launch_narrow((const double *)h->ilu_uell_a, (float *)h->ilu_uell_a32, (int64_t)ne * dpe, st));
-            MLB_CUDA(launch_narrow((const double *)h->ilu_udiag, (float *)h->ilu_udiag32, N * dpe, st));
+            MLB_CUDA(launch_narrow((const double *)h->ilu_lell_a, (float *)h->ilu_lell_a32, h->ilu_nel * dpe, st));
+            MLB_CUDA(launch_narrow((const double *)h->ilu_uell_a, (float *)h->ilu_uell_a32, h->ilu_neu * dpe, st));
+            MLB_CUDA(launch_narrow((const double *)h->ilu_udiag, (float *)h->ilu_udiag32, h->ilu_ndiag * dpe, st));
         }
     }
 

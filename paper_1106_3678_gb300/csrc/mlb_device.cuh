@@ -294,7 +294,7 @@ __device__ __forceinline__ Slot slot_load(const Slot *p) {
 // recorded a failure in bs.  Returns false (uniformly in the warp) then.
 __device__ __forceinline__ bool slots_sum(const Slot *p, unsigned G, unsigned epoch, BarrierState *bs,
                                           uint64_t timeout_ns, double &sum) {
-    constexpr int M = 8;   // slots per lane of one round
+    constexpr int M = 5;   // slots per lane of one round (160 CTAs: every SM of this GPU)
     const unsigned lane = threadIdx.x & 31;
     double total = 0.0;
     for (unsigned b0 = 0; b0 < G; b0 += 32 * M) {
@@ -334,13 +334,12 @@ __device__ __forceinline__ bool slots_sum(const Slot *p, unsigned G, unsigned ep
                 if (__shfl_sync(0xffffffffu, stop, 0)) return false;
             }
         }
-        // the pair tree over 8 terms; terms past the team are zero, so the
+        // the pair tree over 5 terms; terms past the team are zero, so the
         // adds that cannot change the sum are left out
         double part = x[0];
         if (left > 32) part = part + x[1];
         if (left > 64) part = part + (x[2] + x[3]);
-        if (left > 160) part = part + ((x[4] + x[5]) + (x[6] + x[7]));
-        else if (left > 128) part = part + x[4];
+        if (left > 128) part = part + x[4];
         total = b0 == 0 ? part : total + part;
     }
 #pragma unroll

@@ -101,10 +101,15 @@ struct Scalars {
     double rr;       // ||r||^2 (or ||u||^2) of the last update
     double far;      // a ||r||^2 above this is certainly not below tol
     double err;      // ||r|| / ||b|| where it was worked out
-    int64_t iter;
+    double tol;
+    int64_t iter, maxit;
+    unsigned passes; // passes the consumers have finished (thread 0)
+    int rec;         // the residual history is recorded
+    int block;       // j of the running block (thread kErrThread)
     int exit;        // the iteration ends
     int flag, j, i;  // its result
     int act;         // (refined mode) replace the residual
+    int bad;         // ||A u||^2 was zero or not finite
     int conv;        // (refined mode) the true residual met its tolerance
 };
 
@@ -115,6 +120,20 @@ struct Scalars {
 // A (M^{-1} v).  Rows are grouped by level for the triangular solves: a
 // row of level l depends only on rows of lower levels (of L, or of U taken
 // from the last row upwards).  lu == nullptr: no ILU(0) preconditioner.
+// A level of the streamed form of the factors (see IluHost::llev): `ns`
+// slices of 32 rows, `w` entries wide.
+struct IluLevel {
+    int64_t e0;   // its first entry
+    int32_t m0;   // its first slice
+    int32_t ns, w, pad;
+};
+// Slices per tile of that form: values, columns, (row, count) pairs and U's
+// diagonal; 0 when one slice does not fit a stage.
+inline int ilu_slices_per_tile(int64_t w, size_t vbytes) {
+    const int64_t spt = kStageBytes / (32 * (w * (int64_t)(vbytes + 4) + 8 + (int64_t)vbytes));
+    return (int)(spt < kConsumerWarps ? spt : kConsumerWarps);
+}
+
 template <typename T>
 struct IluView {
     const int64_t *rp;          // N+1; columns increase within each row
@@ -132,6 +151,11 @@ struct IluView {
     // kIluEll entries of position q at e * N + q, U's diagonal at q
     const int32_t *lcnt, *ucnt, *lell_c, *uell_c;
     const T *lell_a, *uell_a, *udiag;
+    // few levels: the streamed form (else null); lell/uell and udiag then
+    // hold its entries
+    const IluLevel *llev, *ulev;
+    const int2 *lmeta, *umeta;
+    int spt;                    // its slices per tile
 };
 
 // Device view of one linear system.  Vectors have leading dimension `ld`
@@ -145,7 +169,6 @@ struct SysView {
     const T *sval;
     int spt[3];                 // slices per SpMV tile with 0, 1, 2 epilogue vectors (<= 0: no tiles)
     int ew;                     // 1: scalar entries; 3: 3x3-block entries (three values, one column)
-    int narrow_rows;            // no slice is wider than 7 entries (blocks)
     const T *Q;                 // ld x n
     const T *F;                 // ld x (n-1), F = A^H Q(:,0:n-2)
     T *G, *W;                   // ld x n rings
@@ -167,6 +190,33 @@ struct SolveCtl {
     DevResult *res;
     uint64_t timeout_ns;
 };
+
+// The CTA's views, controls and iteration state (see the_ring).
+template <typename T>
+__device__ __forceinline__ SysView<T> &the_sys() {
+    __shared__ SysView<T> v;
+    return v;
+}
+__device__ __forceinline__ SolveCtl &the_ctl() {
+    __shared__ SolveCtl c;
+    return c;
+}
+__device__ __forceinline__ Acct &the_acct() {
+    __shared__ Acct a;
+    return a;
+}
+template <typename S>
+struct IterState {
+    S c[kMaxN];
+    S bt[kMaxN];
+    Scalars<S> sc;
+    int s_lo, s_hi;   // slices this CTA owns
+};
+template <typename S>
+__device__ __forceinline__ IterState<S> &the_iter() {
+    __shared__ IterState<S> s;
+    return s;
+}
 
 // ---- element helpers used by Engine ---------------------------------------
 __device__ __forceinline__ double subT(double a, double b) { return a - b; }
@@ -278,45 +328,6 @@ __device__ __forceinline__ T sell_slice_sum3(const int32_t *cp, const T *vp, int
     }
     return sum;
 }
-template <typename T>
-__device__ __noinline__ T sell_slice_sum3_wide(const int32_t *cp, const T *vp, int w, const T *xin) {
-    T sum{};
-    for (int k = 0; k < w; ++k) {
-        const int32_t c = cp[32 * k];
-        const T x0 = xin[c], x1 = xin[c + 1], x2 = xin[c + 2];
-        sum = efma(vp[96 * k], x0, sum);
-        sum = efma(vp[96 * k + 1], x1, sum);
-        sum = efma(vp[96 * k + 2], x2, sum);
-    }
-    return sum;
-}
-
-// Row sum of a slice wider than the pipelined path takes, from a stage
-// (values at vp, column indices at cp, lane-strided by 32).  Out of line
-// so that its registers do not weigh on the pipelined loop.
-template <typename T>
-__device__ __noinline__ T sell_slice_sum_wide(const int32_t *cp, const T *vp, int w, const T *xin) {
-    T sum{};
-    int k = 0;
-    for (; k + 8 <= w; k += 8) {
-        T xw[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) xw[u] = xin[cp[32 * (k + u)]];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) sum = efma(vp[32 * (k + u)], xw[u], sum);
-    }
-    if (k < w) {
-        T xw[7];
-#pragma unroll
-        for (int u = 0; u < 7; ++u)
-            if (k + u < w) xw[u] = xin[cp[32 * (k + u)]];
-#pragma unroll
-        for (int u = 0; u < 7; ++u)
-            if (k + u < w) sum = efma(vp[32 * (k + u)], xw[u], sum);
-    }
-    return sum;
-}
-
 // SELL-32 product over the slices [s_lo, s_hi) owned by this CTA: for
 // every row, y = sum_k a_{row,k} xin[col_k], then fin(row, y, e, acc) where
 // e[i] = epi[i][row] for the NE epilogue vectors (rows of this CTA).  The
@@ -329,28 +340,28 @@ __device__ __noinline__ T sell_slice_sum_wide(const int32_t *cp, const T *vp, in
 // and the only global loads on a warp's critical path are the gathers.
 // The epilogue's stores are fenced for later bulk (async-proxy) reads.
 // EW = 3: the 3x3-block storage (see sell_slice_sum3); slice offsets and
-// widths then count blocks.  Slices up to PW entries wide take the
-// pipelined path (PW registers of gathered x per thread), wider ones a
-// direct loop.  Returns false when a tile wait timed out.
+// widths then count blocks.  The first PW entries of a row are pipelined
+// (PW registers of gathered x per thread), further ones follow in batches.
+// No call here: a call in a kernel's loop costs every pass of the kernel
+// registers (saved across it by convention).  Returns false when a tile wait timed out.
 //
 // sell_consume is the consumer warps' part.
 template <int NE, int EW = 1, int PW = 8, typename T, typename Fin, typename AccArr>
-__device__ __forceinline__ bool sell_consume(TileRing *R, unsigned &cseq, uint64_t timeout_ns, int64_t s_lo,
-                                             int64_t s_hi, int spt, const int64_t *slice_ptr, const int32_t *scol,
-                                             const T *sval, const T *xin, const T *const (&epi)[NE > 0 ? NE : 1],
-                                             int lane, Fin fin, AccArr &acc) {
+__device__ __forceinline__ bool sell_consume(TileRing *R, unsigned &cseq, int s_lo, int s_hi, int spt,
+                                             const int64_t *slice_ptr, const int32_t *scol, const T *sval,
+                                             const T *xin, const T *const (&epi)[NE > 0 ? NE : 1], Fin fin,
+                                             AccArr &acc) {
     static_assert(EW == 1 || EW == 3, "scalar entries or 3x3 blocks");
     constexpr int kPipeW = PW;
     constexpr int NEA = NE > 0 ? NE : 1;
-    const int cw = threadIdx.x >> 5;
-    const SliceOffsets off(R, slice_ptr, s_lo, s_hi);
-    bool ok = true;
+    const int cw = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (spt <= 0) {
         // slices too wide for one stage: direct loads, no pipeline
-        for (int64_t s = s_lo + cw; s < s_hi; s += kConsumerWarps) {
+        const SliceOffsets off(R, slice_ptr, s_lo, s_hi);
+        for (int s = s_lo + cw; s < s_hi; s += kConsumerWarps) {
             const int64_t o = off(s);
             const int w = (int)((off(s + 1) - o) >> 5);
-            const int64_t row = s * 32 + lane;
+            const int64_t row = (int64_t)s * 32 + lane;
             T e[NEA];
 #pragma unroll
             for (int i = 0; i < NE; ++i) e[i] = epi[i][row];
@@ -368,105 +379,112 @@ __device__ __forceinline__ bool sell_consume(TileRing *R, unsigned &cseq, uint64
     struct Job {
         int st, o, nv, w;
     };
-    const int nt = (int)((s_hi - s_lo + spt - 1) / spt);
-    // copies in registers (the epilogue's generic stores could alias them)
-    unsigned char *const rbuf = R->buf;
-    const unsigned cs0 = cseq;
-    auto stage_of = [&](const Job &j) { return rbuf + (size_t)j.st * kStageBytes; };
+    const bool cached = R->soff_src == slice_ptr && R->soff_lo == s_lo && R->soff_hi == s_hi;
+    // entries from slice a to slice b of this CTA's range
+    auto span = [&](int a, int b) {
+        if (cached) return the_soff()[b - s_lo] - the_soff()[a - s_lo];
+        return (int)(__ldg(slice_ptr + b) - __ldg(slice_ptr + a));
+    };
+    auto stage_of = [&](const Job &j) { return the_stages() + j.st * kStageBytes; };
     auto vals = [&](const Job &j) { return reinterpret_cast<const T *>(stage_of(j)) + EW * (j.o + lane); };
     auto cols = [&](const Job &j) {
-        return reinterpret_cast<const int32_t *>(stage_of(j) + (size_t)j.nv * EW * sizeof(T)) + j.o + lane;
+        return reinterpret_cast<const int32_t *>(stage_of(j) + j.nv * (int)(EW * sizeof(T))) + j.o + lane;
     };
     // epilogue entry i of this warp's row in the tile
     auto epv = [&](const Job &j, int i) {
-        return reinterpret_cast<const T *>(stage_of(j) + (size_t)j.nv * (EW * sizeof(T) + 4))[(i * spt + cw) * 32 +
-                                                                                             lane];
+        return reinterpret_cast<const T *>(stage_of(j) + j.nv * (int)(EW * sizeof(T) + 4))[(i * spt + cw) * 32 + lane];
     };
-    // wait for tile t and locate this warp's slice in it
-    auto locate = [&](int t, Job &j) -> bool {
-        const unsigned q = cs0 + (unsigned)t;
+    // wait for the tile that starts at slice s0 (its number q) and locate
+    // this warp's slice in it
+    auto locate = [&](int s0, unsigned q, Job &j) -> bool {
         j.st = (int)(q % kStages);
         j.o = j.nv = 0;
         j.w = -1;
-        if (!mbar_wait(&R->full[j.st], (q / kStages) & 1u, timeout_ns)) return false;
-        const int64_t s0 = s_lo + (int64_t)t * spt;
-        const int64_t s1 = s0 + spt < s_hi ? s0 + spt : s_hi;
-        const int64_t s = s0 + cw;
+        if (!mbar_wait(R, &R->full[j.st], (q / kStages) & 1u)) return false;
+        const int s1 = s0 + spt < s_hi ? s0 + spt : s_hi, s = s0 + cw;
         if (s < s1) {
-            const int64_t e0 = off(s0), es = off(s);
-            j.nv = (int)(off(s1) - e0);
-            j.o = (int)(es - e0);
-            j.w = (int)((off(s + 1) - es) >> 5);
+            j.nv = span(s0, s1);
+            j.o = span(s0, s);
+            j.w = span(s, s + 1) >> 5;
         }
         return true;
     };
-    auto row_of = [&](int t) { return (s_lo + (int64_t)t * spt + cw) * 32 + lane; };
-    int done = 0;
-    // x gathers of slice j into xv (pipelined path: widths up to kPipeW)
-    auto gather = [&](const Job &j, T (&xv)[kPipeW * EW]) {
-        if (j.w >= 0 && j.w <= kPipeW) {
-            const int32_t *cp = cols(j);
-#pragma unroll
-            for (int u = 0; u < kPipeW; ++u)
-                if (u < j.w) {
-                    const int32_t c = cp[32 * u];
-#pragma unroll
-                    for (int q = 0; q < EW; ++q) xv[EW * u + q] = xin[c + q];
-                }
-        }
-    };
-    // Tile t (slice jc, its x in xc): the FMAs, each followed by the gather
-    // of slice jn (tile t+1, when `more`) into the register it has just
-    // read; then the epilogue and the release of the stage.  (Gathering two
-    // tiles ahead measured slower: 228 against 206 us per iteration at 128^3.)
-    auto step = [&](int t, const Job &jc, T (&xc)[kPipeW * EW], const Job &jn, bool more) {
-        const bool na = jc.w >= 0 && jc.w <= kPipeW;
-        const bool nb = more && jn.w >= 0 && jn.w <= kPipeW;
+    // Tile jc (its x in xc; its warp's slice s): the FMAs, each followed by
+    // the gather of the slice of tile jn (when `more`) into the register it
+    // has just read; then the epilogue and the release of the stage.
+    // (Gathering two tiles ahead measured slower: 228 against 206 us per
+    // iteration at 128^3.)
+    auto step = [&](int s, const Job &jc, T (&xc)[kPipeW * EW], const Job &jn, bool more) {
         const T *va = vals(jc);
         const int32_t *cb = cols(jn);
         T sum{};
 #pragma unroll
         for (int u = 0; u < kPipeW; ++u) {
-            if (na && u < jc.w) {
+            if (u < jc.w) {
 #pragma unroll
                 for (int q = 0; q < EW; ++q) sum = efma(va[32 * EW * u + q], xc[EW * u + q], sum);
             }
-            if (nb && u < jn.w) {
+            if (more && u < jn.w) {
                 const int32_t c = cb[32 * u];
 #pragma unroll
                 for (int q = 0; q < EW; ++q) xc[EW * u + q] = xin[c + q];
             }
         }
-        if (jc.w > kPipeW) {
-            if constexpr (EW == 3) sum = sell_slice_sum3_wide(cols(jc), va, jc.w, xin);
-            else sum = sell_slice_sum_wide(cols(jc), va, jc.w, xin);
+        constexpr int B = EW == 3 ? 1 : sizeof(T) == 16 ? 2 : 4;   // entries of a wide row at a time
+        const int32_t *ca = cols(jc);
+        for (int k = kPipeW; k < jc.w; k += B) {
+            T xw[B * EW];
+#pragma unroll
+            for (int u = 0; u < B; ++u)
+                if (k + u < jc.w) {
+                    const int32_t c = ca[32 * (k + u)];
+#pragma unroll
+                    for (int q = 0; q < EW; ++q) xw[EW * u + q] = xin[c + q];
+                }
+#pragma unroll
+            for (int u = 0; u < B; ++u)
+                if (k + u < jc.w) {
+#pragma unroll
+                    for (int q = 0; q < EW; ++q) sum = efma(va[32 * EW * (k + u) + q], xw[EW * u + q], sum);
+                }
         }
         if (jc.w >= 0) {
             T e[NEA];
 #pragma unroll
             for (int i = 0; i < NE; ++i) e[i] = epv(jc, i);
-            fin(row_of(t), sum, e, acc);
+            fin((int64_t)s * 32 + lane, sum, e, acc);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&R->empty[jc.st]);
-        ++done;
     };
-    if (nt > 0) {
+    bool ok = true;
+    unsigned q = cseq;
+    if (s_lo < s_hi) {
         Job ja, jb;
         T xv[kPipeW * EW];
-        ok = locate(0, ja);
-        if (ok) gather(ja, xv);
-        for (int t = 0; ok && t < nt; ++t) {
-            const bool more = t + 1 < nt;
-            if (more && !locate(t + 1, jb)) {
+        ok = locate(s_lo, q, ja);
+        if (ok) {
+            const int32_t *cp = cols(ja);
+#pragma unroll
+            for (int u = 0; u < kPipeW; ++u)
+                if (u < ja.w) {
+                    const int32_t c = cp[32 * u];
+#pragma unroll
+                    for (int m = 0; m < EW; ++m) xv[EW * u + m] = xin[c + m];
+                }
+        }
+        for (int s0 = s_lo; ok && s0 < s_hi; s0 += spt) {
+            const bool more = s0 + spt < s_hi;
+            if (more && !locate(s0 + spt, q + 1, jb)) {
                 ok = false;
                 break;
             }
-            step(t, ja, xv, jb, more);
+            step(s0 + cw, ja, xv, jb, more);
+            ++q;
             ja = jb;
         }
     }
-    cseq = cs0 + (unsigned)done;
+    cseq = q;
     fence_proxy_async_global();
     return ok;
 }
@@ -474,22 +492,20 @@ __device__ __forceinline__ bool sell_consume(TileRing *R, unsigned &cseq, uint64
 // Producer and consumers of one product in one call (the fused product's
 // kernel): pseq is the producer lane's tile counter, cseq a consumer's.
 template <int NE, int EW = 1, int PW = 8, typename T, typename Fin, typename AccArr>
-__device__ __forceinline__ bool sell_spmv(TileRing *R, unsigned &pseq, unsigned &cseq, uint64_t timeout_ns,
-                                          int64_t s_lo, int64_t s_hi, int spt, const int64_t *slice_ptr,
-                                          const int32_t *scol, const T *sval, const T *xin,
-                                          const T *const (&epi)[NE > 0 ? NE : 1], int lane, Fin fin, AccArr &acc) {
+__device__ __forceinline__ bool sell_spmv(TileRing *R, unsigned &pseq, unsigned &cseq, int s_lo, int s_hi, int spt,
+                                          const int64_t *slice_ptr, const int32_t *scol, const T *sval,
+                                          const T *xin, const T *const (&epi)[NE > 0 ? NE : 1], Fin fin,
+                                          AccArr &acc) {
     constexpr int NEA = NE > 0 ? NE : 1;
     if ((threadIdx.x >> 5) == kConsumerWarps) {
-        if (lane != 0 || spt <= 0) return true;
+        if ((threadIdx.x & 31) != 0 || spt <= 0) return true;
         const SliceOffsets off(R, slice_ptr, s_lo, s_hi);
         const void *ep[NEA];
 #pragma unroll
         for (int i = 0; i < NE; ++i) ep[i] = epi[i];
-        return produce_sell(R, s_lo, s_hi, spt, off, sval, EW * (int)sizeof(T), (int)sizeof(T), scol, ep, NE, pseq,
-                            timeout_ns);
+        return produce_sell(R, s_lo, s_hi, spt, off, sval, EW * (int)sizeof(T), (int)sizeof(T), scol, ep, NE, pseq);
     }
-    return sell_consume<NE, EW, PW>(R, cseq, timeout_ns, s_lo, s_hi, spt, slice_ptr, scol, sval, xin, epi, lane, fin,
-                                    acc);
+    return sell_consume<NE, EW, PW>(R, cseq, s_lo, s_hi, spt, slice_ptr, scol, sval, xin, epi, fin, acc);
 }
 
 // A 16-byte chunk of input i of a tile, from shared memory.
@@ -507,12 +523,17 @@ __device__ __forceinline__ typename coef_of<T>::type mk_coef(const double *v) {
     else return v[0];
 }
 
+__device__ __forceinline__ RedScratch &the_red() {
+    __shared__ RedScratch r;
+    return r;
+}
+
 // Synchronisation state of one CTA within the team of CTAs that solves one
 // system: the whole grid (a single solve), a group of CTAs of a batch
 // launch (a large system of a batch), or the CTA alone (the other systems
 // of a batch).  Every CTA of a team passes the same sequence of
 // barriers and reductions, so the epochs advance in lock step.
-// Several engines in one kernel share one GridSync.  Its members are called
+// The engines of one kernel share one GridSync (the_gs).  Its members are called
 // by every consumer thread; the producer warp takes no part.
 //
 // The object lives in shared memory, one per CTA (thread-private copies
@@ -528,23 +549,26 @@ struct GridSync {
     unsigned bid;       // this CTA's rank in the team
     BarrierState *bar;
     Slot *slots;        // [2][kMaxSums][nblocks]: exchange e uses half e & 1
-    RedScratch *red;    // shared
     uint64_t timeout_ns;
     unsigned epoch;     // exchanges this CTA has passed
     unsigned bepoch;    // barriers (sync) this CTA has passed
     bool ok;            // false once a barrier or a tile wait failed
-    TileRing *ring;     // shared-memory tile pipeline of this CTA
-    unsigned *seqs;     // shared, kThreads per-thread tile counters
+    unsigned seqs[kThreads];   // per-thread tile counters, kept across systems
 
-    __device__ __forceinline__ unsigned &seq() const { return seqs[threadIdx.x]; }
+    __device__ __forceinline__ unsigned &seq() { return seqs[threadIdx.x]; }
 
     // Team of `nb` CTAs (rank `id`) with their own barrier state and slots;
-    // nb = 1: this CTA alone (b and p null).
-    __device__ GridSync(BarrierState *b, Slot *p, unsigned nb, unsigned id, RedScratch *r, uint64_t to, TileRing *rg,
-                        unsigned *sq)
-        : nblocks(nb), bid(id), bar(b), slots(p), red(r), timeout_ns(to), epoch(0), bepoch(0), ok(!rg->failed),
-          ring(rg), seqs(sq) {
-        r->fail = 0;
+    // nb = 1: this CTA alone (b and p null).  One thread.
+    __device__ __forceinline__ void init(BarrierState *b, Slot *p, unsigned nb, unsigned id, uint64_t to) {
+        nblocks = nb;
+        bid = id;
+        bar = b;
+        slots = p;
+        timeout_ns = to;
+        epoch = bepoch = 0;
+        ok = !the_ring()->failed;
+        the_ring()->timeout_ns = to;
+        the_red().fail = 0;
     }
 
     // Slots of sum k of the exchange `ep`.  Two halves suffice: a CTA
@@ -554,11 +578,10 @@ struct GridSync {
         return slots + ((size_t)(ep & 1u) * kMaxSums + k) * nblocks;
     }
 
-    // The last levels of reduce(), by one warp.  Out of line: its registers
-    // stay out of the passes.
-    __device__ __noinline__ void team_total(int k, bool fence) {
+    // The last levels of reduce(), by one warp.
+    __device__ __forceinline__ void team_total(int k, bool fence) {
         const int lane = threadIdx.x & 31;
-        const double *p = red->part[k] + lane;
+        const double *p = the_red().part[k] + lane;
         double t = p[0] + p[32];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
@@ -571,12 +594,12 @@ struct GridSync {
             }
             const bool got = slots_sum(q, nblocks, ep, bar, timeout_ns, t);
             if (fence) fence_acq_rel_gpu();       // the other CTAs' writes after their slots
-            if (!got && lane == 0) red->fail = 1;
+            if (!got && lane == 0) the_red().fail = 1;
         }
-        if (lane == 0) red->total[k] = t;
+        if (lane == 0) the_red().total[k] = t;
     }
 
-    // Sum K values over the team into red->total[0, K), the same bits in
+    // Sum K values over the team into the_red().total[0, K), the same bits in
     // every CTA.  A dependent FP64 add costs about 60 cycles on this GPU and
     // one warp issues at most one FP64 instruction per ~60 cycles, so the
     // sums are short trees spread over many warps, independent sums
@@ -593,19 +616,20 @@ struct GridSync {
     // fence: what any CTA of the team wrote before is visible to all of them
     // after (needed before a pass that gathers; the streaming passes read
     // their own CTA's rows only).  False (uniformly) when a wait failed.
-    template <int K>
-    __device__ __forceinline__ bool reduce(const double (&v)[K], bool fence) {
-        static_assert(K <= kMaxSums && kMaxSums <= kConsumerWarps && kConsumers == 480, "reduction layout");
+    __device__ __forceinline__ bool reduce_k(const double (&v)[kMaxSums], int K, bool fence) {
+        static_assert(kMaxSums <= kConsumerWarps && kConsumers == 480, "reduction layout");
         constexpr int G1 = 64;
         const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const double h = v[k] + __shfl_down_sync(0xffffffffu, v[k], 16);
-            if (lane < 16) red->part[k][warp * 16 + lane] = h;
+        for (int k = 0; k < kMaxSums; ++k) {
+            if (k < K) {
+                const double h = v[k] + __shfl_down_sync(0xffffffffu, v[k], 16);
+                if (lane < 16) the_red().part[k][warp * 16 + lane] = h;
+            }
         }
         consumer_sync();
         if (tid < K * G1) {
-            double *p = red->part[tid / G1] + tid % G1;
+            double *p = the_red().part[tid / G1] + tid % G1;
             const double a0 = p[0], a1 = p[G1], a2 = p[2 * G1];
             // the last group has 48 partials
             p[0] = (a0 + a1) + (tid % G1 < 48 ? a2 + p[3 * G1] : a2);   // only this task reads slot 0
@@ -614,8 +638,18 @@ struct GridSync {
         if (warp < K) team_total(warp, fence);
         consumer_sync();
         if (tid == 0) epoch += 1;   // read again only after another barrier
-        if (red->fail) { ok = false; return false; }
+        if (the_red().fail) { ok = false; return false; }
         return true;
+    }
+    // The same for the passes outside the iteration (one copy of the code).
+    __device__ __noinline__ bool reduce_ool(double v0, double v1, double v2, double v3, double v4, int K, bool fence) {
+        const double v[kMaxSums] = {v0, v1, v2, v3, v4};
+        return reduce_k(v, K, fence);
+    }
+    template <int K>
+    __device__ __forceinline__ bool reduce(const double (&v)[K], bool fence) {
+        static_assert(K <= kMaxSums && kMaxSums == 5, "sums of a pass");
+        return reduce_ool(v[0], v[K > 1 ? 1 : 0], v[K > 2 ? 2 : 0], v[K > 3 ? 3 : 0], v[K > 4 ? 4 : 0], K, fence);
     }
 
     // Team barrier (a counter: cheaper than an exchange where no value goes
@@ -635,17 +669,17 @@ struct GridSync {
     }
     __device__ __forceinline__ bool wait() {
         if (nblocks == 1) return true;   // arrive()'s barrier ordered the CTA
-        if (threadIdx.x == 0 && !grid_wait(bar, bepoch, nblocks, timeout_ns)) red->fail = 1;
+        if (threadIdx.x == 0 && !grid_wait(bar, bepoch, nblocks, timeout_ns)) the_red().fail = 1;
         consumer_sync();
-        if (red->fail) { ok = false; return false; }
+        if (the_red().fail) { ok = false; return false; }
         return true;
     }
 
     // Hand a command to the producer warp (every consumer thread calls it).
     __device__ __forceinline__ void post(int cmd) {
         if (threadIdx.x == 0) {
-            ring->cmd = cmd;
-            ring->stop = 0;
+            the_ring()->cmd = cmd;
+            the_ring()->stop = 0;
         }
         __syncthreads();
     }
@@ -654,33 +688,39 @@ struct GridSync {
     // `passes`: passes this CTA's consumers have finished.
     __device__ __forceinline__ void end_inner(unsigned &sq, unsigned passes) {
         if (threadIdx.x == 0) {
-            *(volatile int *)&ring->stop = 1;
-            ring->passes = passes;
+            *(volatile int *)&the_ring()->stop = 1;
+            the_ring()->passes = passes;
         }
         __syncthreads();
-        for (const unsigned last = ring->issued; sq != last; ++sq) {
-            if (!mbar_wait(&ring->full[sq % kStages], (sq / kStages) & 1u, timeout_ns)) {
-                ring->failed = 1;
+        for (const unsigned last = the_ring()->issued; sq != last; ++sq) {
+            if (!mbar_wait(the_ring(), &the_ring()->full[sq % kStages], (sq / kStages) & 1u)) {
+                the_ring()->failed = 1;
                 ok = false;
                 break;
             }
             __syncwarp();
-            if ((threadIdx.x & 31) == 0) mbar_arrive(&ring->empty[sq % kStages]);
+            if ((threadIdx.x & 31) == 0) mbar_arrive(&the_ring()->empty[sq % kStages]);
         }
         consumer_sync();
     }
 };
 
+__device__ __forceinline__ GridSync &the_gs() {
+    __shared__ GridSync g;
+    return g;
+}
+
 // One pass of the iteration (Engine::inner) and the pass after it: a
 // function of n alone, which the producer warp follows too.  i: the slot the
 // step builds (ALPHA uses slot i - 1; i = n: the block's last update); s:
 // the column a sweep's pass uses; first: block 0.
-enum { P_SPMV_C, P_ALPHA, P_SPMV_Z, P_OMEGA, P_W_FIRST, P_W_ROUND, P_W_LAST, P_F_ROUND, P_G_J0 };
+enum { P_RESIDUAL, P_SPMV_C, P_ALPHA, P_SPMV_Z, P_OMEGA, P_W_FIRST, P_W_ROUND, P_W_LAST, P_F_ROUND, P_G_J0 };
 struct Step {
     int op = P_SPMV_C, i = 0, s = 0;
     bool first = true;
     __device__ __forceinline__ void advance(int n) {
         switch (op) {
+        case P_RESIDUAL: op = P_SPMV_C; break;
         case P_SPMV_C: ++i; op = P_ALPHA; break;
         case P_ALPHA: op = i == n ? P_SPMV_Z : first ? P_G_J0 : i == n - 1 ? P_W_LAST : P_W_FIRST; break;
         case P_SPMV_Z: op = P_OMEGA; break;
@@ -719,27 +759,31 @@ struct Engine {
     static constexpr int PW = Pack<T>::W;
     static constexpr int CPS = 32 * sizeof(T) / 16;           // 16-byte chunks per slice
 
-    const SysView<T> &sys;
-    const SolveCtl &ctl;
-    GridSync &gs;
-    // shared memory
-    S *c;            // kMaxN
-    S *bt;           // kMaxN
-    Acct *acct;
-    Scalars<S> *sc;
-    // ownership: slices [s_lo, s_hi), chunks [c_lo, c_hi)
-    int64_t s_lo, s_hi, c_lo, c_hi;
+    // The CTA's shared objects; the engine has no state of its own.
+    __device__ __forceinline__ static const SysView<T> &sys() { return the_sys<T>(); }
+    __device__ __forceinline__ static const SolveCtl &ctl() { return the_ctl(); }
+    __device__ __forceinline__ static GridSync &gs() { return the_gs(); }
+    __device__ __forceinline__ static Acct &acct() { return the_acct(); }
+    __device__ __forceinline__ static Scalars<S> &sc() { return the_iter<S>().sc; }
+    __device__ __forceinline__ static S *c() { return the_iter<S>().c; }
+    __device__ __forceinline__ static S *bt() { return the_iter<S>().bt; }
+    // ownership: slices [s_lo(), s_hi()), chunks [c_lo(), c_hi())
+    __device__ __forceinline__ static int s_lo() { return the_iter<S>().s_lo; }
+    __device__ __forceinline__ static int s_hi() { return the_iter<S>().s_hi; }
+    __device__ __forceinline__ static int64_t c_lo() { return (int64_t)s_lo() * CPS; }
+    __device__ __forceinline__ static int64_t c_hi() { return (int64_t)s_hi() * CPS; }
 
-    // Constructed by one thread in shared memory (one engine per CTA; see
-    // GridSync); every thread then calls attach().
-    __device__ Engine(const SysView<T> &s, const SolveCtl &k, GridSync &g, S *c_, S *bt_, Acct *acct_,
-                      Scalars<S> *sc_)
-        : sys(s), ctl(k), gs(g), c(c_), bt(bt_), acct(acct_), sc(sc_) {
-        own_range(s.nslices, g.nblocks, g.bid, s_lo, s_hi);
-        c_lo = s_lo * CPS;
-        c_hi = s_hi * CPS;
+    // Every thread, once the system's view and the team are set.
+    __device__ void attach() {
+        if (threadIdx.x == 0) {
+            int64_t lo, hi;
+            own_range(sys().nslices, gs().nblocks, gs().bid, lo, hi);
+            the_iter<S>().s_lo = (int)lo;
+            the_iter<S>().s_hi = (int)hi;
+        }
+        __syncthreads();
+        soff_load(the_ring(), sys().slice_ptr, s_lo(), s_hi());
     }
-    __device__ void attach() { soff_load(gs.ring, sys.slice_ptr, s_lo, s_hi); }
     // Counts one Table 4.3 operation and its algorithmic floating-point
     // operations (real arithmetic): a product 2 per stored entry; an inner
     // product, AXPY or norm 2 per element; a scaling 1 per element.
@@ -747,34 +791,34 @@ struct Engine {
     // scaling 6.
     __device__ __forceinline__ void op(int which, int cnt = 1) {
         if (threadIdx.x == kAcctThread) {
-            acct->ops[which] += cnt;
+            acct().ops[which] += cnt;
             constexpr bool cx_ = is_cx<T>::value;
-            const int64_t N = sys.N;
+            const int64_t N = sys().N;
             int64_t f;
-            if (which == OP_MATVEC) f = (cx_ ? 8 : 2) * sys.nnz;
+            if (which == OP_MATVEC) f = (cx_ ? 8 : 2) * sys().nnz;
             else if (which == OP_SCALE) f = (cx_ ? 6 : 1) * N;
             else if (which == OP_NORM) f = (cx_ ? 4 : 2) * N;
             else f = (cx_ ? 8 : 2) * N;
-            acct->flops += cnt * f;
+            acct().flops += cnt * f;
         }
     }
 
-    __device__ __forceinline__ const T *Qc(int k) const { return sys.Q + (int64_t)k * sys.ld; }
-    __device__ __forceinline__ const T *Fc(int k) const { return sys.F + (int64_t)k * sys.ld; }
-    __device__ __forceinline__ T *Gc(int k) const { return sys.G + (int64_t)k * sys.ld; }
-    __device__ __forceinline__ T *Wc(int k) const { return sys.W + (int64_t)k * sys.ld; }
+    __device__ __forceinline__ const T *Qc(int k) const { return sys().Q + (int64_t)k * sys().ld; }
+    __device__ __forceinline__ const T *Fc(int k) const { return sys().F + (int64_t)k * sys().ld; }
+    __device__ __forceinline__ T *Gc(int k) const { return sys().G + (int64_t)k * sys().ld; }
+    __device__ __forceinline__ T *Wc(int k) const { return sys().W + (int64_t)k * sys().ld; }
 
     __device__ __forceinline__ void vbytes(int nvec) {
-        if (threadIdx.x == kAcctThread) acct->bytes += nvec * sys.N * (int64_t)sizeof(T);
+        if (threadIdx.x == kAcctThread) acct().bytes += nvec * sys().N * (int64_t)sizeof(T);
     }
     __device__ __forceinline__ void sbytes(int nextra) {
         // SpMV: entries (values, and a column index per stored entry of EW
         // values), row_ptr-equivalent, x read once, y written once, plus
         // `nextra` epilogue vectors.
         if (threadIdx.x == kAcctThread) {
-            acct->bytes += sys.nnz * (int64_t)sizeof(T) + sys.nnz / EW * 4 + 4 * (sys.N + 1) +
-                           (2 + nextra) * sys.N * (int64_t)sizeof(T);
-            acct->spmv++;
+            acct().bytes += sys().nnz * (int64_t)sizeof(T) + sys().nnz / EW * 4 + 4 * (sys().N + 1) +
+                           (2 + nextra) * sys().N * (int64_t)sizeof(T);
+            acct().spmv++;
         }
     }
 
@@ -785,28 +829,30 @@ struct Engine {
     // Issue the tiles of pass `st` (the input order of each pass is that of
     // its consumer side below).
     __device__ __forceinline__ int issue(const Step &st, unsigned &sq) {
-        const int lane = threadIdx.x & 31, n = sys.n, i = st.i, s = st.s;
-        TileRing *const R = gs.ring;
+        const int lane = threadIdx.x & 31, n = sys().n, i = st.i, s = st.s;
+        TileRing *const R = the_ring();
         const T *p = nullptr;
         int ni = 0;
         switch (st.op) {
         case P_SPMV_C:
-        case P_SPMV_Z:
-            return issue_product(st.op == P_SPMV_C ? Qc(i) : sys.r, 1, sq);
+        case P_SPMV_Z: {
+            const int e = issue_ilu(sq);
+            return e ? e : issue_product(st.op == P_SPMV_C ? Qc(i) : sys().r, sys().spt[1], sq);
+        }
         case P_ALPHA: {
             const bool hq = i < n, f0 = st.first && hq;
             ni = 4 + (hq ? 1 : 0) + (f0 ? 1 : 0);
-            p = lane == 0 ? sys.x : lane == 1 ? Gc(i - 1) : lane == 2 ? sys.r : lane == 3 ? Wc(i - 1)
-                : lane == 4 && hq ? Qc(i) : sys.F;
+            p = lane == 0 ? sys().x : lane == 1 ? Gc(i - 1) : lane == 2 ? sys().r : lane == 3 ? Wc(i - 1)
+                : lane == 4 && hq ? Qc(i) : sys().F;
             break;
         }
         case P_OMEGA:
             ni = 4;
-            p = lane == 0 ? sys.x : lane == 1 ? sys.r : lane == 2 ? sys.z : sys.Q;
+            p = lane == 0 ? sys().x : lane == 1 ? sys().r : lane == 2 ? sys().z : sys().Q;
             break;
         case P_W_FIRST:
             ni = 3;
-            p = lane == 0 ? sys.r : lane == 1 ? Wc(i) : Qc(i + 1);
+            p = lane == 0 ? sys().r : lane == 1 ? Wc(i) : Qc(i + 1);
             break;
         case P_W_ROUND:
             ni = 3;
@@ -815,8 +861,8 @@ struct Engine {
         case P_W_LAST: {
             const int nt = n - 1 - i, ntile = nt < kMaxInputs - 4 ? nt : kMaxInputs - 4, f = i > 0 ? 1 : 0;
             ni = 3 + f + ntile;
-            p = lane == 0 ? Wc(i) : lane == 1 ? Gc(i) : lane == 2 ? (i == n - 1 ? sys.r : Wc(n - 1))
-                : lane == 3 && f ? sys.F : Gc(i + 1 + lane - 3 - f);
+            p = lane == 0 ? Wc(i) : lane == 1 ? Gc(i) : lane == 2 ? (i == n - 1 ? sys().r : Wc(n - 1))
+                : lane == 3 && f ? sys().F : Gc(i + 1 + lane - 3 - f);
             break;
         }
         case P_F_ROUND:
@@ -825,23 +871,22 @@ struct Engine {
             break;
         default:   // P_G_J0
             ni = i >= 2 ? 3 : 2;
-            p = lane == 0 ? sys.r : lane == 1 ? sys.G : Fc(1);
+            p = lane == 0 ? sys().r : lane == 1 ? sys().G : Fc(1);
             break;
         }
-        return produce_lanes(R, p, ni, c_lo, c_hi, sq, gs.timeout_ns);
+        return produce_lanes(R, p, ni, c_lo(), c_hi(), sq);
     }
-    // Tiles of a product with `ne` epilogue vectors (lane 2 + k copies
-    // vector k, its own `epi`).
-    __device__ __forceinline__ int issue_product(const T *epi, int ne, unsigned &sq) {
-        if (sys.spt[ne] <= 0) return 0;
-        const SliceOffsets off(gs.ring, sys.slice_ptr, s_lo, s_hi);
-        return produce_sell_lanes(gs.ring, s_lo, s_hi, sys.spt[ne], off, sys.sval, EW * (int)sizeof(T),
-                                  (int)sizeof(T), sys.scol, epi, ne, sq, gs.timeout_ns);
+    // Tiles of a product with one epilogue vector, `spt` slices each.
+    __device__ __forceinline__ int issue_product(const T *epi, int spt, unsigned &sq) {
+        if (spt <= 0) return 0;
+        const SliceOffsets off(the_ring(), sys().slice_ptr, s_lo(), s_hi());
+        return produce_sell_lanes(the_ring(), s_lo(), s_hi(), spt, off, sys().sval, EW * (int)sizeof(T),
+                                  (int)sizeof(T), sys().scol, epi, 1, sq);
     }
     // Wait until the consumers have finished the pass.
     __device__ __forceinline__ int wait_done(unsigned &passes) {
         int st = 0;
-        if ((threadIdx.x & 31) == 0) st = producer_wait(gs.ring, &gs.ring->done, passes & 1u, gs.timeout_ns);
+        if ((threadIdx.x & 31) == 0) st = producer_wait(the_ring(), &the_ring()->done, passes & 1u);
         st = __shfl_sync(0xffffffffu, st, 0);
         if (st == 0) passes += 1;
         return st;
@@ -851,46 +896,44 @@ struct Engine {
     // of r (refined mode).  residual64 issues the FP64 residual's tiles.
     template <bool Decide, typename Fn>
     __device__ __forceinline__ void serve(Fn residual64) {
-        TileRing *const R = gs.ring;
-        unsigned sq = gs.seq(), passes = R->passes;
+        TileRing *const R = the_ring();
+        unsigned sq = gs().seq(), passes = R->passes;
         for (;;) {
             __syncthreads();
             const int cmd = R->cmd;
             if (cmd == kCmdExit) break;
             int st = 0;
             if (cmd == kCmdResidual) {
-                st = issue_product((threadIdx.x & 31) == 2 ? sys.b : sys.Q, 2, sq);
+                st = issue_ilu(sq);
+                if (st == 0) st = issue_product(sys().b, sys().spt[2], sq);
                 if (st == 0) st = wait_done(passes);
             } else if (cmd == kCmdResidual64) {
                 st = residual64(sq);
                 if (st == 0) st = wait_done(passes);
+            } else if (cmd == kCmdIlu) {
+                st = issue_ilu(sq);
             } else {
-                const int n = sys.n;
+                const int n = sys().n;
                 bool met = false;   // the consumers' end_inner has been met at a decision
                 for (Step p; st == 0; p.advance(n)) {
                     st = issue(p, sq);
                     if (st == 0) st = wait_done(passes);
                     if constexpr (Decide) {
-                        if (st == 0 && (p.op == P_ALPHA || p.op == P_OMEGA)) {
+                        // the consumers' commands (a residual replacement)
+                        // until they let the iteration go on or end it
+                        while (st == 0 && (p.op == P_ALPHA || p.op == P_OMEGA)) {
                             if ((threadIdx.x & 31) == 0) R->issued = sq;
                             __syncthreads();
-                            if (R->stop) {
-                                met = true;
-                                break;
-                            }
-                            if (R->cmd == kCmdResidual64) {
+                            met = R->stop != 0;
+                            if (met || R->cmd == kCmdGo) break;
+                            if (R->cmd == kCmdIlu) {
+                                st = issue_ilu(sq);
+                            } else {
                                 st = residual64(sq);
                                 if (st == 0) st = wait_done(passes);
-                                if (st == 0) {
-                                    if ((threadIdx.x & 31) == 0) R->issued = sq;
-                                    __syncthreads();
-                                    if (R->stop) {
-                                        met = true;
-                                        break;
-                                    }
-                                }
                             }
                         }
+                        if (met) break;
                     }
                 }
                 if (st == 2) R->failed = 1;
@@ -904,7 +947,7 @@ struct Engine {
             if (st == 2) R->failed = 1;
             if ((threadIdx.x & 31) == 0) R->passes = passes;
         }
-        gs.seq() = sq;
+        gs().seq() = sq;
         if ((threadIdx.x & 31) == 0) R->passes = passes;
     }
 
@@ -916,8 +959,8 @@ struct Engine {
     // every chunk of this CTA.
     template <typename Fn>
     __device__ __forceinline__ void tiles(int tc, unsigned &sq, Fn fn) {
-        TileRing *const ring = gs.ring;
-        if (!consume(ring, TileGeom{tc, c_lo, c_hi}, sq, gs.timeout_ns, fn)) ring->failed = 1;
+        TileRing *const ring = the_ring();
+        if (!consume(ring, TileGeom{tc, c_lo(), c_hi()}, sq, fn)) ring->failed = 1;
         pass_done(ring);
     }
     template <int K>
@@ -925,42 +968,33 @@ struct Engine {
         double v[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) v[k] = (double)acc[k];
-        return gs.template reduce<K>(v, fence) && ring_ok();
+        return gs().template reduce<K>(v, fence) && ring_ok();
     }
     // A failed tile wait marks the ring; the pass's reduction or barrier
     // then reports it.
     __device__ __forceinline__ bool ring_ok() {
-        if (gs.ring->failed) { gs.ok = false; return false; }
+        if (the_ring()->failed) { gs().ok = false; return false; }
         return true;
     }
 
     // SELL-32 SpMV pass over the owned slices (matrix tiles through the
     // ring).
-    template <int NE, typename Fin, int K>
-    __device__ __forceinline__ void spmv_rows(const T *xin, const T *const (&epi)[NE], unsigned &sq, Fin fin,
+    template <typename Fin, int K>
+    __device__ __forceinline__ void spmv_rows(const T *xin, const T *const (&epi)[1], int spt, unsigned &sq, Fin fin,
                                               ACC (&acc)[K]) {
-        // with ILU(0) the product is A t, t = M^{-1} xin formed by the
-        // caller (ilu_pre) before the pass
+        // with ILU(0) the product is A t, t = M^{-1} xin formed before the
+        // pass
         if constexpr (PC) {
-            if (sys.ilu.lu) xin = sys.ilu.t;
+            if (sys().ilu.lu) xin = sys().ilu.t;
         }
-        bool okw;
-        // FP32 and complex engines: a pipelined width of 7 where the rows
-        // allow it (fewer registers of gathered x); the real FP64 engine
-        // keeps 8 (no gain at 7)
-        if constexpr (is_narrow<T>::value || is_cx<T>::value) {
-            if (sys.narrow_rows)
-                okw = sell_consume<NE, EW, 7>(gs.ring, sq, gs.timeout_ns, s_lo, s_hi, sys.spt[NE], sys.slice_ptr,
-                                              sys.scol, sys.sval, xin, epi, threadIdx.x & 31, fin, acc);
-            else
-                okw = sell_consume<NE, EW>(gs.ring, sq, gs.timeout_ns, s_lo, s_hi, sys.spt[NE], sys.slice_ptr,
-                                           sys.scol, sys.sval, xin, epi, threadIdx.x & 31, fin, acc);
-        } else {
-            okw = sell_consume<NE, EW>(gs.ring, sq, gs.timeout_ns, s_lo, s_hi, sys.spt[NE], sys.slice_ptr, sys.scol,
-                                       sys.sval, xin, epi, threadIdx.x & 31, fin, acc);
-        }
-        if (!okw) gs.ring->failed = 1;
-        pass_done(gs.ring);
+        // FP32 and complex engines: a pipelined width of 7, the widest row of
+        // the 3-D stencils (fewer registers of gathered x); the real FP64
+        // engine keeps 8 (no gain at 7)
+        constexpr int W = is_narrow<T>::value || is_cx<T>::value ? 7 : 8;
+        const bool okw = sell_consume<1, EW, W>(the_ring(), sq, s_lo(), s_hi(), spt, sys().slice_ptr, sys().scol,
+                                                sys().sval, xin, epi, fin, acc);
+        if (!okw) the_ring()->failed = 1;
+        pass_done(the_ring());
     }
 
     // ------------------------------------------------------------------
@@ -985,8 +1019,8 @@ struct Engine {
     __device__ __forceinline__ void ilu_fetch_l(int64_t q, int64_t hi, const T *v, IluRow &R) const {
         R.i = -1;
         if (q >= hi) return;
-        const IluView<T> &M = sys.ilu;
-        const int64_t N = sys.N;
+        const IluView<T> &M = sys().ilu;
+        const int64_t N = sys().N;
         const int i = M.lrows[q];
         const int n = M.lcnt[q];
         const int cnt = n < kIluReg ? n : kIluReg;
@@ -1009,8 +1043,8 @@ struct Engine {
     __device__ __forceinline__ void ilu_fetch_u(int64_t q, int64_t hi, IluRow &R) const {
         R.i = -1;
         if (q >= hi) return;
-        const IluView<T> &M = sys.ilu;
-        const int64_t N = sys.N;
+        const IluView<T> &M = sys().ilu;
+        const int64_t N = sys().N;
         const int i = M.urows[q];
         const int n = M.ucnt[q];
         const int cnt = n < kIluReg ? n : kIluReg;
@@ -1032,7 +1066,7 @@ struct Engine {
     }
     // s - sum of a_e out[c_e] over the row's entries, in pattern order.
     __device__ __forceinline__ T ilu_row_sum(const IluRow &R, T s, const T *out) const {
-        const IluView<T> &M = sys.ilu;
+        const IluView<T> &M = sys().ilu;
 #pragma unroll
         for (int e = 0; e < kIluReg; ++e)
             if (e < R.cnt) s = efma(-R.a[e], ldcg_val(out + R.c[e]), s);
@@ -1048,12 +1082,13 @@ struct Engine {
     // next level (index, entries, right-hand side or diagonal) does not
     // depend on the current level, so it is loaded while the barrier is
     // pending, and only the values of earlier levels are read after it.
-    __device__ __noinline__ bool ilu_solve(const T *v, T *out) {
-        const IluView<T> &M = sys.ilu;
+    __device__ __forceinline__ bool ilu_solve_body(const T *v, T *out) {
+        if (sys().ilu.llev) return ilu_wide(v, out);
+        const IluView<T> &M = sys().ilu;
         // a level's positions split into one contiguous chunk per CTA of
         // ceil(size / CTAs): every CTA shares each level (a level is a few
         // thousand scattered rows), and a warp reads consecutive positions
-        const int64_t G = gs.nblocks, bid = gs.bid;
+        const int64_t G = gs().nblocks, bid = gs().bid;
         const int tid = threadIdx.x;
         auto chunk = [&](const int32_t *ptr, int l, int64_t &q0, int64_t &q1) {
             const int64_t lo = ptr[l], hi = ptr[l + 1], ch = (hi - lo + G - 1) / G;
@@ -1074,7 +1109,7 @@ struct Engine {
                 for (int64_t k = k0; k < kd; ++k) t = efma(-M.lu[k], ldcg_val(out + M.ci[k]), t);
                 out[i] = t;
             }
-            gs.arrive();
+            gs().arrive();
             if (l + 1 < nl) {
                 chunk(M.lptr, l + 1, q0, q1);
                 ilu_fetch_l(q0 + tid, q1, v, R);
@@ -1082,7 +1117,7 @@ struct Engine {
                 chunk(M.uptr, 0, q0, q1);
                 ilu_fetch_u(q0 + tid, q1, R);
             }
-            if (!gs.wait()) return false;
+            if (!gs().wait()) return false;
         }
         for (int l = 0; l < nu; ++l) {
             if (R.i >= 0) out[R.i] = ilu_row_sum(R, ldcg_val(out + R.i), out) / R.v;
@@ -1093,93 +1128,241 @@ struct Engine {
                 for (int64_t k = kd + 1; k < k1; ++k) t = efma(-M.lu[k], ldcg_val(out + M.ci[k]), t);
                 out[i] = t / M.lu[kd];
             }
-            gs.arrive();
+            gs().arrive();
             if (l + 1 < nu) {
                 chunk(M.uptr, l + 1, q0, q1);
                 ilu_fetch_u(q0 + tid, q1, R);
             }
-            if (!gs.wait()) return false;
+            if (!gs().wait()) return false;
         }
-        if (threadIdx.x == kAcctThread) {   // factors and row data once, v read, out written and re-read
-            acct->bytes += M.nnz * (int64_t)(sizeof(T) + 4) + sys.N * (int64_t)(8 + 4 + 8 + 3 * sizeof(T));
-            acct->flops += (is_cx<T>::value ? 8 : 2) * M.nnz;
-        }
+        ilu_count();
         return true;
     }
-
-    // Before a product pass with ILU(0): t = M^{-1} in, where `in` is the
-    // pass's input vector (the pass then multiplies t).  A separate call,
-    // so the product passes themselves carry no call to the solve.
-    __device__ __forceinline__ bool ilu_pre(const T *in) {
-        if constexpr (!PC) {
-            return true;
-        } else {
-            if (!sys.ilu.lu) return true;
-            return ilu_solve(in, sys.ilu.t);
+    // Accounting of one M^{-1}: factors and row data once, v read, out
+    // written and re-read.
+    __device__ __forceinline__ void ilu_count() {
+        if (threadIdx.x == kAcctThread) {
+            acct().bytes += sys().ilu.nnz * (int64_t)(sizeof(T) + 4) + sys().N * (int64_t)(8 + 4 + 8 + 3 * sizeof(T));
+            acct().flops += (is_cx<T>::value ? 8 : 2) * sys().ilu.nnz;
         }
+    }
+
+    // M^{-1} for factors with few levels, as tiles of the ring: each CTA
+    // takes a contiguous share of a level's slices; the producer warp streams
+    // their values, columns, (row, count) pairs and U's diagonal (constant
+    // data, so the next level's tiles arrive during the level's barrier), and
+    // warp w takes slice w of each tile, one row per lane.  As in sell_consume
+    // the gathers and the right-hand side of tile t+1 are issued among the
+    // FMAs of tile t; rows wider than W entries take the rest in batches.
+    // What bounds it: one round of gathers per 480 rows and a barrier per
+    // level.  (With a row's loads one after another (index, row pointer,
+    // entries, values) one M^{-1} at 96^3, four levels, took 95 us, with the
+    // slices read by coalesced loads 100 us.)  Each row is one sequential sum
+    // in pattern order.
+    __device__ __forceinline__ bool ilu_wide(const T *v, T *out) {
+        constexpr int W = sizeof(T) == 16 ? 3 : 6;
+        const int lane = threadIdx.x & 31, cw = threadIdx.x >> 5;
+        TileRing *const R = the_ring();
+        const int nl = sys().ilu.nlev_l, nlev = nl + sys().ilu.nlev_u, spt = sys().ilu.spt;
+        unsigned q = gs().seq();
+        for (int l = 0; l < nlev; ++l) {
+            const bool up = l >= nl;
+            const IluLevel L = up ? sys().ilu.ulev[l - nl] : sys().ilu.llev[l];
+            const T *const rhs = up ? out : v;
+            const int w = L.w;
+            int k0, k1;
+            ilu_share(L.ns, k0, k1);
+            int st = 0, ns = 0;       // stage and slices of the tile at hand
+            int row = -1, cnt = 0;
+            T t{}, x[W];
+            // stage of tile q; its slices; false when the wait failed
+            auto arrived = [&](int k, unsigned tile, int &stage, int &slices) {
+                stage = (int)(tile % kStages);
+                slices = k1 - k < spt ? k1 - k : spt;
+                return mbar_wait(R, &R->full[stage], (tile / kStages) & 1u);
+            };
+            auto vals = [&](int stage) {
+                return reinterpret_cast<const T *>(the_stages() + stage * kStageBytes) + cw * 32 * w + lane;
+            };
+            auto cols = [&](int stage, int slices) {
+                return reinterpret_cast<const int32_t *>(the_stages() + stage * kStageBytes +
+                                                         slices * 32 * w * (int)sizeof(T)) + cw * 32 * w + lane;
+            };
+            auto meta = [&](int stage, int slices) {
+                return reinterpret_cast<const int2 *>(the_stages() + stage * kStageBytes +
+                                                      slices * 32 * w * (int)(sizeof(T) + 4))[cw * 32 + lane];
+            };
+            auto diag = [&](int stage, int slices) {
+                return reinterpret_cast<const T *>(the_stages() + stage * kStageBytes +
+                                                   slices * 32 * (w * (int)(sizeof(T) + 4) + 8))[cw * 32 + lane];
+            };
+            bool ok = k0 >= k1 || arrived(k0, q, st, ns);
+            if (k0 < k1 && ok && cw < ns) {
+                const int2 m = meta(st, ns);
+                row = m.x;
+                cnt = m.y;
+                if (row >= 0) t = ldcg_val(rhs + row);
+                const int32_t *c = cols(st, ns);
+#pragma unroll
+                for (int e = 0; e < W; ++e)
+                    if (e < cnt) x[e] = out[c[32 * e]];
+            }
+            for (int k = k0; ok && k < k1; k += spt, ++q) {
+                int st1 = 0, ns1 = 0, row1 = -1, cnt1 = 0;
+                T t1{};
+                if (k + spt < k1) {
+                    if (!arrived(k + spt, q + 1, st1, ns1)) {
+                        ok = false;
+                        break;
+                    }
+                    if (cw < ns1) {
+                        const int2 m = meta(st1, ns1);
+                        row1 = m.x;
+                        cnt1 = m.y;
+                        if (row1 >= 0) t1 = ldcg_val(rhs + row1);
+                    }
+                }
+                const T *a = vals(st);
+                const int32_t *c = cols(st, ns), *c1 = cols(st1, ns1);
+#pragma unroll
+                for (int e = 0; e < W; ++e) {
+                    if (e < cnt) t = efma(-a[32 * e], x[e], t);
+                    if (e < cnt1) x[e] = out[c1[32 * e]];
+                }
+                for (int e0 = W; e0 < cnt; e0 += 2) {
+                    const T xa = out[c[32 * e0]];
+                    const T xb = e0 + 1 < cnt ? out[c[32 * (e0 + 1)]] : T{};
+                    t = efma(-a[32 * e0], xa, t);
+                    if (e0 + 1 < cnt) t = efma(-a[32 * (e0 + 1)], xb, t);
+                }
+                if (row >= 0) {
+                    if (up) t = t / diag(st, ns);
+                    out[row] = t;
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&R->empty[st]);
+                st = st1;
+                ns = ns1;
+                row = row1;
+                cnt = cnt1;
+                t = t1;
+            }
+            if (!ok) R->failed = 1;
+            if (!gs().sync() || !ring_ok()) return false;
+        }
+        gs().seq() = q;
+        ilu_count();
+        return true;
+    }
+    // This CTA's share [k0, k1) of a level's slices.
+    __device__ __forceinline__ static void ilu_share(int ns, int &k0, int &k1) {
+        const int G = (int)gs().nblocks, ch = (ns + G - 1) / G;
+        k0 = (int)gs().bid * ch;
+        k1 = k0 + ch < ns ? k0 + ch : ns;
+    }
+    // Producer warp: the tiles of ilu_wide (lane 0 the values, 1 the columns,
+    // 2 the (row, count) pairs, 3 U's diagonal).
+    __device__ __forceinline__ int issue_ilu(unsigned &sq) {
+        if constexpr (!PC) {
+            return 0;
+        } else {
+            if (!sys().ilu.llev) return 0;
+            const int lane = threadIdx.x & 31;
+            const int nl = sys().ilu.nlev_l, nlev = nl + sys().ilu.nlev_u, spt = sys().ilu.spt;
+            TileRing *const R = the_ring();
+            for (int l = 0; l < nlev; ++l) {
+                const bool up = l >= nl;
+                const IluLevel L = up ? sys().ilu.ulev[l - nl] : sys().ilu.llev[l];
+                int k0, k1;
+                ilu_share(L.ns, k0, k1);
+                const unsigned ev = 32u * (unsigned)L.w;   // entries of a slice
+                // bytes of a slice of each lane's part, and where the parts
+                // of the share start
+                const unsigned b0 = ev * (unsigned)sizeof(T), b1 = ev * 4u, b2 = 256u,
+                               b3 = up ? 32u * (unsigned)sizeof(T) : 0u;
+                const unsigned mine = lane == 0 ? b0 : lane == 1 ? b1 : lane == 2 ? b2 : lane == 3 ? b3 : 0u;
+                const unsigned before = lane == 0 ? 0u : lane == 1 ? b0 : lane == 2 ? b0 + b1 : b0 + b1 + b2;
+                const unsigned char *src;
+                if (lane == 0) src = (const unsigned char *)((up ? sys().ilu.uell_a : sys().ilu.lell_a) + L.e0);
+                else if (lane == 1) src = (const unsigned char *)((up ? sys().ilu.uell_c : sys().ilu.lell_c) + L.e0);
+                else if (lane == 2) src = (const unsigned char *)((up ? sys().ilu.umeta : sys().ilu.lmeta) + 32 * (int64_t)L.m0);
+                else src = (const unsigned char *)(sys().ilu.udiag + 32 * (int64_t)L.m0);
+                for (int k = k0; k < k1; k += spt, ++sq) {
+                    const int s = (int)(sq % kStages);
+                    const unsigned use = sq / kStages;
+                    int st = 0;
+                    if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u);
+                    st = __shfl_sync(0xffffffffu, st, 0);
+                    if (st) return st;
+                    const unsigned n = (unsigned)(k1 - k < spt ? k1 - k : spt);
+                    if (lane == 0) mbar_arrive_expect_tx(&R->full[s], n * (b0 + b1 + b2 + b3));
+                    __syncwarp();
+                    if (mine)
+                        bulk_g2s(the_stages() + s * kStageBytes + n * before, src + (size_t)k * mine, n * mine,
+                                 &R->full[s]);
+                }
+            }
+            return 0;
+        }
+    }
+
+    // Out of line, for the refined mode's residual replacement; the
+    // iteration's own M^{-1} is inlined in inner().
+    __device__ __noinline__ bool ilu_solve(const T *v, T *out) {
+        if (sys().ilu.llev) gs().post(kCmdIlu);
+        return ilu_solve_body(v, out);
     }
 
     // y_0 = M x_0 = L (U x_0), in place on x: t = U x, then x = L t (two
     // row-parallel products).
-    __device__ __noinline__ bool ilu_to_y() {
-        const IluView<T> &M = sys.ilu;
-        const int64_t nth = (int64_t)gs.nblocks * kConsumers;
-        const int64_t me = (int64_t)gs.bid * kConsumers + threadIdx.x;
-        T *const x = sys.x, *const t = M.t;
-        for (int64_t i = me; i < sys.N; i += nth) {
+    __device__ __forceinline__ bool ilu_to_y() {
+        const IluView<T> &M = sys().ilu;
+        const int64_t nth = (int64_t)gs().nblocks * kConsumers;
+        const int64_t me = (int64_t)gs().bid * kConsumers + threadIdx.x;
+        T *const x = sys().x, *const t = M.t;
+        for (int64_t i = me; i < sys().N; i += nth) {
             const int64_t kd = M.rp[i] + M.dpos[i], k1 = M.rp[i + 1];
             T s{};
             for (int64_t k = kd; k < k1; ++k) s = efma(M.lu[k], x[M.ci[k]], s);
             t[i] = s;
         }
-        if (!gs.sync()) return false;
-        for (int64_t i = me; i < sys.N; i += nth) {
+        if (!gs().sync()) return false;
+        for (int64_t i = me; i < sys().N; i += nth) {
             const int64_t k0 = M.rp[i], kd = k0 + M.dpos[i];
             T s = ldcg_val(t + i);
             for (int64_t k = k0; k < kd; ++k) s = efma(M.lu[k], ldcg_val(t + M.ci[k]), s);
             x[i] = s;
         }
-        return gs.sync();
+        return gs().sync();
     }
 
     // x = M^{-1} y once the final residual pass has formed t = M^{-1} y.
-    __device__ __noinline__ bool ilu_to_x() {
-        const int64_t nth = (int64_t)gs.nblocks * kConsumers;
-        const int64_t me = (int64_t)gs.bid * kConsumers + threadIdx.x;
-        T *const x = sys.x;
-        const T *t = sys.ilu.t;
-        for (int64_t i = me; i < sys.N; i += nth) x[i] = ldcg_val(t + i);
-        return gs.sync();
+    __device__ __forceinline__ bool ilu_to_x() {
+        const int64_t nth = (int64_t)gs().nblocks * kConsumers;
+        const int64_t me = (int64_t)gs().bid * kConsumers + threadIdx.x;
+        T *const x = sys().x;
+        const T *t = sys().ilu.t;
+        for (int64_t i = me; i < sys().N; i += nth) x[i] = ldcg_val(t + i);
+        return gs().sync();
     }
 
     // ------------------------------------------------------------------
-    // passes (sums in gs.red->total)
+    // passes
     // ------------------------------------------------------------------
-
-    // r = b - A x, g_0 = r; sums ||b||^2, ||r||^2, q_1^H r.  The caller has
-    // posted kCmdResidual.
-    __device__ __noinline__ bool ph_residual(bool write_g0) {
-        constexpr int K = 2 + DS;
-        ACC acc[K];
+    // Those of the iteration leave this thread's share of their sums in
+    // sums.v[0, K) and return what ends them (inner() does it, in one place
+    // for all of them).
+    struct Sums {
+        double v[kMaxSums];
+        int K;        // sums; 0: a team barrier (the next pass gathers)
+        bool fence;   // the next pass gathers
+    };
+    template <int K>
+    __device__ __forceinline__ static void take(Sums &r, const ACC (&acc)[K], int used, bool fence) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) acc[k] = ACC(0);
-        T *g0 = Gc(0);
-        const T *epi[2] = {sys.b, Qc(0)};
-        T *const r = sys.r;
-        unsigned sq = gs.seq();
-        // epilogues capture by value: a captured reference would keep the
-        // pointer in memory, reloaded after every store of the loop
-        spmv_rows<2>(sys.x, epi, sq, [=](int64_t row, T y, const T (&e)[2], ACC(&a)[K]) {
-            T rv = subT(e[0], y);
-            r[row] = rv;
-            if (write_g0) g0[row] = rv;
-            acc_nrm(&a[0], e[0]);
-            acc_nrm(&a[1], rv);
-            acc_dot(&a[2], e[1], rv);
-        }, acc);
-        gs.seq() = sq;
-        sbytes(write_g0 ? 4 : 3);
-        return reduce<K>(acc, true);
+        for (int k = 0; k < K; ++k) r.v[k] = (double)acc[k];
+        r.K = used;
+        r.fence = fence;
     }
 
     // Refined mode, inner start with x_0 = 0: b = r = g_0 = src * scale
@@ -1196,10 +1379,10 @@ struct Engine {
         ACC acc[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) acc[k] = ACC(0);
-        T *const bq = sys.b;
-        T *const rq = sys.r;
-        T *const xq = sys.x;
-        const int64_t clo = c_lo, chi = c_hi;
+        T *const bq = sys().b;
+        T *const rq = sys().r;
+        T *const xq = sys().x;
+        const int64_t clo = c_lo(), chi = c_hi();
         {
             for (int64_t ch = clo + threadIdx.x; ch < chi; ch += kConsumers) {
                 const uint4 *sp = reinterpret_cast<const uint4 *>(src) + 2 * ch;
@@ -1229,11 +1412,11 @@ struct Engine {
         double v[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) v[k] = (double)acc[k];
-        if (!gs.template reduce<K>(v, true)) return false;
-        bb = gs.red->total[0];
-        rr = gs.red->total[1];
-        qr = mk_coef<T>(gs.red->total + 2);
-        if (threadIdx.x == kAcctThread) acct->bytes += sys.N * (int64_t)(sizeof(TW) + 5 * sizeof(T));
+        if (!gs().template reduce<K>(v, true)) return false;
+        bb = the_red().total[0];
+        rr = the_red().total[1];
+        qr = mk_coef<T>(the_red().total + 2);
+        if (threadIdx.x == kAcctThread) acct().bytes += sys().N * (int64_t)(sizeof(TW) + 5 * sizeof(T));
         return true;
     }
 
@@ -1252,8 +1435,8 @@ struct Engine {
         ACC acc[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) acc[k] = ACC(0);
-        T *const rq = sys.r;
-        const int64_t clo = c_lo, chi = c_hi;
+        T *const rq = sys().r;
+        const int64_t clo = c_lo(), chi = c_hi();
         {
             for (int64_t ch = clo + threadIdx.x; ch < chi; ch += kConsumers) {
                 const uint4 *sp = reinterpret_cast<const uint4 *>(src) + 2 * ch;
@@ -1282,55 +1465,73 @@ struct Engine {
         double v[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) v[k] = (double)acc[k];
-        if (!gs.template reduce<K>(v, true)) return false;
-        rr = gs.red->total[0];
-        qr = mk_coef<T>(gs.red->total + 1);
-        fr = mk_coef<T>(gs.red->total + 1 + DS);
+        if (!gs().template reduce<K>(v, true)) return false;
+        rr = the_red().total[0];
+        qr = mk_coef<T>(the_red().total + 1);
+        fr = mk_coef<T>(the_red().total + 1 + DS);
         if (threadIdx.x == kAcctThread)
-            acct->bytes += sys.N * (int64_t)(sizeof(TW) + (1 + (qv ? 1 : 0) + (fv ? 1 : 0)) * sizeof(T));
+            acct().bytes += sys().N * (int64_t)(sizeof(TW) + (1 + (qv ? 1 : 0) + (fv ? 1 : 0)) * sizeof(T));
         return true;
     }
 
-    // w_i = A g_i; sum q_i^H w.
-    __device__ __forceinline__ bool ph_spmv_c(int i, unsigned &sq) {
-        ACC acc[DS];
-#pragma unroll
-        for (int k = 0; k < DS; ++k) acc[k] = ACC(0);
-        T *const w = Wc(i);
-        const T *epi[1] = {Qc(i)};
-        spmv_rows<1>(Gc(i), epi, sq, [=](int64_t row, T y, const T (&e)[1], ACC(&a)[DS]) {
-            w[row] = y;
-            acc_dot(&a[0], e[0], y);
-        }, acc);
-        sbytes(1);
-        return reduce<DS>(acc, false);
-    }
-
-    // z = A u (u held in r); sums z^H z, z^H u.
-    __device__ __forceinline__ bool ph_spmv_z(unsigned &sq) {
-        constexpr int K = 1 + DS;
+    // The products, one copy of the code (several crowd each other out of
+    // the registers): P_SPMV_C: w_i = A g_i, sum q_i^H w.  P_SPMV_Z: z = A u
+    // (u held in r), sums z^H z, z^H u.  P_RESIDUAL: r = b - A x, g_0 = r
+    // (write_g0), sums ||b||^2, ||r||^2, q_1^H r (q_1 by direct loads: one
+    // such pass per call of the method).
+    __device__ __forceinline__ void ph_product(int what, int i, bool write_g0, unsigned &sq, Sums &sums) {
+        constexpr int K = 2 + DS;
         ACC acc[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) acc[k] = ACC(0);
-        const T *epi[1] = {sys.r};
-        T *const z = sys.z;
-        spmv_rows<1>(sys.r, epi, sq, [=](int64_t row, T y, const T (&e)[1], ACC(&a)[K]) {
-            z[row] = y;
-            acc_nrm(&a[0], y);
-            acc_dot(&a[1], y, e[0]);
+        const bool az = what == P_SPMV_Z, res = what == P_RESIDUAL;
+        T *const out = az ? sys().z : res ? sys().r : Wc(i);
+        T *const g0 = Gc(0);
+        const T *const q1 = sys().Q;
+        const T *epi[1] = {az ? sys().r : res ? sys().b : Qc(i)};
+        // epilogues capture by value: a captured reference would keep the
+        // pointer in memory, reloaded after every store of the loop
+        spmv_rows(az ? sys().r : res ? sys().x : Gc(i), epi, sys().spt[res ? 2 : 1], sq,
+                  [=](int64_t row, T y, const T (&e)[1], ACC(&a)[K]) {
+            if (res) {
+                const T rv = subT(e[0], y);
+                out[row] = rv;
+                if (write_g0) g0[row] = rv;
+                acc_nrm(&a[0], e[0]);
+                acc_nrm(&a[1], rv);
+                acc_dot(&a[2], ldg_val(q1 + row), rv);
+            } else {
+                out[row] = y;
+                if (az) {
+                    acc_nrm(&a[1], y);
+                    acc_dot(&a[2], y, e[0]);
+                } else {
+                    acc_dot(&a[2], e[0], y);
+                }
+            }
         }, acc);
-        sbytes(1);
-        return reduce<K>(acc, false);
+        sbytes(res ? (write_g0 ? 4 : 3) : 1);
+        // the sums are the last ones of acc
+        const int drop = res ? 0 : az ? 1 : 2;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            ACC v = acc[k];
+            if (drop == 1) v = acc[k + 1 < K ? k + 1 : k];
+            if (drop == 2) v = acc[k + 2 < K ? k + 2 : k];
+            sums.v[k] = (double)v;
+        }
+        sums.K = K - drop;
+        sums.fence = res;
     }
 
     // x += alpha g_sl, r -= alpha w_sl; sums ||r||^2, q_qcol^H r (hq) and
     // (when f0) f_1^H r.
-    __device__ __forceinline__ bool ph_alpha(S alpha, bool hq, bool f0, unsigned &sq) {
+    __device__ __forceinline__ void ph_alpha(S alpha, bool hq, bool f0, unsigned &sq, Sums &sums) {
         constexpr int K = 1 + 2 * DS;
         const T a = to_t<T>(alpha), na = to_t<T>(-alpha);
         const int ni = 4 + (hq ? 1 : 0) + (f0 ? 1 : 0), iff = hq ? 5 : 4;
-        T *const xo = sys.x;
-        T *const ro = sys.r;
+        T *const xo = sys().x;
+        T *const ro = sys().r;
         const int tc = tile_chunks_for(ni);
         ACC acc[K];
 #pragma unroll
@@ -1359,23 +1560,17 @@ struct Engine {
             }
         });
         vbytes(6 + (hq ? 1 : 0) + (f0 ? 1 : 0));
-        if (f0) return reduce<K>(acc, false);
         // without f the sums are ||r||^2 and q^H r, at the block's end (u in
         // r, which the next pass gathers) ||u||^2 alone
-        ACC a1[1 + DS];
-#pragma unroll
-        for (int k = 0; k < 1 + DS; ++k) a1[k] = acc[k];
-        if (hq) return reduce<1 + DS>(a1, false);
-        ACC a0[1] = {acc[0]};
-        return reduce<1>(a0, true);
+        take<K>(sums, acc, f0 ? K : hq ? 1 + DS : 1, !hq);
     }
 
     // x += omega u, r = u - omega z (u in r); sums ||r||^2, q_1^H r.
-    __device__ __forceinline__ bool ph_omega(S omega, unsigned &sq) {
+    __device__ __forceinline__ void ph_omega(S omega, unsigned &sq, Sums &sums) {
         constexpr int K = 1 + DS;
         const T om = to_t<T>(omega), nom = to_t<T>(-omega);
-        T *const xo = sys.x;
-        T *const ro = sys.r;
+        T *const xo = sys().x;
+        T *const ro = sys().r;
         const int tc = tile_chunks_for(4);
         ACC acc[K];
 #pragma unroll
@@ -1397,11 +1592,11 @@ struct Engine {
             }
         });
         vbytes(6);
-        return reduce<K>(acc, false);
+        take<K>(sums, acc, K, false);
     }
 
     // z_w = r + bt0 w_i (first) or z_w += bts w_s, in place; sum q^H z_w.
-    __device__ __forceinline__ bool ph_w(bool first, S coef, int i, unsigned &sq) {
+    __device__ __forceinline__ void ph_w(bool first, S coef, int i, unsigned &sq, Sums &sums) {
         const T b = to_t<T>(coef);
         T *const wp = Wc(i);
         const int tc = tile_chunks_for(3);
@@ -1420,32 +1615,32 @@ struct Engine {
             for (int e = 0; e < PW; ++e) acc_dot(&acc[0], qq.e[e], zw.e[e]);
         });
         vbytes(4);
-        return reduce<DS>(acc, false);
+        take<DS>(sums, acc, DS, false);
     }
 
     // Last pass of the z_w sweep, fused with every deferred g-update of the
     // sweep and the omega-correction:
-    //   first=true : z_w = r + bt[sl] w_sl                (empty s-loop)
-    //   first=false: z_w += bt[last] w_last
-    //   g = bt[sl] g_sl;  g += bt[t] g_t for t = sl+1..n-1;  g = z_w - g/omega
+    //   first=true : z_w = r + bt()[sl] w_sl                (empty s-loop)
+    //   first=false: z_w += bt()[last] w_last
+    //   g = bt()[sl] g_sl;  g += bt()[t] g_t for t = sl+1..n-1;  g = z_w - g/omega
     // sums f_1^H g when with_f.  The first kMaxInputs-4 columns g_t come
     // through the tile pipeline, any further ones by direct loads.
-    __device__ __forceinline__ bool ph_w_last(int sl, unsigned &sq) {
-        const int n = sys.n;
+    __device__ __forceinline__ void ph_w_last(int sl, unsigned &sq, Sums &sums) {
+        const int n = sys().n;
         const int last = n - 1;
         const bool first = sl == last, with_f = sl > 0;
         T *wp = Wc(sl);
         T *gp = Gc(sl);
-        const T bl = to_t<T>(bt[first ? sl : last]);
-        const T b0 = to_t<T>(bt[sl]);
-        const T nio = to_t<T>(-sc->inv_omega);
+        const T bl = to_t<T>(bt()[first ? sl : last]);
+        const T b0 = to_t<T>(bt()[sl]);
+        const T nio = to_t<T>(-sc().inv_omega);
         const int t0 = sl + 1;
         const int nt = n - t0;                                     // g_t columns
         const int ntile = nt < kMaxInputs - 4 ? nt : kMaxInputs - 4;
         const int i_t = with_f ? 4 : 3;
-        const T *const Gb = sys.G;
-        const int64_t ldv = sys.ld;
-        const S *const btl = bt;
+        const T *const Gb = sys().G;
+        const int64_t ldv = sys().ld;
+        const S *const btl = bt();
         const int tc = tile_chunks_for(i_t + ntile);
         ACC acc[DS];
 #pragma unroll
@@ -1478,13 +1673,12 @@ struct Engine {
             }
         });
         vbytes(5 + nt + (with_f ? 1 : 0));
-        if (!with_f) return gs.sync() && ring_ok();   // the next pass gathers g
-        return reduce<DS>(acc, false);
+        take<DS>(sums, acc, with_f ? DS : 0, !with_f);   // without f the next pass gathers g
     }
 
     // g_i += beta g_s, or (block 0's first) g_i = r + beta g_0; sums f^H g_i, or, at the sweep's end (the next pass gathers g_i), a team
     // barrier.
-    __device__ __forceinline__ bool ph_g(S beta, int i, bool with_f, unsigned &sq) {
+    __device__ __forceinline__ void ph_g(S beta, int i, bool with_f, unsigned &sq, Sums &sums) {
         const T bb = to_t<T>(beta);
         T *gp = Gc(i);
         const int tc = tile_chunks_for(with_f ? 3 : 2);
@@ -1503,8 +1697,7 @@ struct Engine {
             }
         });
         vbytes(with_f ? 4 : 3);
-        if (!with_f) return gs.sync() && ring_ok();
-        return reduce<DS>(acc, false);
+        take<DS>(sums, acc, with_f ? DS : 0, !with_f);
     }
 
     // ------------------------------------------------------------------
@@ -1518,9 +1711,9 @@ struct Engine {
     };
 
     __device__ __forceinline__ void record(bool rec, int64_t iter, double err) {
-        if (rec && ctl.err_hist && iter < ctl.hist_cap && gs.bid == 0) ctl.err_hist[iter] = err;
+        if (rec && ctl().err_hist && iter < ctl().hist_cap && gs().bid == 0) ctl().err_hist[iter] = err;
     }
-    __device__ __forceinline__ S total(int k) const { return mk_coef<T>(gs.red->total + k); }
+    __device__ __forceinline__ S total(int k) const { return mk_coef<T>(the_red().total + k); }
 
     // `init` (refined mode only): start from x_0 = 0 with b = init * scale
     // instead of reading b and x.  `hook` (refined mode only, in shared
@@ -1534,307 +1727,371 @@ struct Engine {
     // outer tolerance) and, at block ends, when hook->want(err) (reliable
     // updates); a block end also ends the call when hook->stalled(iter, err).
     //
+    // last: only the residual pass (after the last iteration; ||b||^2 and
+    // ||r||^2 are then in the_red().total).  One call site per kernel, inlined:
+    // this is the kernel's loop, and a call in it costs every pass registers.
+    //
     // After inner() returns, x and r are visible to their own CTA only: a
     // team barrier comes before any pass that gathers them.
     template <typename Hook = NoHook>
-    __device__ Out inner(int64_t maxit, bool rec, double tol,
-                         const typename wide_of<T>::type *init = nullptr, double scale = 1.0,
-                         Hook *hook = nullptr) {
-        const int n = sys.n;
+    __device__ __forceinline__ Out inner(bool last, int64_t maxit, bool rec, double tol,
+                                         const typename wide_of<T>::type *init = nullptr, double scale = 1.0,
+                                         Hook *hook = nullptr) {
         const int tid = threadIdx.x;
-        rec = rec && ctl.err_hist != nullptr;
         Out o{1, 0, 0, 0, 0.0};
-        if (tid == kAcctThread)
-            for (int q = 0; q < 5; ++q) acct->ops[q] = 0;
-
-        // r_0 = b - A x_0 (step 2) with the stopping-rule denominator
-        bool started = false;
-        if constexpr (is_narrow<T>::value) {
-            if (init) {
-                double bb, rr;
-                S e;
-                if (!ph_init_narrow(init, scale, bb, rr, e)) return o;
-                op(OP_NORM, 2);
-                started = true;
-            }
-        }
-        if (!started) {
-            if (!ilu_pre(sys.x)) return o;
-            gs.post(kCmdResidual);
-            if (!ph_residual(true)) return o;
-            op(OP_NORM, 2);
-            op(OP_MATVEC, 1);
-        }
+        if (tid == kAcctThread && !last)
+            for (int q = 0; q < 5; ++q) acct().ops[q] = 0;
         if (tid == 0) {
-            sc->e = total(2);
-            const double t0 = sqrt(gs.red->total[0]);
-            const double bn = t0 == 0.0 ? 1.0 : t0, rr = gs.red->total[1], e0 = sqrt(rr) / bn;
-            sc->bnrm2 = bn;
-            sc->rr = rr;
-            sc->err = e0;
-            // sqrt(rr) / bn < tol is impossible above this (1e-12 covers
-            // the roundings; below 1e-290 the exact test decides)
-            const double t = tol * bn, f = t * t * (1.0 + 1e-12);
-            sc->far = f > 1e-290 ? f : 1e-290;
-            sc->iter = 0;
-            sc->flag = 1;
-            sc->exit = 0;
-            sc->j = sc->i = 0;
-            sc->act = sc->conv = 0;
-            record(rec, 0, e0);
-            if (e0 < tol) {
-                sc->flag = 0;
-                sc->exit = 1;
-            }
-            if constexpr (Hook::kActive) hook->reset(e0);
+            sc().tol = tol;
+            sc().maxit = maxit;
+            sc().rec = rec && ctl().err_hist != nullptr;
         }
-        consumer_sync();
-        o.err = sc->err;
-        if (sc->exit) {
-            o.flag = sc->flag;
-            return o;
-        }
-        // the producer's first step is the product w_0 = A g_0
-        gs.post(kCmdInner);
-        unsigned sq = gs.seq(), passes = 0;
-        const unsigned pass0 = gs.ring->passes;
 
-        int j = 0;
-        for (Step st;; st.advance(n)) {
-            const int i = st.i;
+        Step st;
+        if constexpr (is_narrow<T>::value) {
+            double bb, rr;
+            S e;
+            if (!ph_init_narrow(init, scale, bb, rr, e)) return o;
+            op(OP_NORM, 2);
+            if (tid == 0) start();
+            if (tid == 0 && Hook::kActive) hook->reset(sc().err);
+            consumer_sync();
+            o.err = sc().err;
+            if (sc().exit) {
+                o.flag = sc().flag;
+                return o;
+            }
+            begin_inner();
+        } else {
+            // r_0 = b - A x_0 (step 2) with the stopping-rule denominator
+            st.op = P_RESIDUAL;
+        }
+        unsigned sq = gs().seq();
+
+        // what lives from pass to pass is in shared memory: the registers
+        // belong to the pass
+        for (;; st.advance(sys().n)) {
+            const int i = st.i, n = sys().n;
+            // which of its two forms a sweep's pass has (see the cases)
+            const bool hq = i < n;                      // P_ALPHA: not the block's end
+            const bool f0 = st.first && hq;             // P_ALPHA: block 0's f_1^H r
+            const int s1 = st.op == P_F_ROUND ? st.s + 1 : 1;
+            const bool more = s1 <= i - 1;              // P_F_ROUND, P_G_J0: another f follows
             bool good = true;
-            switch (st.op) {
-            case P_SPMV_C:
-                // steps 31-32, 51 (and w_0 = A g_0): w = A g, c = q_{i+1}^H w
-                good = ilu_pre(Gc(i)) && ph_spmv_c(i, sq);
-                op(OP_MATVEC);
-                op(OP_DOT);
-                if (tid == 0) {
-                    const S cv = total(0);
-                    c[i] = cv;
-                    if (is_zero(cv) || !finite_of(cv)) {
-                        sc->flag = -1;
-                        sc->exit = 1;
-                    }
-                    sc->coef = sc->e / cv;
+            if (!is_narrow<T>::value && st.op == P_RESIDUAL) gs().post(kCmdResidual);
+            if constexpr (PC) {
+                if ((st.op == P_SPMV_C || st.op == P_SPMV_Z || st.op == P_RESIDUAL) && sys().ilu.lu) {
+                    gs().seq() = sq;
+                    good = ilu_solve_body(st.op == P_SPMV_C ? Gc(i) : st.op == P_SPMV_Z ? sys().r : sys().x,
+                                          sys().ilu.t);
+                    sq = gs().seq();
                 }
+            }
+            Sums sums;
+            switch (st.op) {
+            case P_RESIDUAL:
+            case P_SPMV_C:   // steps 31-32, 51 (and w_0 = A g_0): w = A g, c = q_{i+1}^H w
+            case P_SPMV_Z:   // step 38
+                ph_product(st.op, i, !last, sq, sums);
                 break;
-            case P_ALPHA: {
+            case P_ALPHA:
                 // steps 5-8: alpha, x, r, e (and f_1^H r in block 0); steps
                 // 34-36 at the block's end (u kept in r)
-                const bool hq = i < n, f0 = st.first && hq;
-                // the inner product of c_0 belongs to the first block's start
-                if (st.first && i == 1) op(OP_DOT);
-                good = ph_alpha(sc->coef, hq, f0, sq);
-                op(OP_SAXPY, 2);
-                op(OP_NORM);
-                if (tid == kErrThread) {
-                    sc->j = j;
-                    sc->i = i;
-                    residual_norm<Hook>(gs.red->total[0], hq, false, maxit, rec, tol, hook);
-                }
-                if (hq && tid == 0) alpha_coef(i, f0);
+                ph_alpha(sc().coef, hq, f0, sq, sums);
+                break;
+            case P_OMEGA:    // steps 39-41: x += omega u, r = u - omega A u, e = q_1^H r
+                ph_omega(sc().coef, sq, sums);
+                break;
+            case P_W_FIRST:  // steps 10-17, 42-48: sweep the rest of block j-1 with q's
+            case P_W_ROUND:
+                ph_w(st.op == P_W_FIRST, sc().coef, i, sq, sums);
+                break;
+            case P_W_LAST:   // its end, with the omega-correction (steps 18, 50)
+                ph_w_last(i, sq, sums);
+                break;
+            default:         // steps 19-22 (24-28 in block 0): sweep block j with f's
+                ph_g(sc().coef, i, more, sq, sums);
                 break;
             }
-            case P_SPMV_Z:
-                // step 38: omega = (A u)^H u / ||A u||^2, Eq. 5.1 guard
-                good = ilu_pre(sys.r) && ph_spmv_z(sq);
-                op(OP_MATVEC);
-                op(OP_DOT);
-                if (tid == 0) {
-                    const double zz = gs.red->total[0];
+            good = (sums.K ? gs().reduce_k(sums.v, sums.K, sums.fence) : gs().sync()) && good && ring_ok();
+            // the scalars of the next pass, the stopping rule and the
+            // accounting, each on a thread of its own warp
+            if (tid == 0) {
+                switch (st.op) {
+                case P_RESIDUAL:
+                    if (!last) start();
+                    break;
+                case P_SPMV_C: {
+                    const S cv = total(0);
+                    c()[i] = cv;
+                    if (is_zero(cv) || !finite_of(cv)) {
+                        sc().flag = -1;
+                        sc().exit = 1;
+                    }
+                    sc().coef = sc().e / cv;
+                    break;
+                }
+                case P_ALPHA:
+                    if (hq) alpha_coef(i, f0);
+                    break;
+                case P_SPMV_Z: {
+                    // omega = (A u)^H u / ||A u||^2, Eq. 5.1 guard
+                    const double zz = the_red().total[0];
                     const S zu = total(1);
                     const bool bad = zz == 0.0 || !isfinite(zz);
                     S om = zu / zz;
-                    if (ctl.kappa > 0.0) {
-                        const double arho = abs_of(zu) / (sqrt(zz) * sqrt(sc->rr));
-                        if (arho < ctl.kappa && arho != 0.0) om = (ctl.kappa * om) / arho;
+                    if (ctl().kappa > 0.0) {
+                        const double arho = abs_of(zu) / (sqrt(zz) * sqrt(sc().rr));
+                        if (arho < ctl().kappa && arho != 0.0) om = (ctl().kappa * om) / arho;
                     }
                     if (bad || is_zero(om) || !finite_of(om)) {
-                        sc->flag = -1;
-                        sc->exit = 1;
+                        sc().flag = -1;
+                        sc().exit = 1;
                     }
-                    sc->act = bad;   // counted below
-                    sc->coef = om;
-                    sc->omega = om;
+                    sc().bad = bad;
+                    sc().coef = om;
+                    sc().omega = om;
+                    break;
                 }
-                break;
-            case P_OMEGA:
-                // steps 39-41: x += omega u, r = u - omega A u, e = q_1^H r
-                good = ph_omega(sc->coef, sq);
-                op(OP_SAXPY, 2);
-                op(OP_NORM);
-                if (tid == kErrThread) residual_norm<Hook>(gs.red->total[0], true, true, maxit, rec, tol, hook);
-                if (tid == 2 * kErrThread) sc->inv_omega = recip(sc->omega);
-                if (tid == 0) omega_coef();
-                break;
-            case P_W_FIRST:
-            case P_W_ROUND: {
-                // steps 10-17, 42-48: sweep the rest of block j-1 with q's
-                const bool wf = st.op == P_W_FIRST;
-                if (wf) {
-                    op(OP_SAXPY);
-                    op(OP_SCALE);
-                } else {
-                    op(OP_DOT);
-                    op(OP_SAXPY, 2);
+                case P_OMEGA:
+                    omega_coef();
+                    break;
+                case P_W_FIRST:
+                case P_W_ROUND: {
+                    const int s = st.op == P_W_FIRST ? i + 1 : st.s + 1;
+                    const S b = -(total(0) / c()[s]);
+                    bt()[s] = b;
+                    sc().coef = b;
+                    break;
                 }
-                good = ph_w(wf, sc->coef, i, sq);
-                if (tid == 0) {
-                    const int s = wf ? i + 1 : st.s + 1;
-                    const S b = -(total(0) / c[s]);
-                    bt[s] = b;
-                    sc->coef = b;
+                case P_W_LAST:
+                    if (i > 0) sc().coef = -(total(0) / c()[0]);
+                    break;
+                default:
+                    if (more) sc().coef = -(total(0) / c()[s1]);
+                    break;
                 }
-                break;
+            } else if (tid == kErrThread) {
+                if (st.op == P_ALPHA) {
+                    sc().j = sc().block;
+                    sc().i = i;
+                }
+                if (st.op == P_OMEGA) sc().block += 1;
+                if (st.op == P_ALPHA || st.op == P_OMEGA)
+                    residual_norm<Hook>(the_red().total[0], st.op == P_OMEGA || hq, st.op == P_OMEGA, hook);
+            } else if (tid == kAcctThread) {
+                if (st.op == P_OMEGA) sc().inv_omega = recip(sc().omega);
+                if (!last) count(st, n);
             }
-            case P_W_LAST:
-                if (i == n - 1) {
-                    op(OP_SAXPY);
-                    op(OP_SCALE);
-                } else {
-                    op(OP_DOT);
-                    op(OP_SAXPY, 2);
-                }
-                op(OP_SAXPY);   // omega-correction (steps 18, 50)
-                good = ph_w_last(i, sq);
-                if (i > 0 && tid == 0) sc->coef = -(total(0) / c[0]);
-                break;
-            default: {   // P_F_ROUND, P_G_J0
-                // steps 19-22 (24-28 in block 0): sweep block j with f's
-                const int s1 = st.op == P_F_ROUND ? st.s + 1 : 1;
-                const bool more = s1 <= i - 1;
-                op(OP_DOT);
-                op(OP_SAXPY);
-                good = ph_g(sc->coef, i, more, sq);
-                if (more && tid == 0) sc->coef = -(total(0) / c[s1]);
-                break;
-            }
-            }
-            ++passes;
+            if (tid == 0) sc().passes += 1;
             consumer_sync();
+            if (st.op == P_RESIDUAL) {
+                if (!good || last || sc().exit) {
+                    gs().seq() = sq;
+                    if (!last) {
+                        o.err = sc().err;
+                        if (good) o.flag = sc().flag;
+                    }
+                    return o;
+                }
+                begin_inner();
+                continue;
+            }
             if (!good) break;
-            if (st.op == P_SPMV_Z) {
-                if (!sc->act) op(OP_DOT);
-                if (!sc->act && ctl.kappa > 0.0) op(OP_NORM, 2);
+            if (st.op == P_SPMV_Z && !sc().bad) {
+                op(OP_DOT);
+                if (ctl().kappa > 0.0) op(OP_NORM, 2);
             }
             if constexpr (Hook::kActive) {
                 if (st.op == P_ALPHA || st.op == P_OMEGA) {
-                    if (sc->exit) break;
-                    const bool hq = st.op == P_OMEGA || i < n;
-                    if (sc->act) {
-                        const bool f0 = st.op == P_ALPHA && st.first && hq;
-                        gs.seq() = sq;
+                    if (sc().exit) break;
+                    const bool whole = st.op == P_OMEGA || hq;   // not the half step u
+                    const bool f1 = st.op == P_ALPHA && f0;
+                    if (sc().act) {
+                        gs().seq() = sq;
                         double rr;
                         S qr, fr;
                         bool conv;
-                        good = hook->replace(st.op == P_OMEGA ? 0 : hq ? i : -1, f0, rr, qr, fr, conv);
-                        sq = gs.seq();
-                        ++passes;
+                        good = hook->replace(st.op == P_OMEGA ? 0 : hq ? i : -1, f1, rr, qr, fr, conv);
+                        sq = gs().seq();
+                        if (tid == 0) sc().passes += 1;
                         if (!good) break;
-                        if (tid == kErrThread) replaced<Hook>(rr, conv, st.op, hq, maxit, hook);
-                        if (tid == 0 && hq) {
+                        if (tid == kErrThread) replaced<Hook>(rr, conv, st.op, whole, hook);
+                        if (tid == 0 && whole) {
                             if (st.op == P_OMEGA) omega_coef();
-                            else alpha_coef(i, f0);
+                            else alpha_coef(i, f1);
                         }
                         consumer_sync();
-                        if (sc->exit) break;
+                        if (sc().exit) break;
                     }
-                    gs.post(kCmdGo);
+                    gs().post(kCmdGo);
                 }
             }
-            if (sc->exit) break;
-            if (st.op == P_ALPHA && i < n) op(OP_DOT);
-            if (st.op == P_OMEGA) {
-                op(OP_DOT);
-                ++j;
-            }
+            if (sc().exit) break;
+            if (st.op == P_ALPHA && hq) op(OP_DOT);
+            if (st.op == P_OMEGA) op(OP_DOT);
         }
-        gs.end_inner(sq, pass0 + passes);
-        gs.seq() = sq;
-        o.flag = gs.ok ? sc->flag : 1;
-        o.iter = sc->iter;
-        o.j = sc->j;
-        o.i = sc->i;
-        o.err = sqrt(sc->rr) / sc->bnrm2;
+        gs().end_inner(sq, sc().passes);
+        gs().seq() = sq;
+        o.flag = gs().ok ? sc().flag : 1;
+        o.iter = sc().iter;
+        o.j = sc().j;
+        o.i = sc().i;
+        o.err = sqrt(sc().rr) / sc().bnrm2;
         return o;
     }
 
+    // Thread 0: the scalars of a start, from ||b||^2, ||r||^2, q_1^H r.
+    __device__ __forceinline__ void start() {
+        sc().e = total(2);
+        const double t0 = sqrt(the_red().total[0]);
+        const double bn = t0 == 0.0 ? 1.0 : t0, rr = the_red().total[1], e0 = sqrt(rr) / bn;
+        sc().bnrm2 = bn;
+        sc().rr = rr;
+        sc().err = e0;
+        // sqrt(rr) / bn < tol is impossible above this (1e-12 covers the
+        // roundings; below 1e-290 the exact test decides)
+        const double t = sc().tol * bn, f = t * t * (1.0 + 1e-12);
+        sc().far = f > 1e-290 ? f : 1e-290;
+        sc().iter = 0;
+        sc().flag = 1;
+        sc().exit = 0;
+        sc().j = sc().i = sc().block = 0;
+        sc().act = sc().conv = 0;
+        record(sc().rec != 0, 0, e0);
+        if (e0 < sc().tol) {
+            sc().flag = 0;
+            sc().exit = 1;
+        }
+    }
+    // The producer's first step is the product w_0 = A g_0.
+    __device__ __forceinline__ void begin_inner() {
+        gs().post(kCmdInner);
+        if (threadIdx.x == 0) sc().passes = the_ring()->passes;
+    }
+    // Thread kAcctThread: the operations of a pass that are counted before
+    // its exits.
+    __device__ __forceinline__ void count(const Step &st, int n) {
+        const int i = st.i;
+        switch (st.op) {
+        case P_RESIDUAL:
+            op(OP_NORM, 2);
+            op(OP_MATVEC);
+            break;
+        case P_SPMV_C:
+        case P_SPMV_Z:
+            op(OP_MATVEC);
+            op(OP_DOT);
+            break;
+        case P_ALPHA:
+            // the inner product of c_0 belongs to the first block's start
+            if (st.first && i == 1) op(OP_DOT);
+            op(OP_SAXPY, 2);
+            op(OP_NORM);
+            break;
+        case P_OMEGA:
+            op(OP_SAXPY, 2);
+            op(OP_NORM);
+            break;
+        case P_W_LAST:
+            op(OP_SAXPY);   // omega-correction (steps 18, 50)
+            if (i == n - 1) {
+                op(OP_SAXPY);
+                op(OP_SCALE);
+            } else {
+                op(OP_DOT);
+                op(OP_SAXPY, 2);
+            }
+            break;
+        case P_W_FIRST:
+            op(OP_SAXPY);
+            op(OP_SCALE);
+            break;
+        case P_W_ROUND:
+            op(OP_DOT);
+            op(OP_SAXPY, 2);
+            break;
+        default:
+            op(OP_DOT);
+            op(OP_SAXPY);
+            break;
+        }
+    }
     // Thread 0: the coefficient after an update of r within a block
-    // (i: the step's slot): e, then beta~ of the sweep with q's (bt[i]) or,
+    // (i: the step's slot): e, then beta~ of the sweep with q's (bt()[i]) or,
     // in block 0, beta of the one with f's.
     __device__ __forceinline__ void alpha_coef(int i, bool f0) {
         const S e = total(1);
-        sc->e = e;
+        sc().e = e;
         if (f0) {
-            sc->coef = -(total(1 + DS) / c[0]);
+            sc().coef = -(total(1 + DS) / c()[0]);
         } else {
-            const S b = -(e / c[i]);
-            bt[i] = b;
-            sc->coef = b;
+            const S b = -(e / c()[i]);
+            bt()[i] = b;
+            sc().coef = b;
         }
     }
     // Thread 0: the coefficient after the omega step.
     __device__ __forceinline__ void omega_coef() {
         const S e = total(1);
-        sc->e = e;
-        const S b = -(e / c[0]);
-        bt[0] = b;
-        sc->coef = b;
+        sc().e = e;
+        const S b = -(e / c()[0]);
+        bt()[0] = b;
+        sc().coef = b;
     }
     // Thread kErrThread, after an update of r (or of u at the block's end,
     // counts = false): iteration count, stopping rule, iteration limit.
     // The division and the square root of ||r|| / ||b|| are only taken where
     // the value is recorded or can decide.
     template <typename Hook>
-    __device__ __forceinline__ void residual_norm(double rr, bool counts, bool block_end, int64_t maxit, bool rec,
-                                                  double tol, Hook *hook) {
-        sc->rr = rr;
-        int64_t iter = sc->iter + (counts ? 1 : 0);
-        sc->iter = iter;
+    __device__ __forceinline__ void residual_norm(double rr, bool counts, bool block_end, Hook *hook) {
+        const bool rec = sc().rec != 0;
+        sc().rr = rr;
+        int64_t iter = sc().iter + (counts ? 1 : 0);
+        sc().iter = iter;
         bool conv = false;
-        if (Hook::kActive || rec || !(rr > sc->far)) {
-            const double err = sqrt(rr) / sc->bnrm2;
-            conv = err < tol;
+        if (Hook::kActive || rec || !(rr > sc().far)) {
+            const double err = sqrt(rr) / sc().bnrm2;
+            conv = err < sc().tol;
             if constexpr (Hook::kActive) {
                 hook->track(err);
-                sc->act = conv || (block_end && hook->want(err));
-                if (!sc->act) after_norm(err, counts, block_end, maxit, hook);
+                sc().act = conv || (block_end && hook->want(err));
+                if (!sc().act) after_norm(err, counts, block_end, hook);
                 return;
             }
             if (conv && !counts) {
                 iter++;
-                sc->iter = iter;
+                sc().iter = iter;
             }
             if (counts || conv) record(rec, iter, err);
         }
         if (conv) {
-            sc->flag = 0;
-            sc->exit = 1;
-        } else if (counts && iter >= maxit) {
-            sc->exit = 1;
+            sc().flag = 0;
+            sc().exit = 1;
+        } else if (counts && iter >= sc().maxit) {
+            sc().exit = 1;
         }
     }
     // Refined mode: the tests that follow the (possibly replaced) residual.
     template <typename Hook>
-    __device__ __forceinline__ void after_norm(double err, bool counts, bool block_end, int64_t maxit, Hook *hook) {
+    __device__ __forceinline__ void after_norm(double err, bool counts, bool block_end, Hook *hook) {
         if constexpr (Hook::kActive) {
-            if (block_end && hook->stalled(sc->iter, err)) sc->exit = 1;
-            else if (counts && sc->iter >= maxit) sc->exit = 1;
+            if (block_end && hook->stalled(sc().iter, err)) sc().exit = 1;
+            else if (counts && sc().iter >= sc().maxit) sc().exit = 1;
         }
     }
     template <typename Hook>
-    __device__ __forceinline__ void replaced(double rr, bool conv, int op_, bool hq, int64_t maxit, Hook *hook) {
+    __device__ __forceinline__ void replaced(double rr, bool conv, int op_, bool hq, Hook *hook) {
         if constexpr (Hook::kActive) {
-            sc->rr = rr;
-            const double err = sqrt(rr) / sc->bnrm2;
+            sc().rr = rr;
+            const double err = sqrt(rr) / sc().bnrm2;
             hook->reset(err);
             if (conv) {
-                if (!hq) sc->iter += 1;   // the converged half step counts
-                sc->flag = 0;
-                sc->exit = 1;
+                if (!hq) sc().iter += 1;   // the converged half step counts
+                sc().flag = 0;
+                sc().exit = 1;
             } else {
-                after_norm(err, hq, op_ == P_OMEGA, maxit, hook);
+                after_norm(err, hq, op_ == P_OMEGA, hook);
             }
         }
     }

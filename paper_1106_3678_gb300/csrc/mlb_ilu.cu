@@ -29,6 +29,53 @@ void group_levels(const std::vector<int32_t> &lev, int nlev, std::vector<int32_t
     for (size_t i = 0; i < lev.size(); ++i) rows[next[lev[i]]++] = (int32_t)i;
 }
 
+// One triangle in its streamed form (see IluLevel): row rows[q] has cnt[q]
+// entries, the first (upper: after the diagonal) ones of its row.  Sizes
+// first (fill = false), then the entries; U's diagonal by slot into `diag`.
+template <typename V>
+int64_t stream_levels(const IluHost &f, bool upper, bool fill, std::vector<IluLevel> &lev, std::vector<int32_t> &meta,
+                      std::vector<int32_t> &col, std::vector<char> &val, std::vector<char> *diag, int &maxw) {
+    const std::vector<int32_t> &rows = upper ? f.urows : f.lrows, &ptr = upper ? f.uptr : f.lptr;
+    const std::vector<int32_t> &cnt = upper ? f.ucnt : f.lcnt;
+    const V *lu = (const V *)f.lu.data();
+    const int nlev = (int)ptr.size() - 1;
+    int64_t e0 = 0;
+    int32_t m0 = 0;
+    if (!fill) lev.assign(nlev, IluLevel{});
+    for (int l = 0; l < nlev && !fill; ++l) {
+        int32_t w = 0;
+        for (int32_t q = ptr[l]; q < ptr[l + 1]; ++q) w = std::max(w, cnt[q]);
+        const int32_t ns = (ptr[l + 1] - ptr[l] + 31) / 32;
+        lev[l] = IluLevel{e0, m0, ns, w, 0};
+        e0 += 32 * (int64_t)ns * w;
+        m0 += ns;
+        maxw = std::max(maxw, w);
+    }
+    if (!fill) return e0;
+    const int64_t slots = 32 * (int64_t)(lev.back().m0 + lev.back().ns);
+    const int64_t entries = lev.back().e0 + 32 * (int64_t)lev.back().ns * lev.back().w;
+    meta.assign(2 * slots, 0);
+    for (int64_t q = 0; q < slots; ++q) meta[2 * q] = -1;
+    col.assign(entries, 0);
+    val.assign((size_t)entries * sizeof(V), 0);
+    if (diag) diag->assign((size_t)slots * sizeof(V), 0);
+    V *out = (V *)val.data();
+    for (int l = 0; l < nlev; ++l)
+        for (int32_t q = ptr[l]; q < ptr[l + 1]; ++q) {
+            const int64_t k = (q - ptr[l]) / 32, lane = (q - ptr[l]) % 32, m = 32 * (lev[l].m0 + k) + lane;
+            const int64_t i = rows[q], d = f.rp[i] + f.dpos[i], k0 = upper ? d + 1 : f.rp[i];
+            const int64_t p = lev[l].e0 + 32 * k * lev[l].w + lane;
+            meta[2 * m] = (int32_t)i;
+            meta[2 * m + 1] = cnt[q];
+            for (int32_t e = 0; e < cnt[q]; ++e) {
+                col[p + 32 * (int64_t)e] = f.ci[k0 + e];
+                out[p + 32 * (int64_t)e] = lu[k0 + e];
+            }
+            if (diag) ((V *)diag->data())[m] = lu[d];
+        }
+    return entries;
+}
+
 template <typename V>
 int build_t(const mlb_matrix *A, IluHost &f) {
     const int64_t N = A->nrows;
@@ -111,22 +158,37 @@ int build_t(const mlb_matrix *A, IluHost &f) {
     }
     group_levels(lev, nu, f.urows, f.uptr);
     f.nlev_u = nu;
-    // level-position copies (kIluEll entries per row, zero padded)
+    // copies by level: the streamed form (few levels), else kIluEll entries
+    // per row by level position, zero padded
     const V *lu = (const V *)f.lu.data();
     f.lcnt.assign(N, 0);
     f.ucnt.assign(N, 0);
+    for (int64_t q = 0; q < N; ++q) {
+        f.lcnt[q] = f.dpos[f.lrows[q]];
+        const int64_t j = f.urows[q];
+        f.ucnt[q] = (int32_t)(f.rp[j + 1] - f.rp[j] - f.dpos[j] - 1);
+    }
+    if (nl + nu <= kIluWideLevels) {
+        const int64_t filled =
+            stream_levels<V>(f, false, false, f.llev, f.lmeta, f.lell_c, f.lell_a, nullptr, f.maxw) +
+            stream_levels<V>(f, true, false, f.ulev, f.umeta, f.uell_c, f.uell_a, &f.udiag, f.maxw);
+        f.wide = filled <= 2 * f.nnz + 32 * (nl + nu) && ilu_slices_per_tile(f.maxw, sizeof(V)) > 0;
+    }
+    if (f.wide) {
+        stream_levels<V>(f, false, true, f.llev, f.lmeta, f.lell_c, f.lell_a, nullptr, f.maxw);
+        stream_levels<V>(f, true, true, f.ulev, f.umeta, f.uell_c, f.uell_a, &f.udiag, f.maxw);
+        return MLB_OK;
+    }
     f.lell_c.assign((size_t)kIluEll * N, 0);
     f.uell_c.assign((size_t)kIluEll * N, 0);
     std::vector<V> la((size_t)kIluEll * N, V(0)), ua((size_t)kIluEll * N, V(0)), ud(N, V(0));
     for (int64_t q = 0; q < N; ++q) {
         const int64_t i = f.lrows[q], k0 = f.rp[i], d = k0 + f.dpos[i];
-        f.lcnt[q] = (int32_t)(d - k0);
         for (int64_t e = 0; e < kIluEll && k0 + e < d; ++e) {
             f.lell_c[e * N + q] = f.ci[k0 + e];
             la[e * N + q] = lu[k0 + e];
         }
         const int64_t j = f.urows[q], dj = f.rp[j] + f.dpos[j], k1 = f.rp[j + 1];
-        f.ucnt[q] = (int32_t)(k1 - dj - 1);
         for (int64_t e = 0; e < kIluEll && dj + 1 + e < k1; ++e) {
             f.uell_c[e * N + q] = f.ci[dj + 1 + e];
             ua[e * N + q] = lu[dj + 1 + e];

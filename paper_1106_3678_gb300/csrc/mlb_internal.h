@@ -149,6 +149,17 @@ cudaError_t launch_spmv_qdot_tiled(const SysView<T> &sys, int ne, int64_t maxw, 
 // loads are then independent of each other (only the row's right-hand
 // side needs the row index).
 constexpr int kIluEll = 4;
+// Factors whose levels are few and so hold many rows each (a multicolour
+// order: two levels per triangle for the 7-point stencils) are kept in
+// another form instead, which the tile ring can stream (Engine::ilu_wide):
+// each level in slices of 32 rows (the last one filled up), all of one width
+// (the level's widest row): entry e of lane l of the level's slice k at
+// IluLevel::e0 + 32 (k w + e) + l, row number and entry count of the lane at
+// 32 (m0 + k) + l.  The line: at most kIluWideLevels levels in both triangles
+// together, at most twice the entries with the filling, and slices that fit
+// a stage.  A natural order has one level per wavefront (80 at 14^3, 766 at
+// 128^3), where a level is a few rows per CTA and its cost the barrier.
+constexpr int kIluWideLevels = 32;
 struct IluHost {
     std::vector<int64_t> rp;
     std::vector<int32_t> ci, dpos, lrows, lptr, urows, uptr;
@@ -157,6 +168,10 @@ struct IluHost {
     int nlev_l = 0, nlev_u = 0;
     std::vector<int32_t> lcnt, ucnt, lell_c, uell_c;
     std::vector<char> lell_a, uell_a, udiag;
+    bool wide = false;               // the streamed form: lell/uell hold its entries
+    int maxw = 0;                    // its widest slice
+    std::vector<IluLevel> llev, ulev;
+    std::vector<int32_t> lmeta, umeta;   // (row, entry count) pairs; row -1: filling
 };
 // MLB_OK, or MLB_ERR_ARG when a row has no stored diagonal or a pivot is
 // zero or not finite.

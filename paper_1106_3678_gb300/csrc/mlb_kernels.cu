@@ -1,6 +1,5 @@
 // Kernels of the ML(n)BiCGStab library (sm_103a).
 #include <algorithm>
-#include <new>
 
 #include "mlb_internal.h"
 #include "mlb_refine.cuh"
@@ -248,8 +247,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // beside the tile loads (each extra pass re-reads only y)
     constexpr int G = DS == 1 ? 8 : 4;
     using ACC = typename real_of<T>::type;
-    extern __shared__ unsigned char dsm[];
-    __shared__ TileRing ring;
+    TileRing &ring = *the_ring();
     // Programmatic dependent launch: the next product on the stream may be
     // scheduled as soon as every CTA of this one runs.  Its producer warp
     // streams only constant data (A and Q) into its own shared memory, so
@@ -259,14 +257,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     // consumers' through the CTA barriers).  The next product's set-up and
     // first tiles so overlap this one's tail.
     asm volatile("griddepcontrol.launch_dependents;");
-    ring_init(&ring, ring_buffer(dsm));
+    ring_init(&ring, 2000000000ull);
     int64_t s_lo, s_hi;
     own_range(sys.nslices, gridDim.x, blockIdx.x, s_lo, s_hi);
     soff_load(&ring, sys.slice_ptr, s_lo, s_hi);   // constant data
     if ((threadIdx.x >> 5) != kConsumerWarps) asm volatile("griddepcontrol.wait;" ::: "memory");
-    const uint64_t to = 2000000000ull;
     const int n = sys.n;
-    double *const scratch = reinterpret_cast<double *>(ring.buf);   // the stages, free between passes
+    double *const scratch = reinterpret_cast<double *>(the_stages());   // the stages, free between passes
     double *const part = partials + (size_t)blockIdx.x * kQdMaxN * DS;
     unsigned sq = 0;   // this thread's tile counter (issued or consumed)
     bool ok, bad;
@@ -279,8 +276,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int m = 0; m < NE; ++m) epi[m] = sys.Q + (int64_t)m * sys.ld;
         const int64_t nrows = sys.N;
         const bool keep = n > NE;   // later passes read y back
-        ok = sell_spmv<NE, 1, PW>(&ring, sq, sq, to, s_lo, s_hi, spt, sys.slice_ptr, sys.scol, sys.sval, x, epi,
-                           threadIdx.x & 31,
+        ok = sell_spmv<NE, 1, PW>(&ring, sq, sq, (int)s_lo, (int)s_hi, spt, sys.slice_ptr, sys.scol, sys.sval, x, epi,
                            [=](int64_t row, T v, const T (&e)[NE], ACC (&a)[NE * DS]) {
                                if (keep) y[row] = v;                // padded copy
                                if (row < nrows) yout[row] = v;      // the caller's y
@@ -306,9 +302,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int k = 0; k < G * DS; ++k) acc[k] = ACC(0);
         const int tc = P.tc;
         if ((threadIdx.x >> 5) == kConsumerWarps) {
-            if ((threadIdx.x & 31) == 0) ok = produce(&ring, P, sq, to);
+            if ((threadIdx.x & 31) == 0) ok = produce(&ring, P, sq);
         } else {
-            ok = consume(&ring, TileGeom{tc, c_lo, c_hi}, sq, to, [&](int64_t, const unsigned char *st, int k) {
+            ok = consume(&ring, TileGeom{tc, c_lo, c_hi}, sq, [&](int64_t, const unsigned char *st, int k) {
                 const Pack<T> yy = lds<T>(st, tc, 0, k);
 #pragma unroll
                 for (int m = 0; m < G; ++m) {
@@ -324,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!bad) cta_sums(acc, ng * DS, scratch, part + (size_t)g0 * DS);
     }
     if (threadIdx.x == 0) status[blockIdx.x] = bad ? 1 : 0;
-    ring_drain(&ring, sq, sq, to);
+    ring_drain(&ring, sq, sq);
     // The last CTA to finish sums every CTA's partials (fixed order, the
     // same whichever CTA it is) and ORs the status slots into d[n * DS];
     // it resets the ticket for the next launch.  No CTA waits for another.

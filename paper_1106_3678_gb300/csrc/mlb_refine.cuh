@@ -53,43 +53,52 @@ struct RefView {
     T64 *xbest;        // the solution with the smallest true residual so far
 };
 
+template <typename T64>
+__device__ __forceinline__ RefView<T64> &the_ref() {
+    __shared__ RefView<T64> v;
+    return v;
+}
+
 struct RefCtl {
     double delta;         // reliable-update factor (inner_tol of the options)
     int64_t inner_maxit;  // iteration cap of one inner call
     int64_t window;       // stagnation window of one inner call
 };
 
+__device__ __forceinline__ RefCtl &the_refctl() {
+    __shared__ RefCtl c;
+    return c;
+}
+
 template <typename T64, typename T32, int EW = 1>
 struct Refiner {
     using ACC = double;
     static constexpr int DS = dslots<T64>();
-    const RefView<T64> &v;
-    GridSync &gs;
-    Acct *acct;
-    int64_t s_lo, s_hi;   // owned slices (the same rows as the inner engine)
-
-    // Constructed by one thread in shared memory, like the engine.
-    __device__ Refiner(const RefView<T64> &v_, GridSync &g, Acct *a) : v(v_), gs(g), acct(a) {
-        own_range(v_.nslices, g.nblocks, g.bid, s_lo, s_hi);
-    }
+    // shared objects (see Engine)
+    __device__ __forceinline__ static const RefView<T64> &v() { return the_ref<T64>(); }
+    __device__ __forceinline__ static GridSync &gs() { return the_gs(); }
+    __device__ __forceinline__ static Acct &acct() { return the_acct(); }
+    using SI = typename coef_of<T64>::type;
+    __device__ __forceinline__ static int s_lo() { return the_iter<SI>().s_lo; }   // the engine's rows
+    __device__ __forceinline__ static int s_hi() { return the_iter<SI>().s_hi; }
 
     // Producer warp: the tiles of residual().
     __device__ __forceinline__ int issue(unsigned &sq) {
-        if (v.spt[1] <= 0) return 0;
-        const SliceOffsets off(gs.ring, v.slice_ptr, s_lo, s_hi);
-        return produce_sell_lanes(gs.ring, s_lo, s_hi, v.spt[1], off, v.sval, EW * (int)sizeof(T64), (int)sizeof(T64),
-                                  v.scol, v.b, 1, sq, gs.timeout_ns);
+        if (v().spt[1] <= 0) return 0;
+        const SliceOffsets off(the_ring(), v().slice_ptr, s_lo(), s_hi());
+        return produce_sell_lanes(the_ring(), s_lo(), s_hi(), v().spt[1], off, v().sval, EW * (int)sizeof(T64), (int)sizeof(T64),
+                                  v().scol, v().b, 1, sq);
     }
 
     // r = b - A x in FP64; sums ||b||^2, ||r||^2.
     __device__ __noinline__ bool residual(double &bb, double &rr) {
-        gs.post(kCmdResidual64);
+        gs().post(kCmdResidual64);
         double acc[2] = {0.0, 0.0};
-        const T64 *epi[1] = {v.b};
-        T64 *const r = v.r;
-        unsigned sq = gs.seq();
-        const bool okt = sell_consume<1, EW>(gs.ring, sq, gs.timeout_ns, s_lo, s_hi, v.spt[1], v.slice_ptr, v.scol,
-                                             v.sval, v.x, epi, threadIdx.x & 31,
+        const T64 *epi[1] = {v().b};
+        T64 *const r = v().r;
+        unsigned sq = gs().seq();
+        const bool okt = sell_consume<1, EW>(the_ring(), sq, s_lo(), s_hi(), v().spt[1], v().slice_ptr, v().scol,
+                                             v().sval, v().x, epi, 
                                              [=](int64_t row, T64 y, const T64 (&e)[1], double(&a)[2]) {
                                                  T64 rv = subT(e[0], y);
                                                  r[row] = rv;
@@ -97,18 +106,18 @@ struct Refiner {
                                                  acc_nrm(&a[1], rv);
                                              },
                                              acc);
-        gs.seq() = sq;
-        if (!okt) gs.ring->failed = 1;
-        pass_done(gs.ring);
-        if (!gs.template reduce<2>(acc, true)) return false;
-        if (gs.ring->failed) { gs.ok = false; return false; }
-        bb = gs.red->total[0];
-        rr = gs.red->total[1];
+        gs().seq() = sq;
+        if (!okt) the_ring()->failed = 1;
+        pass_done(the_ring());
+        if (!gs().template reduce<2>(acc, true)) return false;
+        if (the_ring()->failed) { gs().ok = false; return false; }
+        bb = the_red().total[0];
+        rr = the_red().total[1];
         if (threadIdx.x == kAcctThread) {
-            acct->bytes += v.nnz * (int64_t)sizeof(T64) + v.nnz / EW * 4 + 4 * (v.N + 1) +
-                           3 * v.N * (int64_t)sizeof(T64);
-            acct->flops += (DS == 2 ? 8 : 2) * v.nnz + (DS == 2 ? 10 : 5) * v.N;
-            acct->spmv++;
+            acct().bytes += v().nnz * (int64_t)sizeof(T64) + v().nnz / EW * 4 + 4 * (v().N + 1) +
+                           3 * v().N * (int64_t)sizeof(T64);
+            acct().flops += (DS == 2 ? 8 : 2) * v().nnz + (DS == 2 ? 10 : 5) * v().N;
+            acct().spmv++;
         }
         return true;
     }
@@ -121,9 +130,9 @@ struct Refiner {
         constexpr int PW = Pack<T32>::W;
         static_assert(PW * sizeof(T64) == 32, "an FP32 chunk maps to two FP64 chunks");
         constexpr int CPS = 32 * sizeof(T32) / 16;   // FP32 chunks per slice
-        const int64_t c_hi = s_hi * CPS;
-        const int64_t c_start = s_lo * CPS + threadIdx.x;
-        T64 *const x64 = v.x;
+        const int64_t c_hi = s_hi() * CPS;
+        const int64_t c_start = s_lo() * CPS + threadIdx.x;
+        T64 *const x64 = v().x;
         for (int64_t ch = c_start; ch < c_hi; ch += kConsumers) {
             Pack<T32> d;
             *reinterpret_cast<uint4 *>(&d) = __ldcg(reinterpret_cast<const uint4 *>(d32) + ch);
@@ -140,20 +149,20 @@ struct Refiner {
         }
         fence_proxy_async_global();
         if (threadIdx.x == kAcctThread)
-            acct->bytes += v.N * (int64_t)(2 * sizeof(T64) + (zero ? 2 : 1) * sizeof(T32));
-        return gs.sync();
+            acct().bytes += v().N * (int64_t)(2 * sizeof(T64) + (zero ? 2 : 1) * sizeof(T32));
+        return gs().sync();
     }
 
     // xbest = x (save) or x = xbest (restore) on the rows of this CTA.
     __device__ __noinline__ bool keep(bool save) {
         constexpr int CPS64 = 32 * sizeof(T64) / 16;   // FP64 chunks per slice
-        const int64_t c_hi = s_hi * CPS64;
-        const int64_t c_start = s_lo * CPS64 + threadIdx.x;
-        uint4 *dst = reinterpret_cast<uint4 *>(save ? v.xbest : v.x);
-        const uint4 *src = reinterpret_cast<const uint4 *>(save ? v.x : v.xbest);
+        const int64_t c_hi = s_hi() * CPS64;
+        const int64_t c_start = s_lo() * CPS64 + threadIdx.x;
+        uint4 *dst = reinterpret_cast<uint4 *>(save ? v().xbest : v().x);
+        const uint4 *src = reinterpret_cast<const uint4 *>(save ? v().x : v().xbest);
         for (int64_t ch = c_start; ch < c_hi; ch += kConsumers) dst[ch] = src[ch];
-        if (threadIdx.x == kAcctThread) acct->bytes += 2 * v.N * (int64_t)sizeof(T64);
-        return gs.sync();
+        if (threadIdx.x == kAcctThread) acct().bytes += 2 * v().N * (int64_t)sizeof(T64);
+        return gs().sync();
     }
 
     __device__ __forceinline__ static double widen_fma(double s, float d, double x) { return fma(s, (double)d, x); }
@@ -176,8 +185,6 @@ template <typename T32, typename T64, bool PC, int EW = 1>
 struct RelUpdate {
     static constexpr bool kActive = true;
     using S = typename coef_of<T32>::type;
-    Engine<T32, PC, EW> *E;
-    Refiner<T64, T32, EW> *R;
     double sigma;      // ||r|| at the start of the call: the inner system is A d = r / sigma
     double bn;         // ||b||
     double tol;        // target of the true relative residual
@@ -207,24 +214,26 @@ struct RelUpdate {
     // The inner iterate into x, the true residual, r replaced (see
     // Engine::inner for the arguments).
     __device__ __noinline__ bool replace(int qcol, bool f0, double &rr, S &qr, S &fr, bool &conv) {
-        const T32 *d = E->sys.x;
+        Engine<T32, PC, EW> E;
+        Refiner<T64, T32, EW> R;
+        const T32 *d = the_sys<T32>().x;
         if constexpr (PC) {
-            if (E->sys.ilu.lu) {
+            if (the_sys<T32>().ilu.lu) {
                 // the iterate's rows of every CTA are read
-                if (!E->gs.sync() || !E->ilu_solve(E->sys.x, E->sys.ilu.t)) return false;
-                d = E->sys.ilu.t;
+                if (!the_gs().sync() || !E.ilu_solve(the_sys<T32>().x, the_sys<T32>().ilu.t)) return false;
+                d = the_sys<T32>().ilu.t;
             }
         }
-        if (!R->update(sigma, d, E->sys.x)) return false;
+        if (!R.update(sigma, d, the_sys<T32>().x)) return false;
         double bb, r64;
-        if (!R->residual(bb, r64)) return false;
+        if (!R.residual(bb, r64)) return false;
         const double te = sqrt(r64) / bn;
         conv = te < tol;
         if (threadIdx.x == 0) {
             true_err = te;
             updates++;
         }
-        return E->ph_replace_narrow(R->v.r, 1.0 / sigma, qcol, f0, rr, qr, fr);
+        return E.ph_replace_narrow(the_ref<T64>().r, 1.0 / sigma, qcol, f0, rr, qr, fr);
     }
 };
 
@@ -233,13 +242,14 @@ struct RelUpdate {
 // one.
 template <typename T32, typename T64, bool PC, int EW = 1>
 __device__ RefineOut refine_solve(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> &R, const SolveCtl &ctl,
-                                  const RefCtl &rc, RelUpdate<T32, T64, PC, EW> &hk) {
+                                  const RefCtl &rc) {
+    __shared__ RelUpdate<T32, T64, PC, EW> hk;
     RefineOut out{1, 0, 0, __longlong_as_double(0x7ff8000000000000LL)};
     double prev = 0.0;   // true residual at the start of the last inner call
     double best = 0.0;   // true residual of the saved solution xbest
     int no_gain = 0;
     auto record = [&](double err) {
-        if (ctl.err_hist && out.outer < ctl.hist_cap && E.gs.bid == 0 && threadIdx.x == 0)
+        if (ctl.err_hist && out.outer < ctl.hist_cap && the_gs().bid == 0 && threadIdx.x == 0)
             ctl.err_hist[out.outer] = err;
     };
     for (;;) {
@@ -281,10 +291,10 @@ __device__ RefineOut refine_solve(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> 
         const double rn = sqrt(rr);
         consumer_sync();   // no thread still reads the last call's state
         if (threadIdx.x == 0)
-            hk = RelUpdate<T32, T64, PC, EW>{&E, &R, rn, bn, ctl.tol, rc.delta, rc.window, 0.0, INFINITY, 0, err, 0};
+            hk = RelUpdate<T32, T64, PC, EW>{rn, bn, ctl.tol, rc.delta, rc.window, 0.0, INFINITY, 0, err, 0};
         consumer_sync();
-        auto o = E.inner(budget, false, ctl.tol * bn / rn, R.v.r, 1.0 / rn, &hk);
-        if (!E.gs.ok) return out;
+        auto o = E.inner(false, budget, false, ctl.tol * bn / rn, the_ref<T64>().r, 1.0 / rn, &hk);
+        if (!the_gs().ok) return out;
         out.iter += o.iter;
         out.outer++;
         if (o.flag == 0) {
@@ -296,11 +306,11 @@ __device__ RefineOut refine_solve(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> 
         }
         if (o.flag == -1 && o.iter == 0) { out.flag = -1; return out; }
         // move what the inner call accumulated since its last update
-        const T32 *d = E.sys.x;
+        const T32 *d = the_sys<T32>().x;
         if constexpr (PC) {
-            if (E.sys.ilu.lu) {
-                if (!E.gs.sync() || !E.ilu_solve(E.sys.x, E.sys.ilu.t)) return out;
-                d = E.sys.ilu.t;
+            if (the_sys<T32>().ilu.lu) {
+                if (!the_gs().sync() || !E.ilu_solve(the_sys<T32>().x, the_sys<T32>().ilu.t)) return out;
+                d = the_sys<T32>().ilu.t;
             }
         }
         if (!R.update(rn, d, nullptr)) return out;

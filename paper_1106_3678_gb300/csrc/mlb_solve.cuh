@@ -6,8 +6,6 @@
 // (PC = true), which compile in parallel.
 #pragma once
 
-#include <new>
-
 #include "mlb_internal.h"
 #include "mlb_refine.cuh"
 
@@ -22,35 +20,38 @@ namespace mlb {
 // against one maxit; then the true residual; the team's rank-0 CTA writes
 // the result record.  Consumer threads only.
 template <typename T, bool PC, int EW>
-__device__ void run_fp64_solve(Engine<T, PC, EW> &E, GridSync &gs, const SolveCtl &ctl, Acct &acct, DevResult *res) {
+__device__ __forceinline__ void run_fp64_solve() {
+    Engine<T, PC, EW> E;
+    GridSync &gs = the_gs();
+    const SolveCtl &ctl = the_ctl();
+    const Acct &acct = the_acct();
+    DevResult *const res = ctl.res;
     int64_t total = 0;
     int outer = 0;
     typename Engine<T, PC, EW>::Out o{1, 0, 0, 0, 0.0};
     // ILU(0): the method iterates on y = M x (y_0 = M x_0; x = M^{-1} y at
     // the end, from the final residual pass, which forms M^{-1} y)
     if constexpr (PC) {
-        if (E.sys.ilu.lu) E.ilu_to_y();
-    }
-    for (;;) {
-        if (!gs.ok) break;
-        o = E.inner(ctl.maxit - total, outer == 0, ctl.tol);
-        if (!gs.ok) break;
-        total += o.iter;
-        gs.sync();   // the residual pass that follows gathers x
-        if (o.flag != 0 || o.iter == 0 || total >= ctl.maxit || outer >= ctl.max_outer) break;
-        outer++;
+        if (E.sys().ilu.lu) E.ilu_to_y();
     }
     double true_rel = __longlong_as_double(0x7ff8000000000000LL);
-    if (gs.ok && E.ilu_pre(E.sys.x)) {
-        gs.post(kCmdResidual);
-        if (E.ph_residual(false)) {
-            double bn = sqrt(gs.red->total[0]);
+    for (bool last = false; gs.ok;) {
+        const auto r = E.inner(last, ctl.maxit - total, outer == 0, ctl.tol);
+        if (!gs.ok) break;
+        if (last) {
+            double bn = sqrt(the_red().total[0]);
             if (bn == 0.0) bn = 1.0;
-            true_rel = sqrt(gs.red->total[1]) / bn;
+            true_rel = sqrt(the_red().total[1]) / bn;
             if constexpr (PC) {
-                if (E.sys.ilu.lu) E.ilu_to_x();
+                if (E.sys().ilu.lu) E.ilu_to_x();
             }
+            break;
         }
+        o = r;
+        total += o.iter;
+        gs.sync();   // the residual pass that follows gathers x
+        last = o.flag != 0 || o.iter == 0 || total >= ctl.maxit || outer >= ctl.max_outer;
+        if (!last) outer++;
     }
     consumer_sync();   // the accounting is complete
     if (gs.bid == 0 && threadIdx.x == 0) {
@@ -71,20 +72,13 @@ __device__ void run_fp64_solve(Engine<T, PC, EW> &E, GridSync &gs, const SolveCt
     }
 }
 
-// Raw shared storage for an object constructed in place by thread 0
-// (per-CTA state shared by all threads of the CTA).
-template <typename X>
-struct alignas(16) SharedSlot {
-    unsigned char raw[sizeof(X)];
-    __device__ X *get() { return reinterpret_cast<X *>(raw); }
-};
-
 // Allow the ring's dynamic shared memory for a kernel (idempotent).
 static cudaError_t allow_ring(const void *fn) {
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingBytes);
 }
 
-__device__ __forceinline__ void acct_reset(Acct &acct) {
+__device__ __forceinline__ void acct_reset() {
+    Acct &acct = the_acct();
     if (threadIdx.x == 0) {
         for (int q = 0; q < 5; ++q) acct.ops[q] = 0;
         acct.spmv = 0;
@@ -96,45 +90,30 @@ __device__ __forceinline__ void acct_reset(Acct &acct) {
 
 // One FP64 solve by a CTA: its producer warp and its consumer warps.
 template <typename T, bool PC, int EW>
-__device__ __forceinline__ void run_cta(Engine<T, PC, EW> &E, GridSync &gs, const SolveCtl &ctl, Acct &acct) {
+__device__ __forceinline__ void run_cta() {
+    Engine<T, PC, EW> E;
+    E.attach();
     if ((threadIdx.x >> 5) == kConsumerWarps) {
         E.template serve<false>([](unsigned &) { return 0; });
     } else {
-        run_fp64_solve(E, gs, ctl, acct, ctl.res);
-        gs.post(kCmdExit);
+        run_fp64_solve<T, PC, EW>();
+        the_gs().post(kCmdExit);
     }
     __syncthreads();
 }
 
 template <typename T, bool PC, int EW = 1>
 __global__ void __launch_bounds__(kThreads, 1) solve_kernel(SysView<T> sys, SolveCtl ctl) {
-    using S = typename coef_of<T>::type;
-    extern __shared__ unsigned char dsm[];
-    __shared__ RedScratch red;
-    __shared__ S cbuf[kMaxN];
-    __shared__ S btbuf[kMaxN];
-    __shared__ Acct acct;
-    __shared__ Scalars<S> scal;
-    __shared__ TileRing ring;
-    __shared__ SysView<T> s_sys;
-    __shared__ SolveCtl s_ctl;
-    __shared__ SharedSlot<GridSync> gs_slot;
-    __shared__ SharedSlot<Engine<T, PC, EW>> e_slot;
-    __shared__ unsigned seqs[kThreads];
-    ring_init(&ring, ring_buffer(dsm));
-    seqs[threadIdx.x] = 0;
+    ring_init(the_ring(), ctl.timeout_ns);
+    the_gs().seq() = 0;
     if (threadIdx.x == 0) {
-        s_sys = sys;
-        s_ctl = ctl;
-        new (gs_slot.get()) GridSync(ctl.bar, ctl.slots, gridDim.x, blockIdx.x, &red, ctl.timeout_ns, &ring, seqs);
-        new (e_slot.get()) Engine<T, PC, EW>(s_sys, s_ctl, *gs_slot.get(), cbuf, btbuf, &acct, &scal);
+        the_sys<T>() = sys;
+        the_ctl() = ctl;
+        the_gs().init(ctl.bar, ctl.slots, gridDim.x, blockIdx.x, ctl.timeout_ns);
     }
-    acct_reset(acct);   // includes the __syncthreads that publishes the objects
-    GridSync &gs = *gs_slot.get();
-    Engine<T, PC, EW> &E = *e_slot.get();
-    E.attach();
-    run_cta(E, gs, s_ctl, acct);
-    ring_drain(&ring, seqs[kConsumers], seqs[0], s_ctl.timeout_ns);
+    acct_reset();   // includes the __syncthreads that publishes the objects
+    run_cta<T, PC, EW>();
+    ring_drain(the_ring(), the_gs().seqs[kConsumers], the_gs().seqs[0]);
 }
 
 // ===========================================================================
@@ -185,38 +164,20 @@ __device__ __forceinline__ void run_batch_plan(const BatchPlan &p, int *sflag, i
 // with CTA-wide barriers and reductions in shared memory.
 template <typename T, bool PC>
 __global__ void __launch_bounds__(kThreads, 1) batch_kernel(const BatchItem<T> *items, BatchPlan plan) {
-    using S = typename coef_of<T>::type;
-    extern __shared__ unsigned char dsm[];
-    __shared__ TileRing ring;
-    __shared__ RedScratch red;
-    __shared__ S cbuf[kMaxN];
-    __shared__ S btbuf[kMaxN];
-    __shared__ Acct acct;
-    __shared__ Scalars<S> scal;
     __shared__ int sflag;
     __shared__ int s_next;
-    __shared__ BatchItem<T> item;
-    __shared__ SharedSlot<GridSync> gs_slot;
-    __shared__ SharedSlot<Engine<T, PC>> e_slot;
-    __shared__ unsigned seqs[kThreads];   // tile counters, kept across systems
-    ring_init(&ring, ring_buffer(dsm));
-    seqs[threadIdx.x] = 0;
-    uint64_t timeout = plan.timeout_ns;
+    ring_init(the_ring(), plan.timeout_ns);
+    the_gs().seq() = 0;
     run_batch_plan(plan, &sflag, &s_next, [&](int idx, unsigned nb, unsigned rk, BarrierState *bar, Slot *slots) {
-        if (threadIdx.x == 0) item = items[idx];
-        acct_reset(acct);   // includes the __syncthreads that publishes `item`
-        timeout = item.ctl.timeout_ns;
         if (threadIdx.x == 0) {
-            GridSync *g = new (gs_slot.get()) GridSync(bar, slots, nb, rk, &red, timeout, &ring, seqs);
-            new (e_slot.get()) Engine<T, PC>(item.sys, item.ctl, *g, cbuf, btbuf, &acct, &scal);
+            the_sys<T>() = items[idx].sys;
+            the_ctl() = items[idx].ctl;
+            the_gs().init(bar, slots, nb, rk, the_ctl().timeout_ns);
         }
-        __syncthreads();
-        GridSync &gs = *gs_slot.get();
-        Engine<T, PC> &E = *e_slot.get();
-        E.attach();
-        run_cta(E, gs, item.ctl, acct);
+        acct_reset();   // includes the __syncthreads that publishes the objects
+        run_cta<T, PC, 1>();
     });
-    ring_drain(&ring, seqs[kConsumers], seqs[0], timeout);
+    ring_drain(the_ring(), the_gs().seqs[kConsumers], the_gs().seqs[0]);
 }
 
 template <typename T, bool PC>
@@ -268,79 +229,62 @@ int solve_blocks_per_sm_pc() {
 // ===========================================================================
 // FP32-inner / FP64-refined persistent solve and batch kernels
 // ===========================================================================
-// One refined solve by a CTA: its producer warp and its consumer warps.
+// One refined solve by a CTA: its producer warp and its consumer warps; the
+// team's rank-0 CTA writes the result record.
 template <typename T32, typename T64, bool PC, int EW>
-__device__ __forceinline__ RefineOut refine_cta(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> &R,
-                                                const SolveCtl &ctl, const RefCtl &rc,
-                                                RelUpdate<T32, T64, PC, EW> &hk) {
+__device__ __forceinline__ void refine_cta() {
+    Engine<T32, PC, EW> E;
+    Refiner<T64, T32, EW> R;
+    E.attach();
     RefineOut o{1, 0, 0, 0.0};
     if ((threadIdx.x >> 5) == kConsumerWarps) {
         E.template serve<true>([&](unsigned &sq) { return R.issue(sq); });
     } else {
-        o = refine_solve<T32, T64, PC, EW>(E, R, ctl, rc, hk);
-        E.gs.post(kCmdExit);
+        o = refine_solve<T32, T64, PC, EW>(E, R, the_ctl(), the_refctl());
+        the_gs().post(kCmdExit);
     }
     __syncthreads();
-    return o;
+    GridSync &gs = the_gs();
+    if (gs.bid == 0 && threadIdx.x == 0) {
+        const Acct &acct = the_acct();
+        DevResult *res = the_ctl().res;
+        res->flag = o.flag;
+        res->j = 0;
+        res->i = 0;
+        res->status = gs.ok ? 0 : (gs.bar ? ld_relaxed_i32(&gs.bar->status) : kStatusTimeout);
+        if (!gs.ok && res->status == 0) res->status = kStatusTimeout;
+        res->iter = o.iter;
+        res->spmv = acct.spmv;
+        res->outer = o.outer;
+        res->err = o.err;
+        res->true_relres = o.err;
+        res->bytes = (double)acct.bytes;
+        res->flops = (double)acct.flops;
+        for (int k = 0; k < 5; ++k) res->ops[k] = acct.ops[k];
+        res->ctas = (int32_t)gs.nblocks;
+    }
+    __syncthreads();
 }
 
 template <typename T32, typename T64, bool PC>
 __global__ void __launch_bounds__(kThreads, 1)
     batch_refine_kernel(const BatchItemR<T32, T64> *items, BatchPlan plan) {
-    using S = typename coef_of<T32>::type;
-    extern __shared__ unsigned char dsm[];
-    __shared__ TileRing ring;
-    __shared__ RedScratch red;
-    __shared__ S cbuf[kMaxN];
-    __shared__ S btbuf[kMaxN];
-    __shared__ Acct acct;
-    __shared__ Scalars<S> scal;
     __shared__ int sflag;
     __shared__ int s_next;
-    __shared__ BatchItemR<T32, T64> item;
-    __shared__ SharedSlot<GridSync> gs_slot;
-    __shared__ SharedSlot<Engine<T32, PC>> e_slot;
-    __shared__ SharedSlot<Refiner<T64, T32>> r_slot;
-    __shared__ SharedSlot<RelUpdate<T32, T64, PC>> h_slot;
-    __shared__ unsigned seqs[kThreads];   // tile counters, kept across systems
-    ring_init(&ring, ring_buffer(dsm));
-    seqs[threadIdx.x] = 0;
-    uint64_t timeout = plan.timeout_ns;
+    ring_init(the_ring(), plan.timeout_ns);
+    the_gs().seq() = 0;
     run_batch_plan(plan, &sflag, &s_next, [&](int idx, unsigned nb, unsigned rk, BarrierState *bar, Slot *slots) {
-        if (threadIdx.x == 0) item = items[idx];
-        acct_reset(acct);
-        timeout = item.ctl.timeout_ns;
         if (threadIdx.x == 0) {
-            GridSync *g = new (gs_slot.get()) GridSync(bar, slots, nb, rk, &red, timeout, &ring, seqs);
-            new (e_slot.get()) Engine<T32, PC>(item.sys, item.ctl, *g, cbuf, btbuf, &acct, &scal);
-            new (r_slot.get()) Refiner<T64, T32>(item.rv, *g, &acct);
+            the_sys<T32>() = items[idx].sys;
+            the_ref<T64>() = items[idx].rv;
+            the_ctl() = items[idx].ctl;
+            the_refctl() = items[idx].rc;
+            the_gs().init(bar, slots, nb, rk, the_ctl().timeout_ns);
         }
-        __syncthreads();
-        GridSync &gs = *gs_slot.get();
-        Engine<T32, PC> &E = *e_slot.get();
-        Refiner<T64, T32> &R = *r_slot.get();
-        E.attach();
-        const RefineOut o = refine_cta<T32, T64, PC, 1>(E, R, item.ctl, item.rc, *h_slot.get());
-        if (gs.bid == 0 && threadIdx.x == 0) {
-            DevResult *res = item.ctl.res;
-            res->flag = o.flag;
-            res->j = 0;
-            res->i = 0;
-            res->status = gs.ok ? 0 : (gs.bar ? ld_relaxed_i32(&gs.bar->status) : kStatusTimeout);
-            if (!gs.ok && res->status == 0) res->status = kStatusTimeout;
-            res->iter = o.iter;
-            res->spmv = acct.spmv;
-            res->outer = o.outer;
-            res->err = o.err;
-            res->true_relres = o.err;
-            res->bytes = (double)acct.bytes;
-            res->flops = (double)acct.flops;
-            for (int k = 0; k < 5; ++k) res->ops[k] = acct.ops[k];
-            res->ctas = (int32_t)nb;
-        }
-        __syncthreads();
+        acct_reset();   // includes the __syncthreads that publishes the objects
+        refine_cta<T32, T64, PC, 1>();
     });
-    ring_drain(&ring, seqs[kConsumers], seqs[0], timeout);
+    ring_drain(the_ring(), the_gs().seqs[kConsumers], the_gs().seqs[0]);
 }
 
 template <typename T32, typename T64, bool PC>
@@ -374,58 +318,18 @@ int batch_refine_blocks_per_sm_pc() {
 template <typename T32, typename T64, bool PC, int EW = 1>
 __global__ void __launch_bounds__(kThreads, 1)
     refine_kernel(SysView<T32> sys, RefView<T64> rv, SolveCtl ctl, RefCtl rc) {
-    using S = typename coef_of<T32>::type;
-    extern __shared__ unsigned char dsm[];
-    __shared__ TileRing ring;
-    __shared__ RedScratch red;
-    __shared__ S cbuf[kMaxN];
-    __shared__ S btbuf[kMaxN];
-    __shared__ Acct acct;
-    __shared__ Scalars<S> scal;
-    __shared__ SysView<T32> s_sys;
-    __shared__ RefView<T64> s_rv;
-    __shared__ SolveCtl s_ctl;
-    __shared__ RefCtl s_rc;
-    __shared__ SharedSlot<GridSync> gs_slot;
-    __shared__ SharedSlot<Engine<T32, PC, EW>> e_slot;
-    __shared__ SharedSlot<Refiner<T64, T32, EW>> r_slot;
-    __shared__ SharedSlot<RelUpdate<T32, T64, PC, EW>> h_slot;
-    __shared__ unsigned seqs[kThreads];
-    ring_init(&ring, ring_buffer(dsm));
-    seqs[threadIdx.x] = 0;
+    ring_init(the_ring(), ctl.timeout_ns);
+    the_gs().seq() = 0;
     if (threadIdx.x == 0) {
-        s_sys = sys;
-        s_rv = rv;
-        s_ctl = ctl;
-        s_rc = rc;
-        GridSync *g = new (gs_slot.get()) GridSync(ctl.bar, ctl.slots, gridDim.x, blockIdx.x, &red, ctl.timeout_ns, &ring, seqs);
-        new (e_slot.get()) Engine<T32, PC, EW>(s_sys, s_ctl, *g, cbuf, btbuf, &acct, &scal);
-        new (r_slot.get()) Refiner<T64, T32, EW>(s_rv, *g, &acct);
+        the_sys<T32>() = sys;
+        the_ref<T64>() = rv;
+        the_ctl() = ctl;
+        the_refctl() = rc;
+        the_gs().init(ctl.bar, ctl.slots, gridDim.x, blockIdx.x, ctl.timeout_ns);
     }
-    acct_reset(acct);   // includes the __syncthreads that publishes the objects
-    GridSync &gs = *gs_slot.get();
-    Engine<T32, PC, EW> &E = *e_slot.get();
-    Refiner<T64, T32, EW> &R = *r_slot.get();
-    E.attach();
-    const RefineOut o = refine_cta<T32, T64, PC, EW>(E, R, s_ctl, s_rc, *h_slot.get());
-    ring_drain(&ring, seqs[kConsumers], seqs[0], ctl.timeout_ns);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        DevResult *res = ctl.res;
-        res->flag = o.flag;
-        res->j = 0;
-        res->i = 0;
-        res->status = gs.ok ? 0 : ld_relaxed_i32(&ctl.bar->status);
-        if (!gs.ok && res->status == 0) res->status = kStatusTimeout;
-        res->iter = o.iter;
-        res->spmv = acct.spmv;
-        res->outer = o.outer;
-        res->err = o.err;
-        res->true_relres = o.err;
-        res->bytes = (double)acct.bytes;
-        res->flops = (double)acct.flops;
-        for (int q = 0; q < 5; ++q) res->ops[q] = acct.ops[q];
-        res->ctas = (int32_t)gridDim.x;
-    }
+    acct_reset();   // includes the __syncthreads that publishes the objects
+    refine_cta<T32, T64, PC, EW>();
+    ring_drain(the_ring(), the_gs().seqs[kConsumers], the_gs().seqs[0]);
 }
 
 template <typename T32, typename T64, bool PC, int EW = 1>

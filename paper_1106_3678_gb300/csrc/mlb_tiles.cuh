@@ -73,15 +73,6 @@ __device__ __forceinline__ bool mbar_probe(uint64_t *b, unsigned phase) {
         : "memory");
     return ok != 0;
 }
-// Bounded wait for the phase with parity `phase` to complete.
-__device__ __forceinline__ bool mbar_wait(uint64_t *b, unsigned phase, uint64_t timeout_ns) {
-    if (mbar_test(b, phase)) return true;
-    const uint64_t t0 = globaltimer_ns();
-    for (unsigned it = 1;; ++it) {
-        if (mbar_test(b, phase)) return true;
-        if ((it & 15u) == 0 && globaltimer_ns() - t0 > timeout_ns) return false;
-    }
-}
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned bytes, uint64_t *bar) {
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -105,12 +96,23 @@ __device__ __forceinline__ uint64_t l2_evict_first_policy() {
 }
 __device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
+// The stages and, after them, the slice-offset cache: the kernels' dynamic
+// shared memory.
+__device__ __forceinline__ unsigned char *the_stages() {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    return dsm;
+}
+__device__ __forceinline__ int32_t *the_soff() {
+    return reinterpret_cast<int32_t *>(the_stages() + (size_t)kStages * kStageBytes);
+}
+
 // Commands of the consumers to the producer warp (TileRing::cmd), handed
 // over by a __syncthreads of the whole CTA.
 enum {
     kCmdExit,        // this system is done
-    kCmdResidual,    // one residual pass of the engine
+    kCmdResidual,    // one residual pass of the engine (with ILU(0), M^{-1} x first)
     kCmdResidual64,  // one residual pass of the refined mode's FP64 side
+    kCmdIlu,         // (refined mode) the tiles of one M^{-1}
     kCmdInner,       // the iteration from its first product on
     kCmdGo,          // (refined mode) go on with the iteration
 };
@@ -121,7 +123,7 @@ struct TileRing {
     uint64_t full[kStages];
     uint64_t empty[kStages];
     uint64_t done;           // completed passes (one arrival per consumer warp)
-    unsigned char *buf;      // kStages * kStageBytes, 128-byte aligned
+    uint64_t timeout_ns;     // limit of every wait
     unsigned issued;         // tiles issued (written by the producer where both sides meet)
     unsigned consumed;       // tiles and passes consumed (written by the consumers there)
     unsigned passes;
@@ -129,25 +131,31 @@ struct TileRing {
     int stop;                // the iteration ended: the producer returns from its waits
     int failed;              // set when a wait timed out
     // Cache of the SELL-32 slice offsets of this CTA's slice range:
-    // soff[i] = slice_ptr[soff_lo + i] - soff_base for i = 0..soff_hi-soff_lo
-    // (kept in the dynamic shared memory after the stages).
-    int32_t *soff;
+    // the_soff()[i] = slice_ptr[soff_lo + i] - soff_base for i = 0..soff_hi-soff_lo
     const int64_t *soff_src; // slice_ptr the cache was filled from (null: empty)
     int64_t soff_lo, soff_hi, soff_base;
 };
 
-__device__ __forceinline__ void ring_init(TileRing *R, unsigned char *buf) {
+// The CTA's ring.  Shared objects of the kernels are reached through
+// functions like this one: their address is then a constant to the compiler,
+// where a pointer kept in memory costs registers in every loop (the product
+// passes spilled 20 values per slice for such pointers).
+__device__ __forceinline__ TileRing *the_ring() {
+    __shared__ TileRing ring;
+    return &ring;
+}
+
+__device__ __forceinline__ void ring_init(TileRing *R, uint64_t timeout_ns) {
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&R->full[s], 1);
             mbar_init(&R->empty[s], kConsumerWarps);
         }
         mbar_init(&R->done, kConsumerWarps);
-        R->buf = buf;
+        R->timeout_ns = timeout_ns;
         R->failed = 0;
         R->stop = 0;
         R->passes = 0;
-        R->soff = reinterpret_cast<int32_t *>(buf + (size_t)kStages * kStageBytes);
         R->soff_src = nullptr;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -159,16 +167,26 @@ __device__ __forceinline__ void consumer_sync() {
     asm volatile("bar.sync 1, %0;" ::"n"(kConsumers) : "memory");
 }
 
+// Bounded wait for the phase with parity `phase` of a barrier of the ring
+// to complete.
+__device__ __forceinline__ bool mbar_wait(TileRing *R, uint64_t *b, unsigned phase) {
+    if (mbar_test(b, phase)) return true;
+    const uint64_t t0 = globaltimer_ns();
+    for (unsigned it = 1;; ++it) {
+        if (mbar_test(b, phase)) return true;
+        if ((it & 15u) == 0 && globaltimer_ns() - t0 > R->timeout_ns) return false;
+    }
+}
 // Bounded wait of the producer's lane 0: 0 when the phase completed, 1 when
 // the consumers ended the iteration, 2 on a timeout.  Twice the consumers'
 // limit, so that a wait of theirs that gives up is reported as such.
-__device__ __forceinline__ int producer_wait(TileRing *R, uint64_t *b, unsigned phase, uint64_t timeout_ns) {
+__device__ __forceinline__ int producer_wait(TileRing *R, uint64_t *b, unsigned phase) {
     if (mbar_probe(b, phase)) return 0;
     const uint64_t t0 = globaltimer_ns();
     for (unsigned it = 1;; ++it) {
         if (mbar_probe(b, phase)) return 0;
         if (*(volatile int *)&R->stop) return 1;
-        if ((it & 63u) == 0 && globaltimer_ns() - t0 > 2 * timeout_ns) return 2;
+        if ((it & 63u) == 0 && globaltimer_ns() - t0 > 2 * R->timeout_ns) return 2;
     }
 }
 
@@ -190,7 +208,7 @@ __device__ __forceinline__ void soff_load(TileRing *R, const int64_t *slice_ptr,
     const bool fits = n + 1 <= kSoffCap && __ldg(slice_ptr + s_hi) - base < ((int64_t)1 << 31);
     if (fits)
         for (int64_t i = threadIdx.x; i <= n; i += blockDim.x)
-            R->soff[i] = (int32_t)(__ldg(slice_ptr + s_lo + i) - base);
+            the_soff()[i] = (int32_t)(__ldg(slice_ptr + s_lo + i) - base);
     if (threadIdx.x == 0) {
         R->soff_src = fits ? slice_ptr : nullptr;
         R->soff_lo = s_lo;
@@ -209,7 +227,7 @@ struct SliceOffsets {
     __device__ __forceinline__ SliceOffsets(const TileRing *R, const int64_t *slice_ptr, int64_t s_lo, int64_t s_hi)
         : so(nullptr), sp(slice_ptr), lo(s_lo), base(0) {
         if (R->soff_src == slice_ptr && R->soff_lo == s_lo && R->soff_hi == s_hi) {
-            so = R->soff;
+            so = the_soff();
             base = R->soff_base;
         }
     }
@@ -218,10 +236,6 @@ struct SliceOffsets {
         return so ? base + so[s - lo] : __ldg(sp + s);
     }
 };
-
-__device__ __forceinline__ unsigned char *ring_buffer(unsigned char *dsm) {
-    return (unsigned char *)(((uintptr_t)dsm + 127) & ~(uintptr_t)127);
-}
 
 // The producer lane's copy descriptor of a streaming pass over the chunk
 // range [c_lo, c_hi) of this CTA: `ni` inputs of 16-byte chunks, tiles of
@@ -248,7 +262,7 @@ __device__ __forceinline__ int tile_chunks_for(int ni) {
 
 // Producer side (lane 0 of the producer warp): issue every tile of pass P.
 // `seq` is this CTA's running tile sequence number.
-__device__ __forceinline__ bool produce(TileRing *R, const TilePass &P, unsigned &seq, uint64_t timeout_ns) {
+__device__ __forceinline__ bool produce(TileRing *R, const TilePass &P, unsigned &seq) {
     // The descriptor lives in memory (its input list is indexed at run
     // time); copy it into registers once, so the issue loop does not wait
     // on a load before every copy.
@@ -257,12 +271,12 @@ __device__ __forceinline__ bool produce(TileRing *R, const TilePass &P, unsigned
     for (int i = 0; i < kMaxInputs; ++i) src[i] = i < P.ni ? (const unsigned char *)P.in[i] : nullptr;
     const int ni = P.ni, tc = P.tc;
     const int64_t c_lo = P.c_lo, c_hi = P.c_hi;
-    unsigned char *const buf = R->buf;
+    unsigned char *const buf = the_stages();
     const int nt = (int)((c_hi - c_lo + tc - 1) / tc);
     for (int t = 0; t < nt; ++t, ++seq) {
         const int s = (int)(seq % kStages);
         const unsigned use = seq / kStages;
-        if (use > 0 && !mbar_wait(&R->empty[s], (use - 1) & 1u, timeout_ns)) return false;
+        if (use > 0 && !mbar_wait(R, &R->empty[s], (use - 1) & 1u)) return false;
         const int64_t c0 = c_lo + (int64_t)t * tc;
         int64_t cn = c_hi - c0;
         if (cn > tc) cn = tc;
@@ -280,17 +294,17 @@ __device__ __forceinline__ bool produce(TileRing *R, const TilePass &P, unsigned
 // for each chunk k of the tile owned by this thread (chunk k is read from
 // stage + i*tc*16 + k*16 for input i), then release the stage.
 template <typename Fn>
-__device__ __forceinline__ bool consume(TileRing *R, const TileGeom g, unsigned &seq, uint64_t timeout_ns, Fn fn) {
+__device__ __forceinline__ bool consume(TileRing *R, const TileGeom g, unsigned &seq, Fn fn) {
     const int tc = g.tc;
     const int64_t c_lo = g.c_lo, c_hi = g.c_hi;
     const int nt = (int)((c_hi - c_lo + tc - 1) / tc);
-    unsigned char *const buf = R->buf;
+    unsigned char *const buf = the_stages();
     unsigned sq = seq;
     const int tid = threadIdx.x;   // < kConsumers
     for (int t = 0; t < nt; ++t, ++sq) {
         const int s = (int)(sq % kStages);
         const unsigned use = sq / kStages;
-        if (!mbar_wait(&R->full[s], use & 1u, timeout_ns)) {
+        if (!mbar_wait(R, &R->full[s], use & 1u)) {
             seq = sq;
             return false;
         }
@@ -318,20 +332,20 @@ __device__ __forceinline__ void pass_done(TileRing *R) {
 // the chunks [c_lo, c_hi), lane i < ni copying input i from `src` (its own
 // pointer).  Returns 0, 1 (stopped) or 2 (timeout), the same in every lane.
 __device__ __forceinline__ int produce_lanes(TileRing *R, const void *src, int ni, int64_t c_lo, int64_t c_hi,
-                                             unsigned &seq, uint64_t timeout_ns) {
+                                             unsigned &seq) {
     const int lane = threadIdx.x & 31, tc = tile_chunks_for(ni);
     for (int64_t c0 = c_lo; c0 < c_hi; c0 += tc, ++seq) {
         const int s = (int)(seq % kStages);
         const unsigned use = seq / kStages;
         int st = 0;
-        if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u, timeout_ns);
+        if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u);
         st = __shfl_sync(0xffffffffu, st, 0);
         if (st) return st;
         const unsigned bytes = (unsigned)(c_hi - c0 < tc ? c_hi - c0 : tc) * 16u;
         if (lane == 0) mbar_arrive_expect_tx(&R->full[s], bytes * (unsigned)ni);
         __syncwarp();
         if (lane < ni)
-            bulk_g2s(R->buf + (size_t)s * kStageBytes + (size_t)lane * tc * 16, (const unsigned char *)src + c0 * 16,
+            bulk_g2s(the_stages() + (size_t)s * kStageBytes + (size_t)lane * tc * 16, (const unsigned char *)src + c0 * 16,
                      bytes, &R->full[s]);
     }
     return 0;
@@ -342,15 +356,14 @@ __device__ __forceinline__ int produce_lanes(TileRing *R, const void *src, int n
 // own pointer).
 __device__ __forceinline__ int produce_sell_lanes(TileRing *R, int64_t s_lo, int64_t s_hi, int spt,
                                                   const SliceOffsets &off, const void *sval, int vbytes, int ebytes,
-                                                  const int32_t *scol, const void *epi, int ne, unsigned &seq,
-                                                  uint64_t timeout_ns) {
+                                                  const int32_t *scol, const void *epi, int ne, unsigned &seq) {
     const uint64_t pol = l2_evict_first_policy();
     const int lane = threadIdx.x & 31;
     for (int64_t s0 = s_lo; s0 < s_hi; s0 += spt, ++seq) {
         const int s = (int)(seq % kStages);
         const unsigned use = seq / kStages;
         int st = 0;
-        if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u, timeout_ns);
+        if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u);
         st = __shfl_sync(0xffffffffu, st, 0);
         if (st) return st;
         const int64_t s1 = s0 + spt < s_hi ? s0 + spt : s_hi;
@@ -360,7 +373,7 @@ __device__ __forceinline__ int produce_sell_lanes(TileRing *R, int64_t s_lo, int
         const unsigned be = (unsigned)(s1 - s0) * 32u * (unsigned)ebytes;
         if (lane == 0) mbar_arrive_expect_tx(&R->full[s], bv + bc + be * (unsigned)ne);
         __syncwarp();
-        unsigned char *const dst = R->buf + (size_t)s * kStageBytes;
+        unsigned char *const dst = the_stages() + (size_t)s * kStageBytes;
         if (lane < 2) {
             if (nv > 0)
                 bulk_g2s_hint(lane == 0 ? dst : dst + bv,
@@ -384,19 +397,19 @@ __device__ __forceinline__ int produce_sell_lanes(TileRing *R, int64_t s_lo, int
 __device__ __forceinline__ bool produce_sell(TileRing *R, int64_t s_lo, int64_t s_hi, int spt,
                                              const SliceOffsets &off, const void *sval, int vbytes, int ebytes,
                                              const int32_t *scol, const void *const *epi, int ne,
-                                             unsigned &seq, uint64_t timeout_ns) {
+                                             unsigned &seq) {
     const uint64_t pol = l2_evict_first_policy();
     for (int64_t s0 = s_lo; s0 < s_hi; s0 += spt, ++seq) {
         const int s = (int)(seq % kStages);
         const unsigned use = seq / kStages;
-        if (use > 0 && !mbar_wait(&R->empty[s], (use - 1) & 1u, timeout_ns)) return false;
+        if (use > 0 && !mbar_wait(R, &R->empty[s], (use - 1) & 1u)) return false;
         const int64_t s1 = s0 + spt < s_hi ? s0 + spt : s_hi;
         const int64_t e0 = off(s0), e1 = off(s1);
         const unsigned nv = (unsigned)(e1 - e0);
         const unsigned bv = nv * (unsigned)vbytes, bc = nv * 4u;
         const unsigned be = (unsigned)(s1 - s0) * 32u * (unsigned)ebytes;
         mbar_arrive_expect_tx(&R->full[s], bv + bc + be * (unsigned)ne);
-        unsigned char *dst = R->buf + (size_t)s * kStageBytes;
+        unsigned char *dst = the_stages() + (size_t)s * kStageBytes;
         if (nv > 0) {
             bulk_g2s_hint(dst, (const unsigned char *)sval + e0 * vbytes, bv, &R->full[s], pol);
             bulk_g2s_hint(dst + bv, scol + e0, bc, &R->full[s], pol);
@@ -413,13 +426,13 @@ __device__ __forceinline__ bool produce_sell(TileRing *R, int64_t s_lo, int64_t 
 // issued has landed, so that no bulk copy is still writing into shared
 // memory when the CTA exits.  In normal operation every issued tile has
 // already been consumed and this returns at once.
-__device__ __forceinline__ void ring_drain(TileRing *R, unsigned pseq, unsigned cseq, uint64_t timeout_ns) {
+__device__ __forceinline__ void ring_drain(TileRing *R, unsigned pseq, unsigned cseq) {
     if ((threadIdx.x >> 5) == kConsumerWarps && (threadIdx.x & 31) == 0) R->issued = pseq;
     if (threadIdx.x == 0) R->consumed = cseq;
     __syncthreads();
     if (threadIdx.x == 0) {
         for (unsigned q = R->consumed; q < R->issued; ++q)
-            if (!mbar_wait(&R->full[q % kStages], (q / kStages) & 1u, timeout_ns)) break;
+            if (!mbar_wait(R, &R->full[q % kStages], (q / kStages) & 1u)) break;
     }
     __syncthreads();
 }
