@@ -14,11 +14,11 @@ namespace mlb {
 namespace {
 
 constexpr int kNaThreads = 256;
+constexpr int kNaWarps = kNaThreads / 32;
 constexpr int kNaMaxN = 64;
-// Scratch: 256 bytes of header (the CTA ticket counter) followed by the
-// per-CTA partial sums, grid * nb * slots doubles.
+constexpr int kNaStages = 3;   // groups of 32 rows in a warp's shared memory
+// Scratch: the CTAs' sums, value by value (value v of CTA b at v * grid + b).
 constexpr int64_t kNaScratchDoubles = 65536;  // 512 KiB
-constexpr int64_t kNaHeaderDoubles = 32;       // 256 bytes
 
 static __device__ __align__(256) double g_noalloc_scratch[kNaScratchDoubles];
 
@@ -50,70 +50,221 @@ __device__ __forceinline__ cdouble ldv(const cdouble *p) {
     return {v.x, v.y};
 }
 
-// One thread per CSR row; each thread keeps NB running inner products
-// conj(q_k) y over its rows; CTA sums go to the scratch array; the last CTA
-// to finish (ticket counter) adds the CTA sums in CTA order and writes d.
-template <typename T, int NB>
-__global__ void __launch_bounds__(kNaThreads)
-    spmv_qdot_csr_kernel(int64_t N, const int64_t *rp, const int32_t *ci, const T *av, const T *x,
-                         const T *Q, int64_t ldq, int n, T *y, T *d, double *scratch) {
-    constexpr int DS = dslots<T>();
-    using ACC = typename real_of<T>::type;
-    __shared__ double red[33 * DS];
-    __shared__ unsigned s_ticket;
-    unsigned *ticket = reinterpret_cast<unsigned *>(scratch);
-    double *part = scratch + kNaHeaderDoubles;
-    ACC acc[NB * DS];
+__device__ __forceinline__ void cp_async(void *dst, const double *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async(void *dst, const cdouble *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async(void *dst, const int32_t *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+}
+
+// Sums of V values (a power of two, at most 8) over a warp: lane l returns
+// the sum of value l / (32 / V).  Each of the first steps halves the values a
+// lane still holds, so it takes V + 1 adds where V trees take 5 V (an FP64
+// instruction occupies the SM's pipe for ~15 cycles).  Fixed order.
+template <int V>
+__device__ __forceinline__ double warp_sums(double (&a)[V]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
 #pragma unroll
-    for (int k = 0; k < NB * DS; ++k) acc[k] = ACC(0);
-    for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < N;
-         row += (int64_t)gridDim.x * blockDim.x) {
-        T sum{};
-        for (int64_t k = __ldg(rp + row), k1 = __ldg(rp + row + 1); k < k1; ++k)
-            sum = efma(ldv(av + k), ldv(x + __ldg(ci + k)), sum);
-        y[row] = sum;
+    for (int h = V / 2; h > 0; h /= 2, o /= 2) {
+        const bool up = (lane & o) != 0;
 #pragma unroll
-        for (int q = 0; q < NB; ++q)
-            if (q < n) acc_dot(&acc[q * DS], ldv(Q + (int64_t)q * ldq + row), sum);
+        for (int k = 0; k < h; ++k) {
+            const double keep = up ? a[k + h] : a[k], give = up ? a[k] : a[k + h];
+            a[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
     }
-    // unrolled over the fixed bound NB so that every index into acc is a
-    // compile-time constant (a run-time index would put acc in local
-    // memory); n is the same in every thread, so the barriers inside
-    // block_sum_all are reached uniformly
+    for (; o > 0; o /= 2) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+    return a[0];
+}
+
+// CTAs an SM holds: as many as the accumulators (NB * DS doubles a thread)
+// and the loads in flight leave registers for.
+template <typename T, int NB>
+constexpr int na_ctas() {
+    return NB * dslots<T>() > 16 ? 1 : 2;
+}
+// Entries of 32 rows that a warp stages (9 a row, complex 7): others are
+// read directly.
+template <typename T>
+constexpr int na_cap() {
+    return 32 * (dslots<T>() == 1 ? 9 : 7);
+}
+template <typename T>
+constexpr size_t na_smem() {
+    return (size_t)kNaWarps * kNaStages * na_cap<T>() * (sizeof(T) + 4);
+}
+
+// One row per lane, 32 rows per warp at a time; each thread keeps NB running
+// inner products conj(q_k) y over its rows.  What bounds it at 1e6 rows of 7
+// entries: HBM (177 MB for n = 8, 26 us) and the FP64 pipe (15 multiply-adds
+// a row, 25 us).  So the warp's entries, which lie one after another, come by
+// coalesced asynchronous copies into its own shared memory, 32 rows ahead
+// (a lane that walks its row itself touches 14 lines per load instruction,
+// and its loads wait for one another), and a row's gathers of x and its
+// entries of Q are in flight together.  us a call, before -> now: 101^3, n = 8:
+// 65 -> 46 (3.8 TB/s), n = 4: 48 -> 44; 40^3: 25 -> 10.  It is as fast with 2 as
+// with 3 CTAs per SM, and a third stage gives 1 us.
+// Rows too long for the staging are read directly.  Each row is one
+// sequential sum in the order of its entries.
+template <typename T, int NB>
+__global__ void __launch_bounds__(kNaThreads, na_ctas<T, NB>())
+    spmv_qdot_csr_kernel(int64_t N, const int64_t *rp, const int32_t *ci, const T *av, const T *x,
+                         const T *Q, int64_t ldq, int n, T *y, double *part) {
+    constexpr int DS = dslots<T>(), V = NB * DS, CAP = na_cap<T>(), ST = kNaStages;
+    constexpr int B = DS == 1 ? 7 : 4;               // gathers of x in flight (8: 47 for 46 us)
+    constexpr int NQ = V <= 8 ? NB : 0;              // entries of Q loaded ahead
+    constexpr int GV = V < 8 ? V : 8;                // sums taken together
+    using ACC = typename real_of<T>::type;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ double red[kNaWarps][V];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T *const vbuf = reinterpret_cast<T *>(smem) + (size_t)warp * ST * CAP;
+    int32_t *const cbuf = reinterpret_cast<int32_t *>(smem + (size_t)kNaWarps * ST * CAP * sizeof(T)) +
+                          (size_t)warp * ST * CAP;
+    ACC acc[V];
 #pragma unroll
-    for (int q = 0; q < NB; ++q) {
-        if (q < n) {
-            double v[DS];
+    for (int k = 0; k < V; ++k) acc[k] = ACC(0);
+    const int64_t ng = (N + 31) / 32, step = (int64_t)gridDim.x * kNaWarps;
+    // the entries [b, e) of this lane's row of group g (empty past the end)
+    auto bounds = [&](int64_t g, int64_t &b, int64_t &e) {
+        const int64_t row = g * 32 + lane;
+        b = g < ng ? __ldg(rp + (row < N ? row : N)) : 0;
+        e = g < ng ? __ldg(rp + (row + 1 < N ? row + 1 : N)) : 0;
+    };
+    // copies of a group into stage st; the first of its entries, or -1 when
+    // it is read directly
+    auto stage = [&](int st, int64_t b, int64_t e) -> int64_t {
+        const int64_t e0 = __shfl_sync(0xffffffffu, b, 0), e1 = __shfl_sync(0xffffffffu, e, 31);
+        const bool fits = __all_sync(0xffffffffu, e1 - e0 <= CAP && b >= e0 && b <= e && e <= e1);
+        if (fits)
+            for (int64_t t = e0 + lane; t < e1; t += 32) {
+                cp_async(vbuf + st * CAP + (t - e0), av + t);
+                cp_async(cbuf + st * CAP + (t - e0), ci + t);
+            }
+        cp_async_commit();
+        return fits ? e0 : -1;
+    };
+    int64_t g = (int64_t)blockIdx.x * kNaWarps + warp;
+    // bounds and first entry of the groups g, g + step, ... in flight, and the
+    // bounds of the one to be copied next
+    int64_t b[ST], e[ST], at[ST];
 #pragma unroll
-            for (int t = 0; t < DS; ++t) v[t] = (double)acc[q * DS + t];
-            block_sum_all<DS>(v, red);
-            if (threadIdx.x == 0) {
+    for (int u = 0; u + 1 < ST; ++u) bounds(g + u * step, b[u], e[u]);
 #pragma unroll
-                for (int t = 0; t < DS; ++t) part[((size_t)blockIdx.x * NB + q) * DS + t] = v[t];
+    for (int u = 0; u + 1 < ST; ++u) at[u] = stage(u, b[u], e[u]);
+    bounds(g + (ST - 1) * step, b[ST - 1], e[ST - 1]);
+    for (int st = 0; g < ng; g += step, st = st + 1 < ST ? st + 1 : 0) {
+        at[ST - 1] = stage(st > 0 ? st - 1 : ST - 1, b[ST - 1], e[ST - 1]);
+        int64_t b2, e2;
+        bounds(g + ST * step, b2, e2);
+        const int64_t row = g * 32 + lane;
+        const bool in = row < N;
+        T qv[NQ > 0 ? NQ : 1];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) qv[q] = in && q < n ? ldv(Q + (int64_t)q * ldq + row) : T{};
+        cp_async_wait<ST - 1>();
+        __syncwarp();
+        T sum{};
+        if (at[0] >= 0) {
+            const T *vp = vbuf + st * CAP + (int)(b[0] - at[0]);
+            const int32_t *cp = cbuf + st * CAP + (int)(b[0] - at[0]);
+            const int len = (int)(e[0] - b[0]);
+            for (int k = 0; k < len; k += B) {
+                T xv[B];
+#pragma unroll
+                for (int u = 0; u < B; ++u)
+                    if (k + u < len) xv[u] = ldv(x + cp[k + u]);
+#pragma unroll
+                for (int u = 0; u < B; ++u)
+                    if (k + u < len) sum = efma(vp[k + u], xv[u], sum);
+            }
+        } else {
+            for (int64_t k = b[0]; k < e[0]; ++k) sum = efma(ldv(av + k), ldv(x + __ldg(ci + k)), sum);
+        }
+        if (in) {
+            y[row] = sum;
+            if constexpr (NQ > 0) {
+#pragma unroll
+                for (int q = 0; q < NB; ++q)
+                    if (q < n) acc_dot(&acc[q * DS], qv[q], sum);
+            } else {
+#pragma unroll
+                for (int q = 0; q < NB; ++q)
+                    if (q < n) acc_dot(&acc[q * DS], ldv(Q + (int64_t)q * ldq + row), sum);
             }
         }
+        __syncwarp();   // the stage is free
+#pragma unroll
+        for (int u = 0; u + 1 < ST; ++u) {
+            at[u] = at[u + 1];
+            b[u] = b[u + 1];
+            e[u] = e[u + 1];
+        }
+        b[ST - 1] = b2;
+        e[ST - 1] = e2;
     }
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_ticket = atomicAdd(ticket, 1u);
+    asm volatile("griddepcontrol.launch_dependents;");
+    // the CTA's sums, GV values at a time (every index into acc a constant:
+    // a run-time index would put acc in local memory)
+#pragma unroll
+    for (int v0 = 0; v0 < V; v0 += GV) {
+        if (v0 < n * DS) {
+            double a[GV];
+#pragma unroll
+            for (int k = 0; k < GV; ++k) a[k] = (double)acc[v0 + k];
+            const double t = warp_sums<GV>(a);
+            if (lane % (32 / GV) == 0) red[warp][v0 + lane / (32 / GV)] = t;
+        }
     }
     __syncthreads();
-    if (s_ticket != gridDim.x - 1) return;
-    __threadfence();
-    for (int q = 0; q < n; ++q) {
-        double v[DS];
+    for (int v = threadIdx.x; v < n * DS; v += kNaThreads) {
+        double t[kNaWarps];
 #pragma unroll
-        for (int t = 0; t < DS; ++t) v[t] = 0.0;
-        for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+        for (int w = 0; w < kNaWarps; ++w) t[w] = red[w][v];
 #pragma unroll
-            for (int t = 0; t < DS; ++t) v[t] += part[((size_t)b * NB + q) * DS + t];
+        for (int h = kNaWarps / 2; h > 0; h /= 2)
+#pragma unroll
+            for (int w = 0; w < h; ++w) t[w] += t[w + h];
+        part[(size_t)v * gridDim.x + blockIdx.x] = t[0];
+    }
+}
+
+// d from the CTAs' sums: one warp per value, lanes over the CTAs in index
+// order, then the warp's tree.  Launched so that it may start as the product
+// ends; in place of a counter that the CTAs take a ticket from (zeroed by a
+// launch of its own on every call, a fence and an atomic per CTA).
+__global__ void __launch_bounds__(1024) sum_parts_kernel(const double *part, int grid, int nv, double *d) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int lane = threadIdx.x & 31;
+    for (int v = threadIdx.x >> 5; v < nv; v += blockDim.x >> 5) {
+        constexpr int M = 16;   // CTA sums in flight per lane
+        double s = 0.0;
+        for (int b = lane; b < grid; b += 32 * M) {
+            double t[M];
+#pragma unroll
+            for (int m = 0; m < M; ++m)
+                t[m] = b + 32 * m < grid ? __ldcg(part + (size_t)v * grid + b + 32 * m) : 0.0;
+#pragma unroll
+            for (int h = M / 2; h > 0; h /= 2)
+#pragma unroll
+                for (int m = 0; m < h; ++m) t[m] += t[m + h];
+            s += t[0];
         }
-        block_sum_all<DS>(v, red);
-        if (threadIdx.x == 0) {
-            double *dd = reinterpret_cast<double *>(d) + (size_t)q * DS;
 #pragma unroll
-            for (int t = 0; t < DS; ++t) dd[t] = v[t];
-        }
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) d[v] = s;
     }
 }
 
@@ -121,25 +272,33 @@ template <typename T, int NB>
 int launch(int dev, int64_t N, const int64_t *rp, const int32_t *ci, const T *av, const T *x, const T *Q,
            int64_t ldq, int n, T *y, T *d, double *scratch, cudaStream_t st) {
     constexpr int DS = dslots<T>();
-    int sms = 0, occ = 0;
+    int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, spmv_qdot_csr_kernel<T, NB>, kNaThreads, 0) !=
-            cudaSuccess) {
+        cudaFuncSetAttribute(spmv_qdot_csr_kernel<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)na_smem<T>()) != cudaSuccess) {
         cudaGetLastError();
         return MLB_ERR_CUDA;
     }
-    int64_t grid = (int64_t)sms * (occ > 0 ? occ : 1);
-    const int64_t fit = (kNaScratchDoubles - kNaHeaderDoubles) / ((int64_t)NB * DS);
+    int64_t grid = (int64_t)sms * na_ctas<T, NB>();
+    const int64_t fit = kNaScratchDoubles / ((int64_t)NB * DS);
     const int64_t need = (N + kNaThreads - 1) / kNaThreads;
     grid = std::min(grid, std::min(fit, need));
-    if (grid < 1) grid = 1;
-    // the ticket counter must start at zero on every call
-    if (cudaMemsetAsync(scratch, 0, sizeof(unsigned), st) != cudaSuccess) {
+    spmv_qdot_csr_kernel<T, NB><<<(int)grid, kNaThreads, na_smem<T>(), st>>>(N, rp, ci, av, x, Q, ldq, n, y, scratch);
+    if (cudaGetLastError() != cudaSuccess) return MLB_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1);
+    cfg.blockDim = dim3(std::min(32 * n * DS, 1024));
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, sum_parts_kernel, (const double *)scratch, (int)grid, n * DS,
+                           reinterpret_cast<double *>(d)) != cudaSuccess) {
         cudaGetLastError();
         return MLB_ERR_CUDA;
     }
-    spmv_qdot_csr_kernel<T, NB><<<(int)grid, kNaThreads, 0, st>>>(N, rp, ci, av, x, Q, ldq, n, y, d, scratch);
-    if (cudaGetLastError() != cudaSuccess) return MLB_ERR_CUDA;
     return MLB_OK;
 }
 

@@ -175,3 +175,37 @@ def test_noalloc_rejects_sizes_beyond_its_scratch_limit():
     with pytest.raises(M.MlbError) as e:
         M.mlbicgstab_spmv_qdot_noalloc(rp, ci, av, x, Q, y, d)
     assert e.value.code == M.MLB_ERR_ARG
+
+
+@pytest.mark.parametrize("case", ["real", "complex"])
+@pytest.mark.parametrize("N,longest", [(1, 1), (31, 3), (33, 9), (1000, 9), (1000, 40), (70001, 12)])
+def test_noalloc_rows_of_any_length(case, N, longest):
+    """Rows of 0 to `longest` entries: 32 rows in one warp's staging, some in
+    and some beyond it, rows wider than one batch of gathers, a last warp with
+    few rows or none.  Bounds as above."""
+    import torch
+    import oracle as O
+    rng = np.random.default_rng(N + longest)
+    cplx, n = case == "complex", 5
+    # long rows stand together, so that some warps stage theirs and others do not
+    lens = np.where((np.arange(N) // 32) % 3 == 1, longest, rng.integers(0, min(longest, 5) + 1, size=N))
+    rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    nnz = int(rp[-1])
+    col = rng.integers(0, N, size=nnz).astype(np.int32)
+    val = _rand(rng, nnz, case)
+    A = W.CSR(row_ptr=rp, col=col, val=val, n_rows=N)
+    x, Q = _rand(rng, N, case), np.stack([_rand(rng, N, case) for _ in range(n)])
+    y_or = O.spmv(A, x)
+    d_or = Q.conj() @ y_or
+    dt = torch.complex128 if cplx else torch.float64
+    dev = [torch.tensor(rp, device="cuda"), torch.tensor(col, device="cuda"), torch.tensor(val, dtype=dt, device="cuda")]
+    y = torch.full((N,), float("nan"), dtype=dt, device="cuda")
+    d = torch.full((n,), float("nan"), dtype=dt, device="cuda")
+    M.mlbicgstab_spmv_qdot_noalloc(*dev, torch.tensor(x, dtype=dt, device="cuda"),
+                                   torch.tensor(Q, dtype=dt, device="cuda"), y, d)
+    torch.cuda.synchronize()
+    yn, dn = y.cpu().numpy(), d.cpu().numpy()
+    bound_y = 2 * _gamma(longest + 1) * _abs_product(A, x)
+    assert np.all(np.abs(yn - y_or) <= bound_y)
+    bound_d = np.abs(Q) @ bound_y + 2 * _gamma(N) * (np.abs(Q) @ np.abs(y_or))
+    assert np.all(np.abs(dn - d_or) <= bound_d)
