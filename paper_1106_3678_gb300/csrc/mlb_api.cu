@@ -40,6 +40,8 @@ struct mlb_handle {
     void *ilu_lell_a = nullptr, *ilu_uell_a = nullptr, *ilu_udiag = nullptr;
     IluLevel *ilu_llev = nullptr, *ilu_ulev = nullptr;    // few levels: the streamed form
     int32_t *ilu_lmeta = nullptr, *ilu_umeta = nullptr;
+    void *ilu_flow = nullptr;                             // many levels: one slot per row of L and of U
+    int32_t *ilu_lwatch = nullptr, *ilu_uwatch = nullptr;
     int ilu_maxw = 0;
     int64_t ilu_nel = 0, ilu_neu = 0, ilu_ndiag = 0;      // values in lell, uell, udiag
     // refined mode with ILU(0): FP32 copies of the factor values and an
@@ -337,6 +339,9 @@ SysView<T> make_view(const mlb_handle *h) {
         v.ilu.ulev = h->ilu_ulev;
         v.ilu.lmeta = (const int2 *)h->ilu_lmeta;
         v.ilu.umeta = (const int2 *)h->ilu_umeta;
+        v.ilu.flow = (decltype(v.ilu.flow))h->ilu_flow;
+        v.ilu.lwatch = h->ilu_lwatch;
+        v.ilu.uwatch = h->ilu_uwatch;
         v.ilu.spt = ilu_slices_per_tile(h->ilu_maxw, sizeof(v.Q[0]));
         v.ilu.lell_c = h->ilu_lell_c;
         v.ilu.uell_c = h->ilu_uell_c;
@@ -388,6 +393,9 @@ SysView<T32> make_view32(const mlb_handle *h) {
         v.ilu.ulev = h->ilu_ulev;
         v.ilu.lmeta = (const int2 *)h->ilu_lmeta;
         v.ilu.umeta = (const int2 *)h->ilu_umeta;
+        v.ilu.flow = (decltype(v.ilu.flow))h->ilu_flow;
+        v.ilu.lwatch = h->ilu_lwatch;
+        v.ilu.uwatch = h->ilu_uwatch;
         v.ilu.spt = ilu_slices_per_tile(h->ilu_maxw, sizeof(v.Q[0]));
         v.ilu.lell_c = h->ilu_lell_c;
         v.ilu.uell_c = h->ilu_uell_c;
@@ -485,7 +493,7 @@ int map_solution(mlb_handle *h, bool to_x, cudaStream_t st) {
 }
 int map_solution(mlb_handle *h, bool to_x) { return map_solution(h, to_x, h->stream); }
 
-static_assert(Engine<double, true>::kIluReg == kIluEll, "ILU(0) entries held by position = entries in registers");
+static_assert(Engine<double, kIluAny>::kIluReg == kIluEll, "ILU(0) entries held by position = entries in registers");
 
 // Jacobi preconditioner M = diag(A) (Algorithm 7.1, right preconditioning):
 // d = diagonal of A (a row's diagonal entries summed), values of A M^{-1}
@@ -696,6 +704,10 @@ int create_impl(mlb_handle *h, const mlb_matrix *A, const mlb_matrix *AH, const 
         if (ih.wide) {
             if ((rc = up(&h->ilu_llev, ih.llev)) || (rc = up(&h->ilu_ulev, ih.ulev)) ||
                 (rc = up(&h->ilu_lmeta, ih.lmeta)) || (rc = up(&h->ilu_umeta, ih.umeta)))
+                return rc;
+        } else if (!cplx) {
+            if ((rc = up(&h->ilu_lwatch, ih.lwatch)) || (rc = up(&h->ilu_uwatch, ih.uwatch)) ||
+                (rc = dev_alloc(h, &h->ilu_flow, (size_t)N * 2 * sizeof(Slot))))
                 return rc;
         }
         if ((rc = dev_alloc_t(h, &h->ilu_lcnt, (size_t)N * 4))) return rc;

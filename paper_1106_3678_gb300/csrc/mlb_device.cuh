@@ -193,6 +193,9 @@ __device__ __forceinline__ int ld_relaxed_i32(const int *p) {
     asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ void st_relaxed_u32(unsigned *p, unsigned v) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 __device__ __forceinline__ uint64_t globaltimer_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -207,7 +210,7 @@ __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_re
 // Barrier state in global memory (zeroed before every launch).
 struct BarrierState {
     unsigned count;   // arrivals since the launch began (monotonic; grid_barrier)
-    unsigned pad0;
+    unsigned progress;   // changes while a triangular solve moves (Engine::ilu_flow)
     int status;       // 0, or an MLB_ERR_* code set by a CTA that gave up
     int pad1;
 };
@@ -218,8 +221,8 @@ constexpr int kStatusTimeout = 4;  // == MLB_ERR_TIMEOUT
 // writes have been ordered before it (a __syncthreads, or thread 0's own
 // writes).  `epoch` counts the barriers this CTA has passed; all CTAs pass
 // the same sequence, so barrier e completes when the counter reaches
-// e * expected.  The spin is bounded by timeout_ns (%globaltimer) and
-// gives up early when another CTA has already recorded a failure.
+// e * expected.  The spin is bounded by timeout_ns (%globaltimer) without
+// progress of a triangular solve and gives up early when another CTA has already recorded a failure.
 // grid_arrive and grid_wait are its two halves, for callers with work to
 // overlap with the wait.  Polls are relaxed loads and one fence orders what
 // follows them.
@@ -231,13 +234,15 @@ __device__ __forceinline__ bool grid_wait(BarrierState *bs, unsigned epoch, unsi
                                           uint64_t timeout_ns) {
     const unsigned target = epoch * expected;
     uint64_t t0 = 0;
-    unsigned spins = 0;
+    unsigned spins = 0, seen = 0;
     while ((int)(ld_relaxed_u32(&bs->count) - target) < 0) {
         if ((++spins & 31u) == 0) {
             if (ld_relaxed_i32(&bs->status) != 0) return false;
             const uint64_t t = globaltimer_ns();
-            if (t0 == 0) {
+            const unsigned at = ld_relaxed_u32(&bs->progress);
+            if (t0 == 0 || at != seen) {
                 t0 = t;
+                seen = at;
             } else if (t - t0 > timeout_ns) {
                 atomicCAS(&bs->status, 0, kStatusTimeout);
                 return false;
@@ -267,7 +272,10 @@ __device__ __forceinline__ bool grid_arrive_wait(BarrierState *bs, unsigned &epo
 // the CTA's two barriers: 1.12 us, with stores 1.59 us, counter and partial
 // sums 1.67 us), and a round of polls loads all its slots before it looks at
 // the first (one at a time: 2.2 us).  Slots are zeroed before a launch;
-// epochs count from 1.
+// epochs count from 1.  A slot's value and epoch belong together only while
+// the load stays one access of 16 bytes, so a reader uses all of its words
+// (the epoch is compared whole): of a load with unused words the compiler may
+// keep the others as accesses of their own.
 struct alignas(16) Slot {
     double v;
     unsigned long long epoch;
@@ -287,6 +295,36 @@ __device__ __forceinline__ Slot slot_load(const Slot *p) {
                  : "memory");
     return Slot{__longlong_as_double((long long)b), ep};
 }
+// Slots of one value each (Engine::ilu_flow): a float and its epoch in 8
+// bytes, a double in a Slot.
+template <int BYTES>
+struct ValueSlot {
+    using type = Slot;
+};
+template <>
+struct ValueSlot<4> {
+    using type = unsigned long long;
+};
+__device__ __forceinline__ void value_put(Slot *p, double v, unsigned epoch) { slot_put(p, v, epoch); }
+__device__ __forceinline__ void value_put(unsigned long long *p, float v, unsigned epoch) {
+    const unsigned long long b = (unsigned long long)epoch << 32 | __float_as_uint(v);
+    asm volatile("{ .reg .b64 o; atom.exch.relaxed.gpu.global.b64 o, [%0], %1; }" ::"l"(p), "l"(b) : "memory");
+}
+__device__ __forceinline__ Slot value_load(const Slot *p) { return slot_load(p); }
+__device__ __forceinline__ unsigned long long value_load(const unsigned long long *p) {
+    unsigned long long b;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(b) : "l"(p) : "memory");
+    return b;
+}
+__device__ __forceinline__ bool value_of(Slot s, unsigned epoch, double &v) {
+    v = s.v;
+    return s.epoch == epoch;
+}
+__device__ __forceinline__ bool value_of(unsigned long long s, unsigned epoch, float &v) {
+    v = __uint_as_float((unsigned)s);
+    return (unsigned)(s >> 32) == epoch;
+}
+
 // One warp waits until all G slots at p carry `epoch` and adds their values:
 // lane l those of CTAs l, l + 32, ... as a pair tree, then an xor tree over
 // the lanes (every lane receives the sum).  The wait is bounded by
@@ -315,7 +353,7 @@ __device__ __forceinline__ bool slots_sum(const Slot *p, unsigned G, unsigned ep
                 if (32 * m < left) s[m] = slot_load(p + b0 + (lane + 32 * m < left ? lane + 32 * m : 0));
 #pragma unroll
             for (int m = 0; m < M; ++m)
-                if ((need >> m & 1u) && (unsigned)s[m].epoch == epoch) {
+                if ((need >> m & 1u) && s[m].epoch == epoch) {
                     x[m] = s[m].v;
                     need &= ~(1u << m);
                 }

@@ -156,6 +156,10 @@ struct IluView {
     const IluLevel *llev, *ulev;
     const int2 *lmeta, *umeta;
     int spt;                    // its slices per tile
+    // many levels, real values: one slot per row of L (i) and of U (N + i)
+    // and, per 32 positions, the row to wait for first (see ilu_flow)
+    typename ValueSlot<sizeof(T)>::type *flow;
+    const int32_t *lwatch, *uwatch;
 };
 
 // Device view of one linear system.  Vectors have leading dimension `ld`
@@ -552,6 +556,7 @@ struct GridSync {
     uint64_t timeout_ns;
     unsigned epoch;     // exchanges this CTA has passed
     unsigned bepoch;    // barriers (sync) this CTA has passed
+    unsigned fepoch;    // triangular solve pairs (Engine::ilu_flow) this CTA has passed
     bool ok;            // false once a barrier or a tile wait failed
     unsigned seqs[kThreads];   // per-thread tile counters, kept across systems
 
@@ -565,7 +570,7 @@ struct GridSync {
         bar = b;
         slots = p;
         timeout_ns = to;
-        epoch = bepoch = 0;
+        epoch = bepoch = fepoch = 0;
         ok = !the_ring()->failed;
         the_ring()->timeout_ns = to;
         the_red().fail = 0;
@@ -744,14 +749,20 @@ struct NoHook {
     static constexpr bool kActive = false;
 };
 
-// PC: built with the ILU(0) preconditioner passes (ilu_pre and the
-// product passes' switch to M^{-1} of their input); without it none of
-// that code is reachable.  EW: the matrix storage of the products (1:
+// PC: the forms of the ILU(0) preconditioner passes that the engine is built
+// with: none, streamed (ilu_wide), by slots (ilu_flow), or those of a batch,
+// whose systems may have either form, and of complex values (ilu_wide and
+// ilu_levels).  What is not built in takes no registers from the kernel's
+// loop: with two forms in one kernel the FP64 one spilled 276 bytes a thread,
+// with the streamed form alone 120 (multicolour ILU(0) at 96^3: 31.0 -> 30.0
+// ms, refined 3x3-block system 2840 -> 2480 us).
+// EW: the matrix storage of the products (1:
 // scalar SELL-32; 3: 3x3 blocks, see sell_slice_sum3).
 //
 // The consumer threads run inner() and the other members; the producer warp
 // runs serve() beside them.
-template <typename T, bool PC = false, int EW = 1>
+enum { kNoIlu, kIluWide, kIluFlow, kIluAny };
+template <typename T, int PC = kNoIlu, int EW = 1>
 struct Engine {
     using S = typename coef_of<T>::type;                      // FP64 coefficient
     using ACC = typename real_of<T>::type;                    // thread accumulator
@@ -984,7 +995,7 @@ struct Engine {
                                               ACC (&acc)[K]) {
         // with ILU(0) the product is A t, t = M^{-1} xin formed before the
         // pass
-        if constexpr (PC) {
+        if constexpr (PC != kNoIlu) {
             if (sys().ilu.lu) xin = sys().ilu.t;
         }
         // FP32 and complex engines: a pipelined width of 7, the widest row of
@@ -1005,6 +1016,7 @@ struct Engine {
     // kIluReg entries (column, factor value) in registers, where the rest
     // of its entries start and end, and the row's right-hand-side entry
     // (forward) or its U diagonal (backward).  i < 0: no row.
+    static constexpr bool kFlow = PC == kIluFlow;   // real values only
     static constexpr int kIluReg = 4;   // == kIluEll (entries stored by position)
     struct IluRow {
         int i, cnt;
@@ -1074,6 +1086,162 @@ struct Engine {
         return s;
     }
 
+    // out = M^{-1} v by a team without a barrier between levels: a row's value
+    // goes to its slot with the number of this M^{-1}, and a row takes the
+    // values it needs from their slots as they arrive.  Warps take 32
+    // positions of the level order at a time, L's and then U's, dealt over
+    // the CTAs; a row only waits for rows at earlier positions, and a warp
+    // takes its positions in increasing order, so the first unfinished
+    // position never waits.  A warp first watches one row two levels back,
+    // so the warps that poll all their rows' slots are those of the next two
+    // levels.  Each row is one sequential sum in pattern order.
+    // What bounds it: the chain of levels, each a slot put, its way through
+    // L2 to a poll, the row's sum and (U) a division.  us a level, FP64, with
+    // barriers (ilu_levels) -> here: 200^2 2.4 -> 1.3, 40^3 2.5 -> 1.7, 48^3 2.5
+    // -> 1.7, 96^3 2.9 -> 2.3; 3x3-block system of 393,216 rows, about ten
+    // entries a triangle and row: 76 -> 55 ms a solve.
+    __device__ __forceinline__ bool ilu_flow(const T *v, T *out) {
+        if constexpr (kFlow) {
+            const IluView<T> &M = sys().ilu;
+            const int lane = threadIdx.x & 31, cw = threadIdx.x >> 5;
+            const unsigned ep = gs().fepoch + 1;
+            const int64_t N = sys().N, nch = (N + 31) / 32, G = gs().nblocks;
+            using VS = typename ValueSlot<sizeof(T)>::type;
+            VS *const zl = M.flow, *const zu = zl + N;
+            BarrierState *const bar = gs().bar;
+            const uint64_t limit = gs().timeout_ns;
+            // progress is told seldom: a store per 32 rows to the word that every
+            // waiting warp reads doubled the time of a solve
+            uint64_t told = globaltimer_ns();
+            bool ok = true;
+            for (int64_t k = gs().bid + G * cw; ok && k < 2 * nch; k += G * kConsumerWarps) {
+                const bool up = k >= nch;
+                const int64_t ch = up ? k - nch : k, q = 32 * ch + lane;
+                VS *const z = up ? zu : zl;
+                const int w = up ? M.uwatch[ch] : M.lwatch[ch];
+                // this lane's row i: n entries, the first ones in c and a, and
+                // the right-hand side (L) or U's diagonal
+                int i = -1, n = 0;
+                int64_t p = 0;          // a longer row's entries in the pattern
+                int32_t c[kIluReg];
+                T a[kIluReg], d{};
+                if (q < N) {
+                    i = up ? M.urows[q] : M.lrows[q];
+                    n = up ? M.ucnt[q] : M.lcnt[q];
+                    const int32_t *const pc = (up ? M.uell_c : M.lell_c) + q;
+                    const T *const pa = (up ? M.uell_a : M.lell_a) + q;
+#pragma unroll
+                    for (int u = 0; u < kIluReg; ++u)
+                        if (u < n) {
+                            c[u] = pc[u * N];
+                            a[u] = pa[u * N];
+                        }
+                    d = up ? M.udiag[q] : v[i];
+                    if (n > kIluReg) p = M.rp[i] + (up ? M.dpos[i] + 1 : 0);
+                }
+                const VS *const watch = w >= 0 ? z + w : up ? zl + ~w : nullptr;
+                uint64_t t0 = 0;
+                unsigned spins = 0, seen = 0;
+                // every 32nd poll: false (uniformly) when the wait is over,
+                // that is after the limit without any warp's progress (a warp
+                // may wait for a whole triangle)
+                auto patience = [&]() -> bool {
+                    if ((++spins & 31u) != 0) return true;
+                    int stop = 0;
+                    if (lane == 0) {
+                        const uint64_t now = globaltimer_ns();
+                        const unsigned at = ld_relaxed_u32(&bar->progress);
+                        if (ld_relaxed_i32(&bar->status) != 0) stop = 1;
+                        else if (t0 == 0 || at != seen) {
+                            t0 = now;
+                            seen = at;
+                        } else if (now - t0 > limit) {
+                            atomicCAS(&bar->status, 0, kStatusTimeout);
+                            stop = 1;
+                        }
+                    }
+                    return __shfl_sync(0xffffffffu, stop, 0) == 0;
+                };
+                T xv;
+                while (ok && watch && !__all_sync(0xffffffffu, value_of(value_load(watch), ep, xv))) ok = patience();
+                int e = up ? -1 : 0;    // next entry; -1: the right-hand side
+                int e0 = 0;             // the entry in c[0] and a[0]
+                T s = d;
+                bool done = i < 0;
+                while (ok && !__all_sync(0xffffffffu, done)) {
+                    if (!done) {
+                        VS r{}, x[kIluReg];
+                        if (e < 0) r = value_load(zl + i);
+#pragma unroll
+                        for (int u = 0; u < kIluReg; ++u)
+                            if (e0 + u >= e && e0 + u < n) x[u] = value_load(z + c[u]);
+                        if (e < 0 && value_of(r, ep, xv)) {
+                            s = xv;
+                            e = 0;
+                        }
+#pragma unroll
+                        for (int u = 0; u < kIluReg; ++u)
+                            if (e0 + u == e && e < n && value_of(x[u], ep, xv)) {
+                                s = efma(-a[u], xv, s);
+                                e = e0 + u + 1;
+                            }
+                        if (e == e0 + kIluReg && e < n) {   // the next entries, from the pattern
+                            e0 = e;
+#pragma unroll
+                            for (int u = 0; u < kIluReg; ++u)
+                                if (e + u < n) {
+                                    c[u] = M.ci[p + e + u];
+                                    a[u] = M.lu[p + e + u];
+                                }
+                        }
+                        if (e == n) {
+                            if (up) {
+                                s = s / d;
+                                out[i] = s;
+                            }
+                            value_put(z + i, s, ep);
+                            done = true;
+                        }
+                    }
+                    if (!__all_sync(0xffffffffu, done)) ok = patience();
+                }
+                if (lane == 0) {
+                    const uint64_t now = globaltimer_ns();
+                    if (now - told > limit / 8) {
+                        st_relaxed_u32(&bar->progress, (unsigned)k + 1u);
+                        told = now;
+                    }
+                }
+            }
+            if (!ok) the_red().fail = 1;
+            const bool good = gs().sync();
+            if (threadIdx.x == 0) gs().fepoch = ep;   // read again only after another barrier
+            ilu_count();
+            return good;
+        } else {
+            return false;
+        }
+    }
+    // Start of a solve: no slot holds a value yet.
+    __device__ __forceinline__ bool ilu_begin() {
+        if constexpr (kFlow) {
+            using VS = typename ValueSlot<sizeof(T)>::type;
+            VS *const z = sys().ilu.flow;
+            const int64_t nth = (int64_t)gs().nblocks * kConsumers;
+            for (int64_t i = (int64_t)gs().bid * kConsumers + threadIdx.x; i < 2 * sys().N; i += nth)
+                z[i] = VS{};
+            return gs().sync();
+        } else {
+            return true;
+        }
+    }
+
+    // out = M^{-1} v.
+    __device__ __forceinline__ bool ilu_solve_body(const T *v, T *out) {
+        if constexpr (PC == kIluWide) return ilu_wide(v, out);
+        else if constexpr (PC == kIluFlow) return ilu_flow(v, out);
+        else return sys().ilu.llev ? ilu_wide(v, out) : ilu_levels(v, out);
+    }
     // out = M^{-1} v: L z = v by forward substitution (unit diagonal), then
     // U out = z by backward substitution, in place.  Level scheduling: all
     // rows of one level at once over the team's threads, a team barrier
@@ -1082,8 +1250,7 @@ struct Engine {
     // next level (index, entries, right-hand side or diagonal) does not
     // depend on the current level, so it is loaded while the barrier is
     // pending, and only the values of earlier levels are read after it.
-    __device__ __forceinline__ bool ilu_solve_body(const T *v, T *out) {
-        if (sys().ilu.llev) return ilu_wide(v, out);
+    __device__ __forceinline__ bool ilu_levels(const T *v, T *out) {
         const IluView<T> &M = sys().ilu;
         // a level's positions split into one contiguous chunk per CTA of
         // ceil(size / CTAs): every CTA shares each level (a level is a few
@@ -1263,7 +1430,7 @@ struct Engine {
     // Producer warp: the tiles of ilu_wide (lane 0 the values, 1 the columns,
     // 2 the (row, count) pairs, 3 U's diagonal).
     __device__ __forceinline__ int issue_ilu(unsigned &sq) {
-        if constexpr (!PC) {
+        if constexpr (PC != kIluWide && PC != kIluAny) {
             return 0;
         } else {
             if (!sys().ilu.llev) return 0;
@@ -1779,7 +1946,7 @@ struct Engine {
             const bool more = s1 <= i - 1;              // P_F_ROUND, P_G_J0: another f follows
             bool good = true;
             if (!is_narrow<T>::value && st.op == P_RESIDUAL) gs().post(kCmdResidual);
-            if constexpr (PC) {
+            if constexpr (PC != kNoIlu) {
                 if ((st.op == P_SPMV_C || st.op == P_SPMV_Z || st.op == P_RESIDUAL) && sys().ilu.lu) {
                     gs().seq() = sq;
                     good = ilu_solve_body(st.op == P_SPMV_C ? Gc(i) : st.op == P_SPMV_Z ? sys().r : sys().x,

@@ -29,6 +29,18 @@ void group_levels(const std::vector<int32_t> &lev, int nlev, std::vector<int32_t
     for (size_t i = 0; i < lev.size(); ++i) rows[next[lev[i]]++] = (int32_t)i;
 }
 
+// The row to wait for first, per 32 positions of a level order.
+void watch_rows(const std::vector<int32_t> &rows, const std::vector<int32_t> &ptr, bool upper,
+                std::vector<int32_t> &watch) {
+    watch.assign((rows.size() + 31) / 32, -1);
+    int l = 0;
+    for (size_t k = 0; k < watch.size(); ++k) {
+        while (ptr[l + 1] <= (int64_t)(32 * k)) ++l;
+        if (l >= 2) watch[k] = rows[ptr[l - 2]];
+        else if (upper) watch[k] = ~rows[32 * k];
+    }
+}
+
 // One triangle in its streamed form (see IluLevel): row rows[q] has cnt[q]
 // entries, the first (upper: after the diagonal) ones of its row.  Sizes
 // first (fill = false), then the entries; U's diagonal by slot into `diag`.
@@ -179,6 +191,8 @@ int build_t(const mlb_matrix *A, IluHost &f) {
         stream_levels<V>(f, true, true, f.ulev, f.umeta, f.uell_c, f.uell_a, &f.udiag, f.maxw);
         return MLB_OK;
     }
+    watch_rows(f.lrows, f.lptr, false, f.lwatch);
+    watch_rows(f.urows, f.uptr, true, f.uwatch);
     f.lell_c.assign((size_t)kIluEll * N, 0);
     f.uell_c.assign((size_t)kIluEll * N, 0);
     std::vector<V> la((size_t)kIluEll * N, V(0)), ua((size_t)kIluEll * N, V(0)), ud(N, V(0));

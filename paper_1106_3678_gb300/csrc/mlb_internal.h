@@ -158,7 +158,11 @@ constexpr int kIluEll = 4;
 // 32 (m0 + k) + l.  The line: at most kIluWideLevels levels in both triangles
 // together, at most twice the entries with the filling, and slices that fit
 // a stage.  A natural order has one level per wavefront (80 at 14^3, 766 at
-// 128^3), where a level is a few rows per CTA and its cost the barrier.
+// 128^3), where a level is a few rows per CTA and its cost the way of its
+// values to the next one (Engine::ilu_flow).  For that, per 32 positions, the
+// row that a warp waits for before it polls all it needs (any row of an
+// earlier position would do): the first one two levels before the first
+// position's; L: -1, none; U: ~row, the row in L instead.
 constexpr int kIluWideLevels = 32;
 struct IluHost {
     std::vector<int64_t> rp;
@@ -172,6 +176,7 @@ struct IluHost {
     int maxw = 0;                    // its widest slice
     std::vector<IluLevel> llev, ulev;
     std::vector<int32_t> lmeta, umeta;   // (row, entry count) pairs; row -1: filling
+    std::vector<int32_t> lwatch, uwatch;
 };
 // MLB_OK, or MLB_ERR_ARG when a row has no stored diagonal or a pivot is
 // zero or not finite.

@@ -11,65 +11,77 @@ namespace mlb {
 // handles that have that preconditioner.
 template <typename T>
 cudaError_t launch_solve(const SysView<T> &sys, const SolveCtl &ctl, int grid, cudaStream_t st) {
-    if constexpr (!is_cx<T>::value) {
+    if constexpr (is_cx<T>::value) {
+        return sys.ilu.lu ? launch_solve_pc<T, kIluAny>(sys, ctl, grid, st)
+                          : launch_solve_pc<T, kNoIlu>(sys, ctl, grid, st);
+    } else {
         if (sys.ew == 3)
-            return sys.ilu.lu ? launch_solve_pc<T, true, 3>(sys, ctl, grid, st)
-                              : launch_solve_pc<T, false, 3>(sys, ctl, grid, st);
+            return !sys.ilu.lu     ? launch_solve_pc<T, kNoIlu, 3>(sys, ctl, grid, st)
+                   : sys.ilu.llev ? launch_solve_pc<T, kIluWide, 3>(sys, ctl, grid, st)
+                                  : launch_solve_pc<T, kIluFlow, 3>(sys, ctl, grid, st);
+        return !sys.ilu.lu     ? launch_solve_pc<T, kNoIlu>(sys, ctl, grid, st)
+               : sys.ilu.llev ? launch_solve_pc<T, kIluWide>(sys, ctl, grid, st)
+                              : launch_solve_pc<T, kIluFlow>(sys, ctl, grid, st);
     }
-    return sys.ilu.lu ? launch_solve_pc<T, true>(sys, ctl, grid, st) : launch_solve_pc<T, false>(sys, ctl, grid, st);
 }
 template <typename T>
 int solve_blocks_per_sm() {
-    int a = solve_blocks_per_sm_pc<T, false>(), b = solve_blocks_per_sm_pc<T, true>();
-    if constexpr (!is_cx<T>::value) {
-        a = std::min(a, solve_blocks_per_sm_pc<T, false, 3>());
-        b = std::min(b, solve_blocks_per_sm_pc<T, true, 3>());
+    int a = solve_blocks_per_sm_pc<T, kNoIlu>();
+    if constexpr (is_cx<T>::value) {
+        a = std::min(a, solve_blocks_per_sm_pc<T, kIluAny>());
+    } else {
+        a = std::min({a, solve_blocks_per_sm_pc<T, kIluWide>(), solve_blocks_per_sm_pc<T, kIluFlow>(),
+                      solve_blocks_per_sm_pc<T, kNoIlu, 3>(), solve_blocks_per_sm_pc<T, kIluWide, 3>(),
+                      solve_blocks_per_sm_pc<T, kIluFlow, 3>()});
     }
-    return a < b ? a : b;
+    return a;
 }
 template <typename T>
 cudaError_t launch_batch(const BatchItem<T> *items, const BatchPlan &plan, int grid, bool ilu, cudaStream_t st) {
-    return ilu ? launch_batch_pc<T, true>(items, plan, grid, st) : launch_batch_pc<T, false>(items, plan, grid, st);
+    return ilu ? launch_batch_pc<T, kIluAny>(items, plan, grid, st) : launch_batch_pc<T, kNoIlu>(items, plan, grid, st);
 }
 template <typename T>
 int batch_blocks_per_sm() {
-    const int a = batch_blocks_per_sm_pc<T, false>(), b = batch_blocks_per_sm_pc<T, true>();
-    return a < b ? a : b;
+    return std::min(batch_blocks_per_sm_pc<T, kNoIlu>(), batch_blocks_per_sm_pc<T, kIluAny>());
 }
 
-// FP32-inner / FP64-refined launches: the kernels with the ILU(0) passes
-// only when a system has that preconditioner.
+// FP32-inner / FP64-refined launches, likewise.
 template <typename T32, typename T64>
 cudaError_t launch_refine(const SysView<T32> &sys, const RefView<T64> &rv, const SolveCtl &ctl,
                           const RefCtl &rc, int grid, cudaStream_t st) {
     if constexpr (!is_cx<T32>::value) {
         if (sys.ew == 3)
-            return sys.ilu.lu ? launch_refine_pc<T32, T64, true, 3>(sys, rv, ctl, rc, grid, st)
-                              : launch_refine_pc<T32, T64, false, 3>(sys, rv, ctl, rc, grid, st);
+            return !sys.ilu.lu     ? launch_refine_pc<T32, T64, kNoIlu, 3>(sys, rv, ctl, rc, grid, st)
+                   : sys.ilu.llev ? launch_refine_pc<T32, T64, kIluWide, 3>(sys, rv, ctl, rc, grid, st)
+                                  : launch_refine_pc<T32, T64, kIluFlow, 3>(sys, rv, ctl, rc, grid, st);
     }
-    return sys.ilu.lu ? launch_refine_pc<T32, T64, true>(sys, rv, ctl, rc, grid, st)
-                      : launch_refine_pc<T32, T64, false>(sys, rv, ctl, rc, grid, st);
+    constexpr int kManyLevels = is_cx<T32>::value ? kIluAny : kIluFlow;
+    return !sys.ilu.lu     ? launch_refine_pc<T32, T64, kNoIlu>(sys, rv, ctl, rc, grid, st)
+           : sys.ilu.llev ? launch_refine_pc<T32, T64, kIluWide>(sys, rv, ctl, rc, grid, st)
+                          : launch_refine_pc<T32, T64, kManyLevels>(sys, rv, ctl, rc, grid, st);
 }
 template <typename T32, typename T64>
 int refine_blocks_per_sm() {
-    int a = refine_blocks_per_sm_pc<T32, T64, false>(), b = refine_blocks_per_sm_pc<T32, T64, true>();
+    constexpr int kManyLevels = is_cx<T32>::value ? kIluAny : kIluFlow;
+    int a = std::min({refine_blocks_per_sm_pc<T32, T64, kNoIlu>(), refine_blocks_per_sm_pc<T32, T64, kIluWide>(),
+                      refine_blocks_per_sm_pc<T32, T64, kManyLevels>()});
     if constexpr (!is_cx<T32>::value) {
-        a = std::min(a, refine_blocks_per_sm_pc<T32, T64, false, 3>());
-        b = std::min(b, refine_blocks_per_sm_pc<T32, T64, true, 3>());
+        a = std::min({a, refine_blocks_per_sm_pc<T32, T64, kNoIlu, 3>(),
+                      refine_blocks_per_sm_pc<T32, T64, kIluWide, 3>(),
+                      refine_blocks_per_sm_pc<T32, T64, kIluFlow, 3>()});
     }
-    return a < b ? a : b;
+    return a;
 }
 template <typename T32, typename T64>
 cudaError_t launch_batch_refine(const BatchItemR<T32, T64> *items, const BatchPlan &plan, int grid, bool ilu,
                                 cudaStream_t st) {
-    return ilu ? launch_batch_refine_pc<T32, T64, true>(items, plan, grid, st)
-               : launch_batch_refine_pc<T32, T64, false>(items, plan, grid, st);
+    return ilu ? launch_batch_refine_pc<T32, T64, kIluAny>(items, plan, grid, st)
+               : launch_batch_refine_pc<T32, T64, kNoIlu>(items, plan, grid, st);
 }
 template <typename T32, typename T64>
 int batch_refine_blocks_per_sm() {
-    const int a = batch_refine_blocks_per_sm_pc<T32, T64, false>(),
-              b = batch_refine_blocks_per_sm_pc<T32, T64, true>();
-    return a < b ? a : b;
+    return std::min(batch_refine_blocks_per_sm_pc<T32, T64, kNoIlu>(),
+                    batch_refine_blocks_per_sm_pc<T32, T64, kIluAny>());
 }
 
 // FP64 -> FP32 copies (matrix values, Q, F); interleaved complex data is a

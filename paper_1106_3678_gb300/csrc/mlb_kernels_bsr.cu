@@ -6,15 +6,20 @@
 
 namespace mlb {
 
-template cudaError_t launch_solve_pc<double, false, 3>(const SysView<double> &, const SolveCtl &, int, cudaStream_t);
-template cudaError_t launch_solve_pc<double, true, 3>(const SysView<double> &, const SolveCtl &, int, cudaStream_t);
-template int solve_blocks_per_sm_pc<double, false, 3>();
-template int solve_blocks_per_sm_pc<double, true, 3>();
-template cudaError_t launch_refine_pc<float, double, false, 3>(const SysView<float> &, const RefView<double> &,
+template cudaError_t launch_solve_pc<double, kNoIlu, 3>(const SysView<double> &, const SolveCtl &, int, cudaStream_t);
+template cudaError_t launch_solve_pc<double, kIluFlow, 3>(const SysView<double> &, const SolveCtl &, int, cudaStream_t);
+template cudaError_t launch_solve_pc<double, kIluWide, 3>(const SysView<double> &, const SolveCtl &, int, cudaStream_t);
+template int solve_blocks_per_sm_pc<double, kNoIlu, 3>();
+template int solve_blocks_per_sm_pc<double, kIluFlow, 3>();
+template int solve_blocks_per_sm_pc<double, kIluWide, 3>();
+template cudaError_t launch_refine_pc<float, double, kNoIlu, 3>(const SysView<float> &, const RefView<double> &,
                                                                const SolveCtl &, const RefCtl &, int, cudaStream_t);
-template cudaError_t launch_refine_pc<float, double, true, 3>(const SysView<float> &, const RefView<double> &,
+template cudaError_t launch_refine_pc<float, double, kIluFlow, 3>(const SysView<float> &, const RefView<double> &,
                                                               const SolveCtl &, const RefCtl &, int, cudaStream_t);
-template int refine_blocks_per_sm_pc<float, double, false, 3>();
-template int refine_blocks_per_sm_pc<float, double, true, 3>();
+template cudaError_t launch_refine_pc<float, double, kIluWide, 3>(const SysView<float> &, const RefView<double> &,
+                                                              const SolveCtl &, const RefCtl &, int, cudaStream_t);
+template int refine_blocks_per_sm_pc<float, double, kNoIlu, 3>();
+template int refine_blocks_per_sm_pc<float, double, kIluFlow, 3>();
+template int refine_blocks_per_sm_pc<float, double, kIluWide, 3>();
 
 }  // namespace mlb

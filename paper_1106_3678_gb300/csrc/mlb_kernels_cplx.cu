@@ -5,16 +5,16 @@
 
 namespace mlb {
 
-template cudaError_t launch_solve_pc<cdouble, false>(const SysView<cdouble> &, const SolveCtl &, int,
+template cudaError_t launch_solve_pc<cdouble, kNoIlu>(const SysView<cdouble> &, const SolveCtl &, int,
                                                      cudaStream_t);
-template cudaError_t launch_solve_pc<cdouble, true>(const SysView<cdouble> &, const SolveCtl &, int, cudaStream_t);
-template int solve_blocks_per_sm_pc<cdouble, false>();
-template int solve_blocks_per_sm_pc<cdouble, true>();
-template cudaError_t launch_batch_pc<cdouble, false>(const BatchItem<cdouble> *, const BatchPlan &, int,
+template cudaError_t launch_solve_pc<cdouble, kIluAny>(const SysView<cdouble> &, const SolveCtl &, int, cudaStream_t);
+template int solve_blocks_per_sm_pc<cdouble, kNoIlu>();
+template int solve_blocks_per_sm_pc<cdouble, kIluAny>();
+template cudaError_t launch_batch_pc<cdouble, kNoIlu>(const BatchItem<cdouble> *, const BatchPlan &, int,
                                                      cudaStream_t);
-template cudaError_t launch_batch_pc<cdouble, true>(const BatchItem<cdouble> *, const BatchPlan &, int,
+template cudaError_t launch_batch_pc<cdouble, kIluAny>(const BatchItem<cdouble> *, const BatchPlan &, int,
                                                     cudaStream_t);
-template int batch_blocks_per_sm_pc<cdouble, false>();
-template int batch_blocks_per_sm_pc<cdouble, true>();
+template int batch_blocks_per_sm_pc<cdouble, kNoIlu>();
+template int batch_blocks_per_sm_pc<cdouble, kIluAny>();
 
 }  // namespace mlb

@@ -5,21 +5,16 @@
 
 namespace mlb {
 
-template cudaError_t launch_solve_pc<double, true>(const SysView<double> &, const SolveCtl &, int, cudaStream_t);
-template cudaError_t launch_batch_pc<double, true>(const BatchItem<double> *, const BatchPlan &, int, cudaStream_t);
-template int solve_blocks_per_sm_pc<double, true>();
-template int batch_blocks_per_sm_pc<double, true>();
-template cudaError_t launch_refine_pc<float, double, true>(const SysView<float> &, const RefView<double> &,
-                                                           const SolveCtl &, const RefCtl &, int, cudaStream_t);
-template cudaError_t launch_refine_pc<cfloat, cdouble, true>(const SysView<cfloat> &, const RefView<cdouble> &,
+template cudaError_t launch_batch_pc<double, kIluAny>(const BatchItem<double> *, const BatchPlan &, int, cudaStream_t);
+template int batch_blocks_per_sm_pc<double, kIluAny>();
+template cudaError_t launch_refine_pc<cfloat, cdouble, kIluAny>(const SysView<cfloat> &, const RefView<cdouble> &,
                                                              const SolveCtl &, const RefCtl &, int, cudaStream_t);
-template int refine_blocks_per_sm_pc<float, double, true>();
-template int refine_blocks_per_sm_pc<cfloat, cdouble, true>();
-template cudaError_t launch_batch_refine_pc<float, double, true>(const BatchItemR<float, double> *,
+template int refine_blocks_per_sm_pc<cfloat, cdouble, kIluAny>();
+template cudaError_t launch_batch_refine_pc<float, double, kIluAny>(const BatchItemR<float, double> *,
                                                                  const BatchPlan &, int, cudaStream_t);
-template cudaError_t launch_batch_refine_pc<cfloat, cdouble, true>(const BatchItemR<cfloat, cdouble> *,
+template cudaError_t launch_batch_refine_pc<cfloat, cdouble, kIluAny>(const BatchItemR<cfloat, cdouble> *,
                                                                    const BatchPlan &, int, cudaStream_t);
-template int batch_refine_blocks_per_sm_pc<float, double, true>();
-template int batch_refine_blocks_per_sm_pc<cfloat, cdouble, true>();
+template int batch_refine_blocks_per_sm_pc<float, double, kIluAny>();
+template int batch_refine_blocks_per_sm_pc<cfloat, cdouble, kIluAny>();
 
 }  // namespace mlb

@@ -181,7 +181,7 @@ struct RefineOut {
 // Residual replacement of one inner call (see the file comment and
 // Engine::inner).  In shared memory; its state is kept by the engine's
 // kErrThread (thread 0 at the start).
-template <typename T32, typename T64, bool PC, int EW = 1>
+template <typename T32, typename T64, int PC, int EW = 1>
 struct RelUpdate {
     static constexpr bool kActive = true;
     using S = typename coef_of<T32>::type;
@@ -217,7 +217,7 @@ struct RelUpdate {
         Engine<T32, PC, EW> E;
         Refiner<T64, T32, EW> R;
         const T32 *d = the_sys<T32>().x;
-        if constexpr (PC) {
+        if constexpr (PC != kNoIlu) {
             if (the_sys<T32>().ilu.lu) {
                 // the iterate's rows of every CTA are read
                 if (!the_gs().sync() || !E.ilu_solve(the_sys<T32>().x, the_sys<T32>().ilu.t)) return false;
@@ -240,7 +240,7 @@ struct RelUpdate {
 // Outer refinement loop (see the file comment).  ctl.err_hist records the
 // true relative residual at the start of every inner call, and the final
 // one.
-template <typename T32, typename T64, bool PC, int EW = 1>
+template <typename T32, typename T64, int PC, int EW = 1>
 __device__ RefineOut refine_solve(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> &R, const SolveCtl &ctl,
                                   const RefCtl &rc) {
     __shared__ RelUpdate<T32, T64, PC, EW> hk;
@@ -252,6 +252,9 @@ __device__ RefineOut refine_solve(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> 
         if (ctl.err_hist && out.outer < ctl.hist_cap && the_gs().bid == 0 && threadIdx.x == 0)
             ctl.err_hist[out.outer] = err;
     };
+    if constexpr (PC != kNoIlu) {
+        if (the_sys<T32>().ilu.lu && !E.ilu_begin()) return out;
+    }
     for (;;) {
         double bb, rr;
         if (!R.residual(bb, rr)) return out;
@@ -307,7 +310,7 @@ __device__ RefineOut refine_solve(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> 
         if (o.flag == -1 && o.iter == 0) { out.flag = -1; return out; }
         // move what the inner call accumulated since its last update
         const T32 *d = the_sys<T32>().x;
-        if constexpr (PC) {
+        if constexpr (PC != kNoIlu) {
             if (the_sys<T32>().ilu.lu) {
                 if (!the_gs().sync() || !E.ilu_solve(the_sys<T32>().x, the_sys<T32>().ilu.t)) return out;
                 d = the_sys<T32>().ilu.t;

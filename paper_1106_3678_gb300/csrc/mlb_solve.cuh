@@ -1,9 +1,9 @@
-// Persistent solve and batch kernels of the FP64 method, templated on PC:
-// PC = true builds the engine with its ILU(0) preconditioner passes, PC =
-// false without them (no call to them anywhere in the kernel, so the
-// unpreconditioned kernels keep their register allocation).  Included by
-// mlb_kernels.cu (PC = false, and the dispatch) and mlb_kernels_ilu.cu
-// (PC = true), which compile in parallel.
+// Persistent solve and batch kernels of the FP64 method, templated on PC, the
+// forms of the ILU(0) passes that the engine is built with (kNoIlu: no call to
+// them anywhere in the kernel, so the unpreconditioned kernels keep their
+// register allocation).  Included by mlb_kernels.cu (kNoIlu, and the dispatch),
+// mlb_kernels_ilu.cu (kIluAny), mlb_kernels_bsr.cu, mlb_kernels_wide.cu
+// (kIluWide) and mlb_kernels_flow.cu (kIluFlow), which compile in parallel.
 #pragma once
 
 #include "mlb_internal.h"
@@ -19,7 +19,7 @@ namespace mlb {
 // residual did not (restart rule of this library), all iterations counted
 // against one maxit; then the true residual; the team's rank-0 CTA writes
 // the result record.  Consumer threads only.
-template <typename T, bool PC, int EW>
+template <typename T, int PC, int EW>
 __device__ __forceinline__ void run_fp64_solve() {
     Engine<T, PC, EW> E;
     GridSync &gs = the_gs();
@@ -31,8 +31,8 @@ __device__ __forceinline__ void run_fp64_solve() {
     typename Engine<T, PC, EW>::Out o{1, 0, 0, 0, 0.0};
     // ILU(0): the method iterates on y = M x (y_0 = M x_0; x = M^{-1} y at
     // the end, from the final residual pass, which forms M^{-1} y)
-    if constexpr (PC) {
-        if (E.sys().ilu.lu) E.ilu_to_y();
+    if constexpr (PC != kNoIlu) {
+        if (E.sys().ilu.lu && E.ilu_begin()) E.ilu_to_y();
     }
     double true_rel = __longlong_as_double(0x7ff8000000000000LL);
     for (bool last = false; gs.ok;) {
@@ -42,7 +42,7 @@ __device__ __forceinline__ void run_fp64_solve() {
             double bn = sqrt(the_red().total[0]);
             if (bn == 0.0) bn = 1.0;
             true_rel = sqrt(the_red().total[1]) / bn;
-            if constexpr (PC) {
+            if constexpr (PC != kNoIlu) {
                 if (E.sys().ilu.lu) E.ilu_to_x();
             }
             break;
@@ -89,7 +89,7 @@ __device__ __forceinline__ void acct_reset() {
 }
 
 // One FP64 solve by a CTA: its producer warp and its consumer warps.
-template <typename T, bool PC, int EW>
+template <typename T, int PC, int EW>
 __device__ __forceinline__ void run_cta() {
     Engine<T, PC, EW> E;
     E.attach();
@@ -102,7 +102,7 @@ __device__ __forceinline__ void run_cta() {
     __syncthreads();
 }
 
-template <typename T, bool PC, int EW = 1>
+template <typename T, int PC, int EW = 1>
 __global__ void __launch_bounds__(kThreads, 1) solve_kernel(SysView<T> sys, SolveCtl ctl) {
     ring_init(the_ring(), ctl.timeout_ns);
     the_gs().seq() = 0;
@@ -162,7 +162,7 @@ __device__ __forceinline__ void run_batch_plan(const BatchPlan &p, int *sflag, i
 // Each system is solved by the same method as a single solve: by a team
 // (the same arithmetic as a solve with grid = team) or by one CTA alone
 // with CTA-wide barriers and reductions in shared memory.
-template <typename T, bool PC>
+template <typename T, int PC>
 __global__ void __launch_bounds__(kThreads, 1) batch_kernel(const BatchItem<T> *items, BatchPlan plan) {
     __shared__ int sflag;
     __shared__ int s_next;
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kThreads, 1) batch_kernel(const BatchItem<T> *
     ring_drain(the_ring(), the_gs().seqs[kConsumers], the_gs().seqs[0]);
 }
 
-template <typename T, bool PC>
+template <typename T, int PC>
 cudaError_t launch_batch_pc(const BatchItem<T> *items, const BatchPlan &plan, int grid, cudaStream_t st) {
     cudaError_t e = allow_ring((const void *)batch_kernel<T, PC>);
     if (e != cudaSuccess) return e;
@@ -193,7 +193,7 @@ cudaError_t launch_batch_pc(const BatchItem<T> *items, const BatchPlan &plan, in
     return cudaLaunchKernel((const void *)batch_kernel<T, PC>, dim3(grid), dim3(kThreads), args, kRingBytes, st);
 }
 
-template <typename T, bool PC>
+template <typename T, int PC>
 int batch_blocks_per_sm_pc() {
     int nb = 0;
     if (allow_ring((const void *)batch_kernel<T, PC>) != cudaSuccess ||
@@ -202,7 +202,7 @@ int batch_blocks_per_sm_pc() {
     return nb;
 }
 
-template <typename T, bool PC, int EW = 1>
+template <typename T, int PC, int EW = 1>
 cudaError_t launch_solve_pc(const SysView<T> &sys, const SolveCtl &ctl, int grid, cudaStream_t st) {
     SysView<T> s = sys;
     SolveCtl c = ctl;
@@ -216,7 +216,7 @@ cudaError_t launch_solve_pc(const SysView<T> &sys, const SolveCtl &ctl, int grid
                                        kRingBytes, st);
 }
 
-template <typename T, bool PC, int EW = 1>
+template <typename T, int PC, int EW = 1>
 int solve_blocks_per_sm_pc() {
     int nb = 0;
     if (allow_ring((const void *)solve_kernel<T, PC, EW>) != cudaSuccess ||
@@ -231,7 +231,7 @@ int solve_blocks_per_sm_pc() {
 // ===========================================================================
 // One refined solve by a CTA: its producer warp and its consumer warps; the
 // team's rank-0 CTA writes the result record.
-template <typename T32, typename T64, bool PC, int EW>
+template <typename T32, typename T64, int PC, int EW>
 __device__ __forceinline__ void refine_cta() {
     Engine<T32, PC, EW> E;
     Refiner<T64, T32, EW> R;
@@ -266,7 +266,7 @@ __device__ __forceinline__ void refine_cta() {
     __syncthreads();
 }
 
-template <typename T32, typename T64, bool PC>
+template <typename T32, typename T64, int PC>
 __global__ void __launch_bounds__(kThreads, 1)
     batch_refine_kernel(const BatchItemR<T32, T64> *items, BatchPlan plan) {
     __shared__ int sflag;
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     ring_drain(the_ring(), the_gs().seqs[kConsumers], the_gs().seqs[0]);
 }
 
-template <typename T32, typename T64, bool PC>
+template <typename T32, typename T64, int PC>
 cudaError_t launch_batch_refine_pc(const BatchItemR<T32, T64> *items, const BatchPlan &plan, int grid,
                                    cudaStream_t st) {
     cudaError_t e = allow_ring((const void *)batch_refine_kernel<T32, T64, PC>);
@@ -302,7 +302,7 @@ cudaError_t launch_batch_refine_pc(const BatchItemR<T32, T64> *items, const Batc
                             kRingBytes, st);
 }
 
-template <typename T32, typename T64, bool PC>
+template <typename T32, typename T64, int PC>
 int batch_refine_blocks_per_sm_pc() {
     int nb = 0;
     if (allow_ring((const void *)batch_refine_kernel<T32, T64, PC>) != cudaSuccess ||
@@ -315,7 +315,7 @@ int batch_refine_blocks_per_sm_pc() {
 // ===========================================================================
 // FP32-inner / FP64-refined persistent solve kernel
 // ===========================================================================
-template <typename T32, typename T64, bool PC, int EW = 1>
+template <typename T32, typename T64, int PC, int EW = 1>
 __global__ void __launch_bounds__(kThreads, 1)
     refine_kernel(SysView<T32> sys, RefView<T64> rv, SolveCtl ctl, RefCtl rc) {
     ring_init(the_ring(), ctl.timeout_ns);
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     ring_drain(the_ring(), the_gs().seqs[kConsumers], the_gs().seqs[0]);
 }
 
-template <typename T32, typename T64, bool PC, int EW = 1>
+template <typename T32, typename T64, int PC, int EW = 1>
 cudaError_t launch_refine_pc(const SysView<T32> &sys, const RefView<T64> &rv, const SolveCtl &ctl,
                           const RefCtl &rc, int grid, cudaStream_t st) {
     SysView<T32> s = sys;
@@ -349,7 +349,7 @@ cudaError_t launch_refine_pc(const SysView<T32> &sys, const RefView<T64> &rv, co
                                        args, kRingBytes, st);
 }
 
-template <typename T32, typename T64, bool PC, int EW = 1>
+template <typename T32, typename T64, int PC, int EW = 1>
 int refine_blocks_per_sm_pc() {
     int nb = 0;
     if (allow_ring((const void *)refine_kernel<T32, T64, PC, EW>) != cudaSuccess ||
@@ -360,55 +360,75 @@ int refine_blocks_per_sm_pc() {
 }
 
 // 3x3-block storage (real values only), instantiated in mlb_kernels_bsr.cu.
-extern template cudaError_t launch_solve_pc<double, false, 3>(const SysView<double> &, const SolveCtl &, int,
+extern template cudaError_t launch_solve_pc<double, kNoIlu, 3>(const SysView<double> &, const SolveCtl &, int,
                                                               cudaStream_t);
-extern template cudaError_t launch_solve_pc<double, true, 3>(const SysView<double> &, const SolveCtl &, int,
+extern template cudaError_t launch_solve_pc<double, kIluFlow, 3>(const SysView<double> &, const SolveCtl &, int,
                                                              cudaStream_t);
-extern template int solve_blocks_per_sm_pc<double, false, 3>();
-extern template int solve_blocks_per_sm_pc<double, true, 3>();
-extern template cudaError_t launch_refine_pc<float, double, false, 3>(const SysView<float> &,
+extern template cudaError_t launch_solve_pc<double, kIluWide, 3>(const SysView<double> &, const SolveCtl &, int,
+                                                             cudaStream_t);
+extern template int solve_blocks_per_sm_pc<double, kNoIlu, 3>();
+extern template int solve_blocks_per_sm_pc<double, kIluFlow, 3>();
+extern template int solve_blocks_per_sm_pc<double, kIluWide, 3>();
+extern template cudaError_t launch_refine_pc<float, double, kNoIlu, 3>(const SysView<float> &,
                                                                       const RefView<double> &, const SolveCtl &,
                                                                       const RefCtl &, int, cudaStream_t);
-extern template cudaError_t launch_refine_pc<float, double, true, 3>(const SysView<float> &,
+extern template cudaError_t launch_refine_pc<float, double, kIluFlow, 3>(const SysView<float> &,
                                                                      const RefView<double> &, const SolveCtl &,
                                                                      const RefCtl &, int, cudaStream_t);
-extern template int refine_blocks_per_sm_pc<float, double, false, 3>();
-extern template int refine_blocks_per_sm_pc<float, double, true, 3>();
+extern template cudaError_t launch_refine_pc<float, double, kIluWide, 3>(const SysView<float> &,
+                                                                     const RefView<double> &, const SolveCtl &,
+                                                                     const RefCtl &, int, cudaStream_t);
+extern template int refine_blocks_per_sm_pc<float, double, kNoIlu, 3>();
+extern template int refine_blocks_per_sm_pc<float, double, kIluFlow, 3>();
+extern template int refine_blocks_per_sm_pc<float, double, kIluWide, 3>();
 
 // Instantiated in mlb_kernels_ilu.cu.
-extern template cudaError_t launch_refine_pc<float, double, true>(const SysView<float> &, const RefView<double> &,
+extern template cudaError_t launch_refine_pc<float, double, kIluWide>(const SysView<float> &, const RefView<double> &,
                                                                   const SolveCtl &, const RefCtl &, int,
                                                                   cudaStream_t);
-extern template cudaError_t launch_refine_pc<cfloat, cdouble, true>(const SysView<cfloat> &,
+extern template cudaError_t launch_refine_pc<cfloat, cdouble, kIluAny>(const SysView<cfloat> &,
                                                                     const RefView<cdouble> &, const SolveCtl &,
                                                                     const RefCtl &, int, cudaStream_t);
-extern template int refine_blocks_per_sm_pc<float, double, true>();
-extern template int refine_blocks_per_sm_pc<cfloat, cdouble, true>();
-extern template cudaError_t launch_batch_refine_pc<float, double, true>(const BatchItemR<float, double> *,
+extern template cudaError_t launch_refine_pc<cfloat, cdouble, kIluWide>(const SysView<cfloat> &,
+                                                                    const RefView<cdouble> &, const SolveCtl &,
+                                                                    const RefCtl &, int, cudaStream_t);
+extern template int refine_blocks_per_sm_pc<float, double, kIluWide>();
+extern template int refine_blocks_per_sm_pc<cfloat, cdouble, kIluAny>();
+extern template int refine_blocks_per_sm_pc<cfloat, cdouble, kIluWide>();
+extern template cudaError_t launch_batch_refine_pc<float, double, kIluAny>(const BatchItemR<float, double> *,
                                                                         const BatchPlan &, int, cudaStream_t);
-extern template cudaError_t launch_batch_refine_pc<cfloat, cdouble, true>(const BatchItemR<cfloat, cdouble> *,
+extern template cudaError_t launch_batch_refine_pc<cfloat, cdouble, kIluAny>(const BatchItemR<cfloat, cdouble> *,
                                                                           const BatchPlan &, int, cudaStream_t);
-extern template int batch_refine_blocks_per_sm_pc<float, double, true>();
-extern template int batch_refine_blocks_per_sm_pc<cfloat, cdouble, true>();
+extern template int batch_refine_blocks_per_sm_pc<float, double, kIluAny>();
+extern template int batch_refine_blocks_per_sm_pc<cfloat, cdouble, kIluAny>();
 
 // Instantiated in mlb_kernels_cplx.cu.
-extern template cudaError_t launch_solve_pc<cdouble, false>(const SysView<cdouble> &, const SolveCtl &, int,
+extern template cudaError_t launch_solve_pc<cdouble, kNoIlu>(const SysView<cdouble> &, const SolveCtl &, int,
                                                             cudaStream_t);
-extern template int solve_blocks_per_sm_pc<cdouble, false>();
-extern template cudaError_t launch_batch_pc<cdouble, false>(const BatchItem<cdouble> *, const BatchPlan &, int,
+extern template int solve_blocks_per_sm_pc<cdouble, kNoIlu>();
+extern template cudaError_t launch_batch_pc<cdouble, kNoIlu>(const BatchItem<cdouble> *, const BatchPlan &, int,
                                                             cudaStream_t);
-extern template int batch_blocks_per_sm_pc<cdouble, false>();
+extern template int batch_blocks_per_sm_pc<cdouble, kNoIlu>();
 
-extern template cudaError_t launch_solve_pc<double, true>(const SysView<double> &, const SolveCtl &, int, cudaStream_t);
-extern template cudaError_t launch_solve_pc<cdouble, true>(const SysView<cdouble> &, const SolveCtl &, int,
+extern template cudaError_t launch_solve_pc<double, kIluWide>(const SysView<double> &, const SolveCtl &, int, cudaStream_t);
+extern template cudaError_t launch_solve_pc<cdouble, kIluAny>(const SysView<cdouble> &, const SolveCtl &, int,
                                                           cudaStream_t);
-extern template cudaError_t launch_batch_pc<double, true>(const BatchItem<double> *, const BatchPlan &, int,
+extern template cudaError_t launch_batch_pc<double, kIluAny>(const BatchItem<double> *, const BatchPlan &, int,
                                                          cudaStream_t);
-extern template cudaError_t launch_batch_pc<cdouble, true>(const BatchItem<cdouble> *, const BatchPlan &, int,
+extern template cudaError_t launch_batch_pc<cdouble, kIluAny>(const BatchItem<cdouble> *, const BatchPlan &, int,
                                                           cudaStream_t);
-extern template int solve_blocks_per_sm_pc<double, true>();
-extern template int solve_blocks_per_sm_pc<cdouble, true>();
-extern template int batch_blocks_per_sm_pc<double, true>();
-extern template int batch_blocks_per_sm_pc<cdouble, true>();
+extern template int solve_blocks_per_sm_pc<double, kIluWide>();
+extern template int solve_blocks_per_sm_pc<cdouble, kIluAny>();
+extern template int batch_blocks_per_sm_pc<double, kIluAny>();
+extern template int batch_blocks_per_sm_pc<cdouble, kIluAny>();
+
+// Instantiated in mlb_kernels_flow.cu.
+extern template cudaError_t launch_solve_pc<double, kIluFlow>(const SysView<double> &, const SolveCtl &, int,
+                                                              cudaStream_t);
+extern template int solve_blocks_per_sm_pc<double, kIluFlow>();
+extern template cudaError_t launch_refine_pc<float, double, kIluFlow>(const SysView<float> &, const RefView<double> &,
+                                                                      const SolveCtl &, const RefCtl &, int,
+                                                                      cudaStream_t);
+extern template int refine_blocks_per_sm_pc<float, double, kIluFlow>();
 
 }  // namespace mlb

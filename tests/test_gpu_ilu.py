@@ -299,3 +299,50 @@ def test_batch_mixing_preconditioners():
         r1, _ = M.mlbicgstab_solve(h1, b, x1, 1e-10, 4000)
         assert (r.iter, r.flag) == (r1.iter, r1.flag), pc
         np.testing.assert_array_equal(x, x1)
+
+
+def _flow_system(kind):
+    if kind == "chain":                      # every level one row, in one warp or across two
+        N = 1000
+        D = 4.0 * np.eye(N) - np.eye(N, k=-1) - 1.5 * np.eye(N, k=1)
+    elif kind == "dense":                    # rows of up to 33 entries, a chain too (no 3x3 blocks: refused in a batch)
+        D = W.random_dense_system(34, seed=71)[1]
+    elif kind == "scattered":                # rows around the 4 entries held in registers
+        return _random_sparse(997, 0.008, seed=72)[0]
+    else:
+        return W.cd3d_lognormal(13)          # 2197 rows: the last positions fill no warp
+    return W.dense_to_csr(D)
+
+
+@pytest.mark.parametrize("kind", ["chain", "dense", "scattered", "stencil"])
+@pytest.mark.parametrize("refined", [False, True])
+def test_ilu_slots_equal_levels_with_barriers(kind, refined):
+    """A single solve passes a row's value to the rows that need it through
+    tagged slots; a batch takes the levels one by one with barriers.  Each row
+    is the same sum, so on one CTA the results are the same bits; over several
+    CTAs (warps with no row, and with many) the solutions agree within the
+    forward error of two residuals below tol."""
+    A = _flow_system(kind)
+    N = A.n_rows
+    opt = dict(n=3, q_seed=0, precond=ILU, precision=M.MLB_PREC_FP32_REFINED if refined else M.MLB_PREC_FP64)
+    b = W.uniform_rhs(N, seed=73)
+    xb = np.zeros(N)
+    hb = M.mlbicgstab_create(A, **opt)
+    rb = M.mlbicgstab_solve_batch([hb], [b], [xb], [1e-10], [2000])[0]
+    assert rb.flag == 0 and rb.true_relres < 1e-10
+    D = np.zeros((N, N))
+    D[np.repeat(np.arange(N), np.diff(A.row_ptr)), A.col] = A.val
+    cond = np.linalg.cond(D)
+    for grid in (1, 2, 7, 152):
+        h = M.mlbicgstab_create(A, grid=grid, **opt)
+        for _ in range(2):
+            x = np.zeros(N)
+            r, _ = M.mlbicgstab_solve(h, b, x, 1e-10, 2000)
+            assert r.flag == 0 and r.true_relres < 1e-10
+            if grid == 1:
+                assert (r.iter, r.outer) == (rb.iter, rb.outer)
+                np.testing.assert_array_equal(x, xb)
+            else:
+                assert np.linalg.norm(x - xb) <= cond * 2e-10 * np.linalg.norm(xb)
+        h.destroy()
+    hb.destroy()
