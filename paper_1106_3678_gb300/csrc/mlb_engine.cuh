@@ -59,7 +59,6 @@ constexpr int kMaxSums = 5;     // doubles reduced per pass (max)
 struct RedScratch {
     double part[kMaxSums][kConsumers / 2];
     double total[kMaxSums];
-    int fail;
 };
 
 // Result record written by CTA 0 at the end of a solve.
@@ -573,7 +572,6 @@ struct GridSync {
         epoch = bepoch = fepoch = 0;
         ok = !the_ring()->failed;
         the_ring()->timeout_ns = to;
-        the_red().fail = 0;
     }
 
     // Slots of sum k of the exchange `ep`.  Two halves suffice: a CTA
@@ -583,13 +581,15 @@ struct GridSync {
         return slots + ((size_t)(ep & 1u) * kMaxSums + k) * nblocks;
     }
 
-    // The last levels of reduce(), by one warp.
-    __device__ __forceinline__ void team_total(int k, bool fence) {
+    // The last levels of reduce(), by one warp; false (uniformly in the warp)
+    // when the wait failed.
+    __device__ __forceinline__ bool team_total(int k, bool fence) {
         const int lane = threadIdx.x & 31;
         const double *p = the_red().part[k] + lane;
         double t = p[0] + p[32];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        bool got = true;
         if (nblocks > 1) {
             const unsigned ep = epoch + 1;
             Slot *const q = slot_of(ep, k);
@@ -597,11 +597,11 @@ struct GridSync {
                 if (fence) fence_acq_rel_gpu();   // this CTA's writes before its slot
                 slot_put(q + bid, t, ep);
             }
-            const bool got = slots_sum(q, nblocks, ep, bar, timeout_ns, t);
+            got = slots_sum(q, nblocks, ep, bar, timeout_ns, t);
             if (fence) fence_acq_rel_gpu();       // the other CTAs' writes after their slots
-            if (!got && lane == 0) the_red().fail = 1;
         }
         if (lane == 0) the_red().total[k] = t;
+        return got;
     }
 
     // Sum K values over the team into the_red().total[0, K), the same bits in
@@ -620,7 +620,8 @@ struct GridSync {
     // Fixed order for a given team size: deterministic.
     // fence: what any CTA of the team wrote before is visible to all of them
     // after (needed before a pass that gathers; the streaming passes read
-    // their own CTA's rows only).  False (uniformly) when a wait failed.
+    // their own CTA's rows only).  False (uniformly) when a wait failed, here
+    // or at a tile of the ring.
     __device__ __forceinline__ bool reduce_k(const double (&v)[kMaxSums], int K, bool fence) {
         static_assert(kMaxSums <= kConsumerWarps && kConsumers == 480, "reduction layout");
         constexpr int G1 = 64;
@@ -640,10 +641,9 @@ struct GridSync {
             p[0] = (a0 + a1) + (tid % G1 < 48 ? a2 + p[3 * G1] : a2);   // only this task reads slot 0
         }
         consumer_sync();
-        if (warp < K) team_total(warp, fence);
-        consumer_sync();
+        const bool lost = warp < K && !team_total(warp, fence);
+        if (consumer_any(lost || the_ring()->failed)) { ok = false; return false; }
         if (tid == 0) epoch += 1;   // read again only after another barrier
-        if (the_red().fail) { ok = false; return false; }
         return true;
     }
     // The same for the passes outside the iteration (one copy of the code).
@@ -659,24 +659,25 @@ struct GridSync {
 
     // Team barrier (a counter: cheaper than an exchange where no value goes
     // with it).
-    __device__ __forceinline__ bool sync() {
+    // lost: a wait of this thread's own failed.
+    __device__ __forceinline__ bool sync(bool lost = false) {
         arrive();
-        return wait();
+        return wait(lost);
     }
 
     // sync() in two halves: arrive() once this CTA's writes are done,
     // wait() before reading other CTAs' writes; work between the two that
     // reads nothing written in this step overlaps the wait.  wait() returns
-    // false (uniformly) when the barrier failed.
+    // false (uniformly) when a wait failed.  A CTA alone needs wait()'s
+    // barrier only.
     __device__ __forceinline__ void arrive() {
+        if (nblocks == 1) return;
         consumer_sync();
-        if (nblocks > 1 && threadIdx.x == 0) grid_arrive(bar, bepoch);
+        if (threadIdx.x == 0) grid_arrive(bar, bepoch);
     }
-    __device__ __forceinline__ bool wait() {
-        if (nblocks == 1) return true;   // arrive()'s barrier ordered the CTA
-        if (threadIdx.x == 0 && !grid_wait(bar, bepoch, nblocks, timeout_ns)) the_red().fail = 1;
-        consumer_sync();
-        if (the_red().fail) { ok = false; return false; }
+    __device__ __forceinline__ bool wait(bool lost = false) {
+        if (nblocks > 1 && threadIdx.x == 0 && !grid_wait(bar, bepoch, nblocks, timeout_ns)) lost = true;
+        if (consumer_any(lost || the_ring()->failed)) { ok = false; return false; }
         return true;
     }
 
@@ -967,25 +968,13 @@ struct Engine {
     // ------------------------------------------------------------------
 
     // Streaming pass through the tile pipeline: fn(chunk, stage, k) for
-    // every chunk of this CTA.
+    // every chunk of this CTA.  A failed tile wait marks the ring; the pass's
+    // reduction or barrier then reports it.
     template <typename Fn>
     __device__ __forceinline__ void tiles(int tc, unsigned &sq, Fn fn) {
         TileRing *const ring = the_ring();
         if (!consume(ring, TileGeom{tc, c_lo(), c_hi()}, sq, fn)) ring->failed = 1;
         pass_done(ring);
-    }
-    template <int K>
-    __device__ __forceinline__ bool reduce(const ACC (&acc)[K], bool fence) {
-        double v[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] = (double)acc[k];
-        return gs().template reduce<K>(v, fence) && ring_ok();
-    }
-    // A failed tile wait marks the ring; the pass's reduction or barrier
-    // then reports it.
-    __device__ __forceinline__ bool ring_ok() {
-        if (the_ring()->failed) { gs().ok = false; return false; }
-        return true;
     }
 
     // SELL-32 SpMV pass over the owned slices (matrix tiles through the
@@ -1213,8 +1202,7 @@ struct Engine {
                     }
                 }
             }
-            if (!ok) the_red().fail = 1;
-            const bool good = gs().sync();
+            const bool good = gs().sync(!ok);
             if (threadIdx.x == 0) gs().fepoch = ep;   // read again only after another barrier
             ilu_count();
             return good;
@@ -1415,7 +1403,7 @@ struct Engine {
                 t = t1;
             }
             if (!ok) R->failed = 1;
-            if (!gs().sync() || !ring_ok()) return false;
+            if (!gs().sync()) return false;
         }
         gs().seq() = q;
         ilu_count();
@@ -1980,7 +1968,7 @@ struct Engine {
                 ph_g(sc().coef, i, more, sq, sums);
                 break;
             }
-            good = (sums.K ? gs().reduce_k(sums.v, sums.K, sums.fence) : gs().sync()) && good && ring_ok();
+            good = (sums.K ? gs().reduce_k(sums.v, sums.K, sums.fence) : gs().sync()) && good;
             // the scalars of the next pass, the stopping rule and the
             // accounting, each on a thread of its own warp
             if (tid == 0) {

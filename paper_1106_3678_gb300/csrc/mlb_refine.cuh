@@ -110,7 +110,6 @@ struct Refiner {
         if (!okt) the_ring()->failed = 1;
         pass_done(the_ring());
         if (!gs().template reduce<2>(acc, true)) return false;
-        if (the_ring()->failed) { gs().ok = false; return false; }
         bb = the_red().total[0];
         rr = the_red().total[1];
         if (threadIdx.x == kAcctThread) {

@@ -166,6 +166,17 @@ __device__ __forceinline__ void ring_init(TileRing *R, uint64_t timeout_ns) {
 __device__ __forceinline__ void consumer_sync() {
     asm volatile("bar.sync 1, %0;" ::"n"(kConsumers) : "memory");
 }
+// The same, and whether `v` holds for any of them: one answer for all, so
+// that what some thread or the producer found out on its own, at a moment of
+// its own, turns every consumer the same way.
+__device__ __forceinline__ bool consumer_any(bool v) {
+    int r;
+    asm volatile("{ .reg .pred p, q; setp.ne.s32 q, %1, 0; bar.red.or.pred p, 1, %2, q; selp.s32 %0, 1, 0, p; }"
+                 : "=r"(r)
+                 : "r"((int)v), "n"(kConsumers)
+                 : "memory");
+    return r != 0;
+}
 
 // Bounded wait for the phase with parity `phase` of a barrier of the ring
 // to complete.
