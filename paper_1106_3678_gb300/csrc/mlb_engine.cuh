@@ -682,22 +682,20 @@ struct GridSync {
     }
 
     // Hand a command to the producer warp (every consumer thread calls it).
+    // Stop and exit also call it out of its waits.
     __device__ __forceinline__ void post(int cmd) {
         if (threadIdx.x == 0) {
             the_ring()->cmd = cmd;
-            the_ring()->stop = 0;
+            *(volatile int *)&the_ring()->stop = cmd == kCmdStop || cmd == kCmdExit;
         }
         __syncthreads();
     }
-    // End of an iteration: stop the producer, meet it, and discard the tiles
-    // it has issued ahead (their stages are released as if consumed).
+    // End of an iteration: stop the producer, and discard the tiles it has
+    // issued ahead (their stages are released as if consumed).
     // `passes`: passes this CTA's consumers have finished.
     __device__ __forceinline__ void end_inner(unsigned &sq, unsigned passes) {
-        if (threadIdx.x == 0) {
-            *(volatile int *)&the_ring()->stop = 1;
-            the_ring()->passes = passes;
-        }
-        __syncthreads();
+        if (threadIdx.x == 0) the_ring()->passes = passes;
+        post(kCmdStop);
         for (const unsigned last = the_ring()->issued; sq != last; ++sq) {
             if (!mbar_wait(the_ring(), &the_ring()->full[sq % kStages], (sq / kStages) & 1u)) {
                 the_ring()->failed = 1;
@@ -792,6 +790,7 @@ struct Engine {
             own_range(sys().nslices, gs().nblocks, gs().bid, lo, hi);
             the_iter<S>().s_lo = (int)lo;
             the_iter<S>().s_hi = (int)hi;
+            the_ring()->stop = 0;
         }
         __syncthreads();
         soff_load(the_ring(), sys().slice_ptr, s_lo(), s_hi());
@@ -903,17 +902,30 @@ struct Engine {
         if (st == 0) passes += 1;
         return st;
     }
+    // Meet the consumers: their next command.  `sq`: tiles issued so far.
+    __device__ __forceinline__ int command(unsigned sq, unsigned &passes) {
+        TileRing *const R = the_ring();
+        if ((threadIdx.x & 31) == 0) R->issued = sq;
+        __syncthreads();
+        const int cmd = R->cmd;
+        // the consumers may have finished a pass that this side did not wait for
+        if (cmd == kCmdStop) passes = R->passes;
+        return cmd;
+    }
     // The producer warp's side of a system: commands of the consumers until
     // kCmdExit.  Decide: the iteration asks the consumers after every update
     // of r (refined mode).  residual64 issues the FP64 residual's tiles.
+    // After a timeout it only takes commands: the consumers find the ring
+    // marked as failed and end the solve.
     template <bool Decide, typename Fn>
     __device__ __forceinline__ void serve(Fn residual64) {
         TileRing *const R = the_ring();
         unsigned sq = gs().seq(), passes = R->passes;
+        bool dead = false;
         for (;;) {
-            __syncthreads();
-            const int cmd = R->cmd;
+            const int cmd = command(sq, passes);
             if (cmd == kCmdExit) break;
+            if (dead || cmd == kCmdStop) continue;
             int st = 0;
             if (cmd == kCmdResidual) {
                 st = issue_ilu(sq);
@@ -926,38 +938,33 @@ struct Engine {
                 st = issue_ilu(sq);
             } else {
                 const int n = sys().n;
-                bool met = false;   // the consumers' end_inner has been met at a decision
-                for (Step p; st == 0; p.advance(n)) {
+                bool over = false;   // ended by a command
+                for (Step p; st == 0 && !over; p.advance(n)) {
                     st = issue(p, sq);
                     if (st == 0) st = wait_done(passes);
                     if constexpr (Decide) {
                         // the consumers' commands (a residual replacement)
                         // until they let the iteration go on or end it
                         while (st == 0 && (p.op == P_ALPHA || p.op == P_OMEGA)) {
-                            if ((threadIdx.x & 31) == 0) R->issued = sq;
-                            __syncthreads();
-                            met = R->stop != 0;
-                            if (met || R->cmd == kCmdGo) break;
-                            if (R->cmd == kCmdIlu) {
+                            const int c = command(sq, passes);
+                            over = c == kCmdStop;
+                            if (over || c == kCmdGo) break;
+                            if (c == kCmdIlu) {
                                 st = issue_ilu(sq);
                             } else {
                                 st = residual64(sq);
                                 if (st == 0) st = wait_done(passes);
                             }
                         }
-                        if (met) break;
                     }
                 }
-                if (st == 2) R->failed = 1;
-                if (!met) {
-                    if ((threadIdx.x & 31) == 0) R->issued = sq;
-                    __syncthreads();
-                }
-                passes = R->passes;
-                continue;
             }
-            if (st == 2) R->failed = 1;
-            if ((threadIdx.x & 31) == 0) R->passes = passes;
+            if (st == 2) {
+                R->failed = 1;
+                dead = true;
+            }
+            // an iteration's count comes from the consumers
+            if (cmd != kCmdInner && (threadIdx.x & 31) == 0) R->passes = passes;
         }
         gs().seq() = sq;
         if ((threadIdx.x & 31) == 0) R->passes = passes;

@@ -106,10 +106,13 @@ __device__ __forceinline__ int32_t *the_soff() {
     return reinterpret_cast<int32_t *>(the_stages() + (size_t)kStages * kStageBytes);
 }
 
-// Commands of the consumers to the producer warp (TileRing::cmd), handed
-// over by a __syncthreads of the whole CTA.
+// Commands of the consumers to the producer warp (TileRing::cmd).  Every
+// __syncthreads of the whole CTA within a system hands one over, so the two
+// sides never take one meeting for another: a producer that has given up
+// meets the consumers for each command and issues nothing.
 enum {
     kCmdExit,        // this system is done
+    kCmdStop,        // the iteration ended
     kCmdResidual,    // one residual pass of the engine (with ILU(0), M^{-1} x first)
     kCmdResidual64,  // one residual pass of the refined mode's FP64 side
     kCmdIlu,         // (refined mode) the tiles of one M^{-1}
@@ -125,10 +128,10 @@ struct TileRing {
     uint64_t done;           // completed passes (one arrival per consumer warp)
     uint64_t timeout_ns;     // limit of every wait
     unsigned issued;         // tiles issued (written by the producer where both sides meet)
-    unsigned consumed;       // tiles and passes consumed (written by the consumers there)
-    unsigned passes;
+    unsigned consumed;       // tiles consumed (written by the consumers there)
+    unsigned passes;         // passes finished, where both sides meet
     int cmd;
-    int stop;                // the iteration ended: the producer returns from its waits
+    int stop;                // the producer returns from its waits, to the next command
     int failed;              // set when a wait timed out
     // Cache of the SELL-32 slice offsets of this CTA's slice range:
     // the_soff()[i] = slice_ptr[soff_lo + i] - soff_base for i = 0..soff_hi-soff_lo
@@ -189,14 +192,14 @@ __device__ __forceinline__ bool mbar_wait(TileRing *R, uint64_t *b, unsigned pha
     }
 }
 // Bounded wait of the producer's lane 0: 0 when the phase completed, 1 when
-// the consumers ended the iteration, 2 on a timeout.  Twice the consumers'
+// the consumers called it off, 2 on a timeout.  Twice the consumers'
 // limit, so that a wait of theirs that gives up is reported as such.
 __device__ __forceinline__ int producer_wait(TileRing *R, uint64_t *b, unsigned phase) {
     if (mbar_probe(b, phase)) return 0;
     const uint64_t t0 = globaltimer_ns();
     for (unsigned it = 1;; ++it) {
         if (mbar_probe(b, phase)) return 0;
-        if (*(volatile int *)&R->stop) return 1;
+        if (*(volatile int *)&R->stop) return mbar_probe(b, phase) ? 0 : 1;
         if ((it & 63u) == 0 && globaltimer_ns() - t0 > 2 * R->timeout_ns) return 2;
     }
 }
