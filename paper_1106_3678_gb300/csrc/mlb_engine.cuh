@@ -102,7 +102,6 @@ struct Scalars {
     double err;      // ||r|| / ||b|| where it was worked out
     double tol;
     int64_t iter, maxit;
-    unsigned passes; // passes the consumers have finished (thread 0)
     int rec;         // the residual history is recorded
     int block;       // j of the running block (thread kErrThread)
     int exit;        // the iteration ends
@@ -682,9 +681,12 @@ struct GridSync {
     }
 
     // Hand a command to the producer warp (every consumer thread calls it).
-    // Stop and exit also call it out of its waits.
-    __device__ __forceinline__ void post(int cmd) {
+    // Stop and exit also call it out of its waits.  The last command and the
+    // call that came with it are only replaced once the producer has taken
+    // them.
+    __device__ __forceinline__ void post(unsigned cmd) {
         if (threadIdx.x == 0) {
+            await_producer(the_ring(), &the_ring()->cmd, kCmdNone);
             the_ring()->cmd = cmd;
             *(volatile int *)&the_ring()->stop = cmd == kCmdStop || cmd == kCmdExit;
         }
@@ -692,9 +694,7 @@ struct GridSync {
     }
     // End of an iteration: stop the producer, and discard the tiles it has
     // issued ahead (their stages are released as if consumed).
-    // `passes`: passes this CTA's consumers have finished.
-    __device__ __forceinline__ void end_inner(unsigned &sq, unsigned passes) {
-        if (threadIdx.x == 0) the_ring()->passes = passes;
+    __device__ __forceinline__ void end_inner(unsigned &sq) {
         post(kCmdStop);
         for (const unsigned last = the_ring()->issued; sq != last; ++sq) {
             if (!mbar_wait(the_ring(), &the_ring()->full[sq % kStages], (sq / kStages) & 1u)) {
@@ -899,17 +899,26 @@ struct Engine {
         int st = 0;
         if ((threadIdx.x & 31) == 0) st = producer_wait(the_ring(), &the_ring()->done, passes & 1u);
         st = __shfl_sync(0xffffffffu, st, 0);
-        if (st == 0) passes += 1;
+        if (st == 0) saw(++passes);
         return st;
     }
+    __device__ __forceinline__ static void saw(unsigned passes) {
+        if ((threadIdx.x & 31) == 0) *(volatile unsigned *)&the_ring()->seen = passes;
+    }
     // Meet the consumers: their next command.  `sq`: tiles issued so far.
-    __device__ __forceinline__ int command(unsigned sq, unsigned &passes) {
+    __device__ __forceinline__ unsigned command(unsigned sq, unsigned &passes) {
         TileRing *const R = the_ring();
         if ((threadIdx.x & 31) == 0) R->issued = sq;
         __syncthreads();
-        const int cmd = R->cmd;
-        // the consumers may have finished a pass that this side did not wait for
-        if (cmd == kCmdStop) passes = R->passes;
+        const unsigned cmd = *(volatile unsigned *)&R->cmd;
+        if (cmd == kCmdStop) {
+            // the consumers may have finished a pass that this side did not
+            // wait for
+            passes = *(volatile unsigned *)&R->finished;
+            saw(passes);
+        }
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) *(volatile unsigned *)&R->cmd = kCmdNone;
         return cmd;
     }
     // The producer warp's side of a system: commands of the consumers until
@@ -920,10 +929,10 @@ struct Engine {
     template <bool Decide, typename Fn>
     __device__ __forceinline__ void serve(Fn residual64) {
         TileRing *const R = the_ring();
-        unsigned sq = gs().seq(), passes = R->passes;
+        unsigned sq = gs().seq(), passes = R->seen;
         bool dead = false;
         for (;;) {
-            const int cmd = command(sq, passes);
+            const unsigned cmd = command(sq, passes);
             if (cmd == kCmdExit) break;
             if (dead || cmd == kCmdStop) continue;
             int st = 0;
@@ -946,7 +955,7 @@ struct Engine {
                         // the consumers' commands (a residual replacement)
                         // until they let the iteration go on or end it
                         while (st == 0 && (p.op == P_ALPHA || p.op == P_OMEGA)) {
-                            const int c = command(sq, passes);
+                            const unsigned c = command(sq, passes);
                             over = c == kCmdStop;
                             if (over || c == kCmdGo) break;
                             if (c == kCmdIlu) {
@@ -963,11 +972,8 @@ struct Engine {
                 R->failed = 1;
                 dead = true;
             }
-            // an iteration's count comes from the consumers
-            if (cmd != kCmdInner && (threadIdx.x & 31) == 0) R->passes = passes;
         }
         gs().seq() = sq;
-        if ((threadIdx.x & 31) == 0) R->passes = passes;
     }
 
     // ------------------------------------------------------------------
@@ -1923,7 +1929,7 @@ struct Engine {
                 o.flag = sc().flag;
                 return o;
             }
-            begin_inner();
+            gs().post(kCmdInner);   // from the product w_0 = A g_0 on
         } else {
             // r_0 = b - A x_0 (step 2) with the stopping-rule denominator
             st.op = P_RESIDUAL;
@@ -2045,7 +2051,6 @@ struct Engine {
                 if (st.op == P_OMEGA) sc().inv_omega = recip(sc().omega);
                 if (!last) count(st, n);
             }
-            if (tid == 0) sc().passes += 1;
             consumer_sync();
             if (st.op == P_RESIDUAL) {
                 if (!good || last || sc().exit) {
@@ -2056,7 +2061,7 @@ struct Engine {
                     }
                     return o;
                 }
-                begin_inner();
+                gs().post(kCmdInner);   // from the product w_0 = A g_0 on
                 continue;
             }
             if (!good) break;
@@ -2076,7 +2081,6 @@ struct Engine {
                         bool conv;
                         good = hook->replace(st.op == P_OMEGA ? 0 : hq ? i : -1, f1, rr, qr, fr, conv);
                         sq = gs().seq();
-                        if (tid == 0) sc().passes += 1;
                         if (!good) break;
                         if (tid == kErrThread) replaced<Hook>(rr, conv, st.op, whole, hook);
                         if (tid == 0 && whole) {
@@ -2093,7 +2097,7 @@ struct Engine {
             if (st.op == P_ALPHA && hq) op(OP_DOT);
             if (st.op == P_OMEGA) op(OP_DOT);
         }
-        gs().end_inner(sq, sc().passes);
+        gs().end_inner(sq);
         gs().seq() = sq;
         o.flag = gs().ok ? sc().flag : 1;
         o.iter = sc().iter;
@@ -2125,11 +2129,6 @@ struct Engine {
             sc().flag = 0;
             sc().exit = 1;
         }
-    }
-    // The producer's first step is the product w_0 = A g_0.
-    __device__ __forceinline__ void begin_inner() {
-        gs().post(kCmdInner);
-        if (threadIdx.x == 0) sc().passes = the_ring()->passes;
     }
     // Thread kAcctThread: the operations of a pass that are counted before
     // its exits.

@@ -111,6 +111,7 @@ __device__ __forceinline__ int32_t *the_soff() {
 // sides never take one meeting for another: a producer that has given up
 // meets the consumers for each command and issues nothing.
 enum {
+    kCmdNone,        // the producer has taken the last command
     kCmdExit,        // this system is done
     kCmdStop,        // the iteration ended
     kCmdResidual,    // one residual pass of the engine (with ILU(0), M^{-1} x first)
@@ -129,8 +130,9 @@ struct TileRing {
     uint64_t timeout_ns;     // limit of every wait
     unsigned issued;         // tiles issued (written by the producer where both sides meet)
     unsigned consumed;       // tiles consumed (written by the consumers there)
-    unsigned passes;         // passes finished, where both sides meet
-    int cmd;
+    unsigned finished;       // passes the consumers have finished (their thread 0)
+    unsigned seen;           // passes the producer has seen the end of
+    unsigned cmd;
     int stop;                // the producer returns from its waits, to the next command
     int failed;              // set when a wait timed out
     // Cache of the SELL-32 slice offsets of this CTA's slice range:
@@ -158,7 +160,8 @@ __device__ __forceinline__ void ring_init(TileRing *R, uint64_t timeout_ns) {
         R->timeout_ns = timeout_ns;
         R->failed = 0;
         R->stop = 0;
-        R->passes = 0;
+        R->finished = R->seen = 0;
+        R->cmd = kCmdNone;
         R->soff_src = nullptr;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -335,11 +338,32 @@ __device__ __forceinline__ bool consume(TileRing *R, const TileGeom g, unsigned 
     return true;
 }
 
+// Consumer thread 0 waits (bounded) until the producer has written `want` to
+// a word of the ring.
+__device__ __forceinline__ void await_producer(TileRing *R, const unsigned *word, unsigned want) {
+    if (*(const volatile unsigned *)word == want) return;
+    const uint64_t t0 = globaltimer_ns();
+    while (*(const volatile unsigned *)word != want)
+        if (globaltimer_ns() - t0 > R->timeout_ns) {
+            R->failed = 1;
+            return;
+        }
+}
 // End of a consumer's part of a pass in the solve kernels (its stores are
-// fenced for the async proxy): the producer may start the next pass.
+// fenced for the async proxy): the producer may start the next pass.  A
+// phase of "done" is told by its parity, so a pass is only reported once the
+// producer has seen the one before.  Where a pass has tiles the consumers
+// could not have got that far; a CTA without rows, or a product whose rows
+// are too wide for a tile, has none.
 __device__ __forceinline__ void pass_done(TileRing *R) {
     __syncwarp();
-    if ((threadIdx.x & 31) == 0) mbar_arrive(&R->done);
+    if ((threadIdx.x & 31) == 0) {
+        if (threadIdx.x == 0) {
+            await_producer(R, &R->seen, R->finished);
+            R->finished += 1;
+        }
+        mbar_arrive(&R->done);
+    }
 }
 
 // Producer warp (all 32 lanes): issue every tile of a streaming pass over
