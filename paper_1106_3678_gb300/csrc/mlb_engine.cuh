@@ -697,7 +697,7 @@ struct GridSync {
     __device__ __forceinline__ void end_inner(unsigned &sq) {
         post(kCmdStop);
         for (const unsigned last = the_ring()->issued; sq != last; ++sq) {
-            if (!mbar_wait(the_ring(), &the_ring()->full[sq % kStages], (sq / kStages) & 1u)) {
+            if (!mbar_wait_for(&the_ring()->full[sq % kStages], (sq / kStages) & 1u, kLandNs)) {
                 the_ring()->failed = 1;
                 ok = false;
                 break;

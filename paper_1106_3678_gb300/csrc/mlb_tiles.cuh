@@ -186,14 +186,21 @@ __device__ __forceinline__ bool consumer_any(bool v) {
 
 // Bounded wait for the phase with parity `phase` of a barrier of the ring
 // to complete.
-__device__ __forceinline__ bool mbar_wait(TileRing *R, uint64_t *b, unsigned phase) {
+__device__ __forceinline__ bool mbar_wait_for(uint64_t *b, unsigned phase, uint64_t limit_ns) {
     if (mbar_test(b, phase)) return true;
     const uint64_t t0 = globaltimer_ns();
     for (unsigned it = 1;; ++it) {
         if (mbar_test(b, phase)) return true;
-        if ((it & 15u) == 0 && globaltimer_ns() - t0 > R->timeout_ns) return false;
+        if ((it & 15u) == 0 && globaltimer_ns() - t0 > limit_ns) return false;
     }
 }
+__device__ __forceinline__ bool mbar_wait(TileRing *R, uint64_t *b, unsigned phase) {
+    return mbar_wait_for(b, phase, R->timeout_ns);
+}
+// Limit of the waits for copies that are under way when a solve or a kernel
+// ends.  Not the solve's own: that one may be as short as the caller likes,
+// and a CTA must not give its shared memory back while a copy writes into it.
+constexpr uint64_t kLandNs = 2000000000ull;
 // Bounded wait of the producer's lane 0: 0 when the phase completed, 1 when
 // the consumers called it off, 2 on a timeout.  Twice the consumers'
 // limit, so that a wait of theirs that gives up is reported as such.
@@ -470,7 +477,7 @@ __device__ __forceinline__ void ring_drain(TileRing *R, unsigned pseq, unsigned 
     __syncthreads();
     if (threadIdx.x == 0) {
         for (unsigned q = R->consumed; q < R->issued; ++q)
-            if (!mbar_wait(R, &R->full[q % kStages], (q / kStages) & 1u)) break;
+            if (!mbar_wait_for(&R->full[q % kStages], (q / kStages) & 1u, kLandNs)) break;
     }
     __syncthreads();
 }
