@@ -402,7 +402,7 @@ __device__ __forceinline__ bool sell_consume(TileRing *R, unsigned &cseq, int s_
         j.st = (int)(q % kStages);
         j.o = j.nv = 0;
         j.w = -1;
-        if (!mbar_wait(R, &R->full[j.st], (q / kStages) & 1u)) return false;
+        if (!mbar_wait_warp(&R->full[j.st], (q / kStages) & 1u, R->timeout_ns)) return false;
         const int s1 = s0 + spt < s_hi ? s0 + spt : s_hi, s = s0 + cw;
         if (s < s1) {
             j.nv = span(s0, s1);
@@ -697,7 +697,7 @@ struct GridSync {
     __device__ __forceinline__ void end_inner(unsigned &sq) {
         post(kCmdStop);
         for (const unsigned last = the_ring()->issued; sq != last; ++sq) {
-            if (!mbar_wait_for(&the_ring()->full[sq % kStages], (sq / kStages) & 1u, kLandNs)) {
+            if (!mbar_wait_warp(&the_ring()->full[sq % kStages], (sq / kStages) & 1u, kLandNs)) {
                 the_ring()->failed = 1;
                 ok = false;
                 break;
@@ -1347,7 +1347,7 @@ struct Engine {
             auto arrived = [&](int k, unsigned tile, int &stage, int &slices) {
                 stage = (int)(tile % kStages);
                 slices = k1 - k < spt ? k1 - k : spt;
-                return mbar_wait(R, &R->full[stage], (tile / kStages) & 1u);
+                return mbar_wait_warp(&R->full[stage], (tile / kStages) & 1u, R->timeout_ns);
             };
             auto vals = [&](int stage) {
                 return reinterpret_cast<const T *>(the_stages() + stage * kStageBytes) + cw * 32 * w + lane;

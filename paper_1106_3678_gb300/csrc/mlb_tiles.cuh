@@ -197,6 +197,17 @@ __device__ __forceinline__ bool mbar_wait_for(uint64_t *b, unsigned phase, uint6
 __device__ __forceinline__ bool mbar_wait(TileRing *R, uint64_t *b, unsigned phase) {
     return mbar_wait_for(b, phase, R->timeout_ns);
 }
+// The same by a whole warp: all of its lanes go on or give up together (lanes
+// that gave up at different polls would wait for each other at the warp's
+// next barriers).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *b, unsigned phase, uint64_t limit_ns) {
+    if (__all_sync(0xffffffffu, mbar_test(b, phase))) return true;
+    const uint64_t t0 = globaltimer_ns();
+    for (unsigned it = 1;; ++it) {
+        if (__all_sync(0xffffffffu, mbar_test(b, phase))) return true;
+        if ((it & 15u) == 0 && __any_sync(0xffffffffu, globaltimer_ns() - t0 > limit_ns)) return false;
+    }
+}
 // Limit of the waits for copies that are under way when a solve or a kernel
 // ends.  Not the solve's own: that one may be as short as the caller likes,
 // and a CTA must not give its shared memory back while a copy writes into it.
@@ -328,7 +339,7 @@ __device__ __forceinline__ bool consume(TileRing *R, const TileGeom g, unsigned 
     for (int t = 0; t < nt; ++t, ++sq) {
         const int s = (int)(sq % kStages);
         const unsigned use = sq / kStages;
-        if (!mbar_wait(R, &R->full[s], use & 1u)) {
+        if (!mbar_wait_warp(&R->full[s], use & 1u, R->timeout_ns)) {
             seq = sq;
             return false;
         }
