@@ -59,6 +59,12 @@ constexpr int kMaxSums = 5;     // doubles reduced per pass (max)
 struct RedScratch {
     double part[kMaxSums][kConsumers / 2];
     double total[kMaxSums];
+    // Whether a wait failed: written before the last barrier of a reduction
+    // or a team barrier, read after it, so that every consumer takes the same
+    // turn.  (The flag of the ring may be set at any time.)  A writer must
+    // find every reader of the barrier before gone: team barriers with no
+    // other barrier between them alternate between the two.
+    int lost[2];
 };
 
 // Result record written by CTA 0 at the end of a solve.
@@ -77,6 +83,10 @@ enum { OP_MATVEC = 0, OP_DOT = 1, OP_SAXPY = 2, OP_SCALE = 3, OP_NORM = 4 };
 // consumer thread kAcctThread: integer adds, beside the threads that work
 // out the pass's scalars.
 constexpr int kAcctThread = 64;
+// The consumer thread that looks at the ring's mark of failure, and at what
+// the producer has seen, for all of them (in a warp that has no sum to add up
+// and no scalar to work out).
+constexpr int kFoldThread = kConsumers - 32;
 struct Acct {
     int64_t ops[5];   // Table 4.3 categories of the current inner call
     int64_t spmv;     // all sparse products of the solve
@@ -213,6 +223,7 @@ struct IterState {
     S bt[kMaxN];
     Scalars<S> sc;
     int s_lo, s_hi;   // slices this CTA owns
+    int bare;         // some pass has no tiles
 };
 template <typename S>
 __device__ __forceinline__ IterState<S> &the_iter() {
@@ -530,6 +541,14 @@ __device__ __forceinline__ RedScratch &the_red() {
     return r;
 }
 
+// A tile wait of this warp failed: its tile counter is no longer that of the
+// next pass, which therefore must not begin.  The reduction or the team
+// barrier (of that turn) that ends the pass reports it.
+__device__ __forceinline__ void tile_lost(int turn = 0) {
+    the_ring()->failed = 1;
+    the_red().lost[turn & 1] = 1;
+}
+
 // Synchronisation state of one CTA within the team of CTAs that solves one
 // system: the whole grid (a single solve), a group of CTAs of a batch
 // launch (a large system of a batch), or the CTA alone (the other systems
@@ -571,6 +590,7 @@ struct GridSync {
         epoch = bepoch = fepoch = 0;
         ok = !the_ring()->failed;
         the_ring()->timeout_ns = to;
+        the_red().lost[0] = the_red().lost[1] = 0;
     }
 
     // Slots of sum k of the exchange `ep`.  Two halves suffice: a CTA
@@ -640,9 +660,11 @@ struct GridSync {
             p[0] = (a0 + a1) + (tid % G1 < 48 ? a2 + p[3 * G1] : a2);   // only this task reads slot 0
         }
         consumer_sync();
-        const bool lost = warp < K && !team_total(warp, fence);
-        if (consumer_any(lost || the_ring()->failed)) { ok = false; return false; }
+        if (warp < K && !team_total(warp, fence)) the_red().lost[0] = 1;
+        if (tid == kFoldThread && the_ring()->failed) the_red().lost[0] = 1;
+        consumer_sync();
         if (tid == 0) epoch += 1;   // read again only after another barrier
+        if (the_red().lost[0]) { ok = false; return false; }
         return true;
     }
     // The same for the passes outside the iteration (one copy of the code).
@@ -658,10 +680,10 @@ struct GridSync {
 
     // Team barrier (a counter: cheaper than an exchange where no value goes
     // with it).
-    // lost: a wait of this thread's own failed.
-    __device__ __forceinline__ bool sync(bool lost = false) {
+    // turn: see RedScratch::lost.
+    __device__ __forceinline__ bool sync(int turn = 0) {
         arrive();
-        return wait(lost);
+        return wait(turn);
     }
 
     // sync() in two halves: arrive() once this CTA's writes are done,
@@ -674,9 +696,12 @@ struct GridSync {
         consumer_sync();
         if (threadIdx.x == 0) grid_arrive(bar, bepoch);
     }
-    __device__ __forceinline__ bool wait(bool lost = false) {
-        if (nblocks > 1 && threadIdx.x == 0 && !grid_wait(bar, bepoch, nblocks, timeout_ns)) lost = true;
-        if (consumer_any(lost || the_ring()->failed)) { ok = false; return false; }
+    __device__ __forceinline__ bool wait(int turn) {
+        int *const l = the_red().lost + (turn & 1);
+        if (nblocks > 1 && threadIdx.x == 0 && !grid_wait(bar, bepoch, nblocks, timeout_ns)) *l = 1;
+        if (threadIdx.x == kFoldThread && the_ring()->failed) *l = 1;
+        consumer_sync();
+        if (*l) { ok = false; return false; }
         return true;
     }
 
@@ -686,7 +711,7 @@ struct GridSync {
     // them.
     __device__ __forceinline__ void post(unsigned cmd) {
         if (threadIdx.x == 0) {
-            await_producer(the_ring(), &the_ring()->cmd, kCmdNone);
+            await_producer(the_ring(), [] { return *(volatile unsigned *)&the_ring()->cmd == kCmdNone; });
             the_ring()->cmd = cmd;
             *(volatile int *)&the_ring()->stop = cmd == kCmdStop || cmd == kCmdExit;
         }
@@ -790,6 +815,7 @@ struct Engine {
             own_range(sys().nslices, gs().nblocks, gs().bid, lo, hi);
             the_iter<S>().s_lo = (int)lo;
             the_iter<S>().s_hi = (int)hi;
+            the_iter<S>().bare = lo >= hi || sys().spt[2] <= 0;
             the_ring()->stop = 0;
         }
         __syncthreads();
@@ -912,10 +938,9 @@ struct Engine {
         __syncthreads();
         const unsigned cmd = *(volatile unsigned *)&R->cmd;
         if (cmd == kCmdStop) {
-            // the consumers may have finished a pass that this side did not
-            // wait for
-            passes = *(volatile unsigned *)&R->finished;
-            saw(passes);
+            // the consumers may have finished the pass that this side was
+            // waiting for or issuing
+            if (mbar_probe(&R->done, passes & 1u)) saw(++passes);
         }
         __syncwarp();
         if ((threadIdx.x & 31) == 0) *(volatile unsigned *)&R->cmd = kCmdNone;
@@ -981,12 +1006,11 @@ struct Engine {
     // ------------------------------------------------------------------
 
     // Streaming pass through the tile pipeline: fn(chunk, stage, k) for
-    // every chunk of this CTA.  A failed tile wait marks the ring; the pass's
-    // reduction or barrier then reports it.
+    // every chunk of this CTA.
     template <typename Fn>
     __device__ __forceinline__ void tiles(int tc, unsigned &sq, Fn fn) {
         TileRing *const ring = the_ring();
-        if (!consume(ring, TileGeom{tc, c_lo(), c_hi()}, sq, fn)) ring->failed = 1;
+        if (!consume(ring, TileGeom{tc, c_lo(), c_hi()}, sq, fn)) tile_lost();
         pass_done(ring);
     }
 
@@ -1006,7 +1030,7 @@ struct Engine {
         constexpr int W = is_narrow<T>::value || is_cx<T>::value ? 7 : 8;
         const bool okw = sell_consume<1, EW, W>(the_ring(), sq, s_lo(), s_hi(), spt, sys().slice_ptr, sys().scol,
                                                 sys().sval, xin, epi, fin, acc);
-        if (!okw) the_ring()->failed = 1;
+        if (!okw) tile_lost();
         pass_done(the_ring());
     }
 
@@ -1215,7 +1239,8 @@ struct Engine {
                     }
                 }
             }
-            const bool good = gs().sync(!ok);
+            if (!ok) the_red().lost[1] = 1;
+            const bool good = gs().sync(1);
             if (threadIdx.x == 0) gs().fepoch = ep;   // read again only after another barrier
             ilu_count();
             return good;
@@ -1285,7 +1310,7 @@ struct Engine {
                 chunk(M.uptr, 0, q0, q1);
                 ilu_fetch_u(q0 + tid, q1, R);
             }
-            if (!gs().wait()) return false;
+            if (!gs().wait(l + 1)) return false;
         }
         for (int l = 0; l < nu; ++l) {
             if (R.i >= 0) out[R.i] = ilu_row_sum(R, ldcg_val(out + R.i), out) / R.v;
@@ -1301,7 +1326,7 @@ struct Engine {
                 chunk(M.uptr, l + 1, q0, q1);
                 ilu_fetch_u(q0 + tid, q1, R);
             }
-            if (!gs().wait()) return false;
+            if (!gs().wait(nl + l + 1)) return false;
         }
         ilu_count();
         return true;
@@ -1415,8 +1440,8 @@ struct Engine {
                 cnt = cnt1;
                 t = t1;
             }
-            if (!ok) R->failed = 1;
-            if (!gs().sync()) return false;
+            if (!ok) tile_lost(l + 1);
+            if (!gs().sync(l + 1)) return false;
         }
         gs().seq() = q;
         ilu_count();
@@ -1478,7 +1503,9 @@ struct Engine {
     // iteration's own M^{-1} is inlined in inner().
     __device__ __noinline__ bool ilu_solve(const T *v, T *out) {
         if (sys().ilu.llev) gs().post(kCmdIlu);
-        return ilu_solve_body(v, out);
+        const bool good = ilu_solve_body(v, out);
+        consumer_sync();   // the next team barrier may have any turn
+        return good;
     }
 
     // y_0 = M x_0 = L (U x_0), in place on x: t = U x, then x = L t (two
@@ -1494,7 +1521,7 @@ struct Engine {
             for (int64_t k = kd; k < k1; ++k) s = efma(M.lu[k], x[M.ci[k]], s);
             t[i] = s;
         }
-        if (!gs().sync()) return false;
+        if (!gs().sync(1)) return false;
         for (int64_t i = me; i < sys().N; i += nth) {
             const int64_t k0 = M.rp[i], kd = k0 + M.dpos[i];
             T s = ldcg_val(t + i);
@@ -2050,6 +2077,8 @@ struct Engine {
             } else if (tid == kAcctThread) {
                 if (st.op == P_OMEGA) sc().inv_omega = recip(sc().omega);
                 if (!last) count(st, n);
+            } else if (tid == kFoldThread) {
+                if (the_iter<S>().bare) await_seen(the_ring());
             }
             consumer_sync();
             if (st.op == P_RESIDUAL) {

@@ -107,11 +107,12 @@ struct Refiner {
                                              },
                                              acc);
         gs().seq() = sq;
-        if (!okt) the_ring()->failed = 1;
+        if (!okt) tile_lost();
         pass_done(the_ring());
         if (!gs().template reduce<2>(acc, true)) return false;
         bb = the_red().total[0];
         rr = the_red().total[1];
+        if (threadIdx.x == kFoldThread) await_seen(the_ring());
         if (threadIdx.x == kAcctThread) {
             acct().bytes += v().nnz * (int64_t)sizeof(T64) + v().nnz / EW * 4 + 4 * (v().N + 1) +
                            3 * v().N * (int64_t)sizeof(T64);
@@ -161,7 +162,7 @@ struct Refiner {
         const uint4 *src = reinterpret_cast<const uint4 *>(save ? v().x : v().xbest);
         for (int64_t ch = c_start; ch < c_hi; ch += kConsumers) dst[ch] = src[ch];
         if (threadIdx.x == kAcctThread) acct().bytes += 2 * v().N * (int64_t)sizeof(T64);
-        return gs().sync();
+        return gs().sync(1);   // after a reduction
     }
 
     __device__ __forceinline__ static double widen_fma(double s, float d, double x) { return fma(s, (double)d, x); }

@@ -130,7 +130,6 @@ struct TileRing {
     uint64_t timeout_ns;     // limit of every wait
     unsigned issued;         // tiles issued (written by the producer where both sides meet)
     unsigned consumed;       // tiles consumed (written by the consumers there)
-    unsigned finished;       // passes the consumers have finished (their thread 0)
     unsigned seen;           // passes the producer has seen the end of
     unsigned cmd;
     int stop;                // the producer returns from its waits, to the next command
@@ -160,7 +159,7 @@ __device__ __forceinline__ void ring_init(TileRing *R, uint64_t timeout_ns) {
         R->timeout_ns = timeout_ns;
         R->failed = 0;
         R->stop = 0;
-        R->finished = R->seen = 0;
+        R->seen = 0;
         R->cmd = kCmdNone;
         R->soff_src = nullptr;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -171,17 +170,6 @@ __device__ __forceinline__ void ring_init(TileRing *R, uint64_t timeout_ns) {
 // Barrier of the consumer warps alone.
 __device__ __forceinline__ void consumer_sync() {
     asm volatile("bar.sync 1, %0;" ::"n"(kConsumers) : "memory");
-}
-// The same, and whether `v` holds for any of them: one answer for all, so
-// that what some thread or the producer found out on its own, at a moment of
-// its own, turns every consumer the same way.
-__device__ __forceinline__ bool consumer_any(bool v) {
-    int r;
-    asm volatile("{ .reg .pred p, q; setp.ne.s32 q, %1, 0; bar.red.or.pred p, 1, %2, q; selp.s32 %0, 1, 0, p; }"
-                 : "=r"(r)
-                 : "r"((int)v), "n"(kConsumers)
-                 : "memory");
-    return r != 0;
 }
 
 // Bounded wait for the phase with parity `phase` of a barrier of the ring
@@ -356,32 +344,31 @@ __device__ __forceinline__ bool consume(TileRing *R, const TileGeom g, unsigned 
     return true;
 }
 
-// Consumer thread 0 waits (bounded) until the producer has written `want` to
-// a word of the ring.
-__device__ __forceinline__ void await_producer(TileRing *R, const unsigned *word, unsigned want) {
-    if (*(const volatile unsigned *)word == want) return;
+// One consumer thread waits (bounded) until `ready` holds, which the producer
+// brings about.
+template <typename Fn>
+__device__ __forceinline__ void await_producer(TileRing *R, Fn ready) {
+    if (ready()) return;
     const uint64_t t0 = globaltimer_ns();
-    while (*(const volatile unsigned *)word != want)
+    while (!ready())
         if (globaltimer_ns() - t0 > R->timeout_ns) {
             R->failed = 1;
             return;
         }
 }
 // End of a consumer's part of a pass in the solve kernels (its stores are
-// fenced for the async proxy): the producer may start the next pass.  A
-// phase of "done" is told by its parity, so a pass is only reported once the
-// producer has seen the one before.  Where a pass has tiles the consumers
-// could not have got that far; a CTA without rows, or a product whose rows
-// are too wide for a tile, has none.
+// fenced for the async proxy): the producer may start the next pass.
 __device__ __forceinline__ void pass_done(TileRing *R) {
     __syncwarp();
-    if ((threadIdx.x & 31) == 0) {
-        if (threadIdx.x == 0) {
-            await_producer(R, &R->seen, R->finished);
-            R->finished += 1;
-        }
-        mbar_arrive(&R->done);
-    }
+    if ((threadIdx.x & 31) == 0) mbar_arrive(&R->done);
+}
+// One consumer thread, once a pass has ended, in a CTA some of whose passes
+// have no tiles (it has no rows, or the rows of a product are too wide for a
+// tile): wait until the producer has seen the end, that is until the phase it
+// looks at is not complete.  A phase of "done" is told by its parity, so the
+// consumers must not be two passes ahead; tiles see to that by themselves.
+__device__ __forceinline__ void await_seen(TileRing *R) {
+    await_producer(R, [=] { return !mbar_probe(&R->done, *(volatile unsigned *)&R->seen & 1u); });
 }
 
 // Producer warp (all 32 lanes): issue every tile of a streaming pass over
