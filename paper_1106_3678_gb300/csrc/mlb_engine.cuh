@@ -717,12 +717,14 @@ struct GridSync {
         }
         __syncthreads();
     }
-    // End of an iteration: stop the producer, and discard the tiles it has
-    // issued ahead (their stages are released as if consumed).
-    __device__ __forceinline__ void end_inner(unsigned &sq) {
-        post(kCmdStop);
+    // End of an iteration (kCmdStop) or of a system (kCmdExit): stop the
+    // producer, and discard the tiles it has issued that no pass has consumed
+    // (their stages are released as if consumed).  What follows, the next
+    // system of a batch too, finds both sides at the same tile.
+    __device__ __forceinline__ void end(unsigned cmd, unsigned &sq) {
+        post(cmd);
         for (const unsigned last = the_ring()->issued; sq != last; ++sq) {
-            if (!mbar_wait_warp(&the_ring()->full[sq % kStages], (sq / kStages) & 1u, kLandNs)) {
+            if (!mbar_wait_warp(&the_ring()->full[sq % kStages], (sq / kStages) & 1u, kOwnNs)) {
                 the_ring()->failed = 1;
                 ok = false;
                 break;
@@ -731,6 +733,11 @@ struct GridSync {
             if ((threadIdx.x & 31) == 0) mbar_arrive(&the_ring()->empty[sq % kStages]);
         }
         consumer_sync();
+    }
+    __device__ __forceinline__ void end_system() {
+        unsigned sq = seq();
+        end(kCmdExit, sq);
+        seq() = sq;
     }
 };
 
@@ -1441,7 +1448,10 @@ struct Engine {
                 t = t1;
             }
             if (!ok) tile_lost(l + 1);
-            if (!gs().sync(l + 1)) return false;
+            if (!gs().sync(l + 1)) {
+                gs().seq() = q;
+                return false;
+            }
         }
         gs().seq() = q;
         ilu_count();
@@ -1972,14 +1982,18 @@ struct Engine {
             const bool f0 = st.first && hq;             // P_ALPHA: block 0's f_1^H r
             const int s1 = st.op == P_F_ROUND ? st.s + 1 : 1;
             const bool more = s1 <= i - 1;              // P_F_ROUND, P_G_J0: another f follows
-            bool good = true;
             if (!is_narrow<T>::value && st.op == P_RESIDUAL) gs().post(kCmdResidual);
             if constexpr (PC != kNoIlu) {
                 if ((st.op == P_SPMV_C || st.op == P_SPMV_Z || st.op == P_RESIDUAL) && sys().ilu.lu) {
                     gs().seq() = sq;
-                    good = ilu_solve_body(st.op == P_SPMV_C ? Gc(i) : st.op == P_SPMV_Z ? sys().r : sys().x,
-                                          sys().ilu.t);
+                    const bool good = ilu_solve_body(
+                        st.op == P_SPMV_C ? Gc(i) : st.op == P_SPMV_Z ? sys().r : sys().x, sys().ilu.t);
                     sq = gs().seq();
+                    if (!good) {
+                        // no product: the ring may still hold M^{-1}'s tiles
+                        if (st.op == P_RESIDUAL) return o;
+                        break;
+                    }
                 }
             }
             Sums sums;
@@ -2008,7 +2022,7 @@ struct Engine {
                 ph_g(sc().coef, i, more, sq, sums);
                 break;
             }
-            good = (sums.K ? gs().reduce_k(sums.v, sums.K, sums.fence) : gs().sync()) && good;
+            bool good = sums.K ? gs().reduce_k(sums.v, sums.K, sums.fence) : gs().sync();
             // the scalars of the next pass, the stopping rule and the
             // accounting, each on a thread of its own warp
             if (tid == 0) {
@@ -2126,7 +2140,7 @@ struct Engine {
             if (st.op == P_ALPHA && hq) op(OP_DOT);
             if (st.op == P_OMEGA) op(OP_DOT);
         }
-        gs().end_inner(sq);
+        gs().end(kCmdStop, sq);
         gs().seq() = sq;
         o.flag = gs().ok ? sc().flag : 1;
         o.iter = sc().iter;

@@ -255,7 +255,7 @@ __device__ RefineOut refine_solve(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> 
     if constexpr (PC != kNoIlu) {
         if (the_sys<T32>().ilu.lu && !E.ilu_begin()) return out;
     }
-    for (;;) {
+    while (the_gs().ok) {   // false from the start when an earlier system of a batch has lost the ring
         double bb, rr;
         if (!R.residual(bb, rr)) return out;
         double bn = sqrt(bb);
@@ -318,6 +318,7 @@ __device__ RefineOut refine_solve(Engine<T32, PC, EW> &E, Refiner<T64, T32, EW> 
         }
         if (!R.update(rn, d, nullptr)) return out;
     }
+    return out;
 }
 
 }  // namespace mlb

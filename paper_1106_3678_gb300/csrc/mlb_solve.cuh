@@ -97,7 +97,7 @@ __device__ __forceinline__ void run_cta() {
         E.template serve<false>([](unsigned &) { return 0; });
     } else {
         run_fp64_solve<T, PC, EW>();
-        the_gs().post(kCmdExit);
+        the_gs().end_system();
     }
     __syncthreads();
 }
@@ -241,7 +241,7 @@ __device__ __forceinline__ void refine_cta() {
         E.template serve<true>([&](unsigned &sq) { return R.issue(sq); });
     } else {
         o = refine_solve<T32, T64, PC, EW>(E, R, the_ctl(), the_refctl());
-        the_gs().post(kCmdExit);
+        the_gs().end_system();
     }
     __syncthreads();
     GridSync &gs = the_gs();

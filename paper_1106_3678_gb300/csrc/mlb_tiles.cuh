@@ -196,10 +196,11 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *b, unsigned phase, uint
         if ((it & 15u) == 0 && __any_sync(0xffffffffu, globaltimer_ns() - t0 > limit_ns)) return false;
     }
 }
-// Limit of the waits for copies that are under way when a solve or a kernel
-// ends.  Not the solve's own: that one may be as short as the caller likes,
-// and a CTA must not give its shared memory back while a copy writes into it.
-constexpr uint64_t kLandNs = 2000000000ull;
+// Limit of the waits that depend on this CTA alone: for copies that are under
+// way when a solve or a kernel ends, and for the producer to take a command.
+// Not the solve's own limit: that one may be as short as the caller likes, and
+// a CTA must not give its shared memory back while a copy writes into it.
+constexpr uint64_t kOwnNs = 2000000000ull;
 // Bounded wait of the producer's lane 0: 0 when the phase completed, 1 when
 // the consumers called it off, 2 on a timeout.  Twice the consumers'
 // limit, so that a wait of theirs that gives up is reported as such.
@@ -351,7 +352,7 @@ __device__ __forceinline__ void await_producer(TileRing *R, Fn ready) {
     if (ready()) return;
     const uint64_t t0 = globaltimer_ns();
     while (!ready())
-        if (globaltimer_ns() - t0 > R->timeout_ns) {
+        if (globaltimer_ns() - t0 > kOwnNs) {
             R->failed = 1;
             return;
         }
@@ -368,7 +369,9 @@ __device__ __forceinline__ void pass_done(TileRing *R) {
 // looks at is not complete.  A phase of "done" is told by its parity, so the
 // consumers must not be two passes ahead; tiles see to that by themselves.
 __device__ __forceinline__ void await_seen(TileRing *R) {
-    await_producer(R, [=] { return !mbar_probe(&R->done, *(volatile unsigned *)&R->seen & 1u); });
+    await_producer(R, [=] {
+        return !mbar_probe(&R->done, *(volatile unsigned *)&R->seen & 1u) || *(volatile int *)&R->failed != 0;
+    });
 }
 
 // Producer warp (all 32 lanes): issue every tile of a streaming pass over
@@ -475,7 +478,7 @@ __device__ __forceinline__ void ring_drain(TileRing *R, unsigned pseq, unsigned 
     __syncthreads();
     if (threadIdx.x == 0) {
         for (unsigned q = R->consumed; q < R->issued; ++q)
-            if (!mbar_wait_for(&R->full[q % kStages], (q / kStages) & 1u, kLandNs)) break;
+            if (!mbar_wait_for(&R->full[q % kStages], (q / kStages) & 1u, kOwnNs)) break;
     }
     __syncthreads();
 }
