@@ -140,8 +140,12 @@ typedef struct {
                              are capped by the maxit of the solve) */
     void *stream;         /* cudaStream_t for all work of this handle;
                              NULL = the legacy default stream */
-    int64_t timeout_ns;   /* limit of every device-side wait (grid barrier
-                             spin); default 2e9 (2 s) */
+    int64_t timeout_ns;   /* limit of every device-side wait on other CTAs
+                             or on copies; default 2e9 (2 s).  Within a
+                             triangular solve of ILU(0) in the order of the
+                             rows the limit is on the time without any
+                             row's progress; the whole solve may last
+                             longer. */
     int32_t precond;      /* MLB_PRECOND_NONE (default), MLB_PRECOND_JACOBI
                              or MLB_PRECOND_ILU0.
                              MLB_PRECOND_JACOBI: Algorithm 7.1 with

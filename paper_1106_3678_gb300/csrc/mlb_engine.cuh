@@ -713,6 +713,7 @@ struct GridSync {
         if (threadIdx.x == 0) {
             await_producer(the_ring(), [] { return *(volatile unsigned *)&the_ring()->cmd == kCmdNone; });
             the_ring()->cmd = cmd;
+            the_ring()->hold = cmd == kCmdResidual || cmd == kCmdResidual64 || cmd == kCmdIlu;
             *(volatile int *)&the_ring()->stop = cmd == kCmdStop || cmd == kCmdExit;
         }
         __syncthreads();
@@ -1983,6 +1984,9 @@ struct Engine {
             const int s1 = st.op == P_F_ROUND ? st.s + 1 : 1;
             const bool more = s1 <= i - 1;              // P_F_ROUND, P_G_J0: another f follows
             if (!is_narrow<T>::value && st.op == P_RESIDUAL) gs().post(kCmdResidual);
+            if (tid == kFoldThread)
+                *(volatile int *)&the_ring()->hold =
+                    st.op == P_RESIDUAL || st.op == P_SPMV_C || st.op == P_SPMV_Z;
             if constexpr (PC != kNoIlu) {
                 if ((st.op == P_SPMV_C || st.op == P_SPMV_Z || st.op == P_RESIDUAL) && sys().ilu.lu) {
                     gs().seq() = sq;

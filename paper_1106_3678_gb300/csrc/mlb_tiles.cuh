@@ -133,6 +133,7 @@ struct TileRing {
     unsigned seen;           // passes the producer has seen the end of
     unsigned cmd;
     int stop;                // the producer returns from its waits, to the next command
+    int hold;                // the consumers are in a pass of a product
     int failed;              // set when a wait timed out
     // Cache of the SELL-32 slice offsets of this CTA's slice range:
     // the_soff()[i] = slice_ptr[soff_lo + i] - soff_base for i = 0..soff_hi-soff_lo
@@ -159,6 +160,7 @@ __device__ __forceinline__ void ring_init(TileRing *R, uint64_t timeout_ns) {
         R->timeout_ns = timeout_ns;
         R->failed = 0;
         R->stop = 0;
+        R->hold = 0;
         R->seen = 0;
         R->cmd = kCmdNone;
         R->soff_src = nullptr;
@@ -203,14 +205,21 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *b, unsigned phase, uint
 constexpr uint64_t kOwnNs = 2000000000ull;
 // Bounded wait of the producer's lane 0: 0 when the phase completed, 1 when
 // the consumers called it off, 2 on a timeout.  Twice the consumers'
-// limit, so that a wait of theirs that gives up is reported as such.
+// limit, so that a wait of theirs that gives up is reported as such, without
+// the time of products: M^{-1} comes before one and may take thousands of
+// levels, rows too wide for a tile any time, and the consumers' waits within
+// have limits of their own.
 __device__ __forceinline__ int producer_wait(TileRing *R, uint64_t *b, unsigned phase) {
     if (mbar_probe(b, phase)) return 0;
-    const uint64_t t0 = globaltimer_ns();
+    uint64_t t0 = globaltimer_ns();
     for (unsigned it = 1;; ++it) {
         if (mbar_probe(b, phase)) return 0;
         if (*(volatile int *)&R->stop) return mbar_probe(b, phase) ? 0 : 1;
-        if ((it & 63u) == 0 && globaltimer_ns() - t0 > 2 * R->timeout_ns) return 2;
+        if ((it & 63u) == 0) {
+            const uint64_t now = globaltimer_ns();
+            if (*(volatile int *)&R->hold) t0 = now;
+            else if (now - t0 > 2 * R->timeout_ns) return 2;
+        }
     }
 }
 

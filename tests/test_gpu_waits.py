@@ -131,3 +131,33 @@ def test_waits_that_run_out_end_a_batch(precond, precision):
                 h.destroy()
 
     _solve_or_timeout(solve, LIMITS)
+
+
+@pytest.mark.parametrize("precision", PRECISIONS)
+@pytest.mark.parametrize("kind,N", [("real", 60000), ("complex", 30000)])
+def test_long_triangular_solves_are_no_timeout(kind, N, precision):
+    """A chain of N levels in each triangle, a microsecond or more each: one
+    M^{-1} (tens of milliseconds) lasts many times the limit of 5 ms, which no
+    single wait of a level comes near.  ILU(0) of a tridiagonal matrix is exact,
+    so that few iterations solve it."""
+    A = _band(N, 1, cplx=kind == "complex")
+    xs = W.uniform_rhs(N, seed=86).astype(A.val.dtype)
+    rows = np.repeat(np.arange(N), np.diff(A.row_ptr))
+    b = np.zeros_like(xs)
+    np.add.at(b, rows, A.val * xs[A.col])
+    h = M.mlbicgstab_create(A, n=2, q_seed=0, precond=M.MLB_PRECOND_ILU0, precision=precision, timeout_ns=5_000_000)
+    x = np.zeros_like(b)
+    r, _ = M.mlbicgstab_solve(h, b, x, 1e-11, 50)
+    assert r.flag == 0 and r.true_relres < 1e-11
+    # at least two M^{-1}, each longer than twice the limit
+    assert r.kernel_ms > 2 * 2 * 5.0
+    # diagonally dominant, ||A^-1||_2 <= 1 / (|d| - off-diagonal sum)
+    d = np.abs(A.val[rows == A.col]).min()
+    off = np.zeros(N)
+    np.add.at(off, rows[rows != A.col], np.abs(A.val[rows != A.col]))
+    offc = np.zeros(N)
+    np.add.at(offc, A.col[rows != A.col], np.abs(A.val[rows != A.col]))
+    gap = d - 0.5 * (off.max() + offc.max())
+    assert gap > 0
+    assert np.linalg.norm(x - xs) <= 1.1e-11 * np.linalg.norm(b) / gap
+    h.destroy()
