@@ -570,11 +570,13 @@ void mlbicgstab_destroy(mlb_handle *h);
 const char *mlbicgstab_strerror(int code);
 
 /*
- * Failure-detection self-test: launches the grid barrier the solve kernel
- * uses with one participant that never arrives, on `grid` CTAs, with a
- * wait limit of `timeout_ns`.  Every wait gives up after the limit and the
- * kernel returns; expected result MLB_ERR_TIMEOUT with the device still
- * usable.  The paper has no counterpart (library robustness only).
+ * Failure-detection self-test: launches, one after another, the three waits
+ * between CTAs that the solve kernels use (the counter barrier, a sum over
+ * the team, a value of a triangular solve) with one participant that never
+ * arrives, on `grid` CTAs, each with a wait limit of `timeout_ns`.  Each
+ * gives up after the limit and its kernel returns; expected result
+ * MLB_ERR_TIMEOUT (all three gave up) with the device still usable.  The
+ * paper has no counterpart (library robustness only).
  */
 int mlbicgstab_selftest_barrier_timeout(int32_t grid, int64_t timeout_ns);
 

@@ -1814,19 +1814,24 @@ int mlbicgstab_selftest_barrier_timeout(int32_t grid, int64_t timeout_ns) {
     BarrierState *bs = nullptr;
     const size_t bytes = 256 + (size_t)(grid + 1) * sizeof(Slot);
     MLB_CUDA(cudaMalloc(&bs, bytes));
-    cudaError_t e = cudaMemset(bs, 0, bytes);
-    if (e == cudaSuccess)
-        e = launch_barrier_selftest(grid, bs, (Slot *)((char *)bs + 256), (uint64_t)timeout_ns, nullptr);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    BarrierState hb;
-    memset(&hb, 0, sizeof(hb));
-    if (e == cudaSuccess) e = cudaMemcpy(&hb, bs, sizeof(hb), cudaMemcpyDeviceToHost);
+    cudaError_t e = cudaSuccess;
+    int ended = 0;
+    for (int wait = 0; wait < kSelftestWaits && e == cudaSuccess; ++wait) {
+        e = cudaMemset(bs, 0, bytes);
+        if (e == cudaSuccess)
+            e = launch_barrier_selftest(wait, grid, bs, (Slot *)((char *)bs + 256), (uint64_t)timeout_ns, nullptr);
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        BarrierState hb;
+        memset(&hb, 0, sizeof(hb));
+        if (e == cudaSuccess) e = cudaMemcpy(&hb, bs, sizeof(hb), cudaMemcpyDeviceToHost);
+        ended += hb.status == kStatusTimeout;
+    }
     cudaFree(bs);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return MLB_ERR_CUDA;
     }
-    return hb.status == kStatusTimeout ? MLB_ERR_TIMEOUT : MLB_OK;
+    return ended == kSelftestWaits ? MLB_ERR_TIMEOUT : MLB_OK;
 }
 
 }  // extern "C"

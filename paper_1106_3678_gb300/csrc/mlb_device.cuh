@@ -325,6 +325,32 @@ __device__ __forceinline__ bool value_of(unsigned long long s, unsigned epoch, f
     return (unsigned)(s >> 32) == epoch;
 }
 
+// Limit of a warp's polls in a triangular solve by value slots: `limit_ns`
+// without any warp's progress (one may wait for a whole triangle).
+struct SlotWait {
+    uint64_t t0 = 0;
+    unsigned spins = 0, seen = 0;
+    // After each round of polls: false (uniformly in the warp) when the wait is
+    // over, or another CTA has recorded a failure in bs.  Looks every 32nd time.
+    __device__ __forceinline__ bool go_on(BarrierState *bs, uint64_t limit_ns) {
+        if ((++spins & 31u) != 0) return true;
+        int stop = 0;
+        if ((threadIdx.x & 31) == 0) {
+            const uint64_t now = globaltimer_ns();
+            const unsigned at = ld_relaxed_u32(&bs->progress);
+            if (ld_relaxed_i32(&bs->status) != 0) stop = 1;
+            else if (t0 == 0 || at != seen) {
+                t0 = now;
+                seen = at;
+            } else if (now - t0 > limit_ns) {
+                atomicCAS(&bs->status, 0, kStatusTimeout);
+                stop = 1;
+            }
+        }
+        return __shfl_sync(0xffffffffu, stop, 0) == 0;
+    }
+};
+
 // One warp waits until all G slots at p carry `epoch` and adds their values:
 // lane l those of CTAs l, l + 32, ... as a pair tree, then an xor tree over
 // the lanes (every lane receives the sum).  The wait is bounded by

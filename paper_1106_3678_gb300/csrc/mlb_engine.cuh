@@ -1174,30 +1174,9 @@ struct Engine {
                     if (n > kIluReg) p = M.rp[i] + (up ? M.dpos[i] + 1 : 0);
                 }
                 const VS *const watch = w >= 0 ? z + w : up ? zl + ~w : nullptr;
-                uint64_t t0 = 0;
-                unsigned spins = 0, seen = 0;
-                // every 32nd poll: false (uniformly) when the wait is over,
-                // that is after the limit without any warp's progress (a warp
-                // may wait for a whole triangle)
-                auto patience = [&]() -> bool {
-                    if ((++spins & 31u) != 0) return true;
-                    int stop = 0;
-                    if (lane == 0) {
-                        const uint64_t now = globaltimer_ns();
-                        const unsigned at = ld_relaxed_u32(&bar->progress);
-                        if (ld_relaxed_i32(&bar->status) != 0) stop = 1;
-                        else if (t0 == 0 || at != seen) {
-                            t0 = now;
-                            seen = at;
-                        } else if (now - t0 > limit) {
-                            atomicCAS(&bar->status, 0, kStatusTimeout);
-                            stop = 1;
-                        }
-                    }
-                    return __shfl_sync(0xffffffffu, stop, 0) == 0;
-                };
+                SlotWait patience;
                 T xv;
-                while (ok && watch && !__all_sync(0xffffffffu, value_of(value_load(watch), ep, xv))) ok = patience();
+                while (ok && watch && !__all_sync(0xffffffffu, value_of(value_load(watch), ep, xv))) ok = patience.go_on(bar, limit);
                 int e = up ? -1 : 0;    // next entry; -1: the right-hand side
                 int e0 = 0;             // the entry in c[0] and a[0]
                 T s = d;
@@ -1237,7 +1216,7 @@ struct Engine {
                             done = true;
                         }
                     }
-                    if (!__all_sync(0xffffffffu, done)) ok = patience();
+                    if (!__all_sync(0xffffffffu, done)) ok = patience.go_on(bar, limit);
                 }
                 if (lane == 0) {
                     const uint64_t now = globaltimer_ns();

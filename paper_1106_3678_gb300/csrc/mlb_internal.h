@@ -199,9 +199,11 @@ void permute_csr(const mlb_matrix *A, const std::vector<int32_t> &perm, const st
 cudaError_t launch_permute(const void *src, void *dst, const int32_t *perm, int64_t N, int es, bool to_perm,
                            cudaStream_t st);
 
-// Failure-detection self-test of the grid barrier (see the C ABI).
-// `slots`: grid + 1 slots, zeroed.
-cudaError_t launch_barrier_selftest(int grid, BarrierState *bs, Slot *slots,
+// Failure-detection self-test (see the C ABI) of one of the waits between
+// CTAs: the counter barrier, a team sum, a value slot of a triangular solve.
+// `bs` and `slots` (grid + 1): zeroed.
+enum { kSelftestBarrier, kSelftestSum, kSelftestValue, kSelftestWaits };
+cudaError_t launch_barrier_selftest(int wait, int grid, BarrierState *bs, Slot *slots,
                                     uint64_t timeout_ns, cudaStream_t st);
 
 }  // namespace mlb

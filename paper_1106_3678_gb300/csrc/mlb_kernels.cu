@@ -414,17 +414,29 @@ cudaError_t launch_spmv_qdot_tiled(const SysView<T> &sys, int ne, int64_t maxw, 
 }
 
 // ===========================================================================
-// failure-detection self-test: a barrier one participant never reaches
+// failure-detection self-test: waits for a participant that never comes
 // ===========================================================================
-__global__ void barrier_selftest_kernel(BarrierState *bs, Slot *slots, uint64_t timeout_ns) {
+__global__ void barrier_selftest_kernel(int wait, BarrierState *bs, Slot *slots, uint64_t timeout_ns) {
+    __shared__ int flag;
+    if (wait == kSelftestBarrier) {
+        unsigned epoch = 0;
+        grid_barrier(bs, epoch, gridDim.x + 1, timeout_ns, &flag);
+        return;
+    }
     if (threadIdx.x >= 32) return;
     if (threadIdx.x == 0) slot_put(slots + blockIdx.x, 0.0, 1u);
     double t;
-    slots_sum(slots, gridDim.x + 1, 1u, bs, timeout_ns, t);
+    if (wait == kSelftestSum) {
+        slots_sum(slots, gridDim.x + 1, 1u, bs, timeout_ns, t);
+    } else {
+        SlotWait patience;
+        while (!value_of(value_load(slots + gridDim.x), 1u, t) && patience.go_on(bs, timeout_ns)) {}
+    }
 }
 
-cudaError_t launch_barrier_selftest(int grid, BarrierState *bs, Slot *slots, uint64_t timeout_ns, cudaStream_t st) {
-    void *args[] = {(void *)&bs, (void *)&slots, (void *)&timeout_ns};
+cudaError_t launch_barrier_selftest(int wait, int grid, BarrierState *bs, Slot *slots, uint64_t timeout_ns,
+                                    cudaStream_t st) {
+    void *args[] = {(void *)&wait, (void *)&bs, (void *)&slots, (void *)&timeout_ns};
     return cudaLaunchCooperativeKernel((const void *)barrier_selftest_kernel, dim3(grid), dim3(64), args, 0,
                                        st);
 }

@@ -161,3 +161,13 @@ def test_long_triangular_solves_are_no_timeout(kind, N, precision):
     assert gap > 0
     assert np.linalg.norm(x - xs) <= 1.1e-11 * np.linalg.norm(b) / gap
     h.destroy()
+
+
+def test_selftest_makes_every_wait_between_ctas_run_out():
+    """The counter barrier, a team sum and a value slot, one after another:
+    three limits pass before the answer."""
+    import time
+    M.mlbicgstab_selftest_barrier_timeout(4, 1_000_000)
+    t = time.perf_counter()
+    assert M.mlbicgstab_selftest_barrier_timeout(4, 60_000_000) == M.MLB_ERR_TIMEOUT
+    assert time.perf_counter() - t >= 3 * 0.060
