@@ -83,9 +83,8 @@ enum { OP_MATVEC = 0, OP_DOT = 1, OP_SAXPY = 2, OP_SCALE = 3, OP_NORM = 4 };
 // consumer thread kAcctThread: integer adds, beside the threads that work
 // out the pass's scalars.
 constexpr int kAcctThread = 64;
-// The consumer thread that looks at the ring's mark of failure, and at what
-// the producer has seen, for all of them (in a warp that has no sum to add up
-// and no scalar to work out).
+// The consumer thread that looks at the ring's mark of failure for all of
+// them (in a warp that has no sum to add up).
 constexpr int kFoldThread = kConsumers - 32;
 struct Acct {
     int64_t ops[5];   // Table 4.3 categories of the current inner call
@@ -223,7 +222,6 @@ struct IterState {
     S bt[kMaxN];
     Scalars<S> sc;
     int s_lo, s_hi;   // slices this CTA owns
-    int bare;         // some pass has no tiles
 };
 template <typename S>
 __device__ __forceinline__ IterState<S> &the_iter() {
@@ -358,8 +356,9 @@ __device__ __forceinline__ T sell_slice_sum3(const int32_t *cp, const T *vp, int
 // No call here: a call in a kernel's loop costs every pass of the kernel
 // registers (saved across it by convention).  Returns false when a tile wait timed out.
 //
-// sell_consume is the consumer warps' part.
-template <int NE, int EW = 1, int PW = 8, typename T, typename Fin, typename AccArr>
+// sell_consume is the consumer warps' part.  EMPTY: a pass without tiles has
+// one empty tile (see consume_empty).
+template <int NE, int EW = 1, int PW = 8, bool EMPTY = false, typename T, typename Fin, typename AccArr>
 __device__ __forceinline__ bool sell_consume(TileRing *R, unsigned &cseq, int s_lo, int s_hi, int spt,
                                              const int64_t *slice_ptr, const int32_t *scol, const T *sval,
                                              const T *xin, const T *const (&epi)[NE > 0 ? NE : 1], Fin fin,
@@ -370,6 +369,7 @@ __device__ __forceinline__ bool sell_consume(TileRing *R, unsigned &cseq, int s_
     const int cw = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (spt <= 0) {
         // slices too wide for one stage: direct loads, no pipeline
+        if (EMPTY && !consume_empty(R, cseq)) return false;
         const SliceOffsets off(R, slice_ptr, s_lo, s_hi);
         for (int s = s_lo + cw; s < s_hi; s += kConsumerWarps) {
             const int64_t o = off(s);
@@ -472,7 +472,7 @@ __device__ __forceinline__ bool sell_consume(TileRing *R, unsigned &cseq, int s_
     };
     bool ok = true;
     unsigned q = cseq;
-    if (s_lo < s_hi) {
+    if (EMPTY || s_lo < s_hi) {
         Job ja, jb;
         T xv[kPipeW * EW];
         ok = locate(s_lo, q, ja);
@@ -486,7 +486,7 @@ __device__ __forceinline__ bool sell_consume(TileRing *R, unsigned &cseq, int s_
                     for (int m = 0; m < EW; ++m) xv[EW * u + m] = xin[c + m];
                 }
         }
-        for (int s0 = s_lo; ok && s0 < s_hi; s0 += spt) {
+        for (int s0 = s_lo; ok && (s0 < s_hi || (EMPTY && s0 == s_lo)); s0 += spt) {
             const bool more = s0 + spt < s_hi;
             if (more && !locate(s0 + spt, q + 1, jb)) {
                 ok = false;
@@ -689,19 +689,19 @@ struct GridSync {
     // sync() in two halves: arrive() once this CTA's writes are done,
     // wait() before reading other CTAs' writes; work between the two that
     // reads nothing written in this step overlaps the wait.  wait() returns
-    // false (uniformly) when a wait failed.  A CTA alone needs wait()'s
-    // barrier only.
+    // false (uniformly) when a wait of the consumers failed (the producer's
+    // own is seen by the next reduction, or starves them of tiles).  A CTA
+    // alone needs arrive()'s barrier only.
     __device__ __forceinline__ void arrive() {
-        if (nblocks == 1) return;
         consumer_sync();
-        if (threadIdx.x == 0) grid_arrive(bar, bepoch);
+        if (nblocks > 1 && threadIdx.x == 0) grid_arrive(bar, bepoch);
     }
     __device__ __forceinline__ bool wait(int turn) {
-        int *const l = the_red().lost + (turn & 1);
-        if (nblocks > 1 && threadIdx.x == 0 && !grid_wait(bar, bepoch, nblocks, timeout_ns)) *l = 1;
-        if (threadIdx.x == kFoldThread && the_ring()->failed) *l = 1;
-        consumer_sync();
-        if (*l) { ok = false; return false; }
+        if (nblocks > 1) {
+            if (threadIdx.x == 0 && !grid_wait(bar, bepoch, nblocks, timeout_ns)) the_red().lost[turn & 1] = 1;
+            consumer_sync();
+        }
+        if (the_red().lost[turn & 1]) { ok = false; return false; }
         return true;
     }
 
@@ -711,9 +711,8 @@ struct GridSync {
     // them.
     __device__ __forceinline__ void post(unsigned cmd) {
         if (threadIdx.x == 0) {
-            await_producer(the_ring(), [] { return *(volatile unsigned *)&the_ring()->cmd == kCmdNone; });
+            await_taken(the_ring());
             the_ring()->cmd = cmd;
-            the_ring()->hold = cmd == kCmdResidual || cmd == kCmdResidual64 || cmd == kCmdIlu;
             *(volatile int *)&the_ring()->stop = cmd == kCmdStop || cmd == kCmdExit;
         }
         __syncthreads();
@@ -823,7 +822,6 @@ struct Engine {
             own_range(sys().nslices, gs().nblocks, gs().bid, lo, hi);
             the_iter<S>().s_lo = (int)lo;
             the_iter<S>().s_hi = (int)hi;
-            the_iter<S>().bare = lo >= hi || sys().spt[2] <= 0;
             the_ring()->stop = 0;
         }
         __syncthreads();
@@ -923,21 +921,17 @@ struct Engine {
     }
     // Tiles of a product with one epilogue vector, `spt` slices each.
     __device__ __forceinline__ int issue_product(const T *epi, int spt, unsigned &sq) {
-        if (spt <= 0) return 0;
         const SliceOffsets off(the_ring(), sys().slice_ptr, s_lo(), s_hi());
         return produce_sell_lanes(the_ring(), s_lo(), s_hi(), spt, off, sys().sval, EW * (int)sizeof(T),
                                   (int)sizeof(T), sys().scol, epi, 1, sq);
     }
     // Wait until the consumers have finished the pass.
-    __device__ __forceinline__ int wait_done(unsigned &passes) {
+    __device__ __forceinline__ int wait_done(unsigned &passes, bool limited) {
         int st = 0;
-        if ((threadIdx.x & 31) == 0) st = producer_wait(the_ring(), &the_ring()->done, passes & 1u);
+        if ((threadIdx.x & 31) == 0) st = producer_wait(the_ring(), &the_ring()->done, passes & 1u, limited);
         st = __shfl_sync(0xffffffffu, st, 0);
-        if (st == 0) saw(++passes);
+        if (st == 0) passes += 1;
         return st;
-    }
-    __device__ __forceinline__ static void saw(unsigned passes) {
-        if ((threadIdx.x & 31) == 0) *(volatile unsigned *)&the_ring()->seen = passes;
     }
     // Meet the consumers: their next command.  `sq`: tiles issued so far.
     __device__ __forceinline__ unsigned command(unsigned sq, unsigned &passes) {
@@ -948,7 +942,7 @@ struct Engine {
         if (cmd == kCmdStop) {
             // the consumers may have finished the pass that this side was
             // waiting for or issuing
-            if (mbar_probe(&R->done, passes & 1u)) saw(++passes);
+            if (mbar_probe(&R->done, passes & 1u)) passes += 1;
         }
         __syncwarp();
         if ((threadIdx.x & 31) == 0) *(volatile unsigned *)&R->cmd = kCmdNone;
@@ -962,7 +956,7 @@ struct Engine {
     template <bool Decide, typename Fn>
     __device__ __forceinline__ void serve(Fn residual64) {
         TileRing *const R = the_ring();
-        unsigned sq = gs().seq(), passes = R->seen;
+        unsigned sq = gs().seq(), passes = R->passes;
         bool dead = false;
         for (;;) {
             const unsigned cmd = command(sq, passes);
@@ -972,10 +966,10 @@ struct Engine {
             if (cmd == kCmdResidual) {
                 st = issue_ilu(sq);
                 if (st == 0) st = issue_product(sys().b, sys().spt[2], sq);
-                if (st == 0) st = wait_done(passes);
+                if (st == 0) st = wait_done(passes, false);
             } else if (cmd == kCmdResidual64) {
                 st = residual64(sq);
-                if (st == 0) st = wait_done(passes);
+                if (st == 0) st = wait_done(passes, false);
             } else if (cmd == kCmdIlu) {
                 st = issue_ilu(sq);
             } else {
@@ -983,7 +977,7 @@ struct Engine {
                 bool over = false;   // ended by a command
                 for (Step p; st == 0 && !over; p.advance(n)) {
                     st = issue(p, sq);
-                    if (st == 0) st = wait_done(passes);
+                    if (st == 0) st = wait_done(passes, p.op != P_SPMV_C && p.op != P_SPMV_Z);
                     if constexpr (Decide) {
                         // the consumers' commands (a residual replacement)
                         // until they let the iteration go on or end it
@@ -995,7 +989,7 @@ struct Engine {
                                 st = issue_ilu(sq);
                             } else {
                                 st = residual64(sq);
-                                if (st == 0) st = wait_done(passes);
+                                if (st == 0) st = wait_done(passes, false);
                             }
                         }
                     }
@@ -1007,6 +1001,7 @@ struct Engine {
             }
         }
         gs().seq() = sq;
+        if ((threadIdx.x & 31) == 0) R->passes = passes;
     }
 
     // ------------------------------------------------------------------
@@ -1018,7 +1013,7 @@ struct Engine {
     template <typename Fn>
     __device__ __forceinline__ void tiles(int tc, unsigned &sq, Fn fn) {
         TileRing *const ring = the_ring();
-        if (!consume(ring, TileGeom{tc, c_lo(), c_hi()}, sq, fn)) tile_lost();
+        if (!consume<true>(ring, TileGeom{tc, c_lo(), c_hi()}, sq, fn)) tile_lost();
         pass_done(ring);
     }
 
@@ -1036,8 +1031,8 @@ struct Engine {
         // the 3-D stencils (fewer registers of gathered x); the real FP64
         // engine keeps 8 (no gain at 7)
         constexpr int W = is_narrow<T>::value || is_cx<T>::value ? 7 : 8;
-        const bool okw = sell_consume<1, EW, W>(the_ring(), sq, s_lo(), s_hi(), spt, sys().slice_ptr, sys().scol,
-                                                sys().sval, xin, epi, fin, acc);
+        const bool okw = sell_consume<1, EW, W, true>(the_ring(), sq, s_lo(), s_hi(), spt, sys().slice_ptr,
+                                                      sys().scol, sys().sval, xin, epi, fin, acc);
         if (!okw) tile_lost();
         pass_done(the_ring());
     }
@@ -1474,7 +1469,7 @@ struct Engine {
                     const int s = (int)(sq % kStages);
                     const unsigned use = sq / kStages;
                     int st = 0;
-                    if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u);
+                    if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u, false);
                     st = __shfl_sync(0xffffffffu, st, 0);
                     if (st) return st;
                     const unsigned n = (unsigned)(k1 - k < spt ? k1 - k : spt);
@@ -1963,9 +1958,6 @@ struct Engine {
             const int s1 = st.op == P_F_ROUND ? st.s + 1 : 1;
             const bool more = s1 <= i - 1;              // P_F_ROUND, P_G_J0: another f follows
             if (!is_narrow<T>::value && st.op == P_RESIDUAL) gs().post(kCmdResidual);
-            if (tid == kFoldThread)
-                *(volatile int *)&the_ring()->hold =
-                    st.op == P_RESIDUAL || st.op == P_SPMV_C || st.op == P_SPMV_Z;
             if constexpr (PC != kNoIlu) {
                 if ((st.op == P_SPMV_C || st.op == P_SPMV_Z || st.op == P_RESIDUAL) && sys().ilu.lu) {
                     gs().seq() = sq;
@@ -2074,8 +2066,6 @@ struct Engine {
             } else if (tid == kAcctThread) {
                 if (st.op == P_OMEGA) sc().inv_omega = recip(sc().omega);
                 if (!last) count(st, n);
-            } else if (tid == kFoldThread) {
-                if (the_iter<S>().bare) await_seen(the_ring());
             }
             consumer_sync();
             if (st.op == P_RESIDUAL) {

@@ -84,7 +84,6 @@ struct Refiner {
 
     // Producer warp: the tiles of residual().
     __device__ __forceinline__ int issue(unsigned &sq) {
-        if (v().spt[1] <= 0) return 0;
         const SliceOffsets off(the_ring(), v().slice_ptr, s_lo(), s_hi());
         return produce_sell_lanes(the_ring(), s_lo(), s_hi(), v().spt[1], off, v().sval, EW * (int)sizeof(T64), (int)sizeof(T64),
                                   v().scol, v().b, 1, sq);
@@ -97,7 +96,7 @@ struct Refiner {
         const T64 *epi[1] = {v().b};
         T64 *const r = v().r;
         unsigned sq = gs().seq();
-        const bool okt = sell_consume<1, EW>(the_ring(), sq, s_lo(), s_hi(), v().spt[1], v().slice_ptr, v().scol,
+        const bool okt = sell_consume<1, EW, 8, true>(the_ring(), sq, s_lo(), s_hi(), v().spt[1], v().slice_ptr, v().scol,
                                              v().sval, v().x, epi, 
                                              [=](int64_t row, T64 y, const T64 (&e)[1], double(&a)[2]) {
                                                  T64 rv = subT(e[0], y);
@@ -112,7 +111,6 @@ struct Refiner {
         if (!gs().template reduce<2>(acc, true)) return false;
         bb = the_red().total[0];
         rr = the_red().total[1];
-        if (threadIdx.x == kFoldThread) await_seen(the_ring());
         if (threadIdx.x == kAcctThread) {
             acct().bytes += v().nnz * (int64_t)sizeof(T64) + v().nnz / EW * 4 + 4 * (v().N + 1) +
                            3 * v().N * (int64_t)sizeof(T64);

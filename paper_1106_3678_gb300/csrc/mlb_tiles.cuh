@@ -130,10 +130,9 @@ struct TileRing {
     uint64_t timeout_ns;     // limit of every wait
     unsigned issued;         // tiles issued (written by the producer where both sides meet)
     unsigned consumed;       // tiles consumed (written by the consumers there)
-    unsigned seen;           // passes the producer has seen the end of
+    unsigned passes;         // passes the producer has seen the end of
     unsigned cmd;
     int stop;                // the producer returns from its waits, to the next command
-    int hold;                // the consumers are in a pass of a product
     int failed;              // set when a wait timed out
     // Cache of the SELL-32 slice offsets of this CTA's slice range:
     // the_soff()[i] = slice_ptr[soff_lo + i] - soff_base for i = 0..soff_hi-soff_lo
@@ -160,8 +159,7 @@ __device__ __forceinline__ void ring_init(TileRing *R, uint64_t timeout_ns) {
         R->timeout_ns = timeout_ns;
         R->failed = 0;
         R->stop = 0;
-        R->hold = 0;
-        R->seen = 0;
+        R->passes = 0;
         R->cmd = kCmdNone;
         R->soff_src = nullptr;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -205,21 +203,17 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *b, unsigned phase, uint
 constexpr uint64_t kOwnNs = 2000000000ull;
 // Bounded wait of the producer's lane 0: 0 when the phase completed, 1 when
 // the consumers called it off, 2 on a timeout.  Twice the consumers'
-// limit, so that a wait of theirs that gives up is reported as such, without
-// the time of products: M^{-1} comes before one and may take thousands of
-// levels, rows too wide for a tile any time, and the consumers' waits within
-// have limits of their own.
-__device__ __forceinline__ int producer_wait(TileRing *R, uint64_t *b, unsigned phase) {
+// limit, so that a wait of theirs that gives up is reported as such, and none
+// in a pass of a product (limited = false): M^{-1} comes before it and may
+// take thousands of levels, rows too wide for a tile any time.  The consumers'
+// own waits there have limits, and they call the producer off when one ends.
+__device__ __forceinline__ int producer_wait(TileRing *R, uint64_t *b, unsigned phase, bool limited) {
     if (mbar_probe(b, phase)) return 0;
     uint64_t t0 = globaltimer_ns();
     for (unsigned it = 1;; ++it) {
         if (mbar_probe(b, phase)) return 0;
         if (*(volatile int *)&R->stop) return mbar_probe(b, phase) ? 0 : 1;
-        if ((it & 63u) == 0) {
-            const uint64_t now = globaltimer_ns();
-            if (*(volatile int *)&R->hold) t0 = now;
-            else if (now - t0 > 2 * R->timeout_ns) return 2;
-        }
+        if (limited && (it & 63u) == 0 && globaltimer_ns() - t0 > 2 * R->timeout_ns) return 2;
     }
 }
 
@@ -325,12 +319,14 @@ __device__ __forceinline__ bool produce(TileRing *R, const TilePass &P, unsigned
 
 // Consumer side: for every tile, wait for it, call fn(chunk, stage, k)
 // for each chunk k of the tile owned by this thread (chunk k is read from
-// stage + i*tc*16 + k*16 for input i), then release the stage.
-template <typename Fn>
+// stage + i*tc*16 + k*16 for input i), then release the stage.  EMPTY: a pass
+// without chunks has one empty tile (see consume_empty).
+template <bool EMPTY = false, typename Fn>
 __device__ __forceinline__ bool consume(TileRing *R, const TileGeom g, unsigned &seq, Fn fn) {
     const int tc = g.tc;
     const int64_t c_lo = g.c_lo, c_hi = g.c_hi;
-    const int nt = (int)((c_hi - c_lo + tc - 1) / tc);
+    int nt = (int)((c_hi - c_lo + tc - 1) / tc);
+    if (EMPTY && nt == 0) nt = 1;
     unsigned char *const buf = the_stages();
     unsigned sq = seq;
     const int tid = threadIdx.x;   // < kConsumers
@@ -354,13 +350,13 @@ __device__ __forceinline__ bool consume(TileRing *R, const TileGeom g, unsigned 
     return true;
 }
 
-// One consumer thread waits (bounded) until `ready` holds, which the producer
-// brings about.
-template <typename Fn>
-__device__ __forceinline__ void await_producer(TileRing *R, Fn ready) {
-    if (ready()) return;
+// One consumer thread waits (bounded) until the producer has taken the last
+// command.
+__device__ __forceinline__ void await_taken(TileRing *R) {
+    const volatile unsigned *cmd = &R->cmd;
+    if (*cmd == kCmdNone) return;
     const uint64_t t0 = globaltimer_ns();
-    while (!ready())
+    while (*cmd != kCmdNone)
         if (globaltimer_ns() - t0 > kOwnNs) {
             R->failed = 1;
             return;
@@ -372,15 +368,17 @@ __device__ __forceinline__ void pass_done(TileRing *R) {
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(&R->done);
 }
-// One consumer thread, once a pass has ended, in a CTA some of whose passes
-// have no tiles (it has no rows, or the rows of a product are too wide for a
-// tile): wait until the producer has seen the end, that is until the phase it
-// looks at is not complete.  A phase of "done" is told by its parity, so the
-// consumers must not be two passes ahead; tiles see to that by themselves.
-__device__ __forceinline__ void await_seen(TileRing *R) {
-    await_producer(R, [=] {
-        return !mbar_probe(&R->done, *(volatile unsigned *)&R->seen & 1u) || *(volatile int *)&R->failed != 0;
-    });
+// A pass without a tile of its own (a CTA without rows, or a product whose
+// rows are too wide for a stage) has an empty one: the end of a pass is told
+// by the parity of "done", so the consumers must not finish a pass before the
+// producer has seen the end of the one before, and waiting for a tile of the
+// pass sees to that.  Consumers: take it, where no loop over tiles does.
+__device__ __forceinline__ bool consume_empty(TileRing *R, unsigned &seq) {
+    const int s = (int)(seq % kStages);
+    if (!mbar_wait_warp(&R->full[s], (seq / kStages) & 1u, R->timeout_ns)) return false;
+    if ((threadIdx.x & 31) == 0) mbar_arrive(&R->empty[s]);
+    ++seq;
+    return true;
 }
 
 // Producer warp (all 32 lanes): issue every tile of a streaming pass over
@@ -389,36 +387,43 @@ __device__ __forceinline__ void await_seen(TileRing *R) {
 __device__ __forceinline__ int produce_lanes(TileRing *R, const void *src, int ni, int64_t c_lo, int64_t c_hi,
                                              unsigned &seq) {
     const int lane = threadIdx.x & 31, tc = tile_chunks_for(ni);
-    for (int64_t c0 = c_lo; c0 < c_hi; c0 += tc, ++seq) {
+    int64_t c0 = c_lo;
+    do {
         const int s = (int)(seq % kStages);
         const unsigned use = seq / kStages;
         int st = 0;
-        if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u);
+        if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u, true);
         st = __shfl_sync(0xffffffffu, st, 0);
         if (st) return st;
         const unsigned bytes = (unsigned)(c_hi - c0 < tc ? c_hi - c0 : tc) * 16u;
         if (lane == 0) mbar_arrive_expect_tx(&R->full[s], bytes * (unsigned)ni);
         __syncwarp();
-        if (lane < ni)
+        if (lane < ni && bytes > 0)
             bulk_g2s(the_stages() + (size_t)s * kStageBytes + (size_t)lane * tc * 16, (const unsigned char *)src + c0 * 16,
                      bytes, &R->full[s]);
-    }
+        ++seq;
+    } while ((c0 += tc) < c_hi);
     return 0;
 }
 
 // The same for SELL-32 tiles (see produce_sell): lane 0 copies the values,
 // lane 1 the column indices, lane 2 + i epilogue vector i from `epi` (its
-// own pointer).
+// own pointer).  spt <= 0: rows too wide for a stage.
 __device__ __forceinline__ int produce_sell_lanes(TileRing *R, int64_t s_lo, int64_t s_hi, int spt,
                                                   const SliceOffsets &off, const void *sval, int vbytes, int ebytes,
                                                   const int32_t *scol, const void *epi, int ne, unsigned &seq) {
+    if (spt <= 0) {
+        s_hi = s_lo;
+        spt = 1;
+    }
     const uint64_t pol = l2_evict_first_policy();
     const int lane = threadIdx.x & 31;
-    for (int64_t s0 = s_lo; s0 < s_hi; s0 += spt, ++seq) {
+    int64_t s0 = s_lo;
+    do {
         const int s = (int)(seq % kStages);
         const unsigned use = seq / kStages;
         int st = 0;
-        if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u);
+        if (lane == 0 && use > 0) st = producer_wait(R, &R->empty[s], (use - 1) & 1u, false);
         st = __shfl_sync(0xffffffffu, st, 0);
         if (st) return st;
         const int64_t s1 = s0 + spt < s_hi ? s0 + spt : s_hi;
@@ -435,11 +440,12 @@ __device__ __forceinline__ int produce_sell_lanes(TileRing *R, int64_t s_lo, int
                               lane == 0 ? (const unsigned char *)sval + e0 * vbytes
                                         : (const unsigned char *)(scol + e0),
                               lane == 0 ? bv : bc, &R->full[s], pol);
-        } else if (lane < 2 + ne) {
+        } else if (lane < 2 + ne && be > 0) {
             bulk_g2s(dst + bv + bc + (size_t)(lane - 2) * spt * 32 * ebytes,
                      (const unsigned char *)epi + s0 * 32 * ebytes, be, &R->full[s]);
         }
-    }
+        ++seq;
+    } while ((s0 += spt) < s_hi);
     return 0;
 }
 
