@@ -781,9 +781,10 @@ struct NoHook {
 };
 
 // PC: the forms of the ILU(0) preconditioner passes that the engine is built
-// with: none, streamed (ilu_wide), by slots (ilu_flow), or those of a batch,
-// whose systems may have either form, and of complex values (ilu_wide and
-// ilu_levels).  What is not built in takes no registers from the kernel's
+// with: none, streamed (ilu_wide), by slots (ilu_flow, single solves of real
+// systems), a barrier per level (ilu_levels), or, for a batch whose systems
+// differ in it, ilu_wide and ilu_levels.  What is not built in takes no
+// registers from the kernel's
 // loop: with two forms in one kernel the FP64 one spilled 276 bytes a thread,
 // with the streamed form alone 120 (multicolour ILU(0) at 96^3: 31.0 -> 30.0
 // ms, refined 3x3-block system 2840 -> 2480 us).
@@ -792,7 +793,7 @@ struct NoHook {
 //
 // The consumer threads run inner() and the other members; the producer warp
 // runs serve() beside them.
-enum { kNoIlu, kIluWide, kIluFlow, kIluAny };
+enum { kNoIlu, kIluWide, kIluFlow, kIluLevels, kIluAny };
 template <typename T, int PC = kNoIlu, int EW = 1>
 struct Engine {
     using S = typename coef_of<T>::type;                      // FP64 coefficient
@@ -1248,6 +1249,7 @@ struct Engine {
     __device__ __forceinline__ bool ilu_solve_body(const T *v, T *out) {
         if constexpr (PC == kIluWide) return ilu_wide(v, out);
         else if constexpr (PC == kIluFlow) return ilu_flow(v, out);
+        else if constexpr (PC == kIluLevels) return ilu_levels(v, out);
         else return sys().ilu.llev ? ilu_wide(v, out) : ilu_levels(v, out);
     }
     // out = M^{-1} v: L z = v by forward substitution (unit diagonal), then
@@ -1335,7 +1337,15 @@ struct Engine {
     // slices read by coalesced loads 100 us.)  Each row is one sequential sum
     // in pattern order.
     __device__ __forceinline__ bool ilu_wide(const T *v, T *out) {
-        constexpr int W = sizeof(T) == 16 ? 3 : 6;
+        // entries gathered a tile ahead, and at a time after those (the six
+        // of a 7-point row's second colour are in flight together with 0 + 6
+        // and 2 + 4).  us of 16 iterations, complex, multicolour, 128x128x64:
+        // 3 + 2 9025, 3 + 3 8670, 2 + 4 8300, 1 + 5 7970, 0 + 6 7770 (held
+        // values spill); of 24 at 96^3, n = 8: 6 + 3 4270, 0 + 6 4180, 2 + 4
+        // 4100; refined 6 + 3 2834, 2 + 4 2790; refined complex 6 + 3 2846,
+        // 0 + 6 2913.
+        constexpr int W = sizeof(T) == 16 ? 0 : is_cx<T>::value ? 6 : 2;
+        constexpr int B = sizeof(T) == 16 ? 6 : is_cx<T>::value ? 3 : 4;
         const int lane = threadIdx.x & 31, cw = threadIdx.x >> 5;
         TileRing *const R = the_ring();
         const int nl = sys().ilu.nlev_l, nlev = nl + sys().ilu.nlev_u, spt = sys().ilu.spt;
@@ -1349,7 +1359,7 @@ struct Engine {
             ilu_share(L.ns, k0, k1);
             int st = 0, ns = 0;       // stage and slices of the tile at hand
             int row = -1, cnt = 0;
-            T t{}, x[W];
+            T t{}, x[W > 0 ? W : 1];
             // stage of tile q; its slices; false when the wait failed
             auto arrived = [&](int k, unsigned tile, int &stage, int &slices) {
                 stage = (int)(tile % kStages);
@@ -1404,11 +1414,14 @@ struct Engine {
                     if (e < cnt) t = efma(-a[32 * e], x[e], t);
                     if (e < cnt1) x[e] = out[c1[32 * e]];
                 }
-                for (int e0 = W; e0 < cnt; e0 += 2) {
-                    const T xa = out[c[32 * e0]];
-                    const T xb = e0 + 1 < cnt ? out[c[32 * (e0 + 1)]] : T{};
-                    t = efma(-a[32 * e0], xa, t);
-                    if (e0 + 1 < cnt) t = efma(-a[32 * (e0 + 1)], xb, t);
+                for (int e0 = W; e0 < cnt; e0 += B) {
+                    T xw[B];
+#pragma unroll
+                    for (int u = 0; u < B; ++u)
+                        if (e0 + u < cnt) xw[u] = out[c[32 * (e0 + u)]];
+#pragma unroll
+                    for (int u = 0; u < B; ++u)
+                        if (e0 + u < cnt) t = efma(-a[32 * (e0 + u)], xw[u], t);
                 }
                 if (row >= 0) {
                     if (up) t = t / diag(st, ns);

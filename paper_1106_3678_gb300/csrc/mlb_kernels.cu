@@ -12,8 +12,9 @@ namespace mlb {
 template <typename T>
 cudaError_t launch_solve(const SysView<T> &sys, const SolveCtl &ctl, int grid, cudaStream_t st) {
     if constexpr (is_cx<T>::value) {
-        return sys.ilu.lu ? launch_solve_pc<T, kIluAny>(sys, ctl, grid, st)
-                          : launch_solve_pc<T, kNoIlu>(sys, ctl, grid, st);
+        return !sys.ilu.lu     ? launch_solve_pc<T, kNoIlu>(sys, ctl, grid, st)
+               : sys.ilu.llev ? launch_solve_pc<T, kIluWide>(sys, ctl, grid, st)
+                              : launch_solve_pc<T, kIluLevels>(sys, ctl, grid, st);
     } else {
         if (sys.ew == 3)
             return !sys.ilu.lu     ? launch_solve_pc<T, kNoIlu, 3>(sys, ctl, grid, st)
@@ -28,7 +29,7 @@ template <typename T>
 int solve_blocks_per_sm() {
     int a = solve_blocks_per_sm_pc<T, kNoIlu>();
     if constexpr (is_cx<T>::value) {
-        a = std::min(a, solve_blocks_per_sm_pc<T, kIluAny>());
+        a = std::min({a, solve_blocks_per_sm_pc<T, kIluWide>(), solve_blocks_per_sm_pc<T, kIluLevels>()});
     } else {
         a = std::min({a, solve_blocks_per_sm_pc<T, kIluWide>(), solve_blocks_per_sm_pc<T, kIluFlow>(),
                       solve_blocks_per_sm_pc<T, kNoIlu, 3>(), solve_blocks_per_sm_pc<T, kIluWide, 3>(),
@@ -55,14 +56,14 @@ cudaError_t launch_refine(const SysView<T32> &sys, const RefView<T64> &rv, const
                    : sys.ilu.llev ? launch_refine_pc<T32, T64, kIluWide, 3>(sys, rv, ctl, rc, grid, st)
                                   : launch_refine_pc<T32, T64, kIluFlow, 3>(sys, rv, ctl, rc, grid, st);
     }
-    constexpr int kManyLevels = is_cx<T32>::value ? kIluAny : kIluFlow;
+    constexpr int kManyLevels = is_cx<T32>::value ? kIluLevels : kIluFlow;
     return !sys.ilu.lu     ? launch_refine_pc<T32, T64, kNoIlu>(sys, rv, ctl, rc, grid, st)
            : sys.ilu.llev ? launch_refine_pc<T32, T64, kIluWide>(sys, rv, ctl, rc, grid, st)
                           : launch_refine_pc<T32, T64, kManyLevels>(sys, rv, ctl, rc, grid, st);
 }
 template <typename T32, typename T64>
 int refine_blocks_per_sm() {
-    constexpr int kManyLevels = is_cx<T32>::value ? kIluAny : kIluFlow;
+    constexpr int kManyLevels = is_cx<T32>::value ? kIluLevels : kIluFlow;
     int a = std::min({refine_blocks_per_sm_pc<T32, T64, kNoIlu>(), refine_blocks_per_sm_pc<T32, T64, kIluWide>(),
                       refine_blocks_per_sm_pc<T32, T64, kManyLevels>()});
     if constexpr (!is_cx<T32>::value) {

@@ -7,9 +7,7 @@ namespace mlb {
 
 template cudaError_t launch_solve_pc<cdouble, kNoIlu>(const SysView<cdouble> &, const SolveCtl &, int,
                                                      cudaStream_t);
-template cudaError_t launch_solve_pc<cdouble, kIluAny>(const SysView<cdouble> &, const SolveCtl &, int, cudaStream_t);
 template int solve_blocks_per_sm_pc<cdouble, kNoIlu>();
-template int solve_blocks_per_sm_pc<cdouble, kIluAny>();
 template cudaError_t launch_batch_pc<cdouble, kNoIlu>(const BatchItem<cdouble> *, const BatchPlan &, int,
                                                      cudaStream_t);
 template cudaError_t launch_batch_pc<cdouble, kIluAny>(const BatchItem<cdouble> *, const BatchPlan &, int,

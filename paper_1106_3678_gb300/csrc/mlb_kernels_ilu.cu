@@ -7,9 +7,6 @@ namespace mlb {
 
 template cudaError_t launch_batch_pc<double, kIluAny>(const BatchItem<double> *, const BatchPlan &, int, cudaStream_t);
 template int batch_blocks_per_sm_pc<double, kIluAny>();
-template cudaError_t launch_refine_pc<cfloat, cdouble, kIluAny>(const SysView<cfloat> &, const RefView<cdouble> &,
-                                                             const SolveCtl &, const RefCtl &, int, cudaStream_t);
-template int refine_blocks_per_sm_pc<cfloat, cdouble, kIluAny>();
 template cudaError_t launch_batch_refine_pc<float, double, kIluAny>(const BatchItemR<float, double> *,
                                                                  const BatchPlan &, int, cudaStream_t);
 template cudaError_t launch_batch_refine_pc<cfloat, cdouble, kIluAny>(const BatchItemR<cfloat, cdouble> *,

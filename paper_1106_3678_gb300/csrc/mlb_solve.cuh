@@ -2,8 +2,9 @@
 // forms of the ILU(0) passes that the engine is built with (kNoIlu: no call to
 // them anywhere in the kernel, so the unpreconditioned kernels keep their
 // register allocation).  Included by mlb_kernels.cu (kNoIlu, and the dispatch),
-// mlb_kernels_ilu.cu (kIluAny), mlb_kernels_bsr.cu, mlb_kernels_wide.cu
-// (kIluWide) and mlb_kernels_flow.cu (kIluFlow), which compile in parallel.
+// mlb_kernels_ilu.cu and mlb_kernels_cplx.cu (the batches' kIluAny),
+// mlb_kernels_bsr.cu, mlb_kernels_wide.cu (kIluWide) and mlb_kernels_flow.cu
+// (kIluFlow, kIluLevels), which compile in parallel.
 #pragma once
 
 #include "mlb_internal.h"
@@ -382,19 +383,23 @@ extern template int refine_blocks_per_sm_pc<float, double, kNoIlu, 3>();
 extern template int refine_blocks_per_sm_pc<float, double, kIluFlow, 3>();
 extern template int refine_blocks_per_sm_pc<float, double, kIluWide, 3>();
 
-// Instantiated in mlb_kernels_ilu.cu.
+// Instantiated in mlb_kernels_wide.cu.
+extern template cudaError_t launch_solve_pc<double, kIluWide>(const SysView<double> &, const SolveCtl &, int,
+                                                              cudaStream_t);
+extern template cudaError_t launch_solve_pc<cdouble, kIluWide>(const SysView<cdouble> &, const SolveCtl &, int,
+                                                               cudaStream_t);
+extern template int solve_blocks_per_sm_pc<double, kIluWide>();
+extern template int solve_blocks_per_sm_pc<cdouble, kIluWide>();
 extern template cudaError_t launch_refine_pc<float, double, kIluWide>(const SysView<float> &, const RefView<double> &,
                                                                   const SolveCtl &, const RefCtl &, int,
                                                                   cudaStream_t);
-extern template cudaError_t launch_refine_pc<cfloat, cdouble, kIluAny>(const SysView<cfloat> &,
-                                                                    const RefView<cdouble> &, const SolveCtl &,
-                                                                    const RefCtl &, int, cudaStream_t);
 extern template cudaError_t launch_refine_pc<cfloat, cdouble, kIluWide>(const SysView<cfloat> &,
                                                                     const RefView<cdouble> &, const SolveCtl &,
                                                                     const RefCtl &, int, cudaStream_t);
 extern template int refine_blocks_per_sm_pc<float, double, kIluWide>();
-extern template int refine_blocks_per_sm_pc<cfloat, cdouble, kIluAny>();
 extern template int refine_blocks_per_sm_pc<cfloat, cdouble, kIluWide>();
+
+// Instantiated in mlb_kernels_ilu.cu.
 extern template cudaError_t launch_batch_refine_pc<float, double, kIluAny>(const BatchItemR<float, double> *,
                                                                         const BatchPlan &, int, cudaStream_t);
 extern template cudaError_t launch_batch_refine_pc<cfloat, cdouble, kIluAny>(const BatchItemR<cfloat, cdouble> *,
@@ -410,15 +415,10 @@ extern template cudaError_t launch_batch_pc<cdouble, kNoIlu>(const BatchItem<cdo
                                                             cudaStream_t);
 extern template int batch_blocks_per_sm_pc<cdouble, kNoIlu>();
 
-extern template cudaError_t launch_solve_pc<double, kIluWide>(const SysView<double> &, const SolveCtl &, int, cudaStream_t);
-extern template cudaError_t launch_solve_pc<cdouble, kIluAny>(const SysView<cdouble> &, const SolveCtl &, int,
-                                                          cudaStream_t);
 extern template cudaError_t launch_batch_pc<double, kIluAny>(const BatchItem<double> *, const BatchPlan &, int,
                                                          cudaStream_t);
 extern template cudaError_t launch_batch_pc<cdouble, kIluAny>(const BatchItem<cdouble> *, const BatchPlan &, int,
                                                           cudaStream_t);
-extern template int solve_blocks_per_sm_pc<double, kIluWide>();
-extern template int solve_blocks_per_sm_pc<cdouble, kIluAny>();
 extern template int batch_blocks_per_sm_pc<double, kIluAny>();
 extern template int batch_blocks_per_sm_pc<cdouble, kIluAny>();
 
@@ -430,5 +430,12 @@ extern template cudaError_t launch_refine_pc<float, double, kIluFlow>(const SysV
                                                                       const SolveCtl &, const RefCtl &, int,
                                                                       cudaStream_t);
 extern template int refine_blocks_per_sm_pc<float, double, kIluFlow>();
+extern template cudaError_t launch_solve_pc<cdouble, kIluLevels>(const SysView<cdouble> &, const SolveCtl &, int,
+                                                                 cudaStream_t);
+extern template int solve_blocks_per_sm_pc<cdouble, kIluLevels>();
+extern template cudaError_t launch_refine_pc<cfloat, cdouble, kIluLevels>(const SysView<cfloat> &,
+                                                                          const RefView<cdouble> &, const SolveCtl &,
+                                                                          const RefCtl &, int, cudaStream_t);
+extern template int refine_blocks_per_sm_pc<cfloat, cdouble, kIluLevels>();
 
 }  // namespace mlb
