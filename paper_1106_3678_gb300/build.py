@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(ROOT, "_build", "obj")
 LIB = os.path.join(HERE, "libmlbicgstab.so")
 HEADER = os.path.join(ROOT, "include", "mlbicgstab.h")
-SOURCES = ["mlb_kernels.cu", "mlb_kernels_ilu.cu", "mlb_kernels_wide.cu",
+SOURCES = ["mlb_kernels.cu", "mlb_kernels_ilu.cu", "mlb_kernels_ilu32.cu", "mlb_kernels_wide.cu",
            "mlb_kernels_flow.cu", "mlb_kernels_cplx.cu", "mlb_kernels_bsr.cu", "mlb_api.cu",
            "mlb_noalloc.cu", "mlb_ilu.cu"]
 

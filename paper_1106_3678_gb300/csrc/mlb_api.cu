@@ -1286,21 +1286,25 @@ int mlbicgstab_solve_batch(mlb_handle *const *hs, int32_t count, const void *con
     }
     MLB_CUDA(cudaMemcpyAsync(dws, hws, off_slots, cudaMemcpyHostToDevice, st));
     if (slot_bytes) MLB_CUDA(cudaMemsetAsync(dws + off_slots, 0, slot_bytes, st));
-    bool any_ilu = false;
-    for (int q = 0; q < count; ++q) any_ilu = any_ilu || has_ilu(hs[q]);
+    int form = kNoIlu;
+    for (int q = 0; q < count; ++q) {
+        if (!has_ilu(hs[q])) continue;
+        const int f = hs[q]->ilu_llev ? kIluWide : kIluLevels;
+        form = form == kNoIlu || form == f ? f : kIluAny;
+    }
     const void *ditems = dws + off_items;
     MLB_CUDA(cudaEventRecord(h0->ev0, st));
     cudaError_t e;
     if (refined) {
         if (cplx)
-            e = launch_batch_refine<cfloat, cdouble>((const BatchItemR<cfloat, cdouble> *)ditems, plan, grid, any_ilu,
+            e = launch_batch_refine<cfloat, cdouble>((const BatchItemR<cfloat, cdouble> *)ditems, plan, grid, form,
                                                      st);
         else
-            e = launch_batch_refine<float, double>((const BatchItemR<float, double> *)ditems, plan, grid, any_ilu, st);
+            e = launch_batch_refine<float, double>((const BatchItemR<float, double> *)ditems, plan, grid, form, st);
     } else if (cplx) {
-        e = launch_batch<cdouble>((const BatchItem<cdouble> *)ditems, plan, grid, any_ilu, st);
+        e = launch_batch<cdouble>((const BatchItem<cdouble> *)ditems, plan, grid, form, st);
     } else {
-        e = launch_batch<double>((const BatchItem<double> *)ditems, plan, grid, any_ilu, st);
+        e = launch_batch<double>((const BatchItem<double> *)ditems, plan, grid, form, st);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();

@@ -78,12 +78,14 @@ struct BatchPlan {
     Slot *sslots;            // per position of order_big: 2 * kMaxSums * team slots (zeroed)
     uint64_t timeout_ns;     // limit of the waits between turns
 };
-// ilu: some item has an ILU(0) preconditioner (the kernel with those passes
-// then runs every item, each by its own view).
+// form: the form of the ILU(0) passes that the items with that preconditioner
+// have (kNoIlu: none has it; kIluWide, kIluLevels; kIluAny: some the one and
+// some the other).  The kernel with those passes runs every item, each by its
+// own view.
 template <typename T>
-cudaError_t launch_batch(const BatchItem<T> *items, const BatchPlan &plan, int grid, bool ilu, cudaStream_t st);
+cudaError_t launch_batch(const BatchItem<T> *items, const BatchPlan &plan, int grid, int form, cudaStream_t st);
 template <typename T32, typename T64>
-cudaError_t launch_batch_refine(const BatchItemR<T32, T64> *items, const BatchPlan &plan, int grid, bool ilu,
+cudaError_t launch_batch_refine(const BatchItemR<T32, T64> *items, const BatchPlan &plan, int grid, int form,
                                 cudaStream_t st);
 template <typename T>
 int batch_blocks_per_sm();

@@ -38,12 +38,16 @@ int solve_blocks_per_sm() {
     return a;
 }
 template <typename T>
-cudaError_t launch_batch(const BatchItem<T> *items, const BatchPlan &plan, int grid, bool ilu, cudaStream_t st) {
-    return ilu ? launch_batch_pc<T, kIluAny>(items, plan, grid, st) : launch_batch_pc<T, kNoIlu>(items, plan, grid, st);
+cudaError_t launch_batch(const BatchItem<T> *items, const BatchPlan &plan, int grid, int form, cudaStream_t st) {
+    return form == kNoIlu     ? launch_batch_pc<T, kNoIlu>(items, plan, grid, st)
+           : form == kIluWide ? launch_batch_pc<T, kIluWide>(items, plan, grid, st)
+           : form == kIluLevels ? launch_batch_pc<T, kIluLevels>(items, plan, grid, st)
+                                : launch_batch_pc<T, kIluAny>(items, plan, grid, st);
 }
 template <typename T>
 int batch_blocks_per_sm() {
-    return std::min(batch_blocks_per_sm_pc<T, kNoIlu>(), batch_blocks_per_sm_pc<T, kIluAny>());
+    return std::min({batch_blocks_per_sm_pc<T, kNoIlu>(), batch_blocks_per_sm_pc<T, kIluWide>(),
+                     batch_blocks_per_sm_pc<T, kIluLevels>(), batch_blocks_per_sm_pc<T, kIluAny>()});
 }
 
 // FP32-inner / FP64-refined launches, likewise.
@@ -74,15 +78,19 @@ int refine_blocks_per_sm() {
     return a;
 }
 template <typename T32, typename T64>
-cudaError_t launch_batch_refine(const BatchItemR<T32, T64> *items, const BatchPlan &plan, int grid, bool ilu,
+cudaError_t launch_batch_refine(const BatchItemR<T32, T64> *items, const BatchPlan &plan, int grid, int form,
                                 cudaStream_t st) {
-    return ilu ? launch_batch_refine_pc<T32, T64, kIluAny>(items, plan, grid, st)
-               : launch_batch_refine_pc<T32, T64, kNoIlu>(items, plan, grid, st);
+    return form == kNoIlu     ? launch_batch_refine_pc<T32, T64, kNoIlu>(items, plan, grid, st)
+           : form == kIluWide ? launch_batch_refine_pc<T32, T64, kIluWide>(items, plan, grid, st)
+           : form == kIluLevels ? launch_batch_refine_pc<T32, T64, kIluLevels>(items, plan, grid, st)
+                                : launch_batch_refine_pc<T32, T64, kIluAny>(items, plan, grid, st);
 }
 template <typename T32, typename T64>
 int batch_refine_blocks_per_sm() {
-    return std::min(batch_refine_blocks_per_sm_pc<T32, T64, kNoIlu>(),
-                    batch_refine_blocks_per_sm_pc<T32, T64, kIluAny>());
+    return std::min({batch_refine_blocks_per_sm_pc<T32, T64, kNoIlu>(),
+                     batch_refine_blocks_per_sm_pc<T32, T64, kIluWide>(),
+                     batch_refine_blocks_per_sm_pc<T32, T64, kIluLevels>(),
+                     batch_refine_blocks_per_sm_pc<T32, T64, kIluAny>()});
 }
 
 // FP64 -> FP32 copies (matrix values, Q, F); interleaved complex data is a
@@ -487,12 +495,12 @@ template cudaError_t launch_refine<cfloat, cdouble>(const SysView<cfloat> &, con
                                                     const SolveCtl &, const RefCtl &, int, cudaStream_t);
 template int refine_blocks_per_sm<float, double>();
 template int refine_blocks_per_sm<cfloat, cdouble>();
-template cudaError_t launch_batch<double>(const BatchItem<double> *, const BatchPlan &, int, bool, cudaStream_t);
-template cudaError_t launch_batch<cdouble>(const BatchItem<cdouble> *, const BatchPlan &, int, bool, cudaStream_t);
+template cudaError_t launch_batch<double>(const BatchItem<double> *, const BatchPlan &, int, int, cudaStream_t);
+template cudaError_t launch_batch<cdouble>(const BatchItem<cdouble> *, const BatchPlan &, int, int, cudaStream_t);
 template cudaError_t launch_batch_refine<float, double>(const BatchItemR<float, double> *, const BatchPlan &, int,
-                                                        bool, cudaStream_t);
+                                                        int, cudaStream_t);
 template cudaError_t launch_batch_refine<cfloat, cdouble>(const BatchItemR<cfloat, cdouble> *, const BatchPlan &,
-                                                          int, bool, cudaStream_t);
+                                                          int, int, cudaStream_t);
 template int batch_blocks_per_sm<double>();
 template int batch_blocks_per_sm<cdouble>();
 template int batch_refine_blocks_per_sm<float, double>();

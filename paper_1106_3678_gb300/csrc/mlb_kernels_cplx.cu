@@ -10,9 +10,6 @@ template cudaError_t launch_solve_pc<cdouble, kNoIlu>(const SysView<cdouble> &, 
 template int solve_blocks_per_sm_pc<cdouble, kNoIlu>();
 template cudaError_t launch_batch_pc<cdouble, kNoIlu>(const BatchItem<cdouble> *, const BatchPlan &, int,
                                                      cudaStream_t);
-template cudaError_t launch_batch_pc<cdouble, kIluAny>(const BatchItem<cdouble> *, const BatchPlan &, int,
-                                                    cudaStream_t);
 template int batch_blocks_per_sm_pc<cdouble, kNoIlu>();
-template int batch_blocks_per_sm_pc<cdouble, kIluAny>();
 
 }  // namespace mlb

@@ -2,7 +2,7 @@
 // forms of the ILU(0) passes that the engine is built with (kNoIlu: no call to
 // them anywhere in the kernel, so the unpreconditioned kernels keep their
 // register allocation).  Included by mlb_kernels.cu (kNoIlu, and the dispatch),
-// mlb_kernels_ilu.cu and mlb_kernels_cplx.cu (the batches' kIluAny),
+// mlb_kernels_ilu.cu and mlb_kernels_ilu32.cu (batches), mlb_kernels_cplx.cu,
 // mlb_kernels_bsr.cu, mlb_kernels_wide.cu (kIluWide) and mlb_kernels_flow.cu
 // (kIluFlow, kIluLevels), which compile in parallel.
 #pragma once
@@ -399,12 +399,24 @@ extern template cudaError_t launch_refine_pc<cfloat, cdouble, kIluWide>(const Sy
 extern template int refine_blocks_per_sm_pc<float, double, kIluWide>();
 extern template int refine_blocks_per_sm_pc<cfloat, cdouble, kIluWide>();
 
-// Instantiated in mlb_kernels_ilu.cu.
+// Instantiated in mlb_kernels_ilu32.cu.
+extern template cudaError_t launch_batch_refine_pc<float, double, kIluWide>(const BatchItemR<float, double> *,
+                                                                   const BatchPlan &, int, cudaStream_t);
+extern template int batch_refine_blocks_per_sm_pc<float, double, kIluWide>();
+extern template cudaError_t launch_batch_refine_pc<float, double, kIluLevels>(const BatchItemR<float, double> *,
+                                                                   const BatchPlan &, int, cudaStream_t);
+extern template int batch_refine_blocks_per_sm_pc<float, double, kIluLevels>();
 extern template cudaError_t launch_batch_refine_pc<float, double, kIluAny>(const BatchItemR<float, double> *,
-                                                                        const BatchPlan &, int, cudaStream_t);
-extern template cudaError_t launch_batch_refine_pc<cfloat, cdouble, kIluAny>(const BatchItemR<cfloat, cdouble> *,
-                                                                          const BatchPlan &, int, cudaStream_t);
+                                                                   const BatchPlan &, int, cudaStream_t);
 extern template int batch_refine_blocks_per_sm_pc<float, double, kIluAny>();
+extern template cudaError_t launch_batch_refine_pc<cfloat, cdouble, kIluWide>(const BatchItemR<cfloat, cdouble> *,
+                                                                   const BatchPlan &, int, cudaStream_t);
+extern template int batch_refine_blocks_per_sm_pc<cfloat, cdouble, kIluWide>();
+extern template cudaError_t launch_batch_refine_pc<cfloat, cdouble, kIluLevels>(const BatchItemR<cfloat, cdouble> *,
+                                                                   const BatchPlan &, int, cudaStream_t);
+extern template int batch_refine_blocks_per_sm_pc<cfloat, cdouble, kIluLevels>();
+extern template cudaError_t launch_batch_refine_pc<cfloat, cdouble, kIluAny>(const BatchItemR<cfloat, cdouble> *,
+                                                                   const BatchPlan &, int, cudaStream_t);
 extern template int batch_refine_blocks_per_sm_pc<cfloat, cdouble, kIluAny>();
 
 // Instantiated in mlb_kernels_cplx.cu.
@@ -415,11 +427,24 @@ extern template cudaError_t launch_batch_pc<cdouble, kNoIlu>(const BatchItem<cdo
                                                             cudaStream_t);
 extern template int batch_blocks_per_sm_pc<cdouble, kNoIlu>();
 
+// Instantiated in mlb_kernels_ilu.cu.
+extern template cudaError_t launch_batch_pc<double, kIluWide>(const BatchItem<double> *, const BatchPlan &, int,
+                                                    cudaStream_t);
+extern template int batch_blocks_per_sm_pc<double, kIluWide>();
+extern template cudaError_t launch_batch_pc<double, kIluLevels>(const BatchItem<double> *, const BatchPlan &, int,
+                                                    cudaStream_t);
+extern template int batch_blocks_per_sm_pc<double, kIluLevels>();
 extern template cudaError_t launch_batch_pc<double, kIluAny>(const BatchItem<double> *, const BatchPlan &, int,
-                                                         cudaStream_t);
-extern template cudaError_t launch_batch_pc<cdouble, kIluAny>(const BatchItem<cdouble> *, const BatchPlan &, int,
-                                                          cudaStream_t);
+                                                    cudaStream_t);
 extern template int batch_blocks_per_sm_pc<double, kIluAny>();
+extern template cudaError_t launch_batch_pc<cdouble, kIluWide>(const BatchItem<cdouble> *, const BatchPlan &, int,
+                                                    cudaStream_t);
+extern template int batch_blocks_per_sm_pc<cdouble, kIluWide>();
+extern template cudaError_t launch_batch_pc<cdouble, kIluLevels>(const BatchItem<cdouble> *, const BatchPlan &, int,
+                                                    cudaStream_t);
+extern template int batch_blocks_per_sm_pc<cdouble, kIluLevels>();
+extern template cudaError_t launch_batch_pc<cdouble, kIluAny>(const BatchItem<cdouble> *, const BatchPlan &, int,
+                                                    cudaStream_t);
 extern template int batch_blocks_per_sm_pc<cdouble, kIluAny>();
 
 // Instantiated in mlb_kernels_flow.cu.
