@@ -1028,10 +1028,13 @@ struct Engine {
         if constexpr (PC != kNoIlu) {
             if (sys().ilu.lu) xin = sys().ilu.t;
         }
-        // FP32 and complex engines: a pipelined width of 7, the widest row of
-        // the 3-D stencils, FP32 with both forms of ILU(0) 4 (fewer registers
-        // of gathered x); the real FP64 engine keeps 8 (no gain at 7)
-        constexpr int W = is_narrow<T>::value && PC == kIluAny ? 4 : is_narrow<T>::value || is_cx<T>::value ? 7 : 8;
+        // pipelined entries: what the registers hold.  FP32 engines 7, the
+        // widest row of the 3-D stencils, 4 with both forms of ILU(0); the real
+        // FP64 engine 8 (no gain at 7); the complex FP64 engine 3 (with 7
+        // gathered values of 16 bytes the loop spilled: batch of 96 small
+        // systems 4.71 -> 4.33 ms, 4.55 before the passes shared one loop;
+        // 128x128x32, 16 iterations, 3.05 -> 2.83 ms)
+        constexpr int W = sizeof(T) == 16 ? 3 : is_narrow<T>::value ? (PC == kIluAny ? 4 : 7) : 8;
         const bool okw = sell_consume<1, EW, W, true>(the_ring(), sq, s_lo(), s_hi(), spt, sys().slice_ptr,
                                                       sys().scol, sys().sval, xin, epi, fin, acc);
         if (!okw) tile_lost();
