@@ -5,6 +5,7 @@
 // device memory instead of caller or library allocations.  Every GPU that
 // loads the library holds this array until the process exits.
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "../../include/mlbicgstab.h"
@@ -89,6 +90,38 @@ __device__ __forceinline__ double warp_sums(double (&a)[V]) {
     return a[0];
 }
 
+// The CTA's sums of the threads' values, one per value and CTA, to `part`.
+template <typename T, int NB>
+__device__ __forceinline__ void cta_parts(const typename real_of<T>::type *acc, int n, double *part) {
+    constexpr int DS = dslots<T>(), V = NB * DS;
+    constexpr int GV = V < 8 ? V : 8;                // sums taken together
+    __shared__ double red[kNaWarps][V];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // GV values at a time (every index into acc a constant: a run-time index
+    // would put acc in local memory)
+#pragma unroll
+    for (int v0 = 0; v0 < V; v0 += GV) {
+        if (v0 < n * DS) {
+            double a[GV];
+#pragma unroll
+            for (int k = 0; k < GV; ++k) a[k] = (double)acc[v0 + k];
+            const double t = warp_sums<GV>(a);
+            if (lane % (32 / GV) == 0) red[warp][v0 + lane / (32 / GV)] = t;
+        }
+    }
+    __syncthreads();
+    for (int v = threadIdx.x; v < n * DS; v += kNaThreads) {
+        double t[kNaWarps];
+#pragma unroll
+        for (int w = 0; w < kNaWarps; ++w) t[w] = red[w][v];
+#pragma unroll
+        for (int h = kNaWarps / 2; h > 0; h /= 2)
+#pragma unroll
+            for (int w = 0; w < h; ++w) t[w] += t[w + h];
+        part[(size_t)v * gridDim.x + blockIdx.x] = t[0];
+    }
+}
+
 // CTAs an SM holds: as many as the accumulators (NB * DS doubles a thread)
 // and the loads in flight leave registers for.
 template <typename T, int NB>
@@ -116,8 +149,9 @@ constexpr size_t na_smem() {
 // entries of Q are in flight together.  us a call, before -> now: 101^3, n = 8:
 // 65 -> 46 (3.8 TB/s), n = 4: 48 -> 44; 40^3: 25 -> 10.  It is as fast with 2 as
 // with 3 CTAs per SM, and a third stage gives 1 us.
-// Rows too long for the staging are read directly.  Each row is one
-// sequential sum in the order of its entries.
+// Rows too long for the staging are read directly (where they are so long on
+// average the kernel below may run instead).  Each row is one sequential sum in
+// the order of its entries.
 template <typename T, int NB>
 __global__ void __launch_bounds__(kNaThreads, na_ctas<T, NB>())
     spmv_qdot_csr_kernel(int64_t N, const int64_t *rp, const int32_t *ci, const T *av, const T *x,
@@ -125,10 +159,8 @@ __global__ void __launch_bounds__(kNaThreads, na_ctas<T, NB>())
     constexpr int DS = dslots<T>(), V = NB * DS, CAP = na_cap<T>(), ST = kNaStages;
     constexpr int B = DS == 1 ? 7 : 4;               // gathers of x in flight (8: 47 for 46 us)
     constexpr int NQ = V <= 8 ? NB : 0;              // entries of Q loaded ahead
-    constexpr int GV = V < 8 ? V : 8;                // sums taken together
     using ACC = typename real_of<T>::type;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ double red[kNaWarps][V];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     T *const vbuf = reinterpret_cast<T *>(smem) + (size_t)warp * ST * CAP;
     int32_t *const cbuf = reinterpret_cast<int32_t *>(smem + (size_t)kNaWarps * ST * CAP * sizeof(T)) +
@@ -216,29 +248,38 @@ __global__ void __launch_bounds__(kNaThreads, na_ctas<T, NB>())
         e[ST - 1] = e2;
     }
     asm volatile("griddepcontrol.launch_dependents;");
-    // the CTA's sums, GV values at a time (every index into acc a constant:
-    // a run-time index would put acc in local memory)
+    cta_parts<T, NB>(acc, n, part);
+}
+
+// The same for long rows and few sums: each lane walks its row.  A row's loads
+// wait for one another, so the threads hide the latency: no staging, 40 to 74
+// registers, as many CTAs as an SM holds (6 of n <= 4; the kernel above holds
+// 2).  us a call, that kernel -> this one: 64x64x32 reservoir matrix (21 entries
+// a row) n = 1 44 -> 39, n = 4 49 -> 41; 27-point 64^3 n = 4 40 -> 37; 30,000
+// rows of 130 39 -> 33; complex, 27-point 48^3 n = 1 41 -> 35, n = 8 47 -> 41,
+// 60 entries a row 39 -> 26.  With more sums the registers take the CTAs away
+// again (real, 130 entries, n = 8 37 -> 41, n = 16 39 -> 54).
+template <typename T, int NB>
+__global__ void __launch_bounds__(kNaThreads)
+    spmv_qdot_csr_long_kernel(int64_t N, const int64_t *rp, const int32_t *ci, const T *av, const T *x,
+                              const T *Q, int64_t ldq, int n, T *y, double *part) {
+    constexpr int DS = dslots<T>(), V = NB * DS;
+    using ACC = typename real_of<T>::type;
+    ACC acc[V];
 #pragma unroll
-    for (int v0 = 0; v0 < V; v0 += GV) {
-        if (v0 < n * DS) {
-            double a[GV];
+    for (int k = 0; k < V; ++k) acc[k] = ACC(0);
+    for (int64_t row = (int64_t)blockIdx.x * kNaThreads + threadIdx.x; row < N;
+         row += (int64_t)gridDim.x * kNaThreads) {
+        T sum{};
+        for (int64_t k = __ldg(rp + row), k1 = __ldg(rp + row + 1); k < k1; ++k)
+            sum = efma(ldv(av + k), ldv(x + __ldg(ci + k)), sum);
+        y[row] = sum;
 #pragma unroll
-            for (int k = 0; k < GV; ++k) a[k] = (double)acc[v0 + k];
-            const double t = warp_sums<GV>(a);
-            if (lane % (32 / GV) == 0) red[warp][v0 + lane / (32 / GV)] = t;
-        }
+        for (int q = 0; q < NB; ++q)
+            if (q < n) acc_dot(&acc[q * DS], ldv(Q + (int64_t)q * ldq + row), sum);
     }
-    __syncthreads();
-    for (int v = threadIdx.x; v < n * DS; v += kNaThreads) {
-        double t[kNaWarps];
-#pragma unroll
-        for (int w = 0; w < kNaWarps; ++w) t[w] = red[w][v];
-#pragma unroll
-        for (int h = kNaWarps / 2; h > 0; h /= 2)
-#pragma unroll
-            for (int w = 0; w < h; ++w) t[w] += t[w + h];
-        part[(size_t)v * gridDim.x + blockIdx.x] = t[0];
-    }
+    asm volatile("griddepcontrol.launch_dependents;");
+    cta_parts<T, NB>(acc, n, part);
 }
 
 // d from the CTAs' sums: one warp per value, lanes over the CTAs in index
@@ -268,22 +309,48 @@ __global__ void __launch_bounds__(1024) sum_parts_kernel(const double *part, int
     }
 }
 
+// CTAs that device `dev` holds of a kernel with `smem` bytes of dynamic shared
+// memory, 0 on failure; asked for once per device (`ctas`: zeroed, one set per
+// kernel).
+template <typename Kernel>
+int device_ctas(int dev, Kernel kernel, size_t smem, std::atomic<int> (&ctas)[256]) {
+    int c = ctas[dev].load(std::memory_order_acquire);
+    if (c > 0) return c;
+    int sms = 0, per_sm = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kNaThreads, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    c = sms * std::max(per_sm, 1);
+    ctas[dev].store(c, std::memory_order_release);
+    return c;
+}
+
 template <typename T, int NB>
-int launch(int dev, int64_t N, const int64_t *rp, const int32_t *ci, const T *av, const T *x, const T *Q,
+int launch(int dev, int64_t N, int64_t nnz, const int64_t *rp, const int32_t *ci, const T *av, const T *x, const T *Q,
            int64_t ldq, int n, T *y, T *d, double *scratch, cudaStream_t st) {
     constexpr int DS = dslots<T>();
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaFuncSetAttribute(spmv_qdot_csr_kernel<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)na_smem<T>()) != cudaSuccess) {
-        cudaGetLastError();
-        return MLB_ERR_CUDA;
+    auto *kernel = spmv_qdot_csr_kernel<T, NB>;
+    size_t smem = na_smem<T>();
+    static std::atomic<int> staged[256], walked[256];
+    auto *held = &staged;
+    // the line: rows that on average do not fit the staging, and as many sums
+    // as the other kernel has registers for (see there)
+    if constexpr (NB <= (DS == 1 ? 4 : 8)) {
+        if (nnz > N * (na_cap<T>() / 32)) {
+            kernel = spmv_qdot_csr_long_kernel<T, NB>;
+            smem = 0;
+            held = &walked;
+        }
     }
-    int64_t grid = (int64_t)sms * na_ctas<T, NB>();
+    const int ctas = device_ctas(dev, kernel, smem, *held);
+    if (ctas == 0) return MLB_ERR_CUDA;
     const int64_t fit = kNaScratchDoubles / ((int64_t)NB * DS);
     const int64_t need = (N + kNaThreads - 1) / kNaThreads;
-    grid = std::min(grid, std::min(fit, need));
-    spmv_qdot_csr_kernel<T, NB><<<(int)grid, kNaThreads, na_smem<T>(), st>>>(N, rp, ci, av, x, Q, ldq, n, y, scratch);
+    const int64_t grid = std::min<int64_t>(ctas, std::min(fit, need));
+    kernel<<<(int)grid, kNaThreads, smem, st>>>(N, rp, ci, av, x, Q, ldq, n, y, scratch);
     if (cudaGetLastError() != cudaSuccess) return MLB_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(1);
@@ -303,13 +370,13 @@ int launch(int dev, int64_t N, const int64_t *rp, const int32_t *ci, const T *av
 }
 
 template <typename T>
-int dispatch(int dev, int64_t N, const int64_t *rp, const int32_t *ci, const T *av, const T *x, const T *Q,
-             int64_t ldq, int n, T *y, T *d, double *scratch, cudaStream_t st) {
-    if (n <= 4) return launch<T, 4>(dev, N, rp, ci, av, x, Q, ldq, n, y, d, scratch, st);
-    if (n <= 8) return launch<T, 8>(dev, N, rp, ci, av, x, Q, ldq, n, y, d, scratch, st);
-    if (n <= 16) return launch<T, 16>(dev, N, rp, ci, av, x, Q, ldq, n, y, d, scratch, st);
-    if (n <= 32) return launch<T, 32>(dev, N, rp, ci, av, x, Q, ldq, n, y, d, scratch, st);
-    return launch<T, kNaMaxN>(dev, N, rp, ci, av, x, Q, ldq, n, y, d, scratch, st);
+int dispatch(int dev, int64_t N, int64_t nnz, const int64_t *rp, const int32_t *ci, const T *av, const T *x,
+             const T *Q, int64_t ldq, int n, T *y, T *d, double *scratch, cudaStream_t st) {
+    if (n <= 4) return launch<T, 4>(dev, N, nnz, rp, ci, av, x, Q, ldq, n, y, d, scratch, st);
+    if (n <= 8) return launch<T, 8>(dev, N, nnz, rp, ci, av, x, Q, ldq, n, y, d, scratch, st);
+    if (n <= 16) return launch<T, 16>(dev, N, nnz, rp, ci, av, x, Q, ldq, n, y, d, scratch, st);
+    if (n <= 32) return launch<T, 32>(dev, N, nnz, rp, ci, av, x, Q, ldq, n, y, d, scratch, st);
+    return launch<T, kNaMaxN>(dev, N, nnz, rp, ci, av, x, Q, ldq, n, y, d, scratch, st);
 }
 
 // Device memory of the current device `dev`, or managed memory.  Memory of
@@ -350,8 +417,8 @@ extern "C" int mlbicgstab_spmv_qdot_noalloc(int64_t nrows, int64_t nnz, const in
     if (rc != MLB_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     if (dtype == MLB_C128)
-        return dispatch<cdouble>(dev, nrows, row_ptr, col_idx, (const cdouble *)values, (const cdouble *)x,
+        return dispatch<cdouble>(dev, nrows, nnz, row_ptr, col_idx, (const cdouble *)values, (const cdouble *)x,
                                  (const cdouble *)Q, ldq, n, (cdouble *)y, (cdouble *)d, scratch, st);
-    return dispatch<double>(dev, nrows, row_ptr, col_idx, (const double *)values, (const double *)x,
+    return dispatch<double>(dev, nrows, nnz, row_ptr, col_idx, (const double *)values, (const double *)x,
                             (const double *)Q, ldq, n, (double *)y, (double *)d, scratch, st);
 }

@@ -209,3 +209,35 @@ def test_noalloc_rows_of_any_length(case, N, longest):
     assert np.all(np.abs(yn - y_or) <= bound_y)
     bound_d = np.abs(Q) @ bound_y + 2 * _gamma(N) * (np.abs(Q) @ np.abs(y_or))
     assert np.all(np.abs(dn - d_or) <= bound_d)
+
+
+@pytest.mark.parametrize("case", ["real", "complex"])
+@pytest.mark.parametrize("N,n", [(1, 1), (255, 1), (257, 4), (1000, 9), (777, 17), (513, 40), (40001, 64)])
+def test_noalloc_long_rows(case, N, n):
+    """Rows of 10 to 40 entries: without staging for few columns of Q, read
+    directly for more, every number of accumulators, CTAs with few rows.
+    Bounds as above."""
+    import torch
+    import oracle as O
+    rng = np.random.default_rng(100 * N + n)
+    lens = rng.integers(10, 41, size=N)
+    lens[N // 2:N // 2 + 3] = 0 if N > 100 else 10
+    rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    nnz = int(rp[-1])
+    A = W.CSR(row_ptr=rp, col=rng.integers(0, N, size=nnz).astype(np.int32), val=_rand(rng, nnz, case), n_rows=N)
+    x, Q = _rand(rng, N, case), np.stack([_rand(rng, N, case) for _ in range(n)])
+    y_or = O.spmv(A, x)
+    d_or = Q.conj() @ y_or
+    dt = torch.complex128 if case == "complex" else torch.float64
+    y = torch.full((N,), float("nan"), dtype=dt, device="cuda")
+    d = torch.full((n,), float("nan"), dtype=dt, device="cuda")
+    M.mlbicgstab_spmv_qdot_noalloc(torch.tensor(rp, device="cuda"), torch.tensor(A.col, device="cuda"),
+                                   torch.tensor(A.val, dtype=dt, device="cuda"),
+                                   torch.tensor(x, dtype=dt, device="cuda"), torch.tensor(Q, dtype=dt, device="cuda"),
+                                   y, d)
+    torch.cuda.synchronize()
+    yn, dn = y.cpu().numpy(), d.cpu().numpy()
+    bound_y = 2 * _gamma(41) * _abs_product(A, x)
+    assert np.all(np.abs(yn - y_or) <= bound_y)
+    bound_d = np.abs(Q) @ bound_y + 2 * _gamma(N) * (np.abs(Q) @ np.abs(y_or))
+    assert np.all(np.abs(dn - d_or) <= bound_d)
