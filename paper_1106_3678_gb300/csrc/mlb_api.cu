@@ -675,19 +675,11 @@ int create_impl(mlb_handle *h, const mlb_matrix *A, const mlb_matrix *AH, const 
         if ((rc = dev_alloc_t(h, &h->ilu_ci, (size_t)ih.nnz * 4))) return rc;
         if ((rc = dev_alloc(h, &h->ilu_lu, (size_t)ih.nnz * es))) return rc;
         if ((rc = dev_alloc_t(h, &h->ilu_dpos, (size_t)N * 4))) return rc;
-        if ((rc = dev_alloc_t(h, &h->ilu_lrows, (size_t)N * 4))) return rc;
-        if ((rc = dev_alloc_t(h, &h->ilu_lptr, ih.lptr.size() * 4))) return rc;
-        if ((rc = dev_alloc_t(h, &h->ilu_urows, (size_t)N * 4))) return rc;
-        if ((rc = dev_alloc_t(h, &h->ilu_uptr, ih.uptr.size() * 4))) return rc;
         if ((rc = dev_alloc(h, &h->ilu_t, vb))) return rc;
         MLB_CUDA(cudaMemcpy(h->ilu_rp, ih.rp.data(), (size_t)(N + 1) * 8, cudaMemcpyHostToDevice));
         MLB_CUDA(cudaMemcpy(h->ilu_ci, ih.ci.data(), (size_t)ih.nnz * 4, cudaMemcpyHostToDevice));
         MLB_CUDA(cudaMemcpy(h->ilu_lu, ih.lu.data(), (size_t)ih.nnz * es, cudaMemcpyHostToDevice));
         MLB_CUDA(cudaMemcpy(h->ilu_dpos, ih.dpos.data(), (size_t)N * 4, cudaMemcpyHostToDevice));
-        MLB_CUDA(cudaMemcpy(h->ilu_lrows, ih.lrows.data(), (size_t)N * 4, cudaMemcpyHostToDevice));
-        MLB_CUDA(cudaMemcpy(h->ilu_lptr, ih.lptr.data(), ih.lptr.size() * 4, cudaMemcpyHostToDevice));
-        MLB_CUDA(cudaMemcpy(h->ilu_urows, ih.urows.data(), (size_t)N * 4, cudaMemcpyHostToDevice));
-        MLB_CUDA(cudaMemcpy(h->ilu_uptr, ih.uptr.data(), ih.uptr.size() * 4, cudaMemcpyHostToDevice));
         MLB_CUDA(cudaMemsetAsync(h->ilu_t, 0, vb, st));
         const size_t nel = ih.lell_c.size(), neu = ih.uell_c.size();
         h->ilu_nel = (int64_t)nel;
@@ -705,20 +697,22 @@ int create_impl(mlb_handle *h, const mlb_matrix *A, const mlb_matrix *AH, const 
             if ((rc = up(&h->ilu_llev, ih.llev)) || (rc = up(&h->ilu_ulev, ih.ulev)) ||
                 (rc = up(&h->ilu_lmeta, ih.lmeta)) || (rc = up(&h->ilu_umeta, ih.umeta)))
                 return rc;
-        } else if (!cplx) {
-            if ((rc = up(&h->ilu_lwatch, ih.lwatch)) || (rc = up(&h->ilu_uwatch, ih.uwatch)) ||
-                (rc = dev_alloc(h, &h->ilu_flow, (size_t)N * 2 * sizeof(Slot))))
+        } else {
+            if ((rc = up(&h->ilu_lrows, ih.lrows)) || (rc = up(&h->ilu_lptr, ih.lptr)) ||
+                (rc = up(&h->ilu_urows, ih.urows)) || (rc = up(&h->ilu_uptr, ih.uptr)) ||
+                (rc = up(&h->ilu_lcnt, ih.lcnt)) || (rc = up(&h->ilu_ucnt, ih.ucnt)))
+                return rc;
+            // a slot per row of each triangle, of the values it runs in
+            const size_t slot = refined ? sizeof(ValueSlot<4>::type) : sizeof(ValueSlot<8>::type);
+            if (!cplx && ((rc = up(&h->ilu_lwatch, ih.lwatch)) || (rc = up(&h->ilu_uwatch, ih.uwatch)) ||
+                          (rc = dev_alloc(h, &h->ilu_flow, (size_t)N * 2 * slot))))
                 return rc;
         }
-        if ((rc = dev_alloc_t(h, &h->ilu_lcnt, (size_t)N * 4))) return rc;
-        if ((rc = dev_alloc_t(h, &h->ilu_ucnt, (size_t)N * 4))) return rc;
         if ((rc = dev_alloc_t(h, &h->ilu_lell_c, nel * 4))) return rc;
         if ((rc = dev_alloc_t(h, &h->ilu_uell_c, neu * 4))) return rc;
         if ((rc = dev_alloc(h, &h->ilu_lell_a, nel * es))) return rc;
         if ((rc = dev_alloc(h, &h->ilu_uell_a, neu * es))) return rc;
         if ((rc = dev_alloc(h, &h->ilu_udiag, ndiag * es))) return rc;
-        MLB_CUDA(cudaMemcpy(h->ilu_lcnt, ih.lcnt.data(), (size_t)N * 4, cudaMemcpyHostToDevice));
-        MLB_CUDA(cudaMemcpy(h->ilu_ucnt, ih.ucnt.data(), (size_t)N * 4, cudaMemcpyHostToDevice));
         MLB_CUDA(cudaMemcpy(h->ilu_lell_c, ih.lell_c.data(), nel * 4, cudaMemcpyHostToDevice));
         MLB_CUDA(cudaMemcpy(h->ilu_uell_c, ih.uell_c.data(), neu * 4, cudaMemcpyHostToDevice));
         MLB_CUDA(cudaMemcpy(h->ilu_lell_a, ih.lell_a.data(), nel * es, cudaMemcpyHostToDevice));

@@ -1,6 +1,6 @@
 // Device building blocks of the ML(n)BiCGStab library (sm_103a):
-// scalar types, 16-byte vector packs, deterministic block/grid reductions
-// and a bounded grid barrier.
+// scalar types, 16-byte vector packs, a bounded grid barrier and the exchange
+// of values between CTAs by tagged slots.
 #pragma once
 
 #include <cstdint>
@@ -138,46 +138,6 @@ __device__ __forceinline__ Pack<T> ldp_ro(const T *base, int64_t c) {
 template <typename T>
 __device__ __forceinline__ void stp(T *base, int64_t c, const Pack<T> &p) {
     reinterpret_cast<uint4 *>(base)[c] = *reinterpret_cast<const uint4 *>(&p);
-}
-
-// ---------------------------------------------------------------------------
-// deterministic reductions
-// ---------------------------------------------------------------------------
-template <int K>
-__device__ __forceinline__ void warp_sum(double (&v)[K]) {
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-}
-
-// Sum K values over the CTA; every thread receives the totals.  `red` is
-// shared scratch of at least 33*K doubles.  Fixed order: deterministic.
-template <int K>
-__device__ __forceinline__ void block_sum_all(double (&v)[K], double *red) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nw = (blockDim.x + 31) >> 5;
-    warp_sum<K>(v);
-    __syncthreads();  // red may still be read by a previous call
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) red[k * 32 + warp] = v[k];
-    }
-    __syncthreads();
-    if (warp == 0) {
-        double t[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) t[k] = lane < nw ? red[k * 32 + lane] : 0.0;
-        warp_sum<K>(t);
-        if (lane == 0) {
-#pragma unroll
-            for (int k = 0; k < K; ++k) red[32 * K + k] = t[k];
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = red[32 * K + k];
 }
 
 // ---------------------------------------------------------------------------

@@ -74,7 +74,7 @@ struct BatchPlan {
     unsigned *queue;         // [0]: next of order_small, [1]: next of order_big (zeroed)
     BarrierState *tbar;      // per team: barrier of the team's turns (zeroed)
     int *team_item;          // per team: 2 slots, the turn's position in order_big
-    BarrierState *sbar;      // per position of order_big: the solve's failure word (zeroed)
+    BarrierState *sbar;      // per position of order_big: the solve's barrier and failure word (zeroed)
     Slot *sslots;            // per position of order_big: 2 * kMaxSums * team slots (zeroed)
     uint64_t timeout_ns;     // limit of the waits between turns
 };
