@@ -1248,13 +1248,18 @@ struct Engine {
         }
     }
 
+    __device__ __noinline__ bool ilu_flow_ool(const T *v, T *out) { return ilu_flow(v, out); }
     __device__ __noinline__ bool ilu_wide_ool(const T *v, T *out) { return ilu_wide(v, out); }
     __device__ __noinline__ bool ilu_levels_ool(const T *v, T *out) { return ilu_levels(v, out); }
-    // out = M^{-1} v.  FP32 with both forms (a refined batch that mixes them):
-    // each a function of its own, since side by side in the loop they crowd it
-    // out of the registers (192 systems: 40.0 -> 38.2 ms; FP64 39.8 -> 40.7 ms).
+    // out = M^{-1} v.  In FP32 a function of its own where the loop of the
+    // refined kernels, which holds more than the FP64 one, crowds its polls
+    // or both forms out of the registers: by slots with scalar storage (24
+    // iterations, ms: 48^3 16.9 -> 13.0, 96^3 n = 8 40.4 -> 34.3, 27-point 40^3
+    // 90.5 -> 55.8; 3x3 blocks 44.9 -> 46.2, FP64 no change: inlined), and a
+    // batch that mixes the forms (192 systems 40.0 -> 38.2; FP64 39.8 -> 40.7).
     __device__ __forceinline__ bool ilu_solve_body(const T *v, T *out) {
         if constexpr (PC == kIluWide) return ilu_wide(v, out);
+        else if constexpr (PC == kIluFlow && is_narrow<T>::value && EW == 1) return ilu_flow_ool(v, out);
         else if constexpr (PC == kIluFlow) return ilu_flow(v, out);
         else if constexpr (PC == kIluLevels) return ilu_levels(v, out);
         else if constexpr (is_narrow<T>::value)
