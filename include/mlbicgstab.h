@@ -231,8 +231,7 @@ typedef struct {
     int64_t device_bytes; /* device memory held by the handle */
     int32_t n_active;     /* shadow vectors the next solve uses (<= n) */
     int32_t ilu_levels;   /* levels of the forward triangular solve of an
-                             ILU(0) handle (one grid barrier each); 0
-                             otherwise */
+                             ILU(0) handle; 0 otherwise */
     double qd_kernel_ms;  /* device time of the last mlbicgstab_spmv_qdot
                              (CUDA events around its launch on the handle's
                              stream); 0 before the first call */

@@ -203,17 +203,18 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *b, unsigned phase, uint
 constexpr uint64_t kOwnNs = 2000000000ull;
 // Bounded wait of the producer's lane 0: 0 when the phase completed, 1 when
 // the consumers called it off, 2 on a timeout.  Twice the consumers'
-// limit, so that a wait of theirs that gives up is reported as such, and none
-// in a pass of a product (limited = false): M^{-1} comes before it and may
-// take thousands of levels, rows too wide for a tile any time.  The consumers'
+// limit, so that a wait of theirs that gives up is reported as such.  In a
+// pass of a product (limited = false) an hour: M^{-1} comes before it and may
+// take millions of levels, rows too wide for a tile any time.  The consumers'
 // own waits there have limits, and they call the producer off when one ends.
+constexpr uint64_t kProductNs = 3600000000000ull;
 __device__ __forceinline__ int producer_wait(TileRing *R, uint64_t *b, unsigned phase, bool limited) {
     if (mbar_probe(b, phase)) return 0;
-    uint64_t t0 = globaltimer_ns();
+    const uint64_t t0 = globaltimer_ns();
     for (unsigned it = 1;; ++it) {
         if (mbar_probe(b, phase)) return 0;
         if (*(volatile int *)&R->stop) return mbar_probe(b, phase) ? 0 : 1;
-        if (limited && (it & 63u) == 0 && globaltimer_ns() - t0 > 2 * R->timeout_ns) return 2;
+        if ((it & 63u) == 0 && globaltimer_ns() - t0 > (limited ? 2 * R->timeout_ns : kProductNs)) return 2;
     }
 }
 
